@@ -5,9 +5,12 @@ Two layers, both marshalling only:
     as in include/dsq.h;
   * functions of the same names taking torch CUDA tensors: they check dtypes,
     allocate the output tensors with torch, pass data pointers and the current
-    CUDA stream, and raise DsqError on a non-zero status.
+    CUDA stream, and raise DsqError on a non-zero status.  Those on the path of
+    a pass (quantise, convolutions, pool, GEMMs, soft quantiser) do that in
+    native code (_dsq_host.so, csrc/dsq_host.cpp).
 """
 import ctypes as C
+import importlib.util
 import os
 
 import torch
@@ -21,6 +24,20 @@ if not os.path.exists(_LIB_PATH):
         "`python -m paper_1908_05033_b200.build` (needs nvcc; there is no "
         "fallback path)")
 lib = C.CDLL(_LIB_PATH)
+
+
+def _load_host():
+    path = os.path.join(_HERE, "_dsq_host.so")
+    if not os.path.exists(path):
+        raise ImportError(f"{path} is missing: build it with "
+                          "`python -m paper_1908_05033_b200.build`")
+    spec = importlib.util.spec_from_file_location("_dsq_host", path)
+    mod = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(mod)
+    return mod
+
+
+_host = _load_host()
 
 
 class dsq_quant_t(C.Structure):
@@ -111,6 +128,9 @@ class DsqError(RuntimeError):
         self.status = status
         msg = lib.dsq_status_string(status).decode()
         super().__init__(f"{where}: {msg} (status {status})")
+
+
+_host.set_error_class(DsqError)
 
 
 def _check(status, where):
@@ -211,16 +231,7 @@ def dsq_unpack(packed, rows, k, bits, signed):
 # ---- quantise -----------------------------------------------------------------
 def dsq_quantize_act(x, bits, lo, hi, out=None):
     """fp32 NHWC [N,H,W,C] -> packed codes uint8 [N,H,W,pitch]."""
-    _need(x, torch.float32, "x")
-    N, H, W, Cc = x.shape
-    pitch = dsq_row_pitch(Cc, bits)
-    if out is None:
-        out = torch.empty((N, H, W, pitch), dtype=torch.uint8, device=x.device)
-    shape = dsq_nhwc_t(N, H, W, Cc)
-    q = dsq_quant_t(bits, lo, hi)
-    _check(lib.dsq_quantize_act(_p(x), C.byref(shape), C.byref(q), _p(out),
-                                out.numel(), _stream()), "dsq_quantize_act")
-    return out
+    return _host.quantize_act(x, bits, lo, hi, out)
 
 
 def dsq_pack_weights(w, bits, lo, hi, ws, depthwise=False, stride=1, pad=0):
@@ -253,108 +264,35 @@ def dsq_pack_weights(w, bits, lo, hi, ws, depthwise=False, stride=1, pad=0):
 
 
 # ---- convolution ----------------------------------------------------------------
-def _epilogue(scale, bias, w_offset, residual, residual_q, requant):
-    ep = dsq_epilogue_t()
-    ep.scale = scale.data_ptr()
-    ep.bias = bias.data_ptr()
-    ep.w_offset = w_offset
-    ep.residual_codes = residual.data_ptr() if residual is not None else None
-    if residual_q is not None:
-        ep.residual_q = dsq_quant_t(*residual_q)
-    if requant is not None:
-        ep.requant = dsq_quant_t(*requant)
-    return ep
-
-
-def _conv_common(fn_name, act, shape, act_q, blob, conv, scale, bias, w_offset,
-                 residual, residual_q, requant, want_f32, want_acc, ws,
-                 out_codes):
-    _need(act, torch.uint8, "act")
-    _need(blob, torch.uint8, "weights")
-    _need(scale, torch.float32, "scale")
-    _need(bias, torch.float32, "bias")
-    N, H, W, Cc = shape
-    bits = act_q[0]
-    Ho = (H + 2 * conv.pad - conv.KH) // conv.stride + 1
-    Wo = (W + 2 * conv.pad - conv.KW) // conv.stride + 1
-    dev = act.device
-    y = torch.empty((N, Ho, Wo, conv.Cout), dtype=torch.float32,
-                    device=dev) if want_f32 else None
-    acc = torch.empty((N, Ho, Wo, conv.Cout), dtype=torch.int32,
-                      device=dev) if want_acc else None
-    codes = None
-    if requant is not None:
-        codes = out_codes if out_codes is not None else torch.empty(
-            (N, Ho, Wo, dsq_row_pitch(conv.Cout, bits)), dtype=torch.uint8,
-            device=dev)
-    ep = _epilogue(scale, bias, w_offset, residual, residual_q, requant)
-    nhwc = dsq_nhwc_t(N, H, W, Cc)
-    aq = dsq_quant_t(*act_q)
-    if fn_name == "dsq_conv2d":
-        st = lib.dsq_conv2d(_p(act), C.byref(nhwc), C.byref(aq), _p(blob),
-                            C.byref(conv), C.byref(ep), _p(y), _p(codes),
-                            _p(acc), _p(ws), ws.numel(), _stream())
-    else:
-        st = lib.dsq_dwconv2d(_p(act), C.byref(nhwc), C.byref(aq), _p(blob),
-                              C.byref(conv), C.byref(ep), _p(y), _p(codes),
-                              _p(acc), _stream())
-    _check(st, fn_name)
-    return codes, y, acc
-
-
 def dsq_conv2d(act, shape, act_q, blob, conv, scale, bias, ws, w_offset=0.0,
                residual=None, residual_q=None, requant=None, want_f32=False,
                want_acc=False, out_codes=None):
     """act: packed codes of NHWC `shape`; act_q / residual_q / requant are
     (bits, lo, hi) tuples.  Returns (codes | None, y_f32 | None, acc | None)."""
-    return _conv_common("dsq_conv2d", act, shape, act_q, blob, conv, scale,
-                        bias, w_offset, residual, residual_q, requant,
-                        want_f32, want_acc, ws, out_codes)
+    return _host.conv2d(False, act, shape, act_q, blob, conv, scale, bias, w_offset, residual,
+                        residual_q, requant, want_f32, want_acc, ws, out_codes)
 
 
 def dsq_dwconv2d(act, shape, act_q, blob, conv, scale, bias, w_offset=0.0,
                  residual=None, residual_q=None, requant=None, want_f32=False,
                  want_acc=False, out_codes=None):
-    return _conv_common("dsq_dwconv2d", act, shape, act_q, blob, conv, scale,
-                        bias, w_offset, residual, residual_q, requant,
-                        want_f32, want_acc, None, out_codes)
+    return _host.conv2d(True, act, shape, act_q, blob, conv, scale, bias, w_offset, residual,
+                        residual_q, requant, want_f32, want_acc, None, out_codes)
 
 
 def dsq_maxpool2x2(codes, shape, bits, out=None):
-    _need(codes, torch.uint8, "codes")
-    N, H, W, Cc = shape
-    pitch = dsq_row_pitch(Cc, bits)
-    if out is None:
-        out = torch.empty((N, H // 2, W // 2, pitch), dtype=torch.uint8,
-                          device=codes.device)
-    nhwc = dsq_nhwc_t(N, H, W, Cc)
-    _check(lib.dsq_maxpool2x2(_p(codes), C.byref(nhwc), bits, _p(out),
-                              out.numel(), _stream()), "dsq_maxpool2x2")
-    return out
+    return _host.maxpool2x2(codes, shape, bits, out)
 
 
 # ---- training side: soft quantiser -----------------------------------------------
 def dsq_soft_quantize_fwd(x, bits, lo, hi, alpha, out=None):
     """y = Q_S(x) (Eq. 5), fp32 CUDA tensor of any shape."""
-    _need(x, torch.float32, "x")
-    y = out if out is not None else torch.empty_like(x)
-    q = dsq_quant_t(bits, lo, hi)
-    _check(lib.dsq_soft_quantize_fwd(_p(x), x.numel(), C.byref(q), alpha, _p(y), _stream()),
-           "dsq_soft_quantize_fwd")
-    return y
+    return _host.soft_fwd(x, bits, lo, hi, alpha, out)
 
 
 def dsq_soft_quantize_bwd(x, grad_y, bits, lo, hi, alpha, out=None, grad_params=None):
     """Returns (grad_x fp32 like x, grad_params fp64 [3] = dL/d(alpha, l, u))."""
-    _need(x, torch.float32, "x")
-    _need(grad_y, torch.float32, "grad_y")
-    gx = out if out is not None else torch.empty_like(x)
-    gp = grad_params if grad_params is not None else torch.empty(
-        3, dtype=torch.float64, device=x.device)
-    q = dsq_quant_t(bits, lo, hi)
-    _check(lib.dsq_soft_quantize_bwd(_p(x), _p(grad_y), x.numel(), C.byref(q), alpha, _p(gx),
-                                     _p(gp), _stream()), "dsq_soft_quantize_bwd")
-    return gx, gp
+    return _host.soft_bwd(x, grad_y, bits, lo, hi, alpha, out, grad_params)
 
 
 # ---- GEMM -------------------------------------------------------------------------
@@ -362,17 +300,7 @@ def dsq_gemm(A, B, M, N, K, bits, ws, row_scale=None, want_i32=True,
              out_i32=None, out_f32=None):
     """A: packed signed codes [M, pitch], B: packed unsigned codes [N, pitch].
     Returns (C int32 [M,N] | None, D fp32 [M,N] | None)."""
-    _need(A, torch.uint8, "A")
-    _need(B, torch.uint8, "B")
-    Cm = out_i32
-    if Cm is None and want_i32:
-        Cm = torch.empty((M, N), dtype=torch.int32, device=A.device)
-    D = out_f32
-    if D is None and row_scale is not None:
-        D = torch.empty((M, N), dtype=torch.float32, device=A.device)
-    _check(lib.dsq_gemm(_p(A), _p(B), M, N, K, bits, _p(Cm), _p(row_scale),
-                        _p(D), _p(ws), ws.numel(), _stream()), "dsq_gemm")
-    return Cm, D
+    return _host.gemm(False, A, B, M, N, K, bits, ws, row_scale, want_i32, out_i32, out_f32)
 
 
 def _sized_workspace(nbytes, device):
@@ -384,31 +312,21 @@ def _sized_workspace(nbytes, device):
 def dsq_binary_gemm(A, B, M, N, K, ws=None, row_scale=None, want_i32=True):
     """A, B: packed 1-bit rows [M, pitch], [N, pitch] (bit 1 = +1, 0 = -1).
     Returns (C int32 [M,N] | None, D fp32 [M,N] | None)."""
-    _need(A, torch.uint8, "A")
-    _need(B, torch.uint8, "B")
     if ws is None:
+        _need(A, torch.uint8, "A")
         ws = _sized_workspace(int(lib.dsq_binary_gemm_workspace_bytes(M, N, K)), A.device)
-    Cm = torch.empty((M, N), dtype=torch.int32, device=A.device) if want_i32 else None
-    D = torch.empty((M, N), dtype=torch.float32, device=A.device) if row_scale is not None else None
-    _check(lib.dsq_binary_gemm(_p(A), _p(B), M, N, K, _p(Cm), _p(row_scale), _p(D), _p(ws),
-                               ws.numel(), _stream()), "dsq_binary_gemm")
+    out = _host.gemm(True, A, B, M, N, K, 1, ws, row_scale, want_i32, None, None)
     check_workspace(ws, "dsq_binary_gemm")
-    return Cm, D
+    return out
 
 
 def dsq_wgemm_bf16(X, W, M, N, K, bits, col_scale, col_bias=None, w_offset=0.5, ws=None,
                    out=None):
     """X: bf16 [M, K]; W: packed signed codes [N, pitch].  Returns Y fp32 [M, N]."""
-    _need(X, torch.bfloat16, "X")
-    _need(W, torch.uint8, "W")
-    _need(col_scale, torch.float32, "col_scale")
     if ws is None:
+        _need(X, torch.bfloat16, "X")
         ws = _sized_workspace(int(lib.dsq_wgemm_workspace_bytes(N, K)), X.device)
-    Y = out if out is not None else torch.empty((M, N), dtype=torch.float32, device=X.device)
-    _check(lib.dsq_wgemm_bf16(_p(X), _p(W), M, N, K, bits, w_offset, _p(col_scale),
-                              _p(col_bias), _p(Y), _p(ws), ws.numel(), _stream()),
-           "dsq_wgemm_bf16")
-    return Y
+    return _host.wgemm(X, W, M, N, K, bits, w_offset, col_scale, col_bias, ws, out)
 
 
 def dsq_set_round_k_steps(ks):

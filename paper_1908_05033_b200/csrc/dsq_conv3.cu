@@ -1066,25 +1066,8 @@ int w3_launch(const CUtensorMap &tb, const CUtensorMap &ta, const W3Params &p, c
         configured.fetch_or(dev_bit, std::memory_order_release);
     }
     const int grid = p.mstep * p.n_tiles;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(W3_THREADS);
-    cfg.dynamicSmemBytes = (size_t)p.smem_bytes;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    int na = 0;
-    if (pdl) {
-        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[na].val.programmaticStreamSerializationAllowed = 1;
-        ++na;
-    }
-    cfg.attrs = attr;
-    cfg.numAttrs = na;
-    if (cudaLaunchKernelEx(&cfg, dsq_win3_kernel<BITS, EPI, TR>, tb, ta, p) != cudaSuccess) {
-        cudaGetLastError();
-        return DSQ_ERR_CUDA;
-    }
-    return dsq_launch_status();
+    return dsq_launch(dsq_win3_kernel<BITS, EPI, TR>, dim3(grid), dim3(W3_THREADS),
+                      (size_t)p.smem_bytes, s, pdl, 0, tb, ta, p);
 }
 
 template <int BITS>
@@ -1173,10 +1156,10 @@ int dsq_w8_build(void *blob, const dsq_conv_t *conv, int bits, cudaStream_t stre
     const uint8_t *packed = (const uint8_t *)blob;
     uint8_t *out = (uint8_t *)blob + w.offset;
     if (bits == 4)
-        w8_build_kernel<4><<<blocks, 256, 0, stream>>>(packed, out, conv->Cout, 9 * P, w.ksteps, kpp, xstep);
-    else
-        w8_build_kernel<2><<<blocks, 256, 0, stream>>>(packed, out, conv->Cout, 9 * P, w.ksteps, kpp, xstep);
-    return cudaGetLastError() == cudaSuccess ? DSQ_OK : DSQ_ERR_CUDA;
+        return dsq_launch(w8_build_kernel<4>, dim3(blocks), dim3(256), 0, stream, 0, 0, packed, out,
+                          conv->Cout, 9 * P, w.ksteps, kpp, xstep);
+    return dsq_launch(w8_build_kernel<2>, dim3(blocks), dim3(256), 0, stream, 0, 0, packed, out,
+                      conv->Cout, 9 * P, w.ksteps, kpp, xstep);
 }
 
 int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,

@@ -6,6 +6,7 @@
 // epilogue.  Inputs and outputs move as packed codes only: bits/8 bytes per
 // element each way.
 #include "dsq_epilogue.cuh"
+#include "dsq_launch.h"
 
 namespace {
 
@@ -388,15 +389,10 @@ extern "C" int dsq_dwconv2d(const void *act_codes, const dsq_nhwc_t *shape,
             if (blocks > (int64_t)sms * 8) blocks = (int64_t)sms * 8;
             blocks = (blocks + units - 1) / units * units;     // blocks * 256 is a multiple of units
             const uint8_t *a8 = (const uint8_t *)act_codes, *w8 = (const uint8_t *)w_packed;
-            if (conv->stride == 1)
-                dwconv3x3_b4_kernel<1><<<(int)blocks, 256, 0, s>>>(a8, w8, shape->N, shape->H, shape->W,
-                                                                  shape->C, Ho, Wo, pitch, e.scale,
-                                                                  e.bias, e.y_codes, f);
-            else
-                dwconv3x3_b4_kernel<2><<<(int)blocks, 256, 0, s>>>(a8, w8, shape->N, shape->H, shape->W,
-                                                                  shape->C, Ho, Wo, pitch, e.scale,
-                                                                  e.bias, e.y_codes, f);
-            return dsq_launch_status();
+            return dsq_launch(conv->stride == 1 ? dwconv3x3_b4_kernel<1> : dwconv3x3_b4_kernel<2>,
+                              dim3((unsigned)blocks), dim3(256), 0, s, 0, 0, a8, w8, shape->N,
+                              shape->H, shape->W, shape->C, Ho, Wo, pitch, e.scale, e.bias,
+                              e.y_codes, f);
         }
     }
     const int64_t total = (int64_t)shape->N * Ho * ((Wo + 3) / 4) *
@@ -405,15 +401,10 @@ extern "C" int dsq_dwconv2d(const void *act_codes, const dsq_nhwc_t *shape,
     if (g > 148 * 32) g = 148 * 32;
     if (g < 1) g = 1;
     const uint8_t *a = (const uint8_t *)act_codes, *w = (const uint8_t *)w_packed;
-#define DSQ_DW_LAUNCH(B, S)                                                               \
-    dwconv3x3_kernel<B, S><<<(int)g, 256, 0, s>>>(a, w, shape->N, shape->H, shape->W, shape->C, \
-                                                  Ho, Wo, pitch, e)
-    if (bits == 4 && conv->stride == 1) DSQ_DW_LAUNCH(4, 1);
-    else if (bits == 4) DSQ_DW_LAUNCH(4, 2);
-    else if (bits == 3 && conv->stride == 1) DSQ_DW_LAUNCH(3, 1);
-    else if (bits == 3) DSQ_DW_LAUNCH(3, 2);
-    else if (conv->stride == 1) DSQ_DW_LAUNCH(2, 1);
-    else DSQ_DW_LAUNCH(2, 2);
-#undef DSQ_DW_LAUNCH
-    return dsq_launch_status();
+    const auto kernel = bits == 4 ? (conv->stride == 1 ? dwconv3x3_kernel<4, 1> : dwconv3x3_kernel<4, 2>)
+                        : bits == 3
+                            ? (conv->stride == 1 ? dwconv3x3_kernel<3, 1> : dwconv3x3_kernel<3, 2>)
+                            : (conv->stride == 1 ? dwconv3x3_kernel<2, 1> : dwconv3x3_kernel<2, 2>);
+    return dsq_launch(kernel, dim3((unsigned)g), dim3(256), 0, s, 0, 0, a, w, shape->N, shape->H,
+                      shape->W, shape->C, Ho, Wo, pitch, e);
 }

@@ -383,18 +383,12 @@ int dsq_quantize_act(const float *x, const dsq_nhwc_t *shape,
         // many more CTAs than SMs: at 8-16 loads per thread the memory system
         // needs the extra resident warps to stay full
         const int grid = grid_for((n_lines + 31) / 32 * 32, 256, 148 * 64);
-        if (bits == 4)
-            quantize_flat_kernel<4><<<grid, 256, 0, s>>>(
-                (const float4 *)x, (uint4 *)codes_out, n_lines, dq);
-        else
-            quantize_flat_kernel<2><<<grid, 256, 0, s>>>(
-                (const float4 *)x, (uint4 *)codes_out, n_lines, dq);
-    } else {
-        const int pw = (int)(pitch / 4);
-        quantize_rows_kernel<<<grid_for(rows * pw, 256), 256, 0, s>>>(
-            x, (uint32_t *)codes_out, rows, k, pw, bits, dq);
+        return dsq_launch(bits == 4 ? quantize_flat_kernel<4> : quantize_flat_kernel<2>, dim3(grid),
+                          dim3(256), 0, s, 0, 0, (const float4 *)x, (uint4 *)codes_out, n_lines, dq);
     }
-    return dsq_launch_status();
+    const int pw = (int)(pitch / 4);
+    return dsq_launch(quantize_rows_kernel, dim3(grid_for(rows * pw, 256)), dim3(256), 0, s, 0, 0, x,
+                      (uint32_t *)codes_out, rows, k, pw, bits, dq);
 }
 
 int dsq_pack_weights(const float *w, const dsq_conv_t *c, int bits,
@@ -418,11 +412,9 @@ int dsq_pack_weights(const float *w, const dsq_conv_t *c, int bits,
     const int rows = dense ? c->Cout * taps : taps;
     const int k = dense ? c->Cin : c->Cout;
     const int pw = (int)(dsq_row_pitch(k, bits) / 4);
-    pack_weights_kernel<<<grid_for((int64_t)rows * pw, 256), 256, 0,
-                          (cudaStream_t)stream>>>(
-        w, (uint32_t *)packed_out, rows, k, pw, bits, taps, dw ? 1 : 0, lo, hi,
-        per_channel ? 1 : 0, (int *)workspace);
-    int st = dsq_launch_status();
+    int st = dsq_launch(pack_weights_kernel, dim3(grid_for((int64_t)rows * pw, 256)), dim3(256), 0,
+                        (cudaStream_t)stream, 0, 0, w, (uint32_t *)packed_out, rows, k, pw, bits,
+                        taps, dw ? 1 : 0, lo, hi, per_channel ? 1 : 0, (int *)workspace);
     if (st == DSQ_OK && dense) st = dsq_w8_build(packed_out, c, bits, (cudaStream_t)stream);
     return st;
 }
@@ -437,9 +429,9 @@ int dsq_pack_codes(const int8_t *codes, int64_t rows, int64_t k, int bits,
     const size_t pitch = dsq_row_pitch(k, bits);
     if (bytes < (size_t)rows * pitch) return DSQ_ERR_SIZE;
     const int pw = (int)(pitch / 4);
-    pack_codes_kernel<<<grid_for(rows * pw, 256), 256, 0, (cudaStream_t)stream>>>(
-        codes, (uint32_t *)packed_out, rows, (int)k, pw, bits);
-    return dsq_launch_status();
+    return dsq_launch(pack_codes_kernel, dim3(grid_for(rows * pw, 256)), dim3(256), 0,
+                      (cudaStream_t)stream, 0, 0, codes, (uint32_t *)packed_out, rows, (int)k, pw,
+                      bits);
 }
 
 int dsq_unpack(const void *packed, int64_t rows, int64_t k, int bits,
@@ -450,10 +442,9 @@ int dsq_unpack(const void *packed, int64_t rows, int64_t k, int bits,
     if (rows <= 0 || k <= 0 || k > (1 << 28)) return DSQ_ERR_SHAPE;
     if (!dsq_aligned16(packed)) return DSQ_ERR_ALIGN;
     const int pw = (int)(dsq_row_pitch(k, bits) / 4);
-    unpack_kernel<<<grid_for(rows * k, 256), 256, 0, (cudaStream_t)stream>>>(
-        (const uint32_t *)packed, codes_out, rows, (int)k, pw, bits,
-        is_signed ? 1 : 0);
-    return dsq_launch_status();
+    return dsq_launch(unpack_kernel, dim3(grid_for(rows * k, 256)), dim3(256), 0,
+                      (cudaStream_t)stream, 0, 0, (const uint32_t *)packed, codes_out, rows, (int)k,
+                      pw, bits, is_signed ? 1 : 0);
 }
 
 int dsq_maxpool2x2(const void *codes_in, const dsq_nhwc_t *shape, int bits,
@@ -469,10 +460,9 @@ int dsq_maxpool2x2(const void *codes_in, const dsq_nhwc_t *shape, int bits,
     const int64_t out_rows = (int64_t)shape->N * (shape->H / 2) * (shape->W / 2);
     if (bytes < (size_t)out_rows * pitch) return DSQ_ERR_SIZE;
     const int pw = (int)(pitch / 4);
-    maxpool_kernel<<<grid_for(out_rows * pw, 256), 256, 0, (cudaStream_t)stream>>>(
-        (const uint32_t *)codes_in, (uint32_t *)codes_out, shape->N, shape->H,
-        shape->W, shape->C, pw, bits);
-    return dsq_launch_status();
+    return dsq_launch(maxpool_kernel, dim3(grid_for(out_rows * pw, 256)), dim3(256), 0,
+                      (cudaStream_t)stream, 0, 0, (const uint32_t *)codes_in, (uint32_t *)codes_out,
+                      shape->N, shape->H, shape->W, shape->C, pw, bits);
 }
 
 const char *dsq_status_string(int status)

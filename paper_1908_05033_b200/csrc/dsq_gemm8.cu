@@ -491,27 +491,11 @@ int launch_pass2(const void *A, size_t a_pitch, const void *B, size_t b_pitch, s
     }
     const int sms = dsq_sm_count() > 0 ? dsq_sm_count() : 148;
     const int pairs = std::min(sms / 2, p.m_tiles * p.n_tiles);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * pairs);
-    cfg.blockDim = dim3(G8_THREADS);
-    cfg.dynamicSmemBytes = G8_SMEM;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    int na = 0;
-    if (dsq_launch_hooks().pdl) {
-        // set-up overlaps the tail of pass 1; the kernel waits for it itself
-        // (griddepcontrol.wait) before the first copy
-        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[na].val.programmaticStreamSerializationAllowed = 1;
-        ++na;
-    }
-    cfg.attrs = attr;
-    cfg.numAttrs = na;
-    if (cudaLaunchKernelEx(&cfg, gemm8_kernel<F16>, ta, tb, p) != cudaSuccess) {
-        cudaGetLastError();
-        return DSQ_ERR_CUDA;
-    }
-    return DSQ_OK;
+    // (dependent launch: set-up overlaps the tail of pass 1; the kernel waits for
+    // it itself before the first copy.  The cluster of two is the kernel's own
+    // attribute.)
+    return dsq_launch(gemm8_kernel<F16>, dim3(2 * pairs), dim3(G8_THREADS), (size_t)G8_SMEM, stream,
+                      dsq_launch_hooks().pdl, 0, ta, tb, p);
 }
 
 // first 1024-byte boundary behind the status words of a caller workspace
@@ -550,12 +534,12 @@ int dsq_gemm8_launch(const void *A_codes, const void *B_codes, int64_t M, int64_
     // whole waves of resident blocks (8 per SM), a few items per thread
     const unsigned blocks = (unsigned)std::min<int64_t>((threads + 255) / 256, (int64_t)sms * 8);
     const uint8_t *A = (const uint8_t *)A_codes, *B = (const uint8_t *)B_codes;
-    switch (bits) {
-    case 2: expand_rows_kernel<2><<<blocks, 256, 0, stream>>>(A, B, M, N, pitch_in, (int)kp, A8, B8); break;
-    case 3: expand_rows_kernel<3><<<blocks, 256, 0, stream>>>(A, B, M, N, pitch_in, (int)kp, A8, B8); break;
-    default: expand_rows_kernel<4><<<blocks, 256, 0, stream>>>(A, B, M, N, pitch_in, (int)kp, A8, B8); break;
-    }
-    if (cudaGetLastError() != cudaSuccess) return DSQ_ERR_CUDA;
+    const int st = dsq_launch(bits == 2   ? expand_rows_kernel<2>
+                              : bits == 3 ? expand_rows_kernel<3>
+                                          : expand_rows_kernel<4>,
+                              dim3(blocks), dim3(256), 0, stream, 0, 0, A, B, M, N, pitch_in,
+                              (int)kp, A8, B8);
+    if (st) return st;
     G8Params p = {};
     p.idesc = idesc_i8(G8_BN, true, false, G8_BM);
     p.C_i32 = C_i32; p.row_scale = row_scale; p.D_f32 = D_f32;
@@ -591,10 +575,11 @@ int dsq_binary_gemm(const void *A_bits, const void *B_bits, int64_t M, int64_t N
     if (ws_bytes < (size_t)(scratch - (uint8_t *)workspace) + need) return DSQ_ERR_SIZE;
     uint8_t *A8 = scratch, *B8 = scratch + round_up((size_t)M * kp, 1024);
     const int64_t threads = (M + N) * (int64_t)(kp / 16);
-    expand_binary_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, (cudaStream_t)stream>>>(
-        (const uint8_t *)A_bits, (const uint8_t *)B_bits, M, N, (int)K,
-        (int)dsq_row_pitch(K, 1), (int)kp, A8, B8);
-    if (cudaGetLastError() != cudaSuccess) return DSQ_ERR_CUDA;
+    const int st = dsq_launch(expand_binary_kernel, dim3((unsigned)((threads + 255) / 256)),
+                              dim3(256), 0, (cudaStream_t)stream, 0, 0, (const uint8_t *)A_bits,
+                              (const uint8_t *)B_bits, M, N, (int)K, (int)dsq_row_pitch(K, 1),
+                              (int)kp, A8, B8);
+    if (st) return st;
     G8Params p = {};
     p.idesc = idesc_i8(G8_BN, true, true, G8_BM);
     p.C_i32 = C_i32; p.row_scale = row_scale; p.D_f32 = D_f32;
@@ -634,13 +619,13 @@ int dsq_wgemm_bf16(const void *X_bf16, const void *W_codes, int64_t M, int64_t N
     const int odd = w_offset == 0.5f;
     const uint8_t *W = (const uint8_t *)W_codes;
     cudaStream_t s = (cudaStream_t)stream;
-    switch (bits) {
-    case 1: expand_w_bf16_kernel<1><<<blocks, 256, 0, s>>>(W, N, (int)K, pitch_in, (int)wp, odd, W16); break;
-    case 2: expand_w_bf16_kernel<2><<<blocks, 256, 0, s>>>(W, N, (int)K, pitch_in, (int)wp, odd, W16); break;
-    case 3: expand_w_bf16_kernel<3><<<blocks, 256, 0, s>>>(W, N, (int)K, pitch_in, (int)wp, odd, W16); break;
-    default: expand_w_bf16_kernel<4><<<blocks, 256, 0, s>>>(W, N, (int)K, pitch_in, (int)wp, odd, W16); break;
-    }
-    if (cudaGetLastError() != cudaSuccess) return DSQ_ERR_CUDA;
+    const int st = dsq_launch(bits == 1   ? expand_w_bf16_kernel<1>
+                              : bits == 2 ? expand_w_bf16_kernel<2>
+                              : bits == 3 ? expand_w_bf16_kernel<3>
+                                          : expand_w_bf16_kernel<4>,
+                              dim3(blocks), dim3(256), 0, s, 0, 0, W, N, (int)K, pitch_in, (int)wp,
+                              odd, W16);
+    if (st) return st;
     G8Params p = {};
     p.idesc = idesc_bf16(G8_BN, G8_BM);
     p.col_scale = col_scale; p.col_bias = col_bias; p.Y_f32 = Y_f32;

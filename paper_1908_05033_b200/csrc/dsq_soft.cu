@@ -3,6 +3,7 @@
 // kernels: 8 bytes per element forward (fp32 in, fp32 out), 12 bytes per
 // element backward (x and dL/dy in, dL/dx out) plus three scalar reductions.
 #include "dsq_common.cuh"
+#include "dsq_launch.h"
 
 namespace {
 
@@ -200,8 +201,8 @@ extern "C" int dsq_soft_quantize_fwd(const float *x, int64_t n, const dsq_quant_
     if (st) return st;
     if (n <= 0) return DSQ_ERR_SHAPE;
     if (!dsq_aligned16(x) || !dsq_aligned16(y)) return DSQ_ERR_ALIGN;
-    soft_fwd_kernel<<<soft_grid(n), 256, 0, (cudaStream_t)stream>>>(x, y, n, p);
-    return dsq_launch_status();
+    return dsq_launch(soft_fwd_kernel, dim3(soft_grid(n)), dim3(256), 0, (cudaStream_t)stream, 0, 0, x,
+                      y, n, p);
 }
 
 extern "C" int dsq_soft_quantize_bwd(const float *x, const float *grad_y, int64_t n,
@@ -218,6 +219,6 @@ extern "C" int dsq_soft_quantize_bwd(const float *x, const float *grad_y, int64_
         return DSQ_ERR_ALIGN;
     cudaStream_t s = (cudaStream_t)stream;
     DSQ_CUDA_TRY(cudaMemsetAsync(grad_params, 0, 3 * sizeof(double), s));
-    soft_bwd_kernel<<<soft_grid(n), 256, 0, s>>>(x, grad_y, grad_x, n, p, grad_params);
-    return dsq_launch_status();
+    return dsq_launch(soft_bwd_kernel, dim3(soft_grid(n)), dim3(256), 0, s, 0, 0, x, grad_y, grad_x, n,
+                      p, grad_params);
 }

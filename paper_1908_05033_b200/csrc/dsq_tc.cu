@@ -1447,6 +1447,7 @@ std::atomic<int> g_skip_b_round{-1};  // dsq_set_test_skip_b_round
 std::atomic<int> g_window3{1};        // dsq_set_conv3_window
 std::atomic<int> g_two_pass{1};       // dsq_set_gemm_two_pass
 std::atomic<int> g_w8{1};             // dsq_set_conv3_expanded_weights
+std::atomic<unsigned> g_generation{0}; // moves with every change of a hook
 
 int pick_bn(int m_tiles, int ncols, int bits)
 {
@@ -1504,34 +1505,9 @@ int launch_tc(const TcMaps &tmap, const TcParams &p, cudaStream_t s)
     q.skip_b_round = g_skip_b_round.load();
     // one cluster of two CTAs (the two SMs of a TPC) per tile in flight
     if (PAIR && grid > sms / 2) grid = sms / 2;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(PAIR ? 2 * grid : grid);
-    cfg.blockDim = dim3(NUM_THREADS);
-    cfg.dynamicSmemBytes = (size_t)smem_bytes;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[2];
-    int na = 0;
-    if (PAIR) {
-        attr[na].id = cudaLaunchAttributeClusterDimension;
-        attr[na].val.clusterDim.x = 2;
-        attr[na].val.clusterDim.y = 1;
-        attr[na].val.clusterDim.z = 1;
-        ++na;
-    }
-    if (g_pdl.load()) {
-        // the kernel waits for its predecessors itself (griddepcontrol.wait)
-        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[na].val.programmaticStreamSerializationAllowed = 1;
-        ++na;
-    }
-    cfg.attrs = attr;
-    cfg.numAttrs = na;
-    if (cudaLaunchKernelEx(&cfg, dsq_tc_kernel<BITS, A_SIGNED, EPI, PM, A_TMA>, tmap.b, tmap.a,
-                           q) != cudaSuccess) {
-        cudaGetLastError();
-        return DSQ_ERR_CUDA;
-    }
-    return dsq_launch_status();
+    return dsq_launch(dsq_tc_kernel<BITS, A_SIGNED, EPI, PM, A_TMA>, dim3(PAIR ? 2 * grid : grid),
+                      dim3(NUM_THREADS), (size_t)smem_bytes, s, g_pdl.load(), PAIR ? 2 : 0,
+                      tmap.b, tmap.a, q);
 }
 
 template <int BITS, int PM>
@@ -1628,6 +1604,8 @@ DsqLaunchHooks dsq_launch_hooks()
     return h;
 }
 
+unsigned dsq_hooks_generation() { return g_generation.load(); }
+
 static void *driver_entry_point(const char *name)
 {
     void *sym = nullptr;
@@ -1666,6 +1644,7 @@ int dsq_set_round_k_steps(int ks)
 {
     if (ks != 0 && ks != 1 && ks != 2) return DSQ_ERR_SHAPE;
     g_forced_ks = ks;
+    ++g_generation;
     return DSQ_OK;
 }
 
@@ -1673,6 +1652,7 @@ int dsq_set_cta_pairs(int mode)
 {
     if (mode < 0 || mode > 2) return DSQ_ERR_SHAPE;
     g_pair_mode = mode;
+    ++g_generation;
     return DSQ_OK;
 }
 
@@ -1680,12 +1660,14 @@ int dsq_set_dependent_launch(int on)
 {
     if (on != 0 && on != 1) return DSQ_ERR_SHAPE;
     g_pdl = on;
+    ++g_generation;
     return DSQ_OK;
 }
 
 int dsq_set_test_skip_b_round(int round)
 {
     g_skip_b_round = round < 0 ? -1 : round;
+    ++g_generation;
     return DSQ_OK;
 }
 
@@ -1693,6 +1675,7 @@ int dsq_set_conv3_window(int mode)
 {
     if (mode < 0 || mode > 4) return DSQ_ERR_SHAPE;
     g_window3 = mode;
+    ++g_generation;
     return DSQ_OK;
 }
 
@@ -1700,6 +1683,7 @@ int dsq_set_wait_limit_ns(long long ns)
 {
     if (ns < 0) return DSQ_ERR_SHAPE;
     g_wait_ns = ns == 0 ? WAIT_LIMIT_NS : (unsigned long long)ns;
+    ++g_generation;
     return DSQ_OK;
 }
 
@@ -1708,6 +1692,7 @@ int dsq_set_tile_n(int bn)
     if (bn != 0 && bn != 32 && bn != 64 && bn != 128 && bn != 192 && bn != 256)
         return DSQ_ERR_SHAPE;
     g_forced_bn = bn;
+    ++g_generation;
     return DSQ_OK;
 }
 
@@ -1740,6 +1725,7 @@ size_t dsq_gemm_workspace_bytes(int64_t M, int64_t N, int64_t K, int bits)
 int dsq_set_conv3_expanded_weights(int on)
 {
     g_w8 = on ? 1 : 0;
+    ++g_generation;
     return DSQ_OK;
 }
 
@@ -1747,6 +1733,7 @@ int dsq_set_gemm_two_pass(int on)
 {
     if (on < 0 || on > 2) return DSQ_ERR_SHAPE;
     g_two_pass = on;
+    ++g_generation;
     return DSQ_OK;
 }
 

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include "dsq_epilogue.cuh"
+#include "dsq_launch.h"
 
 #define DSQ_HIDDEN __attribute__((visibility("hidden")))
 
@@ -18,6 +19,8 @@ struct DsqLaunchHooks {
     int w8;                     // dsq_set_conv3_expanded_weights
 };
 DSQ_HIDDEN DsqLaunchHooks dsq_launch_hooks();
+// a number that changes whenever a hook is set
+DSQ_HIDDEN unsigned dsq_hooks_generation();
 
 typedef CUresult (*DsqEncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
                                      const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
