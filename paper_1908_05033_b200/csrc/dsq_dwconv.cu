@@ -5,8 +5,14 @@
 // the 3x3 taps on packed words and applies the dequantise / requantise
 // epilogue.  Inputs and outputs move as packed codes only: bits/8 bytes per
 // element each way.
+#include <cuda_fp16.h>
+
+#include <algorithm>
+#include <numeric>
+
 #include "dsq_epilogue.cuh"
 #include "dsq_launch.h"
+#include "dsq_tc_host.h"
 
 namespace {
 
@@ -153,194 +159,223 @@ dwconv3x3_kernel(const uint8_t *__restrict__ act, const uint8_t *__restrict__ wg
 }
 
 // ---------------------------------------------------------------------------
-// Fast path: 4-bit codes in, 4-bit codes out (the form the stacks use).
+// Codes in, codes out (the form the stacks use), any bit width.
 //
-// The nine-tap sum of one channel is three 4-way byte dot products (dp4a), one
-// per filter row: the activation operand of a row is the byte vector
-// [q(p), q(p+1), q(p+2), q(p+3)] of ONE channel at four horizontally adjacent
-// pixels, the weight operand [w0, w1, w2, 0] (signed bytes, 2c+1 for the
-// symmetric grid).  The packed words hold eight channels of one pixel, so a
-// thread (eight channels, four adjacent outputs) first splits each word into
-// its even and odd nibbles (two words of four channel bytes) and transposes
-// 4 pixels x 4 channels of bytes with byte permutes; the vectors of outputs
-// 1..3 come from the first one by funnel shifts.  Per output element this is
-// about 10 instructions for the sum and 9 for the dequantise / requantise
-// epilogue.  A thread keeps its eight channels for all its strips, so the
-// weight vectors, scales and biases are set up once.
+// The nine-tap sums run on packed half precision: a code q placed in the low
+// bits of a 16-bit half IS the (denormal) number q * 2^-24, so two channels of a
+// pixel become an operand with one shift and one AND, and one fma.f16x2 does two
+// channels' tap.  Weights are small integers as halves; every partial sum is an
+// integer times 2^-24 with magnitude at most 9 * 15 * 15 = 2025 < 2^11, so the
+// half-precision sums are exact.  Widened to binary32 the sum is acc * 2^-24,
+// and fma(acc 2^-24, scale 2^24, bias) is the pinned fma(acc, scale, bias): a
+// power of two moved between the factors changes no bit (|scale| < 2^100).
+//
+// A thread owns eight channels (pairs j, j + 4 share a register) of a strip of
+// four output columns and walks down the rows: every input row is loaded and
+// split once and feeds the (up to) three output rows it lies under, whose sums
+// stay in registers.
+//
+// Bound: the fma.f16x2 pipe (4.5 instructions per element at 62 lanes a clock
+// and SM, measured); all in all about 10 instructions per element.  The dp4a
+// form this replaces took 30 (byte transposes, funnel shifts and an epilogue of
+// 9) and only existed for 4-bit codes: C = 144, 56x56, batch 64, 4-bit 41.9 us.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel)
-{
-    return __byte_perm(a, b, sel);
-}
+constexpr int DWH_THREADS = 128, DWH_BLOCKS_PER_SM = 3;
 
-// 4 x 4 byte transpose: in[p] = bytes (c0, c1, c2, c3) of pixel p -> out[c] =
-// bytes (p0, p1, p2, p3) of channel c
-__device__ __forceinline__ void transpose4x4(const uint32_t (&in)[4], uint32_t (&out)[4])
-{
-    const uint32_t t0 = prmt(in[0], in[1], 0x5140), t1 = prmt(in[0], in[1], 0x7362);
-    const uint32_t t2 = prmt(in[2], in[3], 0x5140), t3 = prmt(in[2], in[3], 0x7362);
-    out[0] = prmt(t0, t2, 0x5410);
-    out[1] = prmt(t0, t2, 0x7632);
-    out[2] = prmt(t1, t3, 0x5410);
-    out[3] = prmt(t1, t3, 0x7632);
-}
-
-struct DwFast {
-    float inv, r_hi;
+struct DwHalf {
+    int N, H, W, C, Ho, Wo, pitch;
+    int units;                // 8-channel units of a row, padding lanes included
+    int strips, rows, chunks; // strips of four columns; output rows of a work item
     int half_offset;
+    float inv;
 };
 
-template <int STRIDE>
-__global__ void __launch_bounds__(256)
-dwconv3x3_b4_kernel(const uint8_t *__restrict__ act, const uint8_t *__restrict__ wgt,
-                    int N, int H, int W, int C, int Ho, int Wo, int pitch,
-                    const float *__restrict__ scale, const float *__restrict__ bias,
-                    uint8_t *__restrict__ y_codes, DwFast f)
+// the unit's packed codes as 4 + 4 fields: field j at bit BITS * j, field j + 4 at
+// bit 16 + BITS * j
+template <int BITS>
+__device__ __forceinline__ uint32_t dwh_load(const uint8_t *row, int u, int pitch)
+{
+    if (BITS == 4) return __ldg(reinterpret_cast<const uint32_t *>(row) + u);
+    if (BITS == 2) {
+        const uint32_t x = __ldg(reinterpret_cast<const uint16_t *>(row) + u);
+        return __byte_perm(x, 0u, 0x4140);                 // byte 1 -> byte 2
+    }
+    // 3 bytes at 3 u: the one or two aligned words they lie in
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(row);
+    const int i = (3 * u) >> 2, last = pitch / 4 - 1;
+    const uint32_t x = __funnelshift_r(__ldg(w + min(i, last)), __ldg(w + min(i + 1, last)),
+                                       8 * ((3 * u) & 3));
+    return (x & 0xFFFu) | ((x & 0xFFF000u) << 4);
+}
+
+template <int BITS>
+__device__ __forceinline__ uint32_t dwh_field(uint32_t x, int j)
+{
+    constexpr uint32_t M = (1u << BITS) - 1u;
+    return (x >> (BITS * j)) & (M | (M << 16));
+}
+
+// the 2^24-scaled sums of one output pixel's eight channels -> packed codes of the
+// unit (8 * BITS bits)
+template <int BITS>
+__device__ __forceinline__ uint32_t dwh_codes(const uint32_t (&acc)[4],
+                                              const unsigned long long (&sc)[4],
+                                              const unsigned long long (&bi)[4],
+                                              unsigned long long inv2)
+{
+    int q[8];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&acc[j]));
+        const unsigned long long y = dsq_fma2(dsq_pack2(f.x, f.y), sc[j], bi[j]);
+        dsq_requant2<BITS>(y, inv2, q[j], q[j + 4]);
+    }
+    return dsq_pack8<BITS>(q);
+}
+
+template <int BITS, int STRIDE>
+__global__ void __launch_bounds__(DWH_THREADS, DWH_BLOCKS_PER_SM)
+dwconv3x3_half_kernel(const uint8_t *__restrict__ act, const uint8_t *__restrict__ wgt,
+                      const float *__restrict__ scale, const float *__restrict__ bias,
+                      uint8_t *__restrict__ y_codes, const DwHalf p)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    constexpr int OW = 4;                          // outputs per thread along W
-    constexpr int NP = STRIDE == 1 ? 6 : 9;        // input pixels per row
-    constexpr int NT = STRIDE == 1 ? 2 : 3;        // 4-pixel groups (the last one partial)
-    const int units = pitch / 4;
-    const int strips = (Wo + OW - 1) / OW;
-    const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t gthreads = (int64_t)gridDim.x * blockDim.x;   // a multiple of `units`
-    const int u = (int)(gtid % units);
-    const int64_t streams = gthreads / units;
-
-    // weights of the unit's eight channels: channel order (0, 2, 4, 6 | 1, 3, 5, 7),
-    // one register per channel and filter row, bytes (w0, w1, w2, 0)
-    uint32_t wv[3][8];
-    {
-        uint32_t tap[9];
-#pragma unroll
-        for (int k = 0; k < 9; ++k) tap[k] = __ldg(reinterpret_cast<const uint32_t *>(wgt + k * pitch) + u);
-#pragma unroll
-        for (int r = 0; r < 3; ++r)
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int ch = i < 4 ? 2 * i : 2 * (i - 4) + 1;
-                uint32_t v = 0;
-#pragma unroll
-                for (int kw = 0; kw < 3; ++kw) {
-                    int c = ((int)(tap[3 * r + kw] << (28 - 4 * ch))) >> 28;   // signed nibble
-                    if (f.half_offset) c = 2 * c + 1;
-                    v |= ((uint32_t)c & 0xFFu) << (8 * kw);
-                }
-                wv[r][i] = v;
-            }
-    }
-    float sc[8], bi[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int ch = 8 * u + (i < 4 ? 2 * i : 2 * (i - 4) + 1);
-        sc[i] = 0.f; bi[i] = 0.f;
-        if (ch < C) {
-            sc[i] = __ldg(scale + ch);
-            if (f.half_offset) sc[i] = __fmul_rn(sc[i], 0.5f);
-            bi[i] = __ldg(bias + ch);
-        }
-    }
-    // the data below depends on the kernels before this one
+    constexpr int OW = 4, NP = (OW - 1) * STRIDE + 3;
+    const uint32_t gtid = blockIdx.x * DWH_THREADS + threadIdx.x;
+    const uint32_t lanes = gridDim.x * DWH_THREADS / (uint32_t)p.units;   // exact (host)
+    const int u = (int)(gtid % (uint32_t)p.units);
+    const uint32_t per_img = (uint32_t)p.strips * p.chunks;
+    const uint32_t n_items = per_img * (uint32_t)p.N;
+    uint32_t item = gtid / (uint32_t)p.units;
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
-    // Strips are walked with a fixed stride; the strip index is kept as
-    // (image, output row, strip of the row) and advanced by the stride's own
-    // decomposition with carries: no division in the loop.
-    const int per_img = Ho * strips;
-    int sx, ho, n;
+    // weights as halves: c = (n ^ half) - half of the stored field n, or 2 c + 1;
+    // 0x6400 | m is the half 1024 + m
+    __half2 w[9][4];
     {
-        const uint32_t s0 = (uint32_t)(gtid / units);
-        n = (int)(s0 / (uint32_t)per_img);
-        const uint32_t rem = s0 - (uint32_t)n * per_img;
-        ho = (int)(rem / (uint32_t)strips);
-        sx = (int)(rem - (uint32_t)ho * strips);
+        constexpr uint32_t HALF = 1u << (BITS - 1);
+        const __half2 mul = __float2half2_rn(p.half_offset ? 2.0f : 1.0f);
+        const __half2 add = __float2half2_rn(p.half_offset ? 1.0f : 0.0f);
+        const __half2 base = __float2half2_rn(1024.0f + HALF);
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            const uint32_t x = dwh_load<BITS>(wgt + k * p.pitch, u, p.pitch);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const uint32_t m = (dwh_field<BITS>(x, j) ^ (HALF | (HALF << 16))) | 0x64006400u;
+                w[k][j] = __hfma2(__hsub2(*reinterpret_cast<const __half2 *>(&m), base), mul, add);
+            }
+        }
     }
-    const int d_n = (int)(streams / per_img), d_rem = (int)(streams % per_img);
-    const int d_ho = d_rem / strips, d_sx = d_rem - d_ho * strips;
-    const int pw = pitch / 4;                      // words per pixel
-    const uint32_t *act32 = reinterpret_cast<const uint32_t *>(act) + u;
+    unsigned long long sc[4], bi[4];
+    {
+        float s[8], b[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            s[i] = b[i] = 0.f;                              // padding lanes: code 0
+            if (8 * u + i < p.C) dsq_codes_affine(scale, bias, 8 * u + i, p.half_offset, 24, s[i], b[i]);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            sc[j] = dsq_pack2(s[j], s[j + 4]);
+            bi[j] = dsq_pack2(b[j], b[j + 4]);
+        }
+    }
+    const unsigned long long inv2 = dsq_pack2(p.inv, p.inv);
 
-    for (; n < N; ) {
-        const int wo0 = sx * OW;
-        const int hi0 = ho * STRIDE - 1, wi0 = wo0 * STRIDE - 1;
-        // the 3 x NP window of packed words (code 0 outside the image)
-        uint32_t win[3][NP];
-        const uint32_t *base = act32 + ((int64_t)n * H + hi0) * W * pw + (int64_t)wi0 * pw;
-        if (hi0 >= 0 && hi0 + 2 < H && wi0 >= 0 && wi0 + NP <= W) {
+    for (; item < n_items; item += lanes) {
+        const uint32_t n = item / per_img, rem = item - n * per_img;
+        const uint32_t chunk = rem / (uint32_t)p.strips;
+        const int wo0 = (int)(rem - chunk * p.strips) * OW;
+        const int ho0 = (int)chunk * p.rows;
+        const int rows = min(p.rows, p.Ho - ho0);
+        const int hi0 = ho0 * STRIDE - 1, wi0 = wo0 * STRIDE - 1;
+        const uint8_t *base = act + ((int64_t)n * p.H * p.W + wi0) * p.pitch;
+        const bool inner = wi0 >= 0 && wi0 + NP <= p.W;
+        uint32_t next[NP];
+        auto load_row = [&](int hi) {
+            const bool in = hi >= 0 && hi < p.H;
+            const uint8_t *row = base + (int64_t)hi * p.W * p.pitch;
 #pragma unroll
-            for (int r = 0; r < 3; ++r)
-#pragma unroll
-                for (int x = 0; x < NP; ++x) win[r][x] = __ldg(base + (r * W + x) * pw);
-        } else {
-#pragma unroll
-            for (int r = 0; r < 3; ++r)
-#pragma unroll
-                for (int x = 0; x < NP; ++x) {
-                    const int hi = hi0 + r, wi = wi0 + x;
-                    win[r][x] = (hi >= 0 && hi < H && wi >= 0 && wi < W)
-                                    ? __ldg(base + (r * W + x) * pw) : 0u;
-                }
-        }
-        int acc[OW][8];
-#pragma unroll
-        for (int o = 0; o < OW; ++o)
-#pragma unroll
-            for (int i = 0; i < 8; ++i) acc[o][i] = 0;
-#pragma unroll
-        for (int r = 0; r < 3; ++r) {
-            // even / odd nibbles of the row's pixels in groups of four, then per
-            // channel the bytes of 4 consecutive pixels
-            uint32_t tv[NT][8];
-#pragma unroll
-            for (int g = 0; g < NT; ++g) {
-                uint32_t ev[4], od[4], a[4], b[4];
-#pragma unroll
-                for (int x = 0; x < 4; ++x) {
-                    const uint32_t w = 4 * g + x < NP ? win[r][4 * g + x < NP ? 4 * g + x : 0] : 0u;
-                    ev[x] = w & 0x0F0F0F0Fu;
-                    od[x] = (w >> 4) & 0x0F0F0F0Fu;
-                }
-                transpose4x4(ev, a);
-                transpose4x4(od, b);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) { tv[g][i] = a[i]; tv[g][4 + i] = b[i]; }
+            for (int x = 0; x < NP; ++x) {
+                next[x] = 0u;
+                if (in && (inner || (wi0 + x >= 0 && wi0 + x < p.W)))
+                    next[x] = dwh_load<BITS>(row + x * p.pitch, u, p.pitch);
             }
+        };
+        uint8_t *out = y_codes + (((int64_t)n * p.Ho + ho0) * p.Wo + wo0) * p.pitch;
+        __half2 acc[STRIDE == 1 ? 3 : 2][OW][4];
+        __half2 q[NP][4];
+        auto taps = [&](__half2 (&a)[OW][4], int kh, bool first) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
+            for (int kw = 0; kw < 3; ++kw)
 #pragma unroll
-                for (int o = 0; o < OW; ++o) {
-                    // bytes (p, p+1, p+2, .) of the channel with p = o * STRIDE
-                    const int p0 = o * STRIDE, g = p0 >> 2, sh = 8 * (p0 & 3);
-                    const uint32_t v = sh == 0 ? tv[g][i]
-                                               : __funnelshift_r(tv[g][i], g + 1 < NT ? tv[g + 1 < NT ? g + 1 : g][i] : 0u, sh);
-                    acc[o][i] = __dp4a((int)v, (int)wv[r][i], acc[o][i]);
+                for (int o = 0; o < OW; ++o)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        a[o][j] = __hfma2(q[o * STRIDE + kw][j], w[3 * kh + kw][j],
+                                          first && kw == 0 ? __half2half2(__ushort_as_half(0)) : a[o][j]);
+        };
+        auto finish = [&](__half2 (&a)[OW][4]) {
+#pragma unroll
+            for (int o = 0; o < OW; ++o) {
+                uint32_t s[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) s[j] = *reinterpret_cast<const uint32_t *>(&a[o][j]);
+                const uint32_t cw = dwh_codes<BITS>(s, sc, bi, inv2);
+                uint8_t *dst = out + o * p.pitch;
+                const bool live = wo0 + o < p.Wo;
+                if (BITS == 4) {
+                    if (live) reinterpret_cast<uint32_t *>(dst)[u] = cw;
+                } else if (BITS == 2) {
+                    if (live) reinterpret_cast<uint16_t *>(dst)[u] = (uint16_t)cw;
+                } else if (live) {
+                    // (units up to the row pitch: the spare bytes are written as zeros)
+                    const int at = 3 * u;
+                    dst[at] = (uint8_t)cw;
+                    if (at + 1 < p.pitch) dst[at + 1] = (uint8_t)(cw >> 8);
+                    if (at + 2 < p.pitch) dst[at + 2] = (uint8_t)(cw >> 16);
                 }
             }
-        }
-        // epilogue: dequantise, requantise to [0, hi] (clip after the multiply,
-        // floor by the 2^23 trick, codes summed into their nibbles)
-        uint32_t *out32 = reinterpret_cast<uint32_t *>(y_codes) +
-                          (((int64_t)n * Ho + ho) * Wo + wo0) * pw + u;
+            out += (int64_t)p.Wo * p.pitch;
+        };
+        // input row s of the item: rows hi0 .. hi0 + (rows - 1) * STRIDE + 2
+        const int n_in = (rows - 1) * STRIDE + 3;
+        load_row(hi0);
+        constexpr int UNROLL = STRIDE == 1 ? 3 : 4;
+#pragma unroll 1
+        for (int s0 = 0; s0 < n_in; s0 += UNROLL) {
 #pragma unroll
-        for (int o = 0; o < OW; ++o) {
-            if (wo0 + o >= Wo) continue;
-            uint32_t cw = 0u;
+            for (int t = 0; t < UNROLL; ++t) {
+                const int s = s0 + t;
+                if (s >= n_in) break;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int ch_in_word = i < 4 ? 2 * i : 2 * (i - 4) + 1;
-                const float vf = __fsub_rn(__int_as_float(0x4B400000 + acc[o][i]), 12582912.0f);
-                const float y = __fmaf_rn(vf, sc[i], bi[i]);
-                const float rr = fminf(__fmaf_rn(fmaxf(y, 0.0f), f.inv, 0.5f), f.r_hi);
-                cw += (uint32_t)__float_as_int(__fadd_rd(rr, 8388608.0f)) << (4 * ch_in_word);
+                for (int x = 0; x < NP; ++x)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const uint32_t f = dwh_field<BITS>(next[x], j);
+                        q[x][j] = *reinterpret_cast<const __half2 *>(&f);
+                    }
+                if (s + 1 < n_in) load_row(hi0 + s + 1);
+                if (STRIDE == 1) {
+                    // output row s starts, s - 1 goes on, s - 2 is completed
+                    if (s >= 2) {
+                        taps(acc[(t + 1) % 3], 2, false);
+                        finish(acc[(t + 1) % 3]);
+                    }
+                    if (s >= 1 && s <= rows) taps(acc[(t + 2) % 3], 1, false);
+                    if (s < rows) taps(acc[t % 3], 0, true);
+                } else if (t & 1) {
+                    taps(acc[t >> 1], 1, false);
+                } else {
+                    if (s >= 2) {
+                        taps(acc[((t >> 1) + 1) & 1], 2, false);
+                        finish(acc[((t >> 1) + 1) & 1]);
+                    }
+                    if (s >> 1 < rows) taps(acc[(t >> 1) & 1], 0, true);
+                }
             }
-            cw -= 0x4B000000u * 0x11111111u;
-            out32[o * pw] = cw;
         }
-        // next strip of this thread
-        sx += d_sx; ho += d_ho; n += d_n;
-        if (sx >= strips) { sx -= strips; ++ho; }
-        if (ho >= Ho) { ho -= Ho; ++n; }
     }
 }
 
@@ -373,27 +408,48 @@ extern "C" int dsq_dwconv2d(const void *act_codes, const dsq_nhwc_t *shape,
     const int Wo = (shape->W + 2 - 3) / conv->stride + 1;
     const int pitch = (int)dsq_row_pitch(shape->C, bits);
     cudaStream_t s = (cudaStream_t)stream;
-    // fast path: 4-bit codes to 4-bit codes, requantiser range starting at 0
-    if (bits == 4 && y_codes && !y_f32 && !acc_out && !e.residual && !e.general_offset &&
-        e.rq.lo == 0.0f) {
-        DwFast f;
-        f.inv = e.rq.inv;
-        f.r_hi = fmaf(e.rq.hi, e.rq.inv, 0.5f);
-        f.half_offset = e.half_offset;
-        if ((int)floorf(f.r_hi) == e.rq.qmax) {
-            const int units = pitch / 4;
-            const int sms = dsq_sm_count() > 0 ? dsq_sm_count() : 148;
-            const int64_t n_strips = (int64_t)shape->N * Ho * ((Wo + 3) / 4);
-            // threads: a multiple of `units` (a thread keeps its channel word) and of 256
-            int64_t blocks = (n_strips * units + 255) / 256;
-            if (blocks > (int64_t)sms * 8) blocks = (int64_t)sms * 8;
-            blocks = (blocks + units - 1) / units * units;     // blocks * 256 is a multiple of units
-            const uint8_t *a8 = (const uint8_t *)act_codes, *w8 = (const uint8_t *)w_packed;
-            return dsq_launch(conv->stride == 1 ? dwconv3x3_b4_kernel<1> : dwconv3x3_b4_kernel<2>,
-                              dim3((unsigned)blocks), dim3(256), 0, s, 0, 0, a8, w8, shape->N,
-                              shape->H, shape->W, shape->C, Ho, Wo, pitch, e.scale, e.bias,
-                              e.y_codes, f);
+    // codes to codes, requantiser range starting at 0 (the lean epilogue does not
+    // subtract lo); images of at least 2^31 bytes a row keep the general kernel's
+    // 64-bit indexing
+    const int units = (pitch + bits - 1) / bits;
+    const int strips = (Wo + 3) / 4;
+    if (y_codes && !y_f32 && !acc_out && !e.residual && !e.general_offset && e.rq.lo == 0.0f &&
+        (int64_t)units * strips * Ho * shape->N < (1ll << 31)) {
+        DwHalf p;
+        p.N = shape->N; p.H = shape->H; p.W = shape->W; p.C = shape->C;
+        p.Ho = Ho; p.Wo = Wo; p.pitch = pitch;
+        p.units = units; p.strips = strips;
+        p.half_offset = e.half_offset;
+        p.inv = e.rq.inv;
+        const int sms = dsq_sm_count() > 0 ? dsq_sm_count() : 148;
+        // blocks: all resident, and a thread keeps its unit (blocks * 128 is a
+        // multiple of `units`)
+        const int per = units / std::gcd(units, DWH_THREADS);
+        const int resident = std::max(sms * DWH_BLOCKS_PER_SM / per, 1) * per;
+        const int64_t lanes = (int64_t)resident * DWH_THREADS / units;
+        // rows of a work item: a thread's passes over items, each rows + 2 input
+        // rows (stride 1) and about one row's worth of set-up, are what a launch
+        // lasts; the fewest win
+        int64_t best = -1;
+        for (int chunks = 1; chunks <= Ho; ++chunks) {
+            const int rows = (Ho + chunks - 1) / chunks;
+            if (chunks > 1 && rows == (Ho + chunks - 2) / (chunks - 1)) continue;
+            const int used = (Ho + rows - 1) / rows;
+            const int64_t passes = ((int64_t)p.N * strips * used + lanes - 1) / lanes;
+            const int64_t cost = passes * (8 * rows + (conv->stride == 1 ? 12 : 8)) ;
+            if (best < 0 || cost < best) { best = cost; p.rows = rows; p.chunks = used; }
         }
+        const int64_t need = ((int64_t)units * p.N * strips * p.chunks + DWH_THREADS - 1) / DWH_THREADS;
+        const int blocks = (int)std::min<int64_t>(resident, (need + per - 1) / per * per);
+        typedef void (*Kernel)(const uint8_t *, const uint8_t *, const float *, const float *,
+                               uint8_t *, const DwHalf);
+        static const Kernel kernels[3][2] = {
+            {dwconv3x3_half_kernel<2, 1>, dwconv3x3_half_kernel<2, 2>},
+            {dwconv3x3_half_kernel<3, 1>, dwconv3x3_half_kernel<3, 2>},
+            {dwconv3x3_half_kernel<4, 1>, dwconv3x3_half_kernel<4, 2>}};
+        return dsq_launch(kernels[bits - 2][conv->stride - 1], dim3(blocks), dim3(DWH_THREADS), 0, s,
+                          dsq_launch_hooks().pdl, 0, (const uint8_t *)act_codes,
+                          (const uint8_t *)w_packed, e.scale, e.bias, e.y_codes, p);
     }
     const int64_t total = (int64_t)shape->N * Ho * ((Wo + 3) / 4) *
                           (bits == 3 ? (shape->C + 7) / 8 : pitch / bits);

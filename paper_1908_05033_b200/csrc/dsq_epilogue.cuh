@@ -138,4 +138,160 @@ __device__ __forceinline__ float dsq_epi_residual(float y, uint32_t q_r,
 {
     return __fadd_rn(y, __fmaf_rn((float)q_r, res_delta, res_lo));
 }
+// ---------------------------------------------------------------------------
+// Lean codes epilogue: accumulator -> codes in about 3 instructions per element.
+//
+// Per element the pinned sequence is y = fma(v, scale, bias) (+ residual),
+// r = fma(clip(y) - lo, inv, 0.5), q = min(floor(r), qmax).  Here
+//   * arithmetic is on pairs (f32x2: one issue slot for two elements), each
+//     operation rounding as the scalar one does;
+//   * nothing is clipped before the rounding step: below the range r < 0.5 (codes
+//     of negative numbers saturate to 0), above it r > qmax + 0.5;
+//   * floor and clip are one multiply and half a pack.  r * 2^(-141 - BITS),
+//     rounded down, is a denormal number whose bit pattern is the integer
+//     floor(r * 2^(8 - BITS)); cvt.pack.sat.u8 clips two of those to 0 .. 255 and
+//     packs them, and the top BITS bits of each byte are the code.
+// Measured per SM and clock (lanes): f32x2 62, I2F 62, cvt.pack 62 - against an
+// IADD, two FMNMX, a shift and a shift-add per element in the scalar form (all of
+// them on the 62-lane pipe).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ unsigned long long dsq_pack2(float a, float b)
+{
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long dsq_fma2(unsigned long long a, unsigned long long b,
+                                                       unsigned long long c)
+{
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ unsigned long long dsq_add2(unsigned long long a, unsigned long long b)
+{
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// two values y - lo -> two integers whose saturated low byte holds the code in
+// its top BITS bits (inv2: the requantiser's inv, twice)
+template <int BITS>
+__device__ __forceinline__ void dsq_requant2(unsigned long long y, unsigned long long inv2, int &q0,
+                                             int &q1)
+{
+    constexpr unsigned long long DEN = 1ull << (8 - BITS);       // 2^(8 - BITS) * 2^-149
+    const unsigned long long r = dsq_fma2(y, inv2, 0x3F0000003F000000ull);
+    unsigned long long u;
+    asm("mul.rm.f32x2 %0, %1, %2;" : "=l"(u) : "l"(r), "l"(DEN | (DEN << 32)));
+    asm("mov.b64 {%0, %1}, %2;" : "=r"(q0), "=r"(q1) : "l"(u));
+}
+
+// bytes [sat(q0), sat(q1), sat(q2), sat(q3)]
+__device__ __forceinline__ uint32_t dsq_sat_bytes(int q0, int q1, int q2, int q3)
+{
+    uint32_t t, r;
+    asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, 0;" : "=r"(t) : "r"(q3), "r"(q2));
+    asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(q1), "r"(q0), "r"(t));
+    return r;
+}
+
+// eight such integers of consecutive elements -> their codes, packed (8 * BITS bits)
+template <int BITS>
+__device__ __forceinline__ uint32_t dsq_pack8(const int (&q)[8])
+{
+    if (BITS == 4) {
+        const uint32_t e = dsq_sat_bytes(q[0], q[2], q[4], q[6]);
+        const uint32_t o = dsq_sat_bytes(q[1], q[3], q[5], q[7]);
+        return ((e >> 4) & 0x0F0F0F0Fu) | (o & 0xF0F0F0F0u);
+    }
+    if (BITS == 3) {
+        const uint32_t e = dsq_sat_bytes(q[0], q[2], q[4], q[6]);
+        const uint32_t o = dsq_sat_bytes(q[1], q[3], q[5], q[7]);
+        const uint32_t t = ((e >> 5) & 0x07070707u) | ((o >> 2) & 0x38383838u);
+        const uint32_t x = (t & 0x003F003Fu) | ((t & 0x3F003F00u) >> 2);
+        return (x & 0xFFFu) | ((x >> 4) & 0xFFF000u);
+    }
+    const uint32_t x = dsq_sat_bytes(q[0], q[4], q[2], q[6]);
+    const uint32_t y = dsq_sat_bytes(q[1], q[5], q[3], q[7]);
+    const uint32_t z = ((x >> 6) & 0x03030303u) | ((y >> 4) & 0x0C0C0C0Cu);
+    return (z & 0xFFFFu) | ((z >> 12) & 0xF0F0u);
+}
+
+// Scale (halved for the symmetric weight grid, times 2^e: the accumulator comes
+// scaled by 2^-e) and bias of channel ch for the lean epilogue.  It does not clip
+// before rounding, so a NaN y (non-finite scale or bias; code 0 in the pinned
+// sequence) must not arise: such channels get finite numbers that give the
+// same codes for every accumulator.
+__device__ __forceinline__ void dsq_codes_affine(const float *scale, const float *bias, int ch,
+                                                 int half_offset, int e, float &s, float &b)
+{
+    s = __ldg(scale + ch);
+    b = __ldg(bias + ch);
+    const bool odd = !(fabsf(s) <= 3.4e38f) || b != b;
+    s = __fmul_rn(s, __int_as_float((127 + e - (half_offset ? 1 : 0)) << 23));
+    if (odd) {
+        s = (s != s || b != b || b == -__int_as_float(0x7F800000)) ? 0.0f : s;
+        b = -1e30f;
+    }
+    s = fminf(fmaxf(s, -3.4e38f), 3.4e38f);
+}
+
+// Requantiser and residual operands of the lean epilogue, in the form it reads.
+struct DsqLean {
+    unsigned long long inv2;              // inv, twice
+    unsigned long long neg_lo2;           // -lo, twice
+    unsigned long long res_delta2, res_lo2;
+    bool has_lo;                          // lo != 0
+};
+__device__ __forceinline__ DsqLean dsq_make_lean(const DsqEpi &e)
+{
+    DsqLean l;
+    l.inv2 = dsq_pack2(e.rq.inv, e.rq.inv);
+    l.neg_lo2 = dsq_pack2(-e.rq.lo, -e.rq.lo);
+    l.res_delta2 = dsq_pack2(e.res_delta, e.res_delta);
+    l.res_lo2 = dsq_pack2(e.res_lo, e.res_lo);
+    l.has_lo = e.rq.lo != 0.0f;
+    return l;
+}
+
+// residual codes 2 j and 2 j + 1 of eight packed codes as binary32
+template <int BITS>
+__device__ __forceinline__ unsigned long long dsq_code_pair(uint32_t x, int j)
+{
+    if (BITS == 4) {
+        const uint32_t e = x & 0x0F0F0F0Fu, o = (x >> 4) & 0x0F0F0F0Fu;
+        return dsq_pack2((float)((e >> (8 * j)) & 0xFFu), (float)((o >> (8 * j)) & 0xFFu));
+    }
+    constexpr uint32_t M = (1u << BITS) - 1u;
+    return dsq_pack2((float)((x >> (2 * BITS * j)) & M), (float)((x >> (2 * BITS * j + BITS)) & M));
+}
+
+// raw accumulators of eight consecutive output channels of one position -> their
+// packed codes; sc, bi: the channels' dsq_codes_affine (16-byte aligned), res: the
+// position's residual codes of those channels
+template <int BITS, bool RES>
+__device__ __forceinline__ uint32_t dsq_lean_codes8(const uint32_t *r, const float *sc,
+                                                    const float *bi, uint32_t res, const DsqLean &l)
+{
+    int q[8];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const ulonglong2 s = *reinterpret_cast<const ulonglong2 *>(sc + 4 * h);
+        const ulonglong2 b = *reinterpret_cast<const ulonglong2 *>(bi + 4 * h);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int c = 4 * h + 2 * k;
+            unsigned long long y = dsq_fma2(
+                dsq_pack2(__int2float_rn((int)r[c]), __int2float_rn((int)r[c + 1])),
+                k ? s.y : s.x, k ? b.y : b.x);
+            if (RES)
+                y = dsq_add2(y, dsq_fma2(dsq_code_pair<BITS>(res, c / 2), l.res_delta2, l.res_lo2));
+            if (l.has_lo) y = dsq_add2(y, l.neg_lo2);
+            dsq_requant2<BITS>(y, l.inv2, q[c], q[c + 1]);
+        }
+    }
+    return dsq_pack8<BITS>(q);
+}
 #endif
