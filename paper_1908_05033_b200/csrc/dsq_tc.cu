@@ -1841,6 +1841,18 @@ int dsq_conv2d(const void *act_codes, const dsq_nhwc_t *shape, const dsq_quant_t
                           (cudaStream_t)stream);
     if (st != DSQ_ERR_UNSUPPORTED) return st;
 
+    // the lean codes epilogues clip after the requantiser's multiply: they need
+    // floor(fma(hi - lo, inv, 0.5)) = qmax (true for every sane range)
+    const float r_hi = fmaf(e.rq.hi - e.rq.lo, e.rq.inv, 0.5f);
+    const int epi_im2col = epi != EPI_GENERAL && (int)floorf(r_hi) != e.rq.qmax ? EPI_GENERAL : epi;
+    // 1x1 convolutions from codes to codes: weights resident, lean epilogue (the
+    // tile hooks are the im2col kernel's)
+    if (epi_im2col != EPI_GENERAL && !g_forced_bn.load() && !g_forced_ks.load() &&
+        g_pair_mode.load() != 2) {
+        st = dsq_pointwise(act_codes, shape, bits, w_packed, conv, e, workspace, (cudaStream_t)stream);
+        if (st != DSQ_ERR_UNSUPPORTED) return st;
+    }
+
     const size_t P = dsq_row_pitch(conv->Cin, bits);
     const size_t row_bytes = (size_t)taps * P;
     TcParams p = {};
@@ -1887,13 +1899,7 @@ int dsq_conv2d(const void *act_codes, const dsq_nhwc_t *shape, const dsq_quant_t
     st = setup_a_tma(&p, &tmap.a, act_codes, M, bits, ks, plain_rows, shape, conv->KH, pm == 5);
     if (st) return st;
     p.small_acc = small_acc;
-    int epi_im2col = epi;
-    if (epi != EPI_GENERAL) {
-        // the codes epilogue clips after the requantiser's multiply: it needs
-        // floor(fma(hi - lo, inv, 0.5)) = qmax (true for every sane range)
-        p.r_hi = fmaf(e.rq.hi - e.rq.lo, e.rq.inv, 0.5f);
-        if ((int)floorf(p.r_hi) != e.rq.qmax) epi_im2col = EPI_GENERAL;
-    }
+    p.r_hi = r_hi;
     return dispatch_tc(bits, epi_im2col, pm, tmap, p, (cudaStream_t)stream);
 }
 

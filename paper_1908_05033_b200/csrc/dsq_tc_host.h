@@ -49,6 +49,27 @@ DSQ_HIDDEN int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, 
                                 int epi_kind, int small_acc, void *workspace,
                                 cudaStream_t stream);
 
+// 1x1 convolution from codes to codes (dsq_pw.cu).  Arguments are those of
+// dsq_conv2d after validation, `e` writing codes only.  Returns
+// DSQ_ERR_UNSUPPORTED without launching anything where it does not apply.
+DSQ_HIDDEN int dsq_pointwise(const void *act_codes, const dsq_nhwc_t *shape, int bits,
+                             const void *w_packed, const dsq_conv_t *conv, const DsqEpi &e,
+                             void *workspace, cudaStream_t stream);
+
+// Opt-in to large dynamic shared memory, once per kernel and device (an attribute
+// of the function on a device): one bit per device ordinal in *configured.
+static inline int dsq_allow_smem(const void *func, int bytes, std::atomic<unsigned long long> *configured)
+{
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return DSQ_ERR_CUDA;
+    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+    if (configured->load(std::memory_order_acquire) & bit) return DSQ_OK;
+    if (cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess)
+        return DSQ_ERR_CUDA;
+    configured->fetch_or(bit, std::memory_order_release);
+    return DSQ_OK;
+}
+
 // Two-pass GEMM (dsq_gemm8.cu): every packed row is expanded to int8 once
 // into caller-provided scratch, then an 8-bit GEMM reads it by TMA.
 // dsq_gemm8_scratch_bytes: scratch the path needs (0: not a problem it takes;
