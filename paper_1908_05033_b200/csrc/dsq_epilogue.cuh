@@ -243,7 +243,6 @@ struct DsqLean {
     unsigned long long inv2;              // inv, twice
     unsigned long long neg_lo2;           // -lo, twice
     unsigned long long res_delta2, res_lo2;
-    bool has_lo;                          // lo != 0
 };
 __device__ __forceinline__ DsqLean dsq_make_lean(const DsqEpi &e)
 {
@@ -252,7 +251,6 @@ __device__ __forceinline__ DsqLean dsq_make_lean(const DsqEpi &e)
     l.neg_lo2 = dsq_pack2(-e.rq.lo, -e.rq.lo);
     l.res_delta2 = dsq_pack2(e.res_delta, e.res_delta);
     l.res_lo2 = dsq_pack2(e.res_lo, e.res_lo);
-    l.has_lo = e.rq.lo != 0.0f;
     return l;
 }
 
@@ -268,30 +266,35 @@ __device__ __forceinline__ unsigned long long dsq_code_pair(uint32_t x, int j)
     return dsq_pack2((float)((x >> (2 * BITS * j)) & M), (float)((x >> (2 * BITS * j + BITS)) & M));
 }
 
-// raw accumulators of eight consecutive output channels of one position -> their
-// packed codes; sc, bi: the channels' dsq_codes_affine (16-byte aligned), res: the
-// position's residual codes of those channels
-template <int BITS, bool RES>
-__device__ __forceinline__ uint32_t dsq_lean_codes8(const uint32_t *r, const float *sc,
-                                                    const float *bi, uint32_t res, const DsqLean &l)
+// Raw accumulators of eight consecutive output channels of one position -> their
+// packed codes; sc, bi: the channels' dsq_codes_affine in pairs, res: the
+// position's residual codes of those channels.
+template <int BITS, bool RES, bool LO>
+__device__ __forceinline__ uint32_t dsq_lean_codes8(const uint32_t (&v)[8],
+                                                    const unsigned long long (&sc)[4],
+                                                    const unsigned long long (&bi)[4],
+                                                    uint32_t res, const DsqLean &l)
 {
     int q[8];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const ulonglong2 s = *reinterpret_cast<const ulonglong2 *>(sc + 4 * h);
-        const ulonglong2 b = *reinterpret_cast<const ulonglong2 *>(bi + 4 * h);
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int c = 4 * h + 2 * k;
-            unsigned long long y = dsq_fma2(
-                dsq_pack2(__int2float_rn((int)r[c]), __int2float_rn((int)r[c + 1])),
-                k ? s.y : s.x, k ? b.y : b.x);
-            if (RES)
-                y = dsq_add2(y, dsq_fma2(dsq_code_pair<BITS>(res, c / 2), l.res_delta2, l.res_lo2));
-            if (l.has_lo) y = dsq_add2(y, l.neg_lo2);
-            dsq_requant2<BITS>(y, l.inv2, q[c], q[c + 1]);
-        }
+    for (int c = 0; c < 4; ++c) {
+        unsigned long long y = dsq_fma2(
+            dsq_pack2(__int2float_rn((int)v[2 * c]), __int2float_rn((int)v[2 * c + 1])), sc[c], bi[c]);
+        if (RES) y = dsq_add2(y, dsq_fma2(dsq_code_pair<BITS>(res, c), l.res_delta2, l.res_lo2));
+        if (LO) y = dsq_add2(y, l.neg_lo2);
+        dsq_requant2<BITS>(y, l.inv2, q[2 * c], q[2 * c + 1]);
     }
     return dsq_pack8<BITS>(q);
+}
+
+// Which accumulator column holds output channel ch of a group of 32.  The epilogue
+// reads tensor memory in the 16x256b shape, where a lane gets two columns of every
+// block of eight; with the channels laid out like this (the weight rows are put in
+// this order when they are expanded) those are eight CONSECUTIVE channels: one
+// scale and bias set per lane for all its positions - they stay in registers - and
+// a whole word of codes, with no exchange between lanes.
+__host__ __device__ inline int dsq_column_of(int ch)
+{
+    return (ch & ~31) | (((ch >> 1) & 3) << 3) | (((ch >> 3) & 3) << 1) | (ch & 1);
 }
 #endif

@@ -11,10 +11,14 @@
 //   * M tiles are MT x 128 pixels, MT = 1, 2 or 4, each 128 pixels an accumulator
 //     of its own: a hand-off between the roles costs a few hundred clocks
 //     whatever it carries, so a narrow layer hands over 512 pixels at a time;
-//   * twelve epilogue warps run the lean epilogue (dsq_epilogue.cuh), eight warps
-//     expand.
-// Packed pixel rows come by TMA (plain 2-D boxes; im2col boxes with a traversal
-// stride for stride 2), one "plane" of 128 channels per fill.
+//   * sixteen warps run the lean epilogue (dsq_epilogue.cuh), six expand, in two
+//     groups each.  A lane's accumulators are eight consecutive channels of four
+//     pixels, so the scales and biases sit in registers (reading them from shared
+//     memory, one clock of that pipe per number and warp, took 33.6 us for
+//     112x112 16->96 where the kernel without those loads took 22.9).
+//   * the packed rows of a tile are contiguous in memory and come as one untiled
+//     bulk copy (stride 2: im2col boxes with a traversal stride).
+// Input channels are expanded and multiplied in planes of 128.
 //
 // MobileNetV2-shaped layers, batch 64, 4-bit, against the im2col kernel this
 // takes them from: 112x112 16->96 71.8 us, 32->16 49.4 us; 56x56 24->144 30.4 us,
@@ -26,10 +30,13 @@
 
 namespace {
 
-constexpr int PW_WARP_TMA = 0, PW_WARP_MMA = 1, PW_WARP_A0 = 2, PW_A_WARPS = 8, PW_WARP_E0 = 10,
-              PW_E_WARPS = 12, PW_WARPS = 22;
+// Expansion and epilogue are two groups of warps each, working on alternate fills and
+// alternate tiles: what a group waits for (a barrier, a fence, tensor memory) the
+// other one's work covers.
+constexpr int PW_WARP_TMA = 0, PW_WARP_MMA = 1, PW_WARP_A0 = 2, PW_A_GROUP = 3, PW_WARP_E0 = 8,
+              PW_E_GROUP = 8, PW_WARPS = 24;
 constexpr int PW_THREADS = PW_WARPS * 32;
-constexpr int PW_EPQ = PW_E_WARPS / 4;        // epilogue warps per tensor-memory lane quarter
+constexpr int PW_EPQ = PW_E_GROUP / 4;        // warps of a group per tensor-memory lane quarter
 constexpr int PW_A_SLOTS = 2;                 // expanded planes
 constexpr int PW_MAX_STAGES = 4;              // packed planes in flight
 constexpr int PW_BARS = 2 * PW_MAX_STAGES + 2 * PW_A_SLOTS + 4 + 1;
@@ -43,6 +50,7 @@ struct PwParams {
     int m_tiles, mstep;                       // tiles of mt * 128 pixels; tiles between two of a CTA
     int planes, P, PB;                        // planes of 128 channels; packed bytes of a pixel, of a plane
     int stages, tmem_cols;
+    const uint8_t *act;
     int stride, Ho, Wo;                       // stride 2: output image (im2col boxes)
     int box_rows;                             // pixels of a TMA box
     int smem_bytes, shift, out_pitch;
@@ -54,13 +62,14 @@ struct PwParams {
     int *ws;
 };
 
-__host__ inline PwSmem pw_layout(int mt, int BN, int planes, int PB, int stages)
+// row_bytes: packed bytes of a pixel in a stage
+__host__ inline PwSmem pw_layout(int mt, int BN, int planes, int row_bytes, int stages)
 {
     PwSmem L;
     uint32_t o = 0;
     L.a_slots = o; o += PW_A_SLOTS * mt * 128 * 128;
     L.b_tiles = o; o += planes * BN * 128;
-    L.a_stage = o; o += stages * mt * 128 * PB;
+    L.a_stage = o; o += stages * mt * 128 * row_bytes;
     L.epi = o;     o += 2 * BN * 4;
     o = (o + 127u) & ~127u;
     L.bars = o;    o += 8 * PW_BARS;
@@ -105,7 +114,7 @@ __device__ __forceinline__ void pw_store_row3(uint32_t dst, int sw, const uint4 
         }
 }
 
-template <int BITS, bool RES>
+template <int BITS, bool RES, bool LO>
 __global__ void __launch_bounds__(PW_THREADS, 1)
 dsq_pw_kernel(const __grid_constant__ CUtensorMap tmap_a, const PwParams p)
 {
@@ -120,7 +129,11 @@ dsq_pw_kernel(const __grid_constant__ CUtensorMap tmap_a, const PwParams p)
     const int my_tiles = m_first < p.m_tiles ? (p.m_tiles - 1 - m_first) / p.mstep + 1 : 0;
     const int tile_px = p.mt * 128;
     const uint32_t a_slot_bytes = (uint32_t)tile_px * 128u;
-    const uint32_t stage_bytes = (uint32_t)tile_px * p.PB;
+    // a stage holds the tile's packed rows as they lie in memory (stride 1), or its
+    // planes one behind the other
+    const uint32_t px_bytes = p.stride == 1 ? (uint32_t)p.P : (uint32_t)p.PB;
+    const uint32_t plane_at = p.stride == 1 ? (uint32_t)p.PB : (uint32_t)(tile_px * p.PB);
+    const uint32_t stage_bytes = (uint32_t)tile_px * (p.stride == 1 ? p.P : p.planes * p.PB);
     const uint32_t n_fills = (uint32_t)my_tiles * p.planes;
 
     const uint32_t bars = smem_u32(smem + L.bars);
@@ -139,20 +152,20 @@ dsq_pw_kernel(const __grid_constant__ CUtensorMap tmap_a, const PwParams p)
     if (threadIdx.x == 0) {
         for (int s = 0; s < PW_MAX_STAGES; ++s) {
             mbar_init(bar_st_full(s), 1);             // TMA producer (+ bytes)
-            mbar_init(bar_st_empty(s), PW_A_WARPS);
+            mbar_init(bar_st_empty(s), PW_A_GROUP * p.planes);
         }
         for (int s = 0; s < PW_A_SLOTS; ++s) {
-            mbar_init(bar_a_full(s), PW_A_WARPS);
+            mbar_init(bar_a_full(s), PW_A_GROUP);
             mbar_init(bar_a_empty(s), 1);             // tcgen05.commit
         }
         for (int s = 0; s < 2; ++s) {
             mbar_init(bar_acc_full(s), 1);            // tcgen05.commit
-            mbar_init(bar_acc_empty(s), PW_E_WARPS);
+            mbar_init(bar_acc_empty(s), PW_E_GROUP);
         }
         mbar_init(bar_drain, 1);
         *ctl.abort_flag = 0;
         mbar_init_fence();
-        tma_prefetch_desc(&tmap_a);
+        if (p.stride != 1) tma_prefetch_desc(&tmap_a);
     }
     if (warp == PW_WARP_MMA) {
         tmem_alloc(smem_u32((const void *)tmem_slot), (uint32_t)p.tmem_cols);
@@ -162,15 +175,12 @@ dsq_pw_kernel(const __grid_constant__ CUtensorMap tmap_a, const PwParams p)
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
-    // everything above touched no global data; nothing below starts before the
-    // kernels ahead of this one in the stream have completed
-    grid_launch_dependents();
-    grid_dependency_wait();
-
     float *sm_scale = reinterpret_cast<float *>(smem + L.epi);
     float *sm_bias = sm_scale + p.BN;
     if (warp != PW_WARP_TMA) {
         // ---------------- once: weights of this N tile, scales and biases ---------
+        // (before the wait for the kernels ahead in the stream: they are constants of
+        // the network, and no kernel that lets its successors start early writes them)
         const int tid = threadIdx.x - 32;
         constexpr int NT = PW_THREADS - 32;
         const uint32_t bt = smem_u32(smem + L.b_tiles);
@@ -187,7 +197,8 @@ dsq_pw_kernel(const __grid_constant__ CUtensorMap tmap_a, const PwParams p)
                     v[l] = make_uint4(0u, 0u, 0u, 0u);
                     if (at < p.P) v[l] = __ldg(reinterpret_cast<const uint4 *>(w0 + (int64_t)row * p.P + at));
                 }
-                pw_store_row3<true>(bt + (uint32_t)((pl * p.BN + row) * 128), row & 7, v,
+                const int col = dsq_column_of(row);
+                pw_store_row3<true>(bt + (uint32_t)((pl * p.BN + col) * 128), col & 7, v,
                                     pw_groups<3>(p, pl), p.orv);
             }
         } else {
@@ -195,7 +206,8 @@ dsq_pw_kernel(const __grid_constant__ CUtensorMap tmap_a, const PwParams p)
                 const int row = t / cpr, c = t - row * cpr;
                 const uint4 v = __ldg(reinterpret_cast<const uint4 *>(w0) + t);
                 const int pl = c / BITS, ch = c - pl * BITS;     // BITS chunks per plane
-                pw_store_chunk<BITS, true>(bt + (uint32_t)((pl * p.BN + row) * 128), row & 7, ch, v,
+                const int col = dsq_column_of(row);
+                pw_store_chunk<BITS, true>(bt + (uint32_t)((pl * p.BN + col) * 128), col & 7, ch, v,
                                            p.orv);
             }
         }
@@ -210,38 +222,41 @@ dsq_pw_kernel(const __grid_constant__ CUtensorMap tmap_a, const PwParams p)
         fence_proxy_async_smem();
         named_barrier_sync(1, NT);
     }
+    // no activation is read and nothing is written before the kernels ahead of this
+    // one have completed
+    grid_launch_dependents();
+    grid_dependency_wait();
 
     if (warp == PW_WARP_TMA) {
         // ---------------- producer: packed planes --------------------------------
         if (lane == 0) {
             uint32_t issued = 0, ph = 0;
-            int s = 0, pl = 0, tile = m_first;
-            const int boxes = tile_px / p.box_rows;
+            int s = 0, m0 = m_first * tile_px;
 #pragma unroll 1
-            for (uint32_t g = 0; g < n_fills; ++g) {
+            for (int it = 0; it < my_tiles; ++it) {
                 if (!wait_bar(bar_st_empty(s), ph ^ 1u, ctl, 31)) break;
                 const uint32_t dst = smem_u32(smem + L.a_stage) + s * stage_bytes;
+                const int px = min(tile_px, p.M - m0);
                 if (p.stride == 1) {
-                    mbar_arrive_expect_tx(bar_st_full(s), stage_bytes);
-                    for (int i = 0; i < boxes; ++i)
-                        tma_load_2d(dst + (uint32_t)(i * p.box_rows * p.PB), &tmap_a, pl * p.PB,
-                                    tile * tile_px + i * p.box_rows, bar_st_full(s));
+                    mbar_arrive_expect_tx(bar_st_full(s), (uint32_t)(px * p.P));
+                    bulk_load(dst, p.act + (int64_t)m0 * p.P, (uint32_t)(px * p.P), bar_st_full(s));
                 } else {
-                    // boxes that start behind the last pixel are left out (an im2col
+                    // (boxes that start behind the last pixel are left out: an im2col
                     // load starts inside the tensor)
-                    const int left = p.M - tile * tile_px;
-                    const int nb = min(boxes, (left + p.box_rows - 1) / p.box_rows);
-                    mbar_arrive_expect_tx(bar_st_full(s), (uint32_t)(nb * p.box_rows * p.PB));
+                    const int nb = (px + p.box_rows - 1) / p.box_rows;
+                    mbar_arrive_expect_tx(bar_st_full(s), (uint32_t)(nb * p.box_rows * p.planes * p.PB));
                     for (int i = 0; i < nb; ++i) {
-                        const int m = tile * tile_px + i * p.box_rows;
+                        const int m = m0 + i * p.box_rows;
                         const int t = m / p.Wo, n = t / p.Ho;
-                        tma_load_im2col_4d(dst + (uint32_t)(i * p.box_rows * p.PB), &tmap_a, pl * p.PB,
-                                           (m - t * p.Wo) * p.stride, (t - n * p.Ho) * p.stride, n,
-                                           (uint16_t)0, (uint16_t)0, bar_st_full(s));
+                        for (int pl = 0; pl < p.planes; ++pl)
+                            tma_load_im2col_4d(dst + pl * plane_at + (uint32_t)(i * p.box_rows * p.PB),
+                                               &tmap_a, pl * p.PB, (m - t * p.Wo) * p.stride,
+                                               (t - n * p.Ho) * p.stride, n, (uint16_t)0, (uint16_t)0,
+                                               bar_st_full(s));
                     }
                 }
                 ++issued;
-                if (++pl == p.planes) { pl = 0; tile += p.mstep; }
+                m0 += p.mstep * tile_px;
                 if (++s == p.stages) { s = 0; ph ^= 1u; }
             }
             const uint32_t S = (uint32_t)p.stages;
@@ -291,19 +306,28 @@ dsq_pw_kernel(const __grid_constant__ CUtensorMap tmap_a, const PwParams p)
         }
     } else if (warp < PW_WARP_E0) {
         // ---------------- expand the packed planes ---------------------------------
-        const int tid = threadIdx.x - PW_WARP_A0 * 32;
-        constexpr int NT = PW_A_WARPS * 32;
-        int ss = 0, slot = 0, pl = 0;
-        uint32_t phs = 0, pha = 0;
+        const int group = (warp - PW_WARP_A0) / PW_A_GROUP;
+        const int tid = threadIdx.x - (PW_WARP_A0 + group * PW_A_GROUP) * 32;
+        constexpr int NT = PW_A_GROUP * 32;
+        // own fills: g = group, group + 2, ...; slot = group
+        const int slot = group;
+        int ss = 0, pl = group;
+        while (pl >= p.planes) { pl -= p.planes; ++ss; }
+        ss %= p.stages;
+        uint32_t phs = (uint32_t)((group / p.planes) / p.stages) & 1u, pha = 0;
+        // first task (pixel, packed chunk) of this thread and the step to its next, in
+        // a full plane and in the last one
+        const int ch_full = p.PB / 16, ch_last = (p.P - (p.planes - 1) * p.PB) / 16;
+        const int row_f = tid / ch_full, row_l = tid / ch_last, dr_f = NT / ch_full, dr_l = NT / ch_last;
         bool ok = true;
 #pragma unroll 1
-        for (uint32_t g = 0; ok && g < n_fills; ++g) {
+        for (uint32_t g = group; ok && g < n_fills; g += 2) {
             if (!(ok = wait_bar_warp(bar_st_full(ss), phs, ctl, 32))) break;
             if (!(ok = wait_bar_warp(bar_a_empty(slot), pha ^ 1u, ctl, 35))) break;
-            const uint32_t src = smem_u32(smem + L.a_stage) + ss * stage_bytes;
+            const uint32_t src = smem_u32(smem + L.a_stage) + ss * stage_bytes + pl * plane_at;
             const uint32_t dst = smem_u32(smem + L.a_slots) + slot * a_slot_bytes;
             if (BITS == 3) {
-                const int chunks = min(p.PB, p.P - pl * p.PB) / 16;
+                const int chunks = pl == p.planes - 1 ? ch_last : ch_full;
                 const int groups = pw_groups<BITS>(p, pl);
 #pragma unroll 1
                 for (int row = tid; row < tile_px; row += NT) {
@@ -311,18 +335,19 @@ dsq_pw_kernel(const __grid_constant__ CUtensorMap tmap_a, const PwParams p)
 #pragma unroll
                     for (int l = 0; l < 3; ++l) {
                         v[l] = make_uint4(0u, 0u, 0u, 0u);
-                        if (l < chunks) v[l] = lds_128(src + (uint32_t)(row * p.PB + 16 * l));
+                        if (l < chunks) v[l] = lds_128(src + row * px_bytes + 16u * l);
                     }
                     pw_store_row3<false>(dst + (uint32_t)row * 128u, row & 7, v, groups, 0u);
                 }
             } else {
                 // task = (pixel, packed chunk); a thread's next task is NT further
-                const int chunks = min(p.PB, p.P - pl * p.PB) / 16;
-                int row = tid / chunks, ch = tid - row * chunks;
-                const int d_row = NT / chunks, d_ch = NT - d_row * chunks;
+                const bool last = pl == p.planes - 1;
+                const int chunks = last ? ch_last : ch_full;
+                int row = last ? row_l : row_f, ch = tid - row * chunks;
+                const int d_row = last ? dr_l : dr_f, d_ch = NT - d_row * chunks;
 #pragma unroll 2
                 while (row < tile_px) {
-                    const uint4 v = lds_128(src + (uint32_t)(row * p.PB + 16 * ch));
+                    const uint4 v = lds_128(src + row * px_bytes + 16u * ch);
                     pw_store_chunk<BITS, false>(dst + (uint32_t)row * 128u, row & 7, ch, v, 0u);
                     row += d_row;
                     ch += d_ch;
@@ -335,77 +360,105 @@ dsq_pw_kernel(const __grid_constant__ CUtensorMap tmap_a, const PwParams p)
                 mbar_arrive(bar_a_full(slot));
                 mbar_arrive(bar_st_empty(ss));
             }
-            if (++pl == p.planes) pl = 0;
-            if (++ss == p.stages) { ss = 0; phs ^= 1u; }
-            if (++slot == PW_A_SLOTS) { slot = 0; pha ^= 1u; }
+            pha ^= 1u;
+            pl += 2;
+            while (pl >= p.planes) {
+                pl -= p.planes;
+                if (++ss == p.stages) { ss = 0; phs ^= 1u; }
+            }
         }
     } else {
         // ---------------- epilogue -------------------------------------------------
         const int quarter = warp & 3;
-        const int k = (warp - PW_WARP_E0) >> 2;
+        const int group = (warp - PW_WARP_E0) / PW_E_GROUP;
+        const int k = ((warp - PW_WARP_E0) % PW_E_GROUP) >> 2;
         const DsqLean lean = dsq_make_lean(p.e);
-        const int cols = min(p.BN, p.out_pitch * 8 / BITS - n_tile * p.BN);   // columns with a place in the row
-        const int col_units = (cols + 31) / 32;
+        // columns with a place in the output row; unit = 32 columns of a subtile, the
+        // subtiles of the same columns next to each other
+        const int cols = min(p.BN, p.out_pitch * 8 / BITS - n_tile * p.BN);
+        const int col_units = (cols + 31) / 32, units = col_units * p.mt;
+        const int u0 = k * units / PW_EPQ, u1 = (k + 1) * units / PW_EPQ;
+        const int j = lane & 3;                       // eight channels 8 j .. of the 32
+        unsigned long long sc[4], bi[4];
+        int cu_held = -1;
         bool ok = true;
 #pragma unroll 1
-        for (int it = 0; ok && it < my_tiles; ++it) {
-            const int as = it & 1;
-            const int m0 = (m_first + it * p.mstep) * tile_px + quarter * 32 + lane;
+        for (int it = group; ok && it < my_tiles; it += 2) {
+            const int as = group;                     // accumulator of the own tiles
+            const int m0 = (m_first + it * p.mstep) * tile_px + quarter * 32 + (lane >> 2);
             if (!(ok = wait_bar_warp(bar_acc_full(as), (it >> 1) & 1u, ctl, 36))) break;
             tc_fence_after_sync();
-            int mt = 0, cu = k;
-            while (cu >= col_units) { cu -= col_units; ++mt; }
+            int cu = u0 / p.mt, mt = u0 - cu * p.mt;
 #pragma unroll 1
-            while (mt < p.mt) {
-                const int m = m0 + mt * 128;
-                const int byte0 = (n_tile * p.BN + cu * 32) * BITS / 8;
-                uint32_t r[32], res[BITS];
+            for (int u = u0; u < u1; ++u) {
+                uint32_t r[2][16];
+                const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) +
+                                       (as * p.mt + mt) * p.BN + cu * 32;
                 __syncwarp();
-                tmem_ld_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (as * p.mt + mt) * p.BN +
-                                  cu * 32, r);
+                tmem_ld_16x256b_x4(taddr, r[0]);
+                tmem_ld_16x256b_x4(taddr + (16u << 16), r[1]);
+                // this lane's bytes of an output row: BITS bytes at byte0
+                const int byte0 = (n_tile * p.BN + cu * 32) * BITS / 8 + j * BITS;
+                const int mr = m0 + mt * 128;         // + 8 i: this lane's pixels
+                uint32_t res[4];
                 if (RES) {
 #pragma unroll
-                    for (int w = 0; w < BITS; ++w) {
-                        res[w] = 0u;
-                        if (m < p.M && byte0 + 4 * w < p.out_pitch)
-                            res[w] = __ldg(reinterpret_cast<const uint32_t *>(
-                                         p.e.residual + (int64_t)m * p.out_pitch + byte0) + w);
+                    for (int i = 0; i < 4; ++i) {
+                        res[i] = 0u;
+                        const uint8_t *rp = p.e.residual + (int64_t)(mr + 8 * i) * p.out_pitch + byte0;
+                        if (mr + 8 * i >= p.M || byte0 >= p.out_pitch) continue;
+                        if (BITS == 4) res[i] = __ldg(reinterpret_cast<const uint32_t *>(rp));
+                        else if (BITS == 2) res[i] = __ldg(reinterpret_cast<const uint16_t *>(rp));
+                        else {
+                            // three bytes; the row's last lane may reach past its pitch
+#pragma unroll
+                            for (int b = 0; b < 3; ++b)
+                                if (byte0 + b < p.out_pitch) res[i] |= (uint32_t)__ldg(rp + b) << (8 * b);
+                        }
                     }
+                }
+                if (cu != cu_held) {
+                    cu_held = cu;
+                    const ulonglong2 *s2 = reinterpret_cast<const ulonglong2 *>(sm_scale + cu * 32 + 8 * j);
+                    const ulonglong2 *b2 = reinterpret_cast<const ulonglong2 *>(sm_bias + cu * 32 + 8 * j);
+                    sc[0] = s2[0].x; sc[1] = s2[0].y; sc[2] = s2[1].x; sc[3] = s2[1].y;
+                    bi[0] = b2[0].x; bi[1] = b2[0].y; bi[2] = b2[1].x; bi[3] = b2[1].y;
                 }
                 tmem_ld_wait();
                 uint32_t cw[4];
 #pragma unroll
-                for (int h = 0; h < 4; ++h) {
-                    cw[h] = 0u;
-                    if (cu * 32 + 8 * h < cols)
-                        cw[h] = dsq_lean_codes8<BITS, RES>(
-                            r + 8 * h, sm_scale + cu * 32 + 8 * h, sm_bias + cu * 32 + 8 * h,
-                            !RES ? 0u : BITS == 4 ? res[h < BITS ? h : 0]
-                                      : BITS == 2 ? res[h / 2] >> (16 * (h & 1))
-                                      : __funnelshift_r(res[(24 * h) / 32],
-                                                        res[(24 * h) / 32 + 1 < BITS ? (24 * h) / 32 + 1 : 0],
-                                                        (24 * h) & 31),
-                            lean);
+                for (int i = 0; i < 4; ++i) {
+                    const uint32_t (&q)[16] = r[i >> 1];
+                    const int o = 2 * (i & 1);
+                    const uint32_t v[8] = {q[o],     q[o + 1], q[o + 4],  q[o + 5],
+                                           q[o + 8], q[o + 9], q[o + 12], q[o + 13]};
+                    cw[i] = dsq_lean_codes8<BITS, RES, LO>(v, sc, bi, RES ? res[i] : 0u, lean);
                 }
-                if (m < p.M) {
-                    uint32_t *dst = reinterpret_cast<uint32_t *>(p.e.y_codes + (int64_t)m * p.out_pitch +
-                                                                 byte0);
-                    if (BITS == 4) {
-                        *reinterpret_cast<uint4 *>(dst) = make_uint4(cw[0], cw[1], cw[2], cw[3]);
-                    } else if (BITS == 2) {
-                        *reinterpret_cast<uint2 *>(dst) =
-                            make_uint2(cw[0] | (cw[1] << 16), cw[2] | (cw[3] << 16));
-                    } else {
-                        dst[0] = cw[0] | (cw[1] << 24);
-                        if (byte0 + 4 < p.out_pitch) dst[1] = (cw[1] >> 8) | (cw[2] << 16);
-                        if (byte0 + 8 < p.out_pitch) dst[2] = (cw[2] >> 16) | (cw[3] << 8);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int m = mr + 8 * i;
+                    uint32_t word = cw[i];
+                    int at = byte0;
+                    bool live = m < p.M;
+                    if (BITS == 2) {
+                        // two lanes' half words
+                        word |= __shfl_down_sync(0xffffffffu, cw[i], 1) << 16;
+                        live &= (j & 1) == 0;
+                    } else if (BITS == 3) {
+                        // the four lanes' 3 x 4 bytes as three words
+                        const uint32_t nx = __shfl_down_sync(0xffffffffu, cw[i], 1);
+                        word = (cw[i] >> (8 * j)) | (nx << (24 - 8 * j));
+                        at = byte0 + j;
+                        live &= j < 3;
                     }
+                    uint8_t *row = p.e.y_codes + (int64_t)m * p.out_pitch;
+                    if (live && at < p.out_pitch) *reinterpret_cast<uint32_t *>(row + at) = word;
                     // (the last unit may end before the row's pitch does)
-                    if (BITS != 4 && cu == col_units - 1 && n_tile == p.n_tiles - 1)
-                        for (int b = 4 * BITS; byte0 + b < p.out_pitch; b += 4) dst[b / 4] = 0u;
+                    if (BITS != 4 && m < p.M && j == 0 && cu == col_units - 1 && n_tile == p.n_tiles - 1)
+                        for (int b = byte0 + 4 * BITS; b < p.out_pitch; b += 4)
+                            *reinterpret_cast<uint32_t *>(row + b) = 0u;
                 }
-                cu += PW_EPQ;
-                while (cu >= col_units) { cu -= col_units; ++mt; }
+                if (++mt == p.mt) { mt = 0; ++cu; }
             }
             tc_fence_before_sync();
             __syncwarp();
@@ -423,14 +476,24 @@ dsq_pw_kernel(const __grid_constant__ CUtensorMap tmap_a, const PwParams p)
     }
 }
 
-template <int BITS, bool RES>
+template <int BITS, bool RES, bool LO>
 int pw_launch(const CUtensorMap &ta, const PwParams &p, cudaStream_t s, int pdl)
 {
     static std::atomic<unsigned long long> configured{0ull};
-    const int st = dsq_allow_smem((const void *)dsq_pw_kernel<BITS, RES>, 227 * 1024, &configured);
+    const int st = dsq_allow_smem((const void *)dsq_pw_kernel<BITS, RES, LO>, 227 * 1024, &configured);
     if (st) return st;
-    return dsq_launch(dsq_pw_kernel<BITS, RES>, dim3(p.mstep * p.n_tiles), dim3(PW_THREADS),
+    return dsq_launch(dsq_pw_kernel<BITS, RES, LO>, dim3(p.mstep * p.n_tiles), dim3(PW_THREADS),
                       (size_t)p.smem_bytes, s, pdl, 0, ta, p);
+}
+
+template <int BITS>
+int pw_dispatch(const CUtensorMap &ta, const PwParams &p, cudaStream_t s, int pdl)
+{
+    if (p.e.rq.lo != 0.0f)
+        return p.e.residual ? pw_launch<BITS, true, true>(ta, p, s, pdl)
+                            : pw_launch<BITS, false, true>(ta, p, s, pdl);
+    return p.e.residual ? pw_launch<BITS, true, false>(ta, p, s, pdl)
+                        : pw_launch<BITS, false, false>(ta, p, s, pdl);
 }
 
 }  // namespace
@@ -455,7 +518,7 @@ int dsq_pointwise(const void *act_codes, const dsq_nhwc_t *shape, int bits, cons
     if (sms <= 0) return DSQ_ERR_CUDA;
 
     // Tiling: the cheapest in a model of the launch in clocks - per tile the slowest
-    // of epilogue (30 elements a clock), expansion and instructions (120 clocks
+    // of epilogue (25 elements a clock), expansion and instructions (120 clocks
     // each, whatever their N), plus the hand-offs; once per CTA its weights and the
     // fill of the pipeline.
     const int subtiles = (p.M + 127) / 128;
@@ -468,14 +531,15 @@ int dsq_pointwise(const void *act_codes, const dsq_nhwc_t *shape, int bits, cons
         for (int mt = 1; mt <= 4; mt *= 2) {
             if (2 * mt * bn > 512) break;
             int stages = PW_MAX_STAGES;
+            const int row_bytes = p.stride == 1 ? p.P : p.planes * p.PB;
             while (stages >= 2 &&
-                   pw_layout(mt, bn, p.planes, p.PB, stages).total + 1024 > 227u * 1024u)
+                   pw_layout(mt, bn, p.planes, row_bytes, stages).total + 1024 > 227u * 1024u)
                 --stages;
             if (stages < 2) break;
             const int m_tiles = (subtiles + mt - 1) / mt;
             const int mstep = m_tiles < sms / nt ? m_tiles : sms / nt;
             const int per_cta = (m_tiles + mstep - 1) / mstep;
-            const double epi = mt * 128.0 * bn / 30, expand = mt * 2.3 * p.P + 400.0 * p.planes,
+            const double epi = mt * 128.0 * bn / 25, expand = mt * 2.3 * p.P + 400.0 * p.planes,
                          mma = mt * groups * 120.0;
             double tile = epi > expand ? epi : expand;
             tile = (tile > mma ? tile : mma) + 300;
@@ -491,7 +555,8 @@ int dsq_pointwise(const void *act_codes, const dsq_nhwc_t *shape, int bits, cons
     p.tmem_cols = 32;
     while (p.tmem_cols < 2 * p.mt * p.BN) p.tmem_cols *= 2;
     p.box_rows = p.mt * 128 < 256 ? p.mt * 128 : 256;
-    p.L = pw_layout(p.mt, p.BN, p.planes, p.PB, p.stages);
+    p.L = pw_layout(p.mt, p.BN, p.planes, p.stride == 1 ? p.P : p.planes * p.PB, p.stages);
+    p.act = (const uint8_t *)act_codes;
     p.smem_bytes = (int)p.L.total + 1024;
     p.shift = e.half_offset ? 7 - bits : 8 - bits;
     p.orv = e.half_offset ? 0x01010101u << (7 - bits) : 0u;
@@ -501,19 +566,11 @@ int dsq_pointwise(const void *act_codes, const dsq_nhwc_t *shape, int bits, cons
     p.ws = (int *)workspace;
 
     CUtensorMap ta;
-    const cuuint64_t P = (cuuint64_t)p.P;
-    if (p.stride == 1) {
-        DsqEncodeTiledFn enc = dsq_encode_tiled_fn();
-        if (!enc) return DSQ_ERR_CUDA;
-        cuuint64_t dims[2] = {P, (cuuint64_t)p.M}, strides[1] = {P};
-        cuuint32_t box[2] = {(cuuint32_t)p.PB, (cuuint32_t)p.box_rows}, estr[2] = {1, 1};
-        if (enc(&ta, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void *>(act_codes), dims, strides,
-                box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return DSQ_ERR_CUDA;
-    } else {
+    std::memset(&ta, 0, sizeof(ta));
+    if (p.stride != 1) {
         DsqEncodeIm2colFn enc = dsq_encode_im2col_fn();
         if (!enc) return DSQ_ERR_CUDA;
+        const cuuint64_t P = (cuuint64_t)p.P;
         cuuint64_t dims[4] = {P, (cuuint64_t)shape->W, (cuuint64_t)shape->H, (cuuint64_t)shape->N};
         cuuint64_t strides[3] = {P, P * shape->W, P * shape->W * shape->H};
         int lower[2] = {0, 0}, upper[2] = {0, 0};
@@ -524,10 +581,9 @@ int dsq_pointwise(const void *act_codes, const dsq_nhwc_t *shape, int bits, cons
                 CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return DSQ_ERR_UNSUPPORTED;
     }
-    const bool res = e.residual != nullptr;
     switch (bits) {
-    case 2: return res ? pw_launch<2, true>(ta, p, stream, hooks.pdl) : pw_launch<2, false>(ta, p, stream, hooks.pdl);
-    case 3: return res ? pw_launch<3, true>(ta, p, stream, hooks.pdl) : pw_launch<3, false>(ta, p, stream, hooks.pdl);
-    default: return res ? pw_launch<4, true>(ta, p, stream, hooks.pdl) : pw_launch<4, false>(ta, p, stream, hooks.pdl);
+    case 2: return pw_dispatch<2>(ta, p, stream, hooks.pdl);
+    case 3: return pw_dispatch<3>(ta, p, stream, hooks.pdl);
+    default: return pw_dispatch<4>(ta, p, stream, hooks.pdl);
     }
 }
