@@ -42,6 +42,7 @@ constexpr int G8_STAGE_BYTES = 2 * G8_OP_BYTES;          // A then B
 constexpr int G8_WARP_TMA = 0, G8_WARP_MMA = 1, G8_WARP_TMEM = 2, G8_WARP_E0 = 4;
 constexpr int G8_E_WARPS = 8;                // per CTA: two per tensor-memory lane quarter
 constexpr int G8_THREADS = 32 * (G8_WARP_E0 + G8_E_WARPS);
+constexpr int G8_SMALL_M = 64;              // weight-only problems of at most this many rows: dsq_wgemm_small
 constexpr int G8_BARS = 2 * G8_STAGES + 4 + 1;
 constexpr int G8_SMEM = G8_STAGES * G8_STAGE_BYTES + 1024 /* alignment */ + 256 /* barriers */;
 
@@ -613,6 +614,9 @@ int dsq_wgemm_bf16(const void *X_bf16, const void *W_codes, int64_t M, int64_t N
     const size_t wp = round_up((size_t)K, 8) * 2;          // scratch row pitch in bytes
     if (ws_bytes < (size_t)(W16 - (uint8_t *)workspace) + round_up((size_t)N * wp, 1024))
         return DSQ_ERR_SIZE;
+    if (M <= G8_SMALL_M)
+        return dsq_wgemm_small(X_bf16, W_codes, M, N, K, bits, w_offset == 0.5f, col_scale, col_bias,
+                               Y_f32, (cudaStream_t)stream);
     const int pitch_in = (int)dsq_row_pitch(K, bits);
     const int64_t threads = N * (int64_t)(wp / 16);
     const unsigned blocks = (unsigned)((threads + 255) / 256);

@@ -82,6 +82,12 @@ DSQ_HIDDEN int dsq_gemm8_launch(const void *A_codes, const void *B_codes, int64_
                                 float *D_f32, void *workspace, void *scratch,
                                 cudaStream_t stream);
 
+// Weight-only GEMM for few rows (dsq_wgemm_small.cu): arguments as dsq_wgemm_bf16
+// after validation; no workspace.
+DSQ_HIDDEN int dsq_wgemm_small(const void *X, const void *W, int64_t M, int64_t N, int64_t K,
+                               int bits, int odd, const float *col_scale, const float *col_bias,
+                               float *Y, cudaStream_t stream);
+
 // Weights of 3x3 stride-1 pad-1 dense convolutions (2- and 4-bit, 64 or a
 // multiple of 128 input channels) are stored twice in the blob
 // dsq_pack_weights writes: the packed rows, and behind them (1024-byte
