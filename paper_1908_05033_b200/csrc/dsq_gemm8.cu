@@ -22,8 +22,11 @@
 // passes.
 //
 // Every mbarrier wait is bounded (see dsq_tc_common.cuh).
+#include <cuda_bf16.h>
+
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstdint>
 
 #include "dsq_common.cuh"
@@ -42,13 +45,13 @@ constexpr int G8_STAGE_BYTES = 2 * G8_OP_BYTES;          // A then B
 constexpr int G8_WARP_TMA = 0, G8_WARP_MMA = 1, G8_WARP_TMEM = 2, G8_WARP_E0 = 4;
 constexpr int G8_E_WARPS = 8;                // per CTA: two per tensor-memory lane quarter
 constexpr int G8_THREADS = 32 * (G8_WARP_E0 + G8_E_WARPS);
-constexpr int G8_SMALL_M = 64;              // weight-only problems of at most this many rows: dsq_wgemm_small
 constexpr int G8_BARS = 2 * G8_STAGES + 4 + 1;
 constexpr int G8_SMEM = G8_STAGES * G8_STAGE_BYTES + 1024 /* alignment */ + 256 /* barriers */;
 
 struct G8Params {
     int M, N;
     int m_tiles, n_tiles, kblocks;
+    int vec;                 // N is a multiple of 8: 32-byte stores
     uint32_t idesc;          // instruction descriptor (operand types, M = 256, N = 256)
     // integer problems: C = acc, D = (float)acc * row_scale[m]
     int32_t *C_i32;
@@ -63,7 +66,7 @@ struct G8Params {
 };
 
 // ---------------------------------------------------------------------------
-// pass 1: packed codes -> int8.  One thread per 16 codes (16 output bytes).
+// pass 1: packed codes -> int8 or bf16
 // ---------------------------------------------------------------------------
 // bytes (each < 2^BITS) -> two's-complement int8 of the BITS-bit signed code
 template <int BITS>
@@ -74,13 +77,18 @@ __device__ __forceinline__ uint32_t sign_extend_bytes(uint32_t x)
     return (((x ^ HALF) | 0x80808080u) - HALF) ^ 0x80808080u;
 }
 
-// 16 codes (2 BITS bytes at `src`) -> 16 bytes
+// Work item of every expansion: one 16-byte chunk of an output row (16 int8 or 8
+// bf16 values).  A warp's lanes take consecutive chunks of a row, so that it writes
+// 512 contiguous bytes (with 64 bytes a thread every store touched half sectors all
+// over, and the L2 took each sector twice); a thread does the same chunk of four
+// rows, their loads first.
+constexpr int EX_ROWS = 4, EX_THREADS = 256;
+
+// `BITS`-bit codes at bit 0 of a word, ascending -> one code per byte, four a word
 template <int BITS>
-__device__ __forceinline__ uint4 expand_chunk(const uint8_t *src, int bytes_left, bool is_signed)
+__device__ __forceinline__ void spread_bytes(const uint2 v, uint32_t (&o)[4])
 {
-    uint32_t o[4];
     if (BITS == 4) {
-        const uint2 v = __ldcs(reinterpret_cast<const uint2 *>(src));
         const uint32_t w[2] = {v.x, v.y};
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -88,143 +96,215 @@ __device__ __forceinline__ uint4 expand_chunk(const uint8_t *src, int bytes_left
             o[2 * h] = __byte_perm(lo, hi, 0x5140);       // codes 0..3 of the word
             o[2 * h + 1] = __byte_perm(lo, hi, 0x7362);   // codes 4..7
         }
-    } else if (BITS == 2) {
-        const uint32_t v = __ldcs(reinterpret_cast<const uint32_t *>(src));
+    } else if (BITS == 3) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const uint32_t x = (v >> (8 * j)) & 0xFFu;    // four codes
+            const uint32_t x = __funnelshift_r(v.x, v.y, 12 * j) >> (j == 3 ? 4 : 0);
+            const uint32_t y = j == 3 ? v.y >> 4 : x;     // bits 12 j .. 12 j + 11
+            o[j] = (y & 7u) | ((y & 0x38u) << 5) | ((y & 0x1C0u) << 10) | ((y & 0xE00u) << 15);
+        }
+    } else if (BITS == 2) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t x = (v.x >> (8 * j)) & 0xFFu;  // four codes
             o[j] = (x | (x << 6) | (x << 12) | (x << 18)) & 0x03030303u;
         }
     } else {
-        // 16 codes of 3 bits = 6 bytes at an even offset; a row's last chunk may
-        // reach past the row pitch: those bytes are not read
-        uint64_t v = 0;
 #pragma unroll
-        for (int j = 0; j < 3; ++j)
-            if (2 * j < bytes_left)
-                v |= (uint64_t) * reinterpret_cast<const uint16_t *>(src + 2 * j) << (16 * j);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            uint32_t x = 0;
-#pragma unroll
-            for (int t = 0; t < 4; ++t)
-                x |= (uint32_t)((v >> (3 * (4 * j + t))) & 7u) << (8 * t);
-            o[j] = x;
-        }
+        for (int j = 0; j < 4; ++j)
+            o[j] = (((v.x >> (4 * j)) & 0xFu) * 0x00204081u) & 0x01010101u;
     }
-    if (is_signed) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) o[j] = sign_extend_bytes<BITS>(o[j]);
-    }
-    return make_uint4(o[0], o[1], o[2], o[3]);
 }
 
-// One thread per four consecutive chunks of a row (64 output bytes).  Codes
-// past K inside a row's last chunk are spare bits of the packed row: zero.
+// the 2 BITS bytes of chunk c of a packed row (3-bit chunks start at any even byte:
+// the two or three aligned words they lie in, as far as the row goes)
 template <int BITS>
-__global__ void __launch_bounds__(256)
-expand_rows_kernel(const uint8_t *__restrict__ A, const uint8_t *__restrict__ B, int64_t M,
-                   int64_t N, int pitch_in, int pitch_out, uint8_t *__restrict__ A8,
-                   uint8_t *__restrict__ B8)
+__device__ __forceinline__ uint2 load_chunk(const uint8_t *row, int c, int pitch)
 {
-    // lets the second pass (queued behind with programmatic dependent launch)
-    // set itself up while this grid runs; it waits for this grid to complete
-    // before its first copy
+    if (BITS == 4) return __ldg(reinterpret_cast<const uint2 *>(row) + c);
+    if (BITS == 2) return make_uint2(__ldg(reinterpret_cast<const uint32_t *>(row) + c), 0u);
+    if (BITS == 1) return make_uint2(__ldg(reinterpret_cast<const uint16_t *>(row) + c), 0u);
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(row);
+    const int i = (6 * c) >> 2, last = pitch / 4 - 1, sh = 8 * ((6 * c) & 3);
+    const uint32_t a = __ldg(w + i), b = __ldg(w + min(i + 1, last));
+    return make_uint2(__funnelshift_r(a, b, sh), b >> sh);
+}
+
+// Integer operands: rows of A then rows of B.  A's codes are signed, B's unsigned
+// (BITS = 1: both -1 / +1, positions past K 0 so that a row's tail adds nothing;
+// elsewhere the codes past K are spare bits of the packed row: zero).
+template <int BITS>
+__global__ void __launch_bounds__(EX_THREADS)
+expand_rows_kernel(const uint8_t *__restrict__ A, const uint8_t *__restrict__ B, int M, int N, int K,
+                   int pitch_in, int pitch_out, uint8_t *__restrict__ A8, uint8_t *__restrict__ B8)
+{
+    // lets the second pass (queued behind with programmatic dependent launch) set
+    // itself up while this grid runs; it waits for this grid before its first copy
     grid_launch_dependents();
-    const int cpr = pitch_out >> 4;                       // 16-byte chunks per output row
-    const int qpr = (cpr + 3) >> 2;                       // work items per row
-    const int64_t total = (M + N) * qpr;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t row = idx / qpr;
-        const int c0 = (int)(idx - row * qpr) * 4;
-        const bool is_a = row < M;                        // A: signed codes, B: unsigned
-        const uint8_t *src = is_a ? A + row * pitch_in : B + (row - M) * pitch_in;
-        uint8_t *dst = is_a ? A8 + row * pitch_out : B8 + (row - M) * pitch_out;
-        uint4 o[4];
+    const int c = blockIdx.x * EX_THREADS + threadIdx.x;
+    if (16 * c >= pitch_out) return;
+    for (int r0 = blockIdx.y * EX_ROWS; r0 < M + N; r0 += gridDim.y * EX_ROWS) {
+        uint2 v[EX_ROWS];
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (c0 + j < cpr)
-                o[j] = expand_chunk<BITS>(src + (c0 + j) * (2 * BITS),
-                                          pitch_in - (c0 + j) * (2 * BITS), is_a);
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (c0 + j < cpr) *reinterpret_cast<uint4 *>(dst + (c0 + j) * 16) = o[j];
-    }
-}
-
-// Binary operands (Eq. 1): bit 1 -> +1, bit 0 -> -1; positions past K -> 0, so
-// the row tail adds nothing.  One thread per 16 codes of either operand.
-__global__ void __launch_bounds__(256)
-expand_binary_kernel(const uint8_t *__restrict__ A, const uint8_t *__restrict__ B, int64_t M,
-                     int64_t N, int K, int pitch_in, int pitch_out, uint8_t *__restrict__ A8,
-                     uint8_t *__restrict__ B8)
-{
-    const int cpr = pitch_out >> 4;
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t row = idx / cpr;
-    const int c = (int)(idx - row * cpr);
-    if (row >= M + N) return;
-    const bool is_a = row < M;
-    const uint8_t *src = (is_a ? A + row * pitch_in : B + (row - M) * pitch_in) + 2 * c;
-    const uint32_t v = *reinterpret_cast<const uint16_t *>(src);
-    uint32_t o[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        // four bits -> the low bits of four bytes, then 2 x - 1 per byte
-        const uint32_t x = (((v >> (4 * j)) & 0xFu) * 0x00204081u) & 0x01010101u;
-        uint32_t y = (((x << 1) | 0x80808080u) - 0x01010101u) ^ 0x80808080u;
-        const int left = K - (16 * c + 4 * j);            // codes of this word inside the row
-        if (left < 4) y = left <= 0 ? 0u : (y & (0xFFFFFFFFu >> (8 * (4 - left))));
-        o[j] = y;
-    }
-    uint8_t *dst = (is_a ? A8 + row * pitch_out : B8 + (row - M) * pitch_out) + c * 16;
-    *reinterpret_cast<uint4 *>(dst) = make_uint4(o[0], o[1], o[2], o[3]);
-}
-
-// Weight codes -> bf16: value 2c + 1 (grid Delta (c + 1/2), `odd` != 0) or c, c
-// the signed BITS-bit code; positions past K -> 0.  One thread per 8 codes
-// (BITS input bytes, 16 output bytes).
-template <int BITS>
-__global__ void __launch_bounds__(256)
-expand_w_bf16_kernel(const uint8_t *__restrict__ W, int64_t N, int K, int pitch_in, int pitch_out,
-                     int odd, uint8_t *__restrict__ W16)
-{
-    const int cpr = pitch_out >> 4;
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t row = idx / cpr;
-    const int c = (int)(idx - row * cpr);
-    if (row >= N) return;
-    const uint8_t *src = W + row * pitch_in + c * BITS;
-    uint32_t v = 0;
-#pragma unroll
-    for (int j = 0; j < BITS; ++j)
-        if (c * BITS + j < pitch_in) v |= (uint32_t)src[j] << (8 * j);
-    uint32_t o[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        uint32_t pair = 0;
-#pragma unroll
-        for (int t = 0; t < 2; ++t) {
-            const int k = 8 * c + 2 * j + t;
-            int code = (int)((v >> (BITS * (2 * j + t))) & ((1u << BITS) - 1u));
-            if (code >> (BITS - 1)) code -= 1 << BITS;
-            const float f = k < K ? (float)(odd ? 2 * code + 1 : code) : 0.0f;
-            pair |= (__float_as_uint(f) >> 16) << (16 * t);    // small integers: exact in bf16
+        for (int i = 0; i < EX_ROWS; ++i) {
+            const int r = min(r0 + i, M + N - 1);
+            v[i] = load_chunk<BITS>(r < M ? A + (int64_t)r * pitch_in : B + (int64_t)(r - M) * pitch_in,
+                                    c, pitch_in);
         }
-        o[j] = pair;
+#pragma unroll
+        for (int i = 0; i < EX_ROWS; ++i) {
+            const int r = r0 + i;
+            if (r >= M + N) break;
+            uint32_t o[4];
+            spread_bytes<BITS>(v[i], o);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if (BITS == 1) {
+                    // 2 x - 1 per byte
+                    o[j] = (((o[j] << 1) | 0x80808080u) - 0x01010101u) ^ 0x80808080u;
+                    const int left = K - (16 * c + 4 * j);
+                    if (left < 4) o[j] = left <= 0 ? 0u : (o[j] & (0xFFFFFFFFu >> (8 * (4 - left))));
+                } else if (r < M) {
+                    o[j] = sign_extend_bytes<BITS>(o[j]);
+                }
+            }
+            uint8_t *dst = r < M ? A8 + (int64_t)r * pitch_out : B8 + (int64_t)(r - M) * pitch_out;
+            *reinterpret_cast<uint4 *>(dst + 16 * c) = make_uint4(o[0], o[1], o[2], o[3]);
+        }
     }
-    *reinterpret_cast<uint4 *>(W16 + row * pitch_out + c * 16) = make_uint4(o[0], o[1], o[2], o[3]);
+}
+
+// Weight codes -> bf16: value 2 c + 1 (grid Delta (c + 1/2), `odd`) or c, c the
+// signed BITS-bit code; K is a multiple of 8, a chunk of 8 values lies inside the
+// row.  By bit operations: the field (code ^ half) in the low mantissa bits of
+// 128.0 is 128 + field (128 + 2 field + 1), one subtraction leaves the value.
+template <int BITS>
+__global__ void __launch_bounds__(EX_THREADS)
+expand_w_bf16_kernel(const uint8_t *__restrict__ W, int N, int K, int pitch_in, int pitch_out, int odd,
+                     uint8_t *__restrict__ W16)
+{
+    grid_launch_dependents();
+    constexpr uint32_t F = (1u << BITS) - 1u, HALF = 1u << (BITS - 1);
+    const int c = blockIdx.x * EX_THREADS + threadIdx.x;
+    if (8 * c >= K) return;
+    const uint32_t flip = (0x4300u ^ (odd ? (HALF << 1) | 1u : HALF)) * 0x00010001u;
+    const uint32_t base = (0x4300u + (odd ? 2 * HALF : HALF)) * 0x00010001u;
+    const uint32_t mask = (odd ? F << 1 : F) * 0x00010001u;
+    for (int r0 = blockIdx.y * EX_ROWS; r0 < N; r0 += gridDim.y * EX_ROWS) {
+        uint32_t v[EX_ROWS];
+#pragma unroll
+        for (int i = 0; i < EX_ROWS; ++i) {
+            const uint8_t *row = W + (int64_t)min(r0 + i, N - 1) * pitch_in;
+            // eight codes: BITS bytes
+            if (BITS == 4) v[i] = __ldg(reinterpret_cast<const uint32_t *>(row) + c);
+            else if (BITS == 2) v[i] = __ldg(reinterpret_cast<const uint16_t *>(row) + c);
+            else if (BITS == 1) v[i] = __ldg(row + c);
+            else {
+                const uint32_t *w = reinterpret_cast<const uint32_t *>(row);
+                const int q = (3 * c) >> 2;
+                v[i] = __funnelshift_r(__ldg(w + q), __ldg(w + min(q + 1, pitch_in / 4 - 1)),
+                                       8 * ((3 * c) & 3));
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < EX_ROWS; ++i) {
+            if (r0 + i >= N) break;
+            // codes 0..3 in the low half, 4..7 in the high half
+            constexpr uint32_t LOW = BITS == 4 ? 0xFFFFu : (1u << (4 * BITS)) - 1u;
+            const uint32_t x = (v[i] & LOW) | ((v[i] << (16 - 4 * BITS)) & ~0xFFFFu);
+            uint32_t q[4];                                 // values (j, j + 4)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const uint32_t y = odd ? (j == 0 ? x << 1 : x >> (BITS * j - 1)) : x >> (BITS * j);
+                const uint32_t f = (y & mask) ^ flip;
+                const __nv_bfloat162 t = __hsub2(*reinterpret_cast<const __nv_bfloat162 *>(&f),
+                                                 *reinterpret_cast<const __nv_bfloat162 *>(&base));
+                q[j] = *reinterpret_cast<const uint32_t *>(&t);
+            }
+            *reinterpret_cast<uint4 *>(W16 + (int64_t)(r0 + i) * pitch_out + 16 * c) =
+                make_uint4(__byte_perm(q[0], q[1], 0x5410), __byte_perm(q[2], q[3], 0x5410),
+                           __byte_perm(q[0], q[1], 0x7632), __byte_perm(q[2], q[3], 0x7632));
+        }
+    }
+}
+
+// grid of an expansion: about eight resident blocks per SM
+inline dim3 expand_grid(int64_t chunks, int64_t rows)
+{
+    const int sms = dsq_sm_count() > 0 ? dsq_sm_count() : 148;
+    const int64_t gx = (chunks + EX_THREADS - 1) / EX_THREADS;
+    const int64_t gy = std::min<int64_t>((rows + EX_ROWS - 1) / EX_ROWS, std::max<int64_t>(8 * sms / gx, 1));
+    return dim3((unsigned)gx, (unsigned)gy);
 }
 
 // ---------------------------------------------------------------------------
 // pass 2: int8 GEMM, CTA pairs
 // ---------------------------------------------------------------------------
+// 32 lanes x 32 columns in the 16x256b shape: r[2 e], r[2 e + 1] are two adjacent
+// columns 8 ((e >> 1) & 3) + 2 (lane & 3) of row lane / 4 + 8 (e & 1) + 16 (e >> 3).
+// A store instruction then covers eight rows x 32 contiguous bytes.
+__device__ __forceinline__ void g8_load_pairs(uint32_t taddr, uint32_t (&r)[32])
+{
+    uint32_t lo[16], hi[16];
+    tmem_ld_16x256b_x4(taddr, lo);
+    tmem_ld_16x256b_x4(taddr + (16u << 16), hi);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) { r[i] = lo[i]; r[16 + i] = hi[i]; }
+}
+
+// outputs of such a block; m, n: this lane's first row and column
+template <bool F16>
+__device__ __forceinline__ void g8_store_pairs(const G8Params &p, int m, int n, const uint32_t (&r)[32])
+{
+    const bool even = (p.N & 1) == 0;      // (bases are 16-byte aligned: pairs at even offsets)
+    float cs[8], cb[8];
+    if (F16) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int c = min(n + 8 * (i >> 1) + (i & 1), p.N - 1);
+            cs[i] = __ldg(p.col_scale + c);
+            cb[i] = p.col_bias ? __ldg(p.col_bias + c) : 0.0f;
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+        const int row = m + 8 * (e & 1) + 16 * (e >> 3), b = (e >> 1) & 3, c = n + 8 * b;
+        if (row >= p.M || c >= p.N) continue;
+        const int64_t at = (int64_t)row * p.N + c;
+        const bool two = c + 1 < p.N;
+        auto put = [&](void *base, uint32_t x, uint32_t y) {
+            uint32_t *dst = reinterpret_cast<uint32_t *>(base) + at;
+            if (even) *reinterpret_cast<uint2 *>(dst) = make_uint2(x, y);
+            else {
+                dst[0] = x;
+                if (two) dst[1] = y;
+            }
+        };
+        if (F16) {
+            put(p.Y_f32, __float_as_uint(__fmaf_rn(__uint_as_float(r[2 * e]), cs[2 * b], cb[2 * b])),
+                __float_as_uint(__fmaf_rn(__uint_as_float(r[2 * e + 1]), cs[2 * b + 1], cb[2 * b + 1])));
+            continue;
+        }
+        if (p.C_i32) put(p.C_i32, r[2 * e], r[2 * e + 1]);
+        if (p.D_f32) {
+            const float rs = __ldg(p.row_scale + row);
+            put(p.D_f32, __float_as_uint(__fmul_rn((float)(int)r[2 * e], rs)),
+                __float_as_uint(__fmul_rn((float)(int)r[2 * e + 1], rs)));
+        }
+    }
+}
+
 // F16 = false: 8-bit integer operands, s32 accumulators (kind::i8);
 // F16 = true: bf16 operands, f32 accumulators (kind::f16).  A stage row is 128
 // bytes of K either way (128 or 64 elements), four instructions per stage.
-template <bool F16>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(G8_THREADS, 1)
+//
+// S > 1: few tiles and a long K.  A cluster is S pairs on ONE tile, pair s taking the
+// s-th part of K; when all are done, pair s gets the other pairs' partial sums of
+// columns s * 256 / S .. through distributed shared memory (into the stage ring,
+// which nothing reads any more), adds them to its own in a fixed order and writes
+// those columns.  One tile per cluster.
+template <bool F16, int S>
+__global__ void __launch_bounds__(G8_THREADS, 1)
 gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
              const __grid_constant__ CUtensorMap tmap_b, const G8Params p)
 {
@@ -236,7 +316,10 @@ gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(tail + 8 * G8_BARS);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tail + 8 * G8_BARS + 8);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t rank = cluster_ctarank();
+    const uint32_t crank = cluster_ctarank();
+    const uint32_t rank = crank & 1u, split = crank >> 1;       // in the pair; which part of K
+    const uint32_t leader = crank & ~1u;
+    const uint16_t pair_mask = (uint16_t)(3u << leader);
     Ctl ctl{abort_flag, p.ws, p.wait_ns};
 
     // full: operand bytes of BOTH CTAs' stage s have landed (counted on the
@@ -280,7 +363,9 @@ gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
     tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_slot;
 
-    const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
+    const int pair = blockIdx.x / (2 * S), npairs = gridDim.x / (2 * S);
+    const int kb0 = S == 1 ? 0 : (int)split * p.kblocks / S;
+    const int kb1 = S == 1 ? p.kblocks : ((int)split + 1) * p.kblocks / S;
     const int total_tiles = p.m_tiles * p.n_tiles;
     grid_dependency_wait();
 
@@ -292,10 +377,10 @@ gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
             for (int tile = pair; ok && tile < total_tiles; tile += npairs) {
                 const int m0 = (tile / p.n_tiles) * G8_BM + (int)rank * G8_ROWS;
                 const int n0 = (tile % p.n_tiles) * G8_BN + (int)rank * G8_ROWS;
-                for (int kb = 0; kb < p.kblocks; ++kb, ++g) {
+                for (int kb = kb0; kb < kb1; ++kb, ++g) {
                     const int s = g % G8_STAGES;
                     if (!(ok = wait_bar(bar_empty(s), ((g / G8_STAGES) & 1u) ^ 1u, ctl, 21))) break;
-                    const uint32_t full0 = map_to_cta(bar_full(s), 0u);
+                    const uint32_t full0 = map_to_cta(bar_full(s), leader);
                     if (rank == 0) mbar_arrive_expect_tx(bar_full(s), 2 * G8_STAGE_BYTES);
                     const uint32_t dst = smem_u32(smem + s * G8_STAGE_BYTES);
                     tma_load_2d_pair(dst, &tmap_a, kb * G8_KB, m0, full0);
@@ -320,7 +405,7 @@ gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
                     break;
                 tc_fence_after_sync();
                 const uint32_t d_tmem = tmem_base + b * G8_BN;
-                for (int kb = 0; kb < p.kblocks; ++kb, ++g) {
+                for (int kb = kb0; kb < kb1; ++kb, ++g) {
                     const int s = g % G8_STAGES;
                     if (!(ok = wait_bar_warp<true>(bar_full(s), (g / G8_STAGES) & 1u, ctl, 23)))
                         break;
@@ -331,14 +416,14 @@ gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
                     if (F16)
                         mma_f16_ss_pair_x4_elect(d_tmem, (uint32_t)ad, (uint32_t)(ad >> 32),
                                                  (uint32_t)bd, (uint32_t)(bd >> 32), idesc,
-                                                 (uint32_t)kb);
+                                                 (uint32_t)(kb - kb0));
                     else
                         mma_i8_ss_pair_x4_elect(d_tmem, (uint32_t)ad, (uint32_t)(ad >> 32),
                                                 (uint32_t)bd, (uint32_t)(bd >> 32), idesc,
-                                                (uint32_t)kb);
-                    mma_commit_pair_elect(bar_empty(s), (uint16_t)3);
+                                                (uint32_t)(kb - kb0));
+                    mma_commit_pair_elect(bar_empty(s), pair_mask);
                 }
-                if (ok) mma_commit_pair_elect(bar_acc_full(b), (uint16_t)3);
+                if (ok) mma_commit_pair_elect(bar_acc_full(b), pair_mask);
             }
             if (!ok) {
                 // instructions already issued still read shared memory and write
@@ -347,6 +432,9 @@ gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
                 wait_bar_drain(bar_drain, 0u);
             }
         }
+    } else if (S > 1 && warp >= G8_WARP_E0) {
+        // (the exchange below starts when every pair's instructions are done)
+        wait_bar_warp(bar_acc_full(0), 0u, ctl, 24);
     } else if (warp >= G8_WARP_E0) {
         // ---------------- epilogue: eight warps per CTA ----------------------
         const int quarter = warp & 3;                      // tensor-memory lane quarter
@@ -360,76 +448,114 @@ gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
             if (!(ok = wait_bar_warp(bar_acc_full(b), (it >> 1) & 1u, ctl, 24))) break;
             tc_fence_after_sync();
             const float rs = (!F16 && p.D_f32 && m < p.M) ? __ldg(p.row_scale + m) : 0.0f;
+            const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + b * G8_BN + half * 128;
 #pragma unroll 1
             for (int c0 = 0; c0 < 128; c0 += 32) {
                 uint32_t r[32];
-                tmem_ld_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + b * G8_BN +
-                                  half * 128 + c0,
-                              r);
+                if (p.vec) tmem_ld_32x32(taddr + c0, r);
+                else g8_load_pairs(taddr + c0, r);
                 tmem_ld_wait();
                 if (c0 == 96) {
                     // the accumulator is in registers: hand it back
                     tc_fence_before_sync();
                     __syncwarp();
                     if (lane == 0) {
-                        if (rank != 0) mbar_arrive_cluster(map_to_cta(bar_acc_empty(b), 0u));
+                        if (rank != 0) mbar_arrive_cluster(map_to_cta(bar_acc_empty(b), leader));
                         else mbar_arrive(bar_acc_empty(b));
                     }
                 }
                 const int n = n0 + c0;
-                if (m >= p.M || n >= p.N) continue;
-                const int64_t at = (int64_t)m * p.N + n;
-                if (F16) {
-                    // Y = fma(acc, col_scale[n], col_bias[n])
-                    const bool vec = n + 32 <= p.N &&
-                                     (reinterpret_cast<uintptr_t>(p.Y_f32 + at) & 31u) == 0;
-#pragma unroll
-                    for (int j = 0; j < 32; j += 8) {
-                        uint32_t f[8];
-#pragma unroll
-                        for (int t = 0; t < 8; ++t) {
-                            const int nn = min(n + j + t, p.N - 1);
-                            const float cb = p.col_bias ? __ldg(p.col_bias + nn) : 0.0f;
-                            f[t] = __float_as_uint(
-                                __fmaf_rn(__uint_as_float(r[j + t]), __ldg(p.col_scale + nn), cb));
-                        }
-                        if (vec)
-                            stg_256(p.Y_f32 + at + j, f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7]);
-                        else
-                            for (int t = 0; t < 8 && n + j + t < p.N; ++t)
-                                p.Y_f32[at + j + t] = __uint_as_float(f[t]);
-                    }
+                if (!p.vec) {
+                    g8_store_pairs<F16>(p, m - lane + (lane >> 2), n + 2 * (lane & 3), r);
                     continue;
                 }
-                const bool vec =
-                    n + 32 <= p.N &&
-                    (!p.C_i32 || (reinterpret_cast<uintptr_t>(p.C_i32 + at) & 31u) == 0) &&
-                    (!p.D_f32 || (reinterpret_cast<uintptr_t>(p.D_f32 + at) & 31u) == 0);
-                if (vec) {
-                    if (p.C_i32) {
-                        int32_t *dst = p.C_i32 + at;
+                // N is a multiple of 8: every group of eight columns of a row is a full
+                // 32-byte sector, inside or outside the matrix as a whole
+                if (m >= p.M || n >= p.N) continue;
+                const int64_t at = (int64_t)m * p.N + n;
 #pragma unroll
-                        for (int j = 0; j < 32; j += 8)
-                            stg_256(dst + j, r[j], r[j + 1], r[j + 2], r[j + 3], r[j + 4], r[j + 5],
-                                    r[j + 6], r[j + 7]);
+                for (int j = 0; j < 32; j += 8) {
+                    if (n + j >= p.N) break;
+                    uint32_t f[8];
+                    if (F16) {
+#pragma unroll
+                        for (int t = 0; t < 8; ++t)
+                            f[t] = __float_as_uint(
+                                __fmaf_rn(__uint_as_float(r[j + t]), __ldg(p.col_scale + n + j + t),
+                                          p.col_bias ? __ldg(p.col_bias + n + j + t) : 0.0f));
+                        stg_256(p.Y_f32 + at + j, f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7]);
+                        continue;
                     }
+                    if (p.C_i32)
+                        stg_256(p.C_i32 + at + j, r[j], r[j + 1], r[j + 2], r[j + 3], r[j + 4], r[j + 5],
+                                r[j + 6], r[j + 7]);
                     if (p.D_f32) {
-                        float *dst = p.D_f32 + at;
 #pragma unroll
-                        for (int j = 0; j < 32; j += 8) {
-                            uint32_t f[8];
-#pragma unroll
-                            for (int t = 0; t < 8; ++t)
-                                f[t] = __float_as_uint(__fmul_rn((float)(int)r[j + t], rs));
-                            stg_256(dst + j, f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7]);
-                        }
-                    }
-                } else {
-                    for (int j = 0; j < 32 && n + j < p.N; ++j) {
-                        if (p.C_i32) p.C_i32[at + j] = (int)r[j];
-                        if (p.D_f32) p.D_f32[at + j] = __fmul_rn((float)(int)r[j], rs);
+                        for (int t = 0; t < 8; ++t)
+                            f[t] = __float_as_uint(__fmul_rn((float)(int)r[j + t], rs));
+                        stg_256(p.D_f32 + at + j, f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7]);
                     }
                 }
+            }
+        }
+    }
+
+    if (S > 1) {
+        // ---------------- exchange of the partial sums --------------------------
+        constexpr int COLS = G8_BN / S;                    // columns a pair writes
+        constexpr uint32_t BLOCK = 128u * COLS * 4u;       // one pair's sums of them, 128 rows
+        // [row][COLS] words, 16-byte units XOR-ed with the row: conflict-free for a
+        // lane per row and for eight rows per load
+        auto unit = [](int row, int u) { return (uint32_t)(row * (COLS * 4) + ((u ^ (row & 7)) << 4)); };
+        const int quarter = warp & 3, k = (warp - G8_WARP_E0) >> 2;
+        const uint32_t ring = smem_u32(smem);
+        const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16);
+        tc_fence_after_sync();
+        __syncwarp();
+        cluster_sync_all();                                // every pair's instructions are done
+        if (warp >= G8_WARP_E0) {
+            const int row = quarter * 32 + lane;
+#pragma unroll 1
+            for (int c0 = 32 * k; c0 < G8_BN; c0 += 64) {
+                const uint32_t d = (uint32_t)c0 / COLS;    // the pair these columns belong to
+                if (d == split) continue;
+                uint32_t r[32];
+                tmem_ld_32x32(taddr + c0, r);
+                tmem_ld_wait();
+                const uint32_t dst = map_to_cta(ring, 2 * d + rank) + (split - (split > d)) * BLOCK;
+#pragma unroll
+                for (int v = 0; v < 8; ++v)
+                    st_cluster_128(dst + unit(row, (c0 % COLS) / 4 + v), r[4 * v], r[4 * v + 1],
+                                   r[4 * v + 2], r[4 * v + 3]);
+            }
+        }
+        __syncwarp();
+        cluster_sync_all();
+        if (warp >= G8_WARP_E0 && pair < total_tiles) {
+            const int row = quarter * 32 + (lane >> 2), j = lane & 3;
+            const int m = (pair / p.n_tiles) * G8_BM + (int)rank * G8_ROWS + row;
+            const int n0 = (pair % p.n_tiles) * G8_BN + (int)split * COLS;
+#pragma unroll 1
+            for (int c0 = 32 * k; c0 < COLS; c0 += 64) {
+                uint32_t r[32];
+                g8_load_pairs(taddr + split * COLS + c0, r);
+                tmem_ld_wait();
+#pragma unroll
+                for (int o = 0; o < S - 1; ++o)
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) {
+                        // r[2 e], r[2 e + 1]: row + 8 (e & 1) + 16 (e >> 3), columns of block (e >> 1) & 3
+                        const int rr = row + 8 * (e & 1) + 16 * (e >> 3), cc = c0 + 8 * ((e >> 1) & 3) + 2 * j;
+                        const uint2 v = lds_64(ring + o * BLOCK + unit(rr, cc >> 2) + 4 * (cc & 3));
+                        if (F16) {
+                            r[2 * e] = __float_as_uint(__uint_as_float(r[2 * e]) + __uint_as_float(v.x));
+                            r[2 * e + 1] = __float_as_uint(__uint_as_float(r[2 * e + 1]) + __uint_as_float(v.y));
+                        } else {
+                            r[2 * e] += v.x;
+                            r[2 * e + 1] += v.y;
+                        }
+                    }
+                g8_store_pairs<F16>(p, m, n0 + c0 + 2 * j, r);
             }
         }
     }
@@ -464,6 +590,50 @@ int make_rows128_tmap(CUtensorMap *map, const void *base, uint64_t k_bytes, uint
 
 inline size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
+template <bool F16, int S>
+int launch_split(const CUtensorMap &ta, const CUtensorMap &tb, const G8Params &p, int clusters,
+                 cudaStream_t stream)
+{
+    static std::atomic<unsigned long long> configured{0};
+    const int st = dsq_allow_smem((const void *)gemm8_kernel<F16, S>, G8_SMEM, &configured);
+    if (st) return st;
+    // (dependent launch: set-up overlaps the tail of pass 1; the kernel waits for it
+    // itself before the first copy)
+    return dsq_launch(gemm8_kernel<F16, S>, dim3(2 * S * clusters), dim3(G8_THREADS), (size_t)G8_SMEM,
+                      stream, dsq_launch_hooks().pdl, 2 * S, ta, tb, p);
+}
+
+// Clusters of S pairs that fit on the GPU at once (a cluster lives inside one group
+// of SMs, so this is less than SMs / 2 S).
+template <bool F16, int S>
+int resident_clusters()
+{
+    static std::atomic<int> cached[DSQ_MAX_DEVICES];
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= DSQ_MAX_DEVICES) return 0;
+    int n = cached[dev].load(std::memory_order_relaxed);
+    if (n) return n;
+    if (cudaFuncSetAttribute(gemm8_kernel<F16, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, G8_SMEM) !=
+        cudaSuccess)
+        return 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * S);
+    cfg.blockDim = dim3(G8_THREADS);
+    cfg.dynamicSmemBytes = G8_SMEM;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2 * S;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&n, gemm8_kernel<F16, S>, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        n = 0;
+    }
+    cached[dev].store(n, std::memory_order_relaxed);
+    return n;
+}
+
 // Pass 2 over operands that are rows of k_bytes bytes of K (byte maps: the
 // kernel never looks at an element, only the tensor core does).
 template <bool F16>
@@ -481,22 +651,18 @@ int launch_pass2(const void *A, size_t a_pitch, const void *B, size_t b_pitch, s
     st = make_rows128_tmap(&tb, B, k_bytes, (uint64_t)N, b_pitch);
     if (st) return st;
 
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= DSQ_MAX_DEVICES) return DSQ_ERR_CUDA;
-    static std::atomic<unsigned long long> configured{0};
-    if (!(configured.load() >> dev & 1ull)) {
-        if (cudaFuncSetAttribute(gemm8_kernel<F16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 G8_SMEM) != cudaSuccess)
-            return DSQ_ERR_CUDA;
-        configured.fetch_or(1ull << dev);
-    }
+    p.vec = N % 8 == 0 && (!p.C_i32 || (reinterpret_cast<uintptr_t>(p.C_i32) & 31u) == 0) &&
+            (!p.D_f32 || (reinterpret_cast<uintptr_t>(p.D_f32) & 31u) == 0) &&
+            (!p.Y_f32 || (reinterpret_cast<uintptr_t>(p.Y_f32) & 31u) == 0);
     const int sms = dsq_sm_count() > 0 ? dsq_sm_count() : 148;
-    const int pairs = std::min(sms / 2, p.m_tiles * p.n_tiles);
-    // (dependent launch: set-up overlaps the tail of pass 1; the kernel waits for
-    // it itself before the first copy.  The cluster of two is the kernel's own
-    // attribute.)
-    return dsq_launch(gemm8_kernel<F16>, dim3(2 * pairs), dim3(G8_THREADS), (size_t)G8_SMEM, stream,
-                      dsq_launch_hooks().pdl, 0, ta, tb, p);
+    const int tiles = p.m_tiles * p.n_tiles;
+    // K split over the two pairs of a cluster where all the tiles' clusters are resident
+    // at once (33 of them) and a part still has twelve K blocks: the exchange costs
+    // about as much as eight.  (Four pairs a cluster gained nothing more: 15 such
+    // clusters are resident and the exchange doubles.)
+    if (p.kblocks >= 24 && tiles <= sms / 4 && tiles <= resident_clusters<F16, 2>())
+        return launch_split<F16, 2>(ta, tb, p, tiles, stream);
+    return launch_split<F16, 1>(ta, tb, p, std::min(sms / 2, tiles), stream);
 }
 
 // first 1024-byte boundary behind the status words of a caller workspace
@@ -510,12 +676,11 @@ inline uint8_t *scratch_of(void *workspace)
 
 // Scratch the two-pass path needs behind the status words (0: the problem is
 // one the fused kernel keeps).
-size_t dsq_gemm8_scratch_bytes(int64_t M, int64_t N, int64_t K, int force)
+size_t dsq_gemm8_scratch_bytes(int64_t M, int64_t N, int64_t K, int bits, int force)
 {
-    // below this the fused kernel's single launch wins (measured: 2048^3 takes
-    // 22.5 us fused and 25.6 us in two passes, 4096^3 85 and 71 us)
-    if (!force && (M < 1024 || N < 1024 || K < 1024 ||
-                   (double)M * (double)N * (double)K < 34359738368.0 /* 2^35 */))
+    const double work = (double)M * (double)N * (double)K;
+    if (!force && (M < 256 || N < 256 || K < 256 || work <= (bits == 3 ? 134217728.0 /* 2^27 */
+                                                                       : 8589934592.0 /* 2^33 */)))
         return 0;
     const size_t kp = round_up((size_t)K, 16);
     return round_up((size_t)M * kp, 1024) + round_up((size_t)N * kp, 1024);
@@ -530,16 +695,12 @@ int dsq_gemm8_launch(const void *A_codes, const void *B_codes, int64_t M, int64_
     uint8_t *A8 = (uint8_t *)scratch;
     uint8_t *B8 = A8 + round_up((size_t)M * kp, 1024);
     const int pitch_in = (int)dsq_row_pitch(K, bits);
-    const int64_t threads = (M + N) * (int64_t)((kp / 16 + 3) / 4);
-    const int sms = dsq_sm_count() > 0 ? dsq_sm_count() : 148;
-    // whole waves of resident blocks (8 per SM), a few items per thread
-    const unsigned blocks = (unsigned)std::min<int64_t>((threads + 255) / 256, (int64_t)sms * 8);
     const uint8_t *A = (const uint8_t *)A_codes, *B = (const uint8_t *)B_codes;
     const int st = dsq_launch(bits == 2   ? expand_rows_kernel<2>
                               : bits == 3 ? expand_rows_kernel<3>
                                           : expand_rows_kernel<4>,
-                              dim3(blocks), dim3(256), 0, stream, 0, 0, A, B, M, N, pitch_in,
-                              (int)kp, A8, B8);
+                              expand_grid((int64_t)kp / 16, M + N), dim3(EX_THREADS), 0, stream, 0, 0,
+                              A, B, (int)M, (int)N, (int)K, pitch_in, (int)kp, A8, B8);
     if (st) return st;
     G8Params p = {};
     p.idesc = idesc_i8(G8_BN, true, false, G8_BM);
@@ -575,11 +736,10 @@ int dsq_binary_gemm(const void *A_bits, const void *B_bits, int64_t M, int64_t N
     const size_t need = round_up((size_t)M * kp, 1024) + round_up((size_t)N * kp, 1024);
     if (ws_bytes < (size_t)(scratch - (uint8_t *)workspace) + need) return DSQ_ERR_SIZE;
     uint8_t *A8 = scratch, *B8 = scratch + round_up((size_t)M * kp, 1024);
-    const int64_t threads = (M + N) * (int64_t)(kp / 16);
-    const int st = dsq_launch(expand_binary_kernel, dim3((unsigned)((threads + 255) / 256)),
-                              dim3(256), 0, (cudaStream_t)stream, 0, 0, (const uint8_t *)A_bits,
-                              (const uint8_t *)B_bits, M, N, (int)K, (int)dsq_row_pitch(K, 1),
-                              (int)kp, A8, B8);
+    const int st = dsq_launch(expand_rows_kernel<1>, expand_grid((int64_t)kp / 16, M + N),
+                              dim3(EX_THREADS), 0, (cudaStream_t)stream, 0, 0, (const uint8_t *)A_bits,
+                              (const uint8_t *)B_bits, (int)M, (int)N, (int)K,
+                              (int)dsq_row_pitch(K, 1), (int)kp, A8, B8);
     if (st) return st;
     G8Params p = {};
     p.idesc = idesc_i8(G8_BN, true, true, G8_BM);
@@ -591,6 +751,22 @@ int dsq_binary_gemm(const void *A_bits, const void *B_bits, int64_t M, int64_t N
 // ---------------------------------------------------------------------------
 // weight-only low-bit GEMM: bf16 activations x b-bit weights
 // ---------------------------------------------------------------------------
+// Whether dsq_wgemm_small takes the problem: always up to 64 rows (23 us against 24
+// at 64 x 4096 x 4096, 6 against 24 at 16 rows), and beyond while its launch - waves
+// of blocks of 64 x 16 outputs, 2.6 us for every 1024 of K (measured) - is shorter
+// than the two passes: 9 us of launches and set-up, the expansion, 0.27 us a K block.
+static bool wgemm_prefers_small(int64_t M, int64_t N, int64_t K)
+{
+    if (M <= 64) return true;
+    const int sms = dsq_sm_count() > 0 ? dsq_sm_count() : 148;
+    const double blocks = (double)((N + 15) / 16) * (double)((M + 63) / 64);
+    const double small = 2.2 + std::ceil(blocks / sms) * (double)((K + 1023) / 1024) * 2.6;
+    const double tiles = (double)((M + G8_BM - 1) / G8_BM) * (double)((N + G8_BN - 1) / G8_BN);
+    const double kb = (double)((K + 63) / 64);
+    const double main_loop = (tiles <= 33 && kb >= 24 ? 0.5 : std::ceil(tiles / (sms / 2))) * kb * 0.27;
+    return small < 9.0 + 5.2e-7 * (double)N * (double)K + main_loop;
+}
+
 size_t dsq_wgemm_workspace_bytes(int64_t N, int64_t K)
 {
     if (N <= 0 || K <= 0) return DSQ_WS_BYTES;
@@ -614,12 +790,10 @@ int dsq_wgemm_bf16(const void *X_bf16, const void *W_codes, int64_t M, int64_t N
     const size_t wp = round_up((size_t)K, 8) * 2;          // scratch row pitch in bytes
     if (ws_bytes < (size_t)(W16 - (uint8_t *)workspace) + round_up((size_t)N * wp, 1024))
         return DSQ_ERR_SIZE;
-    if (M <= G8_SMALL_M)
+    if (wgemm_prefers_small(M, N, K))
         return dsq_wgemm_small(X_bf16, W_codes, M, N, K, bits, w_offset == 0.5f, col_scale, col_bias,
                                Y_f32, (cudaStream_t)stream);
     const int pitch_in = (int)dsq_row_pitch(K, bits);
-    const int64_t threads = N * (int64_t)(wp / 16);
-    const unsigned blocks = (unsigned)((threads + 255) / 256);
     const int odd = w_offset == 0.5f;
     const uint8_t *W = (const uint8_t *)W_codes;
     cudaStream_t s = (cudaStream_t)stream;
@@ -627,8 +801,8 @@ int dsq_wgemm_bf16(const void *X_bf16, const void *W_codes, int64_t M, int64_t N
                               : bits == 2 ? expand_w_bf16_kernel<2>
                               : bits == 3 ? expand_w_bf16_kernel<3>
                                           : expand_w_bf16_kernel<4>,
-                              dim3(blocks), dim3(256), 0, s, 0, 0, W, N, (int)K, pitch_in, (int)wp,
-                              odd, W16);
+                              expand_grid(K / 8, N), dim3(EX_THREADS), 0, s, 0, 0, W, (int)N,
+                              (int)K, pitch_in, (int)wp, odd, W16);
     if (st) return st;
     G8Params p = {};
     p.idesc = idesc_bf16(G8_BN, G8_BM);

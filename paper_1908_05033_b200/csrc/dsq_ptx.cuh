@@ -162,6 +162,18 @@ __device__ __forceinline__ void sts_128(uint32_t addr, uint32_t a, uint32_t b, u
                  : "memory");
 }
 // 256-bit global store (one full 32-byte sector per lane); dst 32-byte aligned
+// 16 bytes into another CTA's shared memory (address from map_to_cta)
+__device__ __forceinline__ void st_cluster_128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d)
+                 : "memory");
+}
+__device__ __forceinline__ uint2 lds_64(uint32_t addr)
+{
+    uint2 v;
+    asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr));
+    return v;
+}
 __device__ __forceinline__ void stg_256(void *dst, uint32_t a, uint32_t b, uint32_t c, uint32_t d,
                                         uint32_t e, uint32_t f, uint32_t g, uint32_t h)
 {

@@ -1718,7 +1718,7 @@ size_t dsq_gemm_workspace_bytes(int64_t M, int64_t N, int64_t K, int bits)
 {
     if (bits < 2 || bits > 4 || M <= 0 || N <= 0 || K <= 0) return DSQ_WS_BYTES;
     const int mode = g_two_pass.load();
-    const size_t need = mode ? dsq_gemm8_scratch_bytes(M, N, K, mode == 2) : 0;
+    const size_t need = mode ? dsq_gemm8_scratch_bytes(M, N, K, bits, mode == 2) : 0;
     return need ? DSQ_WS_BYTES + 1024 + need : DSQ_WS_BYTES;
 }
 
@@ -1751,7 +1751,7 @@ int dsq_gemm(const void *A_codes, const void *B_codes, int64_t M, int64_t N, int
     // operands (dsq_gemm_workspace_bytes): expand every row once, then an
     // 8-bit GEMM fed by TMA alone
     const int two_pass = g_two_pass.load();
-    const size_t scratch_need = two_pass ? dsq_gemm8_scratch_bytes(M, N, K, two_pass == 2) : 0;
+    const size_t scratch_need = two_pass ? dsq_gemm8_scratch_bytes(M, N, K, bits, two_pass == 2) : 0;
     if (scratch_need) {
         const uintptr_t w0 = reinterpret_cast<uintptr_t>(workspace);
         const uintptr_t s0 = (w0 + DSQ_WS_BYTES + 1023u) & ~(uintptr_t)1023u;

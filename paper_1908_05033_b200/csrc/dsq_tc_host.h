@@ -76,7 +76,7 @@ static inline int dsq_allow_smem(const void *func, int bytes, std::atomic<unsign
 // force: whatever the size).
 // dsq_gemm8_launch: arguments as dsq_gemm after validation, `scratch`
 // 1024-byte aligned and at least that large.
-DSQ_HIDDEN size_t dsq_gemm8_scratch_bytes(int64_t M, int64_t N, int64_t K, int force);
+DSQ_HIDDEN size_t dsq_gemm8_scratch_bytes(int64_t M, int64_t N, int64_t K, int bits, int force);
 DSQ_HIDDEN int dsq_gemm8_launch(const void *A_codes, const void *B_codes, int64_t M, int64_t N,
                                 int64_t K, int bits, int32_t *C_i32, const float *row_scale,
                                 float *D_f32, void *workspace, void *scratch,
