@@ -678,10 +678,14 @@ inline uint8_t *scratch_of(void *workspace)
 // one the fused kernel keeps).
 size_t dsq_gemm8_scratch_bytes(int64_t M, int64_t N, int64_t K, int bits, int force)
 {
+    // Measured, fused / two passes in us: 4-bit 1500x1500x6000 (1.4e10) 22 / 31,
+    // 2048x2048x4096 (1.7e10) 22 / 21, 3072^3 33 / 26, 4096^3 75 / 52.  3-bit rows,
+    // which the fused kernel takes one K step a round: 1024^3 10.6 / 12, 128x6144x6144
+    // (4.8e9) 41 / 26, 2048^3 24 / 15.  Where N is not a multiple of 4 the fused
+    // kernel stores words: 4-bit 1023^2 outputs 11 / 16, 2500x1111 29 / 20.
     const double work = (double)M * (double)N * (double)K;
-    if (!force && (M < 256 || N < 256 || K < 256 || work <= (bits == 3 ? 134217728.0 /* 2^27 */
-                                                                       : 8589934592.0 /* 2^33 */)))
-        return 0;
+    const bool large = work >= (bits == 3 ? 1.5e9 : 1.5e10) || (N % 4 != 0 && (double)M * (double)N >= 1.5e6);
+    if (!force && (M < 128 || N < 128 || K < 128 || !large)) return 0;
     const size_t kp = round_up((size_t)K, 16);
     return round_up((size_t)M * kp, 1024) + round_up((size_t)N * kp, 1024);
 }
