@@ -56,6 +56,12 @@ DSQ_HIDDEN int dsq_pointwise(const void *act_codes, const dsq_nhwc_t *shape, int
                              const void *w_packed, const dsq_conv_t *conv, const DsqEpi &e,
                              void *workspace, cudaStream_t stream);
 
+// Dense convolution with little work (dsq_conv_small.cu).  Arguments as dsq_pointwise,
+// any outputs; lean: codes only, with a requantiser the lean epilogue takes.
+DSQ_HIDDEN int dsq_conv_small(const void *act_codes, const dsq_nhwc_t *shape, int bits,
+                              const void *w_packed, const dsq_conv_t *conv, const DsqEpi &e,
+                              int lean, cudaStream_t stream);
+
 // Opt-in to large dynamic shared memory, once per kernel and device (an attribute
 // of the function on a device): one bit per device ordinal in *configured.
 static inline int dsq_allow_smem(const void *func, int bytes, std::atomic<unsigned long long> *configured)
