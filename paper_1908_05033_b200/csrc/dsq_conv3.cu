@@ -113,6 +113,7 @@ struct W3Params {
     // (< Hp), padded columns (< Wp)
     int ld_dn[3], ld_dh[3], ld_dw[3];
     int smem_bytes;
+    int early;                         // dsq_early_constants
     unsigned long long wait_ns;
     int skip_b_round;
     int base_offset_mode;              // probe: put the row phase into the descriptor
@@ -370,9 +371,12 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
     // everything above touched no global data; nothing below starts before the
     // kernels ahead of this one in the stream have completed
     W3_STAMP(13, 1);
-    grid_launch_dependents();
-    // (the window producer first works out its coordinates, then waits)
-    if (warp != W3_WARP_TMA_A) grid_dependency_wait();
+    // (the window producer first works out its coordinates, then waits; the weights'
+    // producer does not wait where its constants may be read early)
+    if (warp != W3_WARP_TMA_A && !(warp == W3_WARP_TMA_B && p.early)) {
+        grid_dependency_wait();
+        grid_launch_dependents();
+    }
     W3_STAMP(13, 2);
 
     if (warp == W3_WARP_TMA_B) {
@@ -1317,6 +1321,7 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     }
     p.wait_ns = hooks.wait_ns;
     p.skip_b_round = hooks.skip_b_round;
+    p.early = dsq_early_constants();
     p.base_offset_mode = hooks.window3 == 2;   // (probe)
     p.e = e;
     p.r_hi = r_hi;

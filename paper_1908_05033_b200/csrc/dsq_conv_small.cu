@@ -37,6 +37,7 @@ struct CsParams {
     int upt, chunks;                  // units per tap; chunks of four units
     int units, d_tap, d_s;            // all units; a warp's step of 4 * warps units as taps, units
     int shift, out_pitch, lean;
+    int early;                        // dsq_early_constants
     uint32_t orv;
     DsqEpi e;
 };
@@ -91,7 +92,6 @@ conv_small_kernel(const CsParams p)
 {
     constexpr int WORDS = Unit<BITS>::WORDS, UNIT_BYTES = 4 * WORDS;
     extern __shared__ int4 part[];                    // [warp][MT * NT][lane]
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
     const int g = lane >> 2, j = lane & 3;
     const int n0 = blockIdx.x * 8 * NT, m0 = blockIdx.y * 16 * MT;
@@ -110,6 +110,7 @@ conv_small_kernel(const CsParams p)
             load_unit<BITS>(p.w + (int64_t)row * p.w_row + at, in && row < p.Ncols, p.P - s * UNIT_BYTES, wv[t]);
         }
     };
+    if (!p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
     load_w();
     // this lane's pixels (rows g and g + 8 of every tile): corner of the filter window
     int hb[MT][2], wb[MT][2], at0[MT][2];
@@ -150,6 +151,7 @@ conv_small_kernel(const CsParams p)
         }
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     uint32_t res = 0u;
     if (e.residual && mine && byte0 < p.out_pitch) {
         const uint8_t *rp = e.residual + (int64_t)px * p.out_pitch + byte0;
@@ -358,6 +360,7 @@ int dsq_conv_small(const void *act_codes, const dsq_nhwc_t *shape, int bits, con
     p.chunks = (p.units + 3) / 4;
     p.out_pitch = (int)dsq_row_pitch(conv->Cout, bits);
     p.lean = lean;
+    p.early = dsq_early_constants();
     p.shift = e.half_offset ? 7 - bits : 8 - bits;
     p.orv = e.half_offset ? 0x01010101u << (7 - bits) : 0u;
     p.e = e;

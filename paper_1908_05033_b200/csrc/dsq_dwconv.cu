@@ -187,6 +187,7 @@ struct DwHalf {
     int units;                // 8-channel units of a row, padding lanes included
     int strips, rows, chunks; // strips of four columns; output rows of a work item
     int half_offset;
+    int early;                // dsq_early_constants
     float inv;
 };
 
@@ -239,7 +240,6 @@ dwconv3x3_half_kernel(const uint8_t *__restrict__ act, const uint8_t *__restrict
                       const float *__restrict__ scale, const float *__restrict__ bias,
                       uint8_t *__restrict__ y_codes, const DwHalf p)
 {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     constexpr int OW = 4, NP = (OW - 1) * STRIDE + 3;
     const uint32_t gtid = blockIdx.x * DWH_THREADS + threadIdx.x;
     const uint32_t lanes = gridDim.x * DWH_THREADS / (uint32_t)p.units;   // exact (host)
@@ -247,7 +247,7 @@ dwconv3x3_half_kernel(const uint8_t *__restrict__ act, const uint8_t *__restrict
     const uint32_t per_img = (uint32_t)p.strips * p.chunks;
     const uint32_t n_items = per_img * (uint32_t)p.N;
     uint32_t item = gtid / (uint32_t)p.units;
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (!p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
 
     // weights as halves: c = (n ^ half) - half of the stored field n, or 2 c + 1;
     // 0x6400 | m is the half 1024 + m
@@ -282,6 +282,8 @@ dwconv3x3_half_kernel(const uint8_t *__restrict__ act, const uint8_t *__restrict
         }
     }
     const unsigned long long inv2 = dsq_pack2(p.inv, p.inv);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     for (; item < n_items; item += lanes) {
         const uint32_t n = item / per_img, rem = item - n * per_img;
@@ -421,6 +423,7 @@ extern "C" int dsq_dwconv2d(const void *act_codes, const dsq_nhwc_t *shape,
         p.units = units; p.strips = strips;
         p.half_offset = e.half_offset;
         p.inv = e.rq.inv;
+        p.early = dsq_early_constants();
         const int sms = dsq_sm_count() > 0 ? dsq_sm_count() : 148;
         // blocks: all resident, and a thread keeps its unit (blocks * 128 is a
         // multiple of `units`)

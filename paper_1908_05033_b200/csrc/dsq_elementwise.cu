@@ -2,6 +2,7 @@
 // (Algorithm 1 steps 1 and 3), weight quantise + pack, code pack / unpack,
 // 2x2 max-pool on codes.  All are HBM-bound streaming kernels.
 #include "dsq_common.cuh"
+#include "dsq_epilogue.cuh"
 #include "dsq_tc_host.h"
 
 namespace {
@@ -82,9 +83,9 @@ __global__ void __launch_bounds__(256)
 quantize_flat_kernel(const float4 *__restrict__ x, uint4 *__restrict__ out,
                      int64_t n_lines, DsqQ q)
 {
-    // lets a tensor-core kernel queued behind this one (programmatic dependent
-    // launch) set itself up while this grid runs; it still waits for this grid
-    // to complete before touching global data
+    // waits for the kernels ahead, then lets the one queued behind (programmatic
+    // dependent launch) start its set-up (in this order: see dsq_early_constants)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     constexpr int NF = (BITS == 4) ? 1 : 2;
     constexpr int F4_PER_LINE = 8 * NF;
@@ -158,9 +159,9 @@ __global__ void __launch_bounds__(256)
 quantize_rows_kernel(const float *__restrict__ x, uint32_t *__restrict__ out,
                      int64_t rows, int k, int pitch_words, int bits, DsqQ q)
 {
-    // lets a tensor-core kernel queued behind this one (programmatic dependent
-    // launch) set itself up while this grid runs; it still waits for this grid
-    // to complete before touching global data
+    // waits for the kernels ahead, then lets the one queued behind (programmatic
+    // dependent launch) start its set-up (in this order: see dsq_early_constants)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int64_t total = rows * pitch_words;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
@@ -170,6 +171,64 @@ quantize_rows_kernel(const float *__restrict__ x, uint32_t *__restrict__ out,
         const float *row = x + r * k;
         out[i] = build_word(wi, k, bits,
                             [&](int j) { return dsq_code(__ldg(row + j), q); });
+    }
+}
+
+// Activation quantise for 2- and 3-bit rows with padding behind the codes (and 3-bit
+// rows without): C a multiple of 32.  A lane takes eight elements (one 256-bit load),
+// four lanes of a group the 32 whose codes are whole words: the 3-bit pieces (24 bits)
+// are put together with one shuffle, the group's lanes write the words and the row's
+// spare bytes.  HBM-bound; quantize_rows_kernel, one thread per output word with a
+// chain of strided loads, took 4.2 times as long (64 channels, 3-bit).
+template <int BITS>
+__global__ void __launch_bounds__(256)
+quantize_groups_kernel(const float *__restrict__ x, uint32_t *__restrict__ out, int64_t groups,
+                       int groups_row, int pitch_words, DsqQ q)
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    constexpr int UNROLL = 4;
+    const int j = threadIdx.x & 3;
+    const unsigned long long inv2 = dsq_pack2(q.inv, q.inv), lo2 = dsq_pack2(-q.lo, -q.lo);
+    const int64_t step = (int64_t)gridDim.x * 64;
+    for (int64_t g0 = (int64_t)blockIdx.x * 64 + (threadIdx.x >> 2); g0 - (threadIdx.x >> 2) < groups;
+         g0 += step * UNROLL) {
+        float f[UNROLL][8];
+#pragma unroll
+        for (int i = 0; i < UNROLL; ++i) {
+            const int64_t g = g0 + i * step;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) f[i][k] = 0.f;
+            if (g < groups)
+                asm volatile("ld.global.nc.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                             : "=f"(f[i][0]), "=f"(f[i][1]), "=f"(f[i][2]), "=f"(f[i][3]), "=f"(f[i][4]),
+                               "=f"(f[i][5]), "=f"(f[i][6]), "=f"(f[i][7])
+                             : "l"(x + g * 32 + 8 * j));
+        }
+#pragma unroll
+        for (int i = 0; i < UNROLL; ++i) {
+            const int64_t g = g0 + i * step;
+            int c[8];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                // (fmaxf: NaN is code 0; the other end saturates in the pack)
+                dsq_requant2<BITS>(dsq_add2(dsq_pack2(fmaxf(f[i][2 * k], q.lo), fmaxf(f[i][2 * k + 1], q.lo)), lo2),
+                                   inv2, c[2 * k], c[2 * k + 1]);
+            const uint32_t mine = dsq_pack8<BITS>(c);
+            const uint32_t next = __shfl_down_sync(0xffffffffu, mine, 1);
+            if (g >= groups) continue;
+            // groups_row > 0: pitch_words words a row, groups_row groups of BITS words
+            const int64_t row = g / groups_row;
+            const int gr = (int)(g - row * groups_row);
+            uint32_t *dst = out + row * pitch_words + gr * BITS;
+            if (BITS == 3) {
+                if (j < 3) dst[j] = (mine >> (8 * j)) | (next << (24 - 8 * j));
+            } else if ((j & 1) == 0) {
+                dst[j >> 1] = mine | (next << 16);
+            }
+            if (gr == groups_row - 1)
+                for (int w = BITS * groups_row + j; w < pitch_words; w += 4) out[row * pitch_words + w] = 0u;
+        }
     }
 }
 
@@ -255,9 +314,9 @@ __global__ void __launch_bounds__(256)
 maxpool_kernel(const uint32_t *__restrict__ in, uint32_t *__restrict__ out,
                int N, int H, int W, int C, int pitch_words, int bits)
 {
-    // lets a tensor-core kernel queued behind this one (programmatic dependent
-    // launch) set itself up while this grid runs; it still waits for this grid
-    // to complete before touching global data
+    // waits for the kernels ahead, then lets the one queued behind (programmatic
+    // dependent launch) start its set-up (in this order: see dsq_early_constants)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int Ho = H / 2, Wo = W / 2;
     const int64_t total = (int64_t)N * Ho * Wo * pitch_words;
@@ -407,11 +466,20 @@ int dsq_quantize_act(const float *x, const dsq_nhwc_t *shape,
         // needs the extra resident warps to stay full
         const int grid = grid_for((n_lines + 31) / 32 * 32, 256, 148 * 64);
         return dsq_launch(bits == 4 ? quantize_flat_kernel<4> : quantize_flat_kernel<2>, dim3(grid),
-                          dim3(256), 0, s, 0, 0, (const float4 *)x, (uint4 *)codes_out, n_lines, dq);
+                          dim3(256), 0, s, dsq_launch_hooks().pdl, 0, (const float4 *)x,
+                          (uint4 *)codes_out, n_lines, dq);
     }
     const int pw = (int)(pitch / 4);
-    return dsq_launch(quantize_rows_kernel, dim3(grid_for(rows * pw, 256)), dim3(256), 0, s, 0, 0, x,
-                      (uint32_t *)codes_out, rows, k, pw, bits, dq);
+    // (the lean rounding wants floor(fma(hi - lo, inv, 0.5)) = qmax: every sane range)
+    if (bits < 4 && k % 32 == 0 && ((uintptr_t)x & 31u) == 0 &&
+        (int)floorf(fmaf(dq.hi - dq.lo, dq.inv, 0.5f)) == dq.qmax) {
+        const int64_t groups = rows * (k / 32);
+        return dsq_launch(bits == 3 ? quantize_groups_kernel<3> : quantize_groups_kernel<2>,
+                          dim3(grid_for((groups + 3) / 4 * 4, 256, 148 * 32)), dim3(256), 0, s,
+                          dsq_launch_hooks().pdl, 0, x, (uint32_t *)codes_out, groups, k / 32, pw, dq);
+    }
+    return dsq_launch(quantize_rows_kernel, dim3(grid_for(rows * pw, 256)), dim3(256), 0, s,
+                      dsq_launch_hooks().pdl, 0, x, (uint32_t *)codes_out, rows, k, pw, bits, dq);
 }
 
 int dsq_pack_weights(const float *w, const dsq_conv_t *c, int bits,
@@ -484,7 +552,7 @@ int dsq_maxpool2x2(const void *codes_in, const dsq_nhwc_t *shape, int bits,
     if (bytes < (size_t)out_rows * pitch) return DSQ_ERR_SIZE;
     const int pw = (int)(pitch / 4);
     return dsq_launch(maxpool_kernel, dim3(grid_for(out_rows * pw, 256)), dim3(256), 0,
-                      (cudaStream_t)stream, 0, 0, (const uint32_t *)codes_in, (uint32_t *)codes_out,
+                      (cudaStream_t)stream, dsq_launch_hooks().pdl, 0, (const uint32_t *)codes_in, (uint32_t *)codes_out,
                       shape->N, shape->H, shape->W, shape->C, pw, bits);
 }
 

@@ -41,6 +41,18 @@ struct dsq_plan {
 // the plan the calling thread records into, or nullptr
 __attribute__((visibility("hidden"))) dsq_plan *&dsq_recording_plan();
 
+// Whether a kernel launched now may read a layer's constants (packed weights, scales,
+// biases) before griddepcontrol.wait.  Every kernel of the library waits for the
+// kernels ahead of it before it lets the next one start, so when a kernel starts,
+// everything but its immediate predecessor has completed and is visible.  Behind
+// another launch of the same plan that predecessor is a layer of the network, which
+// writes activations only; elsewhere it may be what wrote the constants.
+inline int dsq_early_constants()
+{
+    const dsq_plan *plan = dsq_recording_plan();
+    return plan && !plan->recs.empty();
+}
+
 inline int dsq_launch_args(const DsqGrid &g, void *const *argv, cudaStream_t s)
 {
     cudaLaunchConfig_t cfg = {};

@@ -50,6 +50,7 @@ struct PwParams {
     int m_tiles, mstep;                       // tiles of mt * 128 pixels; tiles between two of a CTA
     int planes, P, PB;                        // planes of 128 channels; packed bytes of a pixel, of a plane
     int stages, tmem_cols;
+    int early;                                // dsq_early_constants
     const uint8_t *act;
     int stride, Ho, Wo;                       // stride 2: output image (im2col boxes)
     int box_rows;                             // pixels of a TMA box
@@ -179,8 +180,8 @@ dsq_pw_kernel(const __grid_constant__ CUtensorMap tmap_a, const PwParams p)
     float *sm_bias = sm_scale + p.BN;
     if (warp != PW_WARP_TMA) {
         // ---------------- once: weights of this N tile, scales and biases ---------
-        // (before the wait for the kernels ahead in the stream: they are constants of
-        // the network, and no kernel that lets its successors start early writes them)
+        // (early: before the wait for the kernel ahead in the stream)
+        if (!p.early) grid_dependency_wait();
         const int tid = threadIdx.x - 32;
         constexpr int NT = PW_THREADS - 32;
         const uint32_t bt = smem_u32(smem + L.b_tiles);
@@ -224,8 +225,8 @@ dsq_pw_kernel(const __grid_constant__ CUtensorMap tmap_a, const PwParams p)
     }
     // no activation is read and nothing is written before the kernels ahead of this
     // one have completed
-    grid_launch_dependents();
     grid_dependency_wait();
+    grid_launch_dependents();
 
     if (warp == PW_WARP_TMA) {
         // ---------------- producer: packed planes --------------------------------
@@ -557,6 +558,7 @@ int dsq_pointwise(const void *act_codes, const dsq_nhwc_t *shape, int bits, cons
     p.box_rows = p.mt * 128 < 256 ? p.mt * 128 : 256;
     p.L = pw_layout(p.mt, p.BN, p.planes, p.stride == 1 ? p.P : p.planes * p.PB, p.stages);
     p.act = (const uint8_t *)act_codes;
+    p.early = dsq_early_constants();
     p.smem_bytes = (int)p.L.total + 1024;
     p.shift = e.half_offset ? 7 - bits : 8 - bits;
     p.orv = e.half_offset ? 0x01010101u << (7 - bits) : 0u;

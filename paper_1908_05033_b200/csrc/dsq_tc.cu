@@ -367,8 +367,8 @@ dsq_tc_kernel(const __grid_constant__ CUtensorMap tmap_b,
     // descriptor prefetch) touched no global data, so it may run while the
     // kernel before this one is still finishing; nothing below starts before
     // that kernel has completed.  The kernel behind this one may set up likewise.
-    grid_launch_dependents();
     grid_dependency_wait();
+    grid_launch_dependents();
 
     // Epilogue roles.  epi_idx >= 0: the warp takes part in the epilogue of every
     // tile (p.epw warps per TMEM lane quarter).  join_idx >= 0: it takes part in

@@ -88,7 +88,6 @@ wgemm_small_kernel(const WsParams p)
     constexpr bool ALL = MT <= 2;              // X of a whole chunk in registers
     constexpr int XG = ALL ? GROUPS : 1;
     __shared__ float part[8][MT * NT][32][4];
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n = lane >> 2, j = lane & 3;
     const int n0 = blockIdx.x * 8 * NT, m0 = blockIdx.y * 16 * MT;
@@ -99,6 +98,7 @@ wgemm_small_kernel(const WsParams p)
     constexpr uint32_t BASE = (0x4300u + (ODD ? 2 * HALF : HALF)) * 0x00010001u;
     const int chunks = (p.K + 127) / 128;
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     float acc[MT][NT][4];
 #pragma unroll
