@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 
 #include <cstring>
+#include <mutex>
 #include <type_traits>
 #include <vector>
 
@@ -33,9 +34,17 @@ struct DsqLaunchRec {
 
 struct dsq_plan {
     std::vector<DsqLaunchRec> recs;
-    unsigned hooks_generation;          // of the process-wide hooks when recorded
-    int device;
-    int status;                         // first failure while recording
+    unsigned hooks_generation = 0;      // of the process-wide hooks when recorded
+    int device = -1;
+    int status = DSQ_OK;                // first failure while recording
+    // the launches as a CUDA graph, made on the third run (dsq_plan_run); guarded
+    mutable std::mutex lock;
+    mutable int runs = 0;
+    mutable cudaGraphExec_t graph = nullptr;
+    ~dsq_plan()
+    {
+        if (graph) cudaGraphExecDestroy(graph);
+    }
 };
 
 // the plan the calling thread records into, or nullptr

@@ -4,6 +4,48 @@
 #include "dsq_launch.h"
 #include "dsq_tc_host.h"
 
+namespace {
+
+// A pass whose kernels are short waits for its launches (3 us each of host time,
+// against 2 to 4 us of GPU time a layer at batch 1): from the third run on they go as
+// one CUDA graph.  Plans that run once or twice do not pay for making it; neither do
+// passes that are being captured.
+constexpr int GRAPH_AFTER = 3;
+constexpr size_t MIN_GRAPH = 4;
+
+int launch_all(const dsq_plan *plan, cudaStream_t s)
+{
+    void *argv[DsqLaunchRec::MAX_ARGS];
+    for (const DsqLaunchRec &r : plan->recs) {
+        for (int i = 0; i < r.n_args; ++i)
+            argv[i] = const_cast<unsigned char *>(r.args) + r.arg_at[i];
+        const int st = dsq_launch_args(r.g, argv, s);
+        if (st) return st;
+    }
+    return DSQ_OK;
+}
+
+// nullptr where it cannot be made: the launches then go one by one
+cudaGraphExec_t make_graph(const dsq_plan *plan)
+{
+    cudaStream_t s = nullptr;
+    cudaGraph_t g = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess &&
+        cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+        const int st = launch_all(plan, s);
+        if (cudaStreamEndCapture(s, &g) != cudaSuccess || st ||
+            cudaGraphInstantiate(&exec, g, 0) != cudaSuccess)
+            exec = nullptr;
+    }
+    if (g) cudaGraphDestroy(g);
+    if (s) cudaStreamDestroy(s);
+    cudaGetLastError();
+    return exec;
+}
+
+}  // namespace
+
 dsq_plan *&dsq_recording_plan()
 {
     static thread_local dsq_plan *plan = nullptr;
@@ -51,14 +93,20 @@ int dsq_plan_valid(const dsq_plan *plan)
 int dsq_plan_run(const dsq_plan *plan, void *stream)
 {
     if (!plan) return DSQ_ERR_NULL;
-    void *argv[DsqLaunchRec::MAX_ARGS];
-    for (const DsqLaunchRec &r : plan->recs) {
-        for (int i = 0; i < r.n_args; ++i)
-            argv[i] = const_cast<unsigned char *>(r.args) + r.arg_at[i];
-        const int st = dsq_launch_args(r.g, argv, (cudaStream_t)stream);
-        if (st) return st;
+    cudaStream_t s = (cudaStream_t)stream;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (plan->recs.size() >= MIN_GRAPH && cudaStreamIsCapturing(s, &cap) == cudaSuccess &&
+        cap == cudaStreamCaptureStatusNone) {
+        std::lock_guard<std::mutex> guard(plan->lock);
+        if (plan->runs < GRAPH_AFTER && ++plan->runs == GRAPH_AFTER) plan->graph = make_graph(plan);
+        if (plan->graph) {
+            if (cudaGraphLaunch(plan->graph, s) == cudaSuccess) return DSQ_OK;
+            cudaGetLastError();
+            return DSQ_ERR_CUDA;
+        }
     }
-    return DSQ_OK;
+    cudaGetLastError();
+    return launch_all(plan, s);
 }
 
 }  // extern "C"
