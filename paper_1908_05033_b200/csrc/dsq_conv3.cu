@@ -741,7 +741,6 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
             constexpr int CWU = 16 / E;                      // code words per unit: 2 (4-bit), 1 (2-bit)
             constexpr uint32_t MASK = (1u << BITS) - 1u;
             const DsqEpi &e = p.e;
-            const float *lut = reinterpret_cast<const float *>(smem + L.lut);
             // (dup: lanes 64..127 repeat channels 0..63; quarters 2, 3 take columns 128..255)
             const int chq = p.dup ? (quarter & 1) * 32 : quarter * 32;
             const int colbase = p.dup ? 128 * (quarter >> 1) + 32 * k : 64 * k;
@@ -751,12 +750,19 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
             // channels past Cout are padding lanes of the packed row and get zeros
             // (warp-uniform)
             const bool warp_live = (n_tile * 128 + chq) * BITS / 8 < p.out_pitch;
-            float sc = 0.f, bi = 0.f;
+            constexpr bool LEAN = EPI == DSQ_EPI_CODES || EPI == DSQ_EPI_CODES_RES;
+            float sc = 0.f, bi = LEAN ? -1e30f : 0.f;        // padding lanes: code 0
             if (ch < p.Ncols) {
-                sc = __ldg(e.scale + ch);
-                if (e.half_offset) sc = __fmul_rn(sc, 0.5f);
-                bi = __ldg(e.bias + ch);
+                if (LEAN) dsq_codes_affine(e.scale, e.bias, ch, e.half_offset, -p.shift, sc, bi);
+                else {
+                    sc = __ldg(e.scale + ch);
+                    if (e.half_offset) sc = __fmul_rn(sc, 0.5f);
+                    bi = __ldg(e.bias + ch);
+                }
             }
+            const DsqLean lean = dsq_make_lean(e);
+            const unsigned long long scp = dsq_pack2(sc, sc), bip = dsq_pack2(bi, bi);
+            const unsigned long long sc4[4] = {scp, scp, scp, scp}, bi4[4] = {bip, bip, bip, bip};
             const int pw = p.out_pitch / 4;                  // words of an output pixel
             const int cg = (n_tile * 128 + chq + (lane & ~(E - 1))) / E;   // this lane group's word
             const uint32_t *res32 = reinterpret_cast<const uint32_t *>(e.residual);
@@ -829,24 +835,25 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                         cw[w] = 0u;
                     }
                     tmem_ld_wait();
+                    if constexpr (LEAN) {
+                        // eight positions of this lane's channel at a time
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        // column 16 u + j of the warp: held by lane 8 u + j / 2
-                        const int mj = __shfl_sync(0xffffffffu, (j & 1) ? m1 : m0, 8 * u + (j >> 1));
-                        const int vi = (int)r[j] >> p.shift;
-                        if constexpr (EPI == DSQ_EPI_CODES || EPI == DSQ_EPI_CODES_RES) {
-                            const float vf = __fsub_rn(__int_as_float(0x4B400000 + vi), 12582912.0f);
-                            float y = __fmaf_rn(vf, sc, bi);
-                            if (EPI == DSQ_EPI_CODES_RES) {
-                                // (positions without an output and channels past Cout
-                                // carry no residual: their codes are not stored / are 0)
-                                const uint32_t qr = (resT[(j * BITS) >> 5] >> ((j * BITS) & 31)) & MASK;
-                                y = __fadd_rn(y, ch < p.Ncols ? lut[qr] : 0.0f);
-                            }
-                            const float rr = fminf(__fmaf_rn(fmaxf(y, 0.0f), e.rq.inv, 0.5f), p.r_hi);
-                            cw[(j * BITS) >> 5] +=
-                                (uint32_t)__float_as_int(__fadd_rd(rr, 8388608.0f)) << ((j * BITS) & 31);
-                        } else {
+                        for (int h = 0; h < 2; ++h) {
+                            uint32_t v[8];
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) v[j] = r[8 * h + j];
+                            const uint32_t rw = BITS == 4 ? resT[h < CWU ? h : 0] : resT[0] >> (16 * h);
+                            const uint32_t x = dsq_lean_codes8<BITS, EPI == DSQ_EPI_CODES_RES, false>(
+                                v, sc4, bi4, rw, lean);
+                            if (BITS == 4) cw[h < CWU ? h : 0] = x;
+                            else cw[0] |= x << (16 * h);
+                        }
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) {
+                            // column 16 u + j of the warp: held by lane 8 u + j / 2
+                            const int mj = __shfl_sync(0xffffffffu, (j & 1) ? m1 : m0, 8 * u + (j >> 1));
+                            const int vi = (int)r[j] >> p.shift;
                             if (mj >= 0 && ch < p.Ncols) {
                                 if (e.acc_out) e.acc_out[(int64_t)mj * p.Ncols + ch] = vi;
                                 float y;
@@ -869,11 +876,6 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                                 if (e.y_f32) e.y_f32[(int64_t)mj * p.Ncols + ch] = y;
                             }
                         }
-                    }
-                    if constexpr (EPI == DSQ_EPI_CODES || EPI == DSQ_EPI_CODES_RES) {
-                        constexpr uint32_t FIELDS = BITS == 4 ? 0x11111111u : 0x55555555u;
-#pragma unroll
-                        for (int w = 0; w < CWU; ++w) cw[w] -= 0x4B000000u * FIELDS;
                     }
                     if (e.y_codes) {
                         // fields of E positions of one channel -> fields of the E
@@ -1191,12 +1193,12 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     //  * otherwise plain tiles.
     const bool tiny_deep = shape->H * shape->W <= 64 && Cin >= 512;
     if (hooks.window3 == 1 && tiny_deep) return DSQ_ERR_UNSUPPORTED;
-    // the lean codes epilogue wants the requantiser range to start at 0, the
-    // accumulator to fit the 2^22 conversion trick and floor(r_hi) = qmax
+    // the codes epilogues want the requantiser range to start at 0 and
+    // floor(r_hi) = qmax
     float r_hi = 0.f;
     if (epi_kind != DSQ_EPI_GENERAL) {
         r_hi = fmaf(e.rq.hi - e.rq.lo, e.rq.inv, 0.5f);
-        if (e.rq.lo != 0.0f || !small_acc || (int)floorf(r_hi) != e.rq.qmax)
+        if (e.rq.lo != 0.0f || (int)floorf(r_hi) != e.rq.qmax)
             epi_kind = DSQ_EPI_GENERAL;
     }
     W3Params p = {};
@@ -1295,6 +1297,8 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     if (bits != 3 && want_tr) found = configure(1);
     if (!found) found = configure(0);
     if (!found) return DSQ_ERR_UNSUPPORTED;
+    // (plain tiles convert accumulators by the 2^22 trick)
+    if (!p.tr && !small_acc) epi_kind = DSQ_EPI_GENERAL;
     p.L = w3_layout(p.apx, p.BN, bits, p.PB, p.as_slots, p.b_stages, p.bp_slots, p.cout_pad);
     p.smem_bytes = (int)p.L.total + 1024;
     // grid: a multiple of n_tiles; CTA c takes N tile c % n_tiles and every
