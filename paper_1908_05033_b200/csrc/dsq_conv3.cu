@@ -1184,14 +1184,13 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     if (shape->W + 2 > 32000 || shape->H + 2 > 32000) return DSQ_ERR_UNSUPPORTED;
     // Which kernel (hook value 1 = automatic; measured on the ResNet-18- and
     // VGG-16-shaped layers, per layer, 20 launches back to back):
-    //  * transposed tiles wherever they fit, except 7x7-sized images with >= 512
-    //    input channels (a handful of tiles with very long K loops, where the
-    //    im2col kernel is as fast or faster).  With up to 64 output channels the
+    //  * transposed tiles wherever they fit (3-bit codes: not on 7x7-sized images with
+    //    >= 512 input channels).  With up to 64 output channels the
     //    transposed form needs the weight rows twice in its A operand (`dup`),
     //    which it only gets from the blob's expanded copy: 64->64 at 56x56 runs
     //    in 18 us against 22.5 us on plain tiles;
     //  * otherwise plain tiles.
-    const bool tiny_deep = shape->H * shape->W <= 64 && Cin >= 512;
+    const bool tiny_deep = bits == 3 && shape->H * shape->W <= 64 && Cin >= 512;
     if (hooks.window3 == 1 && tiny_deep) return DSQ_ERR_UNSUPPORTED;
     // the codes epilogues want the requantiser range to start at 0 and
     // floor(r_hi) = qmax

@@ -23,6 +23,8 @@
 // K is a list of units: 16 bytes of one filter tap of a pixel row (32 codes of 4 bits,
 // 64 of 2; 12 bytes = 32 codes at 3 bits), four units - lanes j = 0 .. 3 - a chunk.
 // The order of K inside a unit is free as long as both operands agree.
+#include <cmath>
+
 #include "dsq_tc_common.cuh"
 #include "dsq_tc_host.h"
 
@@ -327,14 +329,19 @@ double estimate(const CsParams &p, int bits, int mt, int warps)
 
 // and what the other kernel for the layer takes, likewise: a floor that grows with K
 // (the few CTAs such a layer has walk it alone) plus its work at full rate
-double estimate_other(const CsParams &p, int Cin, double macs, int lean)
+double estimate_other(const CsParams &p, int bits, int Cin, double macs, int lean)
 {
+    const int sms = dsq_sm_count() > 0 ? dsq_sm_count() : 148;
     const double ksteps = p.ksize * p.ksize * Cin / 128.0;
-    double floor_us = 4.3 + 0.23 * ksteps;                         // im2col kernel
-    if (p.ksize == 1 && lean) floor_us = 2.9 + (double)p.M * p.Ncols / 3.7e6;
-    else if (p.ksize == 3 && p.stride == 1 && p.pad == 1 && (Cin == 64 || Cin % 128 == 0))
-        floor_us = Cin == 64 ? 5.5 : Cin <= 256 ? 7.8 + 0.26 * ksteps : 14.0;
-    return floor_us + macs / 4.5e8;
+    if (p.ksize == 1 && lean) return 2.9 + (double)p.M * p.Ncols / 3.7e6;
+    if (p.ksize == 3 && p.stride == 1 && p.pad == 1 && bits != 3 && (Cin == 64 || Cin % 128 == 0)) {
+        // window kernel: waves of tiles of 256 positions x 128 channels
+        const double tiles = std::ceil((double)p.M / p.H / p.W * (p.H + 2) * (p.W + 2) / 256) *
+                             ((p.Ncols + 127) / 128);
+        return (Cin == 64 ? 4.3 : Cin <= 256 ? 7.7 : 5.5) +
+               std::ceil(tiles / sms) * ksteps * (Cin == 64 ? 0.4 : 0.27);
+    }
+    return 4.3 + 0.23 * ksteps + macs / 4.5e8;                     // im2col kernel
 }
 
 }  // namespace
@@ -374,7 +381,7 @@ int dsq_conv_small(const void *act_codes, const dsq_nhwc_t *shape, int bits, con
             if (t < best) { best = t; mt = m; warps = w; }
         }
     const double macs = (double)p.M * p.Ncols * taps * conv->Cin;
-    if (best > estimate_other(p, conv->Cin, macs, lean)) return DSQ_ERR_UNSUPPORTED;
+    if (best > estimate_other(p, bits, conv->Cin, macs, lean)) return DSQ_ERR_UNSUPPORTED;
     switch (bits) {
     case 2: return pick<2>(p, mt, warps, stream);
     case 3: return pick<3>(p, mt, warps, stream);

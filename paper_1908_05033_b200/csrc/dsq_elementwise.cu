@@ -358,6 +358,48 @@ maxpool_kernel(const uint32_t *__restrict__ in, uint32_t *__restrict__ out,
     }
 }
 
+// fields-wise maximum of two words of 2- or 4-bit codes: a field is at least the other
+// where subtracting leaves its guard bit (bit BITS of the split field) set
+template <int BITS>
+__device__ __forceinline__ uint32_t max_fields(uint32_t a, uint32_t b)
+{
+    constexpr uint32_t F = BITS == 4 ? 0x0F0F0F0Fu : 0x33333333u, G = BITS == 4 ? 0x10101010u : 0x44444444u;
+    uint32_t r = 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const uint32_t x = (a >> (BITS * h)) & F, y = (b >> (BITS * h)) & F;
+        const uint32_t ge = ((x | G) - y) & G;
+        const uint32_t m = ge - (ge >> BITS);             // the field's bits where x >= y
+        r |= ((x & m) | (y & ~m)) << (BITS * h);
+    }
+    return r;
+}
+
+// 2x2 max-pool on 2- and 4-bit codes: a thread does 16 bytes of one output pixel.
+// HBM-bound (224x224x64 at 2 bits, batch 32: 24.5 us with a thread per word and
+// 64-bit index divisions).
+template <int BITS>
+__global__ void __launch_bounds__(256)
+maxpool_chunks_kernel(const uint4 *__restrict__ in, uint4 *__restrict__ out, int total, int H, int W,
+                      int chunks)
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int Wo = W / 2, Ho = H / 2;
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < total; i += gridDim.x * 256) {
+        const int pix = i / chunks, c = i - pix * chunks;
+        const int row = pix / Wo, wo = pix - row * Wo;     // row: of all images
+        const int n = row / Ho, ho = row - n * Ho;
+        const uint4 *p = in + ((int64_t)(n * H + 2 * ho) * W + 2 * wo) * chunks + c;
+        const uint4 v00 = __ldg(p), v01 = __ldg(p + chunks), v10 = __ldg(p + (int64_t)W * chunks),
+                    v11 = __ldg(p + (int64_t)W * chunks + chunks);
+        out[i] = make_uint4(max_fields<BITS>(max_fields<BITS>(v00.x, v01.x), max_fields<BITS>(v10.x, v11.x)),
+                            max_fields<BITS>(max_fields<BITS>(v00.y, v01.y), max_fields<BITS>(v10.y, v11.y)),
+                            max_fields<BITS>(max_fields<BITS>(v00.z, v01.z), max_fields<BITS>(v10.z, v11.z)),
+                            max_fields<BITS>(max_fields<BITS>(v00.w, v01.w), max_fields<BITS>(v10.w, v11.w)));
+    }
+}
+
 // Hands a workspace's status word to the host and clears it.  Written straight into
 // page-locked host memory: a copy to pageable memory is staged and took about 10 us
 // more of every call that reads the status.
@@ -551,6 +593,12 @@ int dsq_maxpool2x2(const void *codes_in, const dsq_nhwc_t *shape, int bits,
     const int64_t out_rows = (int64_t)shape->N * (shape->H / 2) * (shape->W / 2);
     if (bytes < (size_t)out_rows * pitch) return DSQ_ERR_SIZE;
     const int pw = (int)(pitch / 4);
+    const int64_t items = out_rows * (int64_t)(pitch / 16);
+    if (bits != 3 && items < (1ll << 31) - (1 << 26))
+        return dsq_launch(bits == 4 ? maxpool_chunks_kernel<4> : maxpool_chunks_kernel<2>,
+                          dim3(grid_for(items, 256, 148 * 32)), dim3(256), 0, (cudaStream_t)stream,
+                          dsq_launch_hooks().pdl, 0, (const uint4 *)codes_in, (uint4 *)codes_out,
+                          (int)items, shape->H, shape->W, (int)(pitch / 16));
     return dsq_launch(maxpool_kernel, dim3(grid_for(out_rows * pw, 256)), dim3(256), 0,
                       (cudaStream_t)stream, dsq_launch_hooks().pdl, 0, (const uint32_t *)codes_in, (uint32_t *)codes_out,
                       shape->N, shape->H, shape->W, shape->C, pw, bits);
