@@ -96,6 +96,9 @@ struct W3Params {
     int npl, kpp, ksteps;              // planes of 128 channels, K steps per plane, total
     int PB, cpp;                       // packed bytes per pixel and plane; 16-byte chunks of it
     int two_taps;                      // 64-channel rows of 2 / 4 bits: a K step is two filter taps
+    int rb;                            // bytes of a window row: 128, or 64 (transposed tiles over 64
+                                       // channels: half the shared memory, which is what leaves room
+                                       // for resident weights beside the window of a wide image)
     int xstep;                         // bytes between two K steps of a plane in a weight row
     int apx;                           // pixels of an A slot
     int a_box, a_nload, nbands, band_px;
@@ -129,12 +132,13 @@ struct W3Params {
 };
 
 
-__host__ __device__ inline W3Smem w3_layout(int apx, int BN, int bits, int PB, int as_slots,
+__host__ __device__ inline W3Smem w3_layout(int apx, int rb, int BN, int bits, int PB, int as_slots,
                                             int b_stages, int bp_slots, int cout_pad)
 {
     W3Smem L;
     uint32_t o = 0;
-    L.a_slots = o;  o += W3_A_SLOTS * apx * 128;           // apx is a multiple of 8
+    L.a_slots = o;  o += W3_A_SLOTS * apx * rb;            // apx is a multiple of 8
+    o = (o + 1023u) & ~1023u;
     L.b_tiles = o;  o += b_stages * BN * 128;              // BN is a multiple of 8
     L.a_stage = o;  o += as_slots * apx * PB;
     L.b_packed = o; o += bp_slots * BN * 16 * bits;
@@ -272,7 +276,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
     const uint32_t n_b_fills =
         my_tiles == 0 ? 0u : (p.b_res ? (uint32_t)p.ksteps : (uint32_t)my_tiles * p.ksteps);
     const uint32_t n_a_fills = (uint32_t)my_tiles * p.npl;
-    const uint32_t a_slot_bytes = (uint32_t)p.apx * 128u;
+    const uint32_t a_slot_bytes = (uint32_t)(p.apx * p.rb);
     const uint32_t a_stage_bytes = (uint32_t)p.apx * p.PB;
     const uint32_t b_stage_bytes = (uint32_t)BN * 128u;
     const uint32_t b_packed_bytes = (uint32_t)BN * 16u * BITS;
@@ -340,7 +344,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
             const int within = p.two_taps ? 32 * (j & 1) : 32 * j;
             const int kh = tap / 3, kw = tap - 3 * kh;
             tab[i] = tap < 9 && within < p.E
-                         ? (uint32_t)((kh * p.tap_stride + kw) * 8 + (within >> 4))
+                         ? (uint32_t)((kh * p.tap_stride + kw) * (p.rb >> 4) + (within >> 4))
                          : 0xFFFFFFFFu;
         }
     }
@@ -508,6 +512,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
         const uint32_t idesc = TR ? idesc_i8(256, true, false, 128) : idesc_i8(BN, false, true, W3_BM);
         const uint64_t desc0 = smem_desc_sw128(0u);
         const uint32_t desc_hi = (uint32_t)(desc0 >> 32), desc_lo = (uint32_t)desc0;
+        const uint32_t win_hi = p.rb == 64 ? (uint32_t)(smem_desc_sw64(0u) >> 32) : desc_hi;
         const uint32_t a_lo_base = desc_lo + (smem_u32(smem + L.a_slots) >> 4);
         const uint32_t b_lo_base = desc_lo + (smem_u32(smem + L.b_tiles) >> 4);
         const uint4 *tab = reinterpret_cast<const uint4 *>(smem + L.a_tab);
@@ -543,7 +548,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                         mma_i8_ss_x4b_elect(d_tmem, b_lo_base + st * (b_stage_bytes >> 4), desc_hi,
                                             a_lo + t.x, t.y == 0xFFFFFFFFu ? t.y : a_lo + t.y,
                                             t.z == 0xFFFFFFFFu ? t.z : a_lo + t.z,
-                                            t.w == 0xFFFFFFFFu ? t.w : a_lo + t.w, desc_hi, idesc,
+                                            t.w == 0xFFFFFFFFu ? t.w : a_lo + t.w, win_hi, idesc,
                                             first);
                     else
                     mma_i8_ss_x4_elect(d_tmem, a_lo + t.x, t.y == 0xFFFFFFFFu ? t.y : a_lo + t.y,
@@ -616,8 +621,9 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
             for (int t = tid; t < n_tasks; t += W3_NUM_A_WARPS * 32) {
                 const int px = t >> lcpp, ch = t & (p.cpp - 1);
                 const uint4 v = lds_128(src + 16u * t);
-                const uint32_t row = dst + (uint32_t)px * 128u;
-                const int sw = px & 7;
+                // (16-byte chunks XOR-ed with address bits 7..9, of 64-byte rows bits 7..8)
+                const uint32_t row = dst + (uint32_t)(px * p.rb);
+                const int sw = p.rb == 64 ? (px >> 1) & 3 : px & 7;
 #pragma unroll
                 for (int c = 0; c < OUT; ++c)
                     sts_128(row + (uint32_t)(((ch * OUT + c) ^ sw) << 4),
@@ -1224,6 +1230,7 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     const bool w8_ok = hooks.w8 && w8.enabled && e.half_offset && bits != 3;
     auto configure = [&](int tr) -> int {
         p.tr = tr;
+        p.rb = tr && p.two_taps ? 64 : 128;
         // transposed tiles for <= 64 output channels: the weight rows twice in the
         // A operand (two TMA boxes of the expanded copy), so that all 128 lanes of
         // the accumulator, and all epilogue warps, carry data
@@ -1259,7 +1266,7 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
         if (p.ksteps <= W3_MAX_BST) {
             for (int as = W3_MAX_AS; as >= 2; --as) {
                 const int bp = p.w8 ? 0 : 2;
-                const W3Smem L = w3_layout(p.apx, p.BN, bits, p.PB, as, p.ksteps, bp, p.cout_pad);
+                const W3Smem L = w3_layout(p.apx, p.rb, p.BN, bits, p.PB, as, p.ksteps, bp, p.cout_pad);
                 if (L.total + 1024 <= 227u * 1024u) {
                     p.b_res = 1; p.b_stages = p.ksteps; p.as_slots = as; p.bp_slots = bp;
                     return 1;
@@ -1272,7 +1279,7 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
             // no packed ring: the operand ring itself hides the latency of the loads
             for (int as = W3_MAX_AS; as >= 1; --as)
                 for (int bst = 6; bst >= 2; --bst) {
-                    const W3Smem L = w3_layout(p.apx, p.BN, bits, p.PB, as, bst, 0, p.cout_pad);
+                    const W3Smem L = w3_layout(p.apx, p.rb, p.BN, bits, p.PB, as, bst, 0, p.cout_pad);
                     if (L.total + 1024 <= 227u * 1024u) {
                         p.as_slots = as; p.b_stages = bst; p.bp_slots = 0;
                         return 1;
@@ -1282,7 +1289,7 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
         }
         const int tries[6][3] = {{3, 3, 4}, {2, 3, 4}, {2, 2, 4}, {2, 2, 3}, {2, 2, 2}, {1, 2, 2}};
         for (int t = 0; t < 6; ++t) {
-            const W3Smem L = w3_layout(p.apx, p.BN, bits, p.PB, tries[t][0], tries[t][1],
+            const W3Smem L = w3_layout(p.apx, p.rb, p.BN, bits, p.PB, tries[t][0], tries[t][1],
                                        tries[t][2], p.cout_pad);
             if (L.total + 1024 <= 227u * 1024u) {
                 p.as_slots = tries[t][0]; p.b_stages = tries[t][1]; p.bp_slots = tries[t][2];
@@ -1298,7 +1305,7 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     if (!found) return DSQ_ERR_UNSUPPORTED;
     // (plain tiles convert accumulators by the 2^22 trick)
     if (!p.tr && !small_acc) epi_kind = DSQ_EPI_GENERAL;
-    p.L = w3_layout(p.apx, p.BN, bits, p.PB, p.as_slots, p.b_stages, p.bp_slots, p.cout_pad);
+    p.L = w3_layout(p.apx, p.rb, p.BN, bits, p.PB, p.as_slots, p.b_stages, p.bp_slots, p.cout_pad);
     p.smem_bytes = (int)p.L.total + 1024;
     // grid: a multiple of n_tiles; CTA c takes N tile c % n_tiles and every
     // mstep-th M tile

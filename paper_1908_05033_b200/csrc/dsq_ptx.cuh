@@ -645,6 +645,18 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t smem_addr)
     return d;
 }
 
+// The same with the 64-byte swizzle: rows of 64 bytes, 8-row groups 512 bytes apart.
+__device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t smem_addr)
+{
+    uint64_t d = 0;
+    d |= (uint64_t)((smem_addr >> 4) & 0x3FFF);
+    d |= (uint64_t)1 << 16;
+    d |= (uint64_t)(512 >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)4 << 61;                       // SWIZZLE_64B
+    return d;
+}
+
 // Instruction descriptor for kind::i8: s32 accumulator, K-major A and B.
 __host__ __device__ inline uint32_t idesc_i8(int n, bool a_signed, bool b_signed, int m = 128)
 {
