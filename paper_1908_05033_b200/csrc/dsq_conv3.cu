@@ -95,7 +95,8 @@ struct W3Params {
     int E;                             // int8 bytes per pixel = Cin
     int npl, kpp, ksteps;              // planes of 128 channels, K steps per plane, total
     int PB, cpp;                       // packed bytes per pixel and plane; 16-byte chunks of it
-    int two_taps;                      // 64-channel rows of 2 / 4 bits: a K step is two filter taps
+    int two_taps;                      // 64-channel rows (3-bit: transposed tiles): a K step is two filter taps
+    int pk;                            // packed bytes of a K step in a weight row
     int rb;                            // bytes of a window row: 128, or 64 (transposed tiles over 64
                                        // channels: half the shared memory, which is what leaves room
                                        // for resident weights beside the window of a wide image)
@@ -132,7 +133,7 @@ struct W3Params {
 };
 
 
-__host__ __device__ inline W3Smem w3_layout(int apx, int rb, int BN, int bits, int PB, int as_slots,
+__host__ __device__ inline W3Smem w3_layout(int apx, int rb, int BN, int pk, int PB, int as_slots,
                                             int b_stages, int bp_slots, int cout_pad)
 {
     W3Smem L;
@@ -141,7 +142,7 @@ __host__ __device__ inline W3Smem w3_layout(int apx, int rb, int BN, int bits, i
     o = (o + 1023u) & ~1023u;
     L.b_tiles = o;  o += b_stages * BN * 128;              // BN is a multiple of 8
     L.a_stage = o;  o += as_slots * apx * PB;
-    L.b_packed = o; o += bp_slots * BN * 16 * bits;
+    L.b_packed = o; o += bp_slots * BN * pk;
     L.epi = o;      o += 2 * cout_pad * 4;                  // scale[cout_pad], bias[cout_pad]
     L.lut = o;      o += 16 * 4;
     L.a_tab = o;    o += 9 * 16;                            // four A offsets per K step of a plane
@@ -228,7 +229,12 @@ __device__ __forceinline__ W3Pos w3_add(W3Pos a, int dn, int dh, int dw, int Hp,
 // the tensor-memory lanes and POSITIONS in the columns: an epilogue thread owns
 // one channel, gathers its codes of 8 (16 at 2 bits) positions in a word and an
 // 8 x 8 (16 x 16) transpose of bit fields across the lanes of a channel group
-// (shuffles) turns that into the packed NHWC words of those positions.
+// (shuffles) turns that into the packed NHWC words of those positions.  3-bit codes
+// take four-bit fields up to there; then a lane's eight channels are 24 bits and the
+// four groups of a quarter put three words together.
+//
+// 3-bit, batch 64, plain tiles or the im2col kernel before -> transposed: 64->64 at 56x56
+// 70.9 -> 18.6 us, 128->128 at 28x28 28.7 -> 15.7, 512->512 at 7x7 40 -> 21.
 template <int BITS>
 __device__ __forceinline__ uint32_t w3_transpose_fields(uint32_t x, int lane)
 {
@@ -252,7 +258,6 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
     constexpr int CH = Chunks<BITS>::CH;       // packed 16-byte chunks per 128 codes
     constexpr int OUT = Chunks<BITS>::OUT;     // int8 chunks per packed chunk
     constexpr int TP = TR ? 256 : W3_BM;       // positions of a tile
-    static_assert(!TR || BITS != 3, "transposed tiles: 2- and 4-bit codes");
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     if ((threadIdx.x >> 5) == 1) W3_STAMP(13, 0);
     uint8_t *smem = reinterpret_cast<uint8_t *>(
@@ -279,7 +284,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
     const uint32_t a_slot_bytes = (uint32_t)(p.apx * p.rb);
     const uint32_t a_stage_bytes = (uint32_t)p.apx * p.PB;
     const uint32_t b_stage_bytes = (uint32_t)BN * 128u;
-    const uint32_t b_packed_bytes = (uint32_t)BN * 16u * BITS;
+    const uint32_t b_packed_bytes = (uint32_t)BN * p.pk;
     const int img_positions = p.Hp * p.Wp;
 
     const uint32_t bars = smem_u32(smem + L.bars);
@@ -598,6 +603,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                 // 3-bit rows: one task per pixel (8 codes per 3 bytes from the
                 // row's start): its 32 or 48 packed bytes -> 64 or 128 int8 bytes
                 const int nq = p.E >= 128 ? 8 : 4;
+                const bool half_rows = p.rb == 64;
 #pragma unroll 1
                 for (int px = tid; px < p.apx; px += W3_NUM_A_WARPS * 32) {
                     uint32_t w[12];
@@ -607,8 +613,8 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                         if (l < p.cpp) v = lds_128(src + (uint32_t)(px * p.PB + 16 * l));
                         w[4 * l] = v.x; w[4 * l + 1] = v.y; w[4 * l + 2] = v.z; w[4 * l + 3] = v.w;
                     }
-                    const uint32_t row = dst + (uint32_t)px * 128u;
-                    const int sw = px & 7;
+                    const uint32_t row = dst + (uint32_t)(px * p.rb);
+                    const int sw = half_rows ? (px >> 1) & 3 : px & 7;
 #pragma unroll
                     for (int q = 0; q < 8; ++q)
                         if (q < nq) {
@@ -663,7 +669,37 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
             const uint4 *src = reinterpret_cast<const uint4 *>(smem + L.b_packed + sp * b_packed_bytes);
             uint8_t *rowp = smem + L.b_tiles + st * b_stage_bytes + row0 * 128;
             bool waited = p.b_res != 0;
-            if (BITS == 3) {
+            if (BITS == 3 && TR) {
+                // one thread per operand row: 48 packed bytes of a tap and plane, or the
+                // 24 bytes of each of two taps (rows 64 .. 127 repeat 0 .. 63: dup)
+                const int row = tid;
+                const uint4 *r4 = reinterpret_cast<const uint4 *>(
+                    smem + L.b_packed + sp * b_packed_bytes + (p.dup ? row & 63 : row) * p.pk);
+                uint32_t w[12], w1[12];
+#pragma unroll
+                for (int l = 0; l < 3; ++l) {
+                    const uint4 v = r4[l];
+                    w[4 * l] = v.x; w[4 * l + 1] = v.y; w[4 * l + 2] = v.z; w[4 * l + 3] = v.w;
+                }
+                if (p.two_taps) {
+                    const uint4 v = r4[3];
+#pragma unroll
+                    for (int l = 0; l < 4; ++l) w1[l] = w[8 + l];
+                    w1[4] = v.x; w1[5] = v.y;
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_bp_empty(sp));
+                if (!waited && !(ok = wait_bar_warp(bar_b_empty(st), phu ^ 1u, ctl, 7))) break;
+                uint8_t *rp = smem + L.b_tiles + st * b_stage_bytes + row * 128;
+                const int sw3 = row & 7;
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    uint4 c;
+                    if (q >= 4 && p.two_taps) c = expand3_chunk<true>(w1, q & 3, p.orv);
+                    else c = expand3_chunk<true>(w, q, p.orv);
+                    *reinterpret_cast<uint4 *>(rp + ((q ^ sw3) << 4)) = c;
+                }
+            } else if (BITS == 3) {
                 // 3-bit rows: one thread per row of 48 packed bytes
                 uint32_t w[2][12];
 #pragma unroll
@@ -743,9 +779,10 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
         if constexpr (TR) {
             // thread = output channel (tensor-memory lane), columns = positions;
             // warp k of a quarter takes columns 64 k .. 64 k + 63 in units of 16
-            constexpr int E = 32 / BITS;                     // positions per code word
-            constexpr int CWU = 16 / E;                      // code words per unit: 2 (4-bit), 1 (2-bit)
-            constexpr uint32_t MASK = (1u << BITS) - 1u;
+            constexpr int SB = BITS == 3 ? 4 : BITS;         // bits of a field
+            constexpr int E = 32 / SB;                       // positions per code word
+            constexpr int CWU = 16 / E;                      // code words per unit: 2 (1 at 2 bits)
+            constexpr uint32_t MASK = (1u << SB) - 1u;
             const DsqEpi &e = p.e;
             // (dup: lanes 64..127 repeat channels 0..63; quarters 2, 3 take columns 128..255)
             const int chq = p.dup ? (quarter & 1) * 32 : quarter * 32;
@@ -770,7 +807,8 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
             const unsigned long long scp = dsq_pack2(sc, sc), bip = dsq_pack2(bi, bi);
             const unsigned long long sc4[4] = {scp, scp, scp, scp}, bi4[4] = {bip, bip, bip, bip};
             const int pw = p.out_pitch / 4;                  // words of an output pixel
-            const int cg = (n_tile * 128 + chq + (lane & ~(E - 1))) / E;   // this lane group's word
+            const int cg = (n_tile * 128 + chq + (lane & ~(E - 1))) / E;   // this lane group's word (3-bit: 24 bits)
+            const int cw3 = (n_tile * 128 + chq) / 32 * 3;   // 3-bit: the quarter's first word
             const uint32_t *res32 = reinterpret_cast<const uint32_t *>(e.residual);
             uint32_t *y32 = reinterpret_cast<uint32_t *>(e.y_codes);
             // output pixel (or -1) of the warp's columns: lane L follows columns
@@ -813,7 +851,13 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                         const int mp_b = __shfl_sync(0xffffffffu, m1, cpos >> 1);
                         mpn[w] = (cpos & 1) ? mp_b : mp_a;
                         wordn[w] = 0u;
-                        if (EPI != DSQ_EPI_CODES && e.residual && mpn[w] >= 0 && 4 * cg < p.out_pitch)
+                        if (BITS == 3) {
+                            // (the quarter's three words, one per lane group; the 24-bit
+                            // pieces are cut from them by shuffle)
+                            const int wi = cw3 + (lane >> 3 < 2 ? lane >> 3 : 2);
+                            if (EPI != DSQ_EPI_CODES && e.residual && mpn[w] >= 0 && wi < pw)
+                                wordn[w] = __ldg(res32 + (int64_t)mpn[w] * pw + wi);
+                        } else if (EPI != DSQ_EPI_CODES && e.residual && mpn[w] >= 0 && 4 * cg < p.out_pitch)
                             wordn[w] = __ldg(res32 + (int64_t)mpn[w] * pw + cg);
                     }
                 };
@@ -837,7 +881,15 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
 #pragma unroll
                     for (int w = 0; w < CWU; ++w) {
                         resT[w] = 0u;
-                        if (EPI != DSQ_EPI_CODES) resT[w] = w3_transpose_fields<BITS>(word[w], lane);
+                        if (BITS == 3 && EPI != DSQ_EPI_CODES) {
+                            const int grp = lane >> 3;
+                            const uint32_t low = __shfl_up_sync(0xffffffffu, word[w], 8);
+                            const uint32_t x = __funnelshift_rc(low, word[w], 32 - 8 * grp);
+                            const uint32_t y = (x & 0xFFFu) | ((x << 4) & 0x0FFF0000u);
+                            const uint32_t z = (y & 0x003F003Fu) | ((y << 2) & 0x3F003F00u);
+                            word[w] = (z & 0x07070707u) | ((z << 1) & 0x70707070u);
+                        }
+                        if (EPI != DSQ_EPI_CODES) resT[w] = w3_transpose_fields<SB>(word[w], lane);
                         cw[w] = 0u;
                     }
                     tmem_ld_wait();
@@ -848,10 +900,10 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                             uint32_t v[8];
 #pragma unroll
                             for (int j = 0; j < 8; ++j) v[j] = r[8 * h + j];
-                            const uint32_t rw = BITS == 4 ? resT[h < CWU ? h : 0] : resT[0] >> (16 * h);
-                            const uint32_t x = dsq_lean_codes8<BITS, EPI == DSQ_EPI_CODES_RES, false>(
+                            const uint32_t rw = SB == 4 ? resT[h < CWU ? h : 0] : resT[0] >> (16 * h);
+                            const uint32_t x = dsq_lean_codes8<BITS, EPI == DSQ_EPI_CODES_RES, false, SB>(
                                 v, sc4, bi4, rw, lean);
-                            if (BITS == 4) cw[h < CWU ? h : 0] = x;
+                            if (SB == 4) cw[h < CWU ? h : 0] = x;
                             else cw[0] |= x << (16 * h);
                         }
                     } else {
@@ -874,11 +926,11 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                                     y = dsq_epi_y(vi, sc, bi);
                                 }
                                 if (e.residual) {
-                                    const uint32_t qr = (resT[(j * BITS) >> 5] >> ((j * BITS) & 31)) & MASK;
+                                    const uint32_t qr = (resT[(j * SB) >> 5] >> ((j * SB) & 31)) & MASK;
                                     y = dsq_epi_residual(y, qr, e.res_delta, e.res_lo);
                                 }
                                 if (e.has_requant)
-                                    cw[(j * BITS) >> 5] |= dsq_code(y, e.rq) << ((j * BITS) & 31);
+                                    cw[(j * SB) >> 5] |= dsq_code(y, e.rq) << ((j * SB) & 31);
                                 if (e.y_f32) e.y_f32[(int64_t)mj * p.Ncols + ch] = y;
                             }
                         }
@@ -888,8 +940,25 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                         // channels of this lane group at one position
 #pragma unroll
                         for (int w = 0; w < CWU; ++w) {
-                            const uint32_t word = w3_transpose_fields<BITS>(cw[w], lane);
-                            if (mp[w] >= 0 && 4 * cg < p.out_pitch) y32[(int64_t)mp[w] * pw + cg] = word;
+                            uint32_t word = w3_transpose_fields<SB>(cw[w], lane);
+                            if (BITS == 3) {
+                                // the position's 24-bit pieces of the four lane groups are
+                                // three words; groups 0..2 store one each, and the spare words
+                                // of a 64-channel row come from group 3
+                                word = (word & 0x07070707u) | ((word & 0x70707070u) >> 1);
+                                word = (word & 0x003F003Fu) | ((word & 0x3F003F00u) >> 2);
+                                word = (word & 0xFFFu) | ((word >> 4) & 0xFFF000u);
+                                const uint32_t next = __shfl_down_sync(0xffffffffu, word, 8);
+                                const int grp = lane >> 3;
+                                word = (word >> (8 * grp)) | (next << (24 - 8 * grp));
+                                const int wi = cw3 + grp;
+                                uint32_t *row = y32 + (int64_t)mp[w] * pw;
+                                if (grp < 3) {
+                                    if (mp[w] >= 0 && wi < pw) row[wi] = word;
+                                } else if (p.dup && mp[w] >= 0 && wi == 6) {
+                                    for (int i = wi; i < pw; ++i) row[i] = 0u;
+                                }
+                            } else if (mp[w] >= 0 && 4 * cg < p.out_pitch) y32[(int64_t)mp[w] * pw + cg] = word;
                         }
                     }
                 }
@@ -1093,11 +1162,14 @@ int w3_dispatch(int epi, const CUtensorMap &tb, const CUtensorMap &ta, const W3P
         default: return w3_launch<BITS, DSQ_EPI_GENERAL, true>(tb, ta, p, s, pdl);
         }
     }
-    switch (epi) {
-    case DSQ_EPI_CODES: return w3_launch<BITS, DSQ_EPI_CODES>(tb, ta, p, s, pdl);
-    case DSQ_EPI_CODES_RES: return w3_launch<BITS, DSQ_EPI_CODES_RES>(tb, ta, p, s, pdl);
-    default: return w3_launch<BITS, DSQ_EPI_GENERAL>(tb, ta, p, s, pdl);
+    if constexpr (BITS != 3) {
+        switch (epi) {
+        case DSQ_EPI_CODES: return w3_launch<BITS, DSQ_EPI_CODES>(tb, ta, p, s, pdl);
+        case DSQ_EPI_CODES_RES: return w3_launch<BITS, DSQ_EPI_CODES_RES>(tb, ta, p, s, pdl);
+        default: break;
+        }
     }
+    return w3_launch<BITS, DSQ_EPI_GENERAL>(tb, ta, p, s, pdl);
 }
 
 }  // namespace
@@ -1183,21 +1255,14 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     if (conv->KH != 3 || conv->KW != 3 || conv->stride != 1 || conv->pad != 1)
         return DSQ_ERR_UNSUPPORTED;
     if (bits < 2 || bits > 4) return DSQ_ERR_UNSUPPORTED;
-    if (bits == 3) epi_kind = DSQ_EPI_GENERAL;   // the lean codes epilogue packs whole nibbles / pairs
     if (e.general_offset) epi_kind = DSQ_EPI_GENERAL;
     const int Cin = conv->Cin, Cout = conv->Cout;
     if (!(Cin == 64 || (Cin % 128 == 0 && Cin <= 1024))) return DSQ_ERR_UNSUPPORTED;
     if (shape->W + 2 > 32000 || shape->H + 2 > 32000) return DSQ_ERR_UNSUPPORTED;
-    // Which kernel (hook value 1 = automatic; measured on the ResNet-18- and
-    // VGG-16-shaped layers, per layer, 20 launches back to back):
-    //  * transposed tiles wherever they fit (3-bit codes: not on 7x7-sized images with
-    //    >= 512 input channels).  With up to 64 output channels the
-    //    transposed form needs the weight rows twice in its A operand (`dup`),
-    //    which it only gets from the blob's expanded copy: 64->64 at 56x56 runs
-    //    in 18 us against 22.5 us on plain tiles;
-    //  * otherwise plain tiles.
-    const bool tiny_deep = bits == 3 && shape->H * shape->W <= 64 && Cin >= 512;
-    if (hooks.window3 == 1 && tiny_deep) return DSQ_ERR_UNSUPPORTED;
+    // Which form: transposed tiles wherever they fit.  With up to 64 output channels they
+    // need the weight rows twice in the A operand (`dup`), from the blob's expanded copy
+    // or, at 3 bits, by the expansion warps: 64->64 at 56x56 runs in 18 us against 22.5 us
+    // on plain tiles.  Otherwise plain tiles.
     // the codes epilogues want the requantiser range to start at 0 and
     // floor(r_hi) = qmax
     float r_hi = 0.f;
@@ -1213,14 +1278,10 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     if (G > (1ll << 30)) return DSQ_ERR_UNSUPPORTED;
     p.Ncols = Cout;
     p.E = Cin;
-    p.two_taps = Cin == 64 && bits != 3;
     p.npl = Cin == 64 ? 1 : Cin / 128;
-    p.kpp = p.two_taps ? 5 : 9;
-    p.ksteps = p.npl * p.kpp;
     const int P = (int)dsq_row_pitch(Cin, bits);           // packed bytes per pixel
     p.PB = Cin == 64 ? P : 16 * bits;
     p.cpp = p.PB / 16;
-    p.xstep = p.two_taps ? 16 * bits : P;
     // Tiling, window and shared memory for one of the two kernel forms.
     // Transposed (tr): tiles of 256 positions x 128 output channels, A = weights.
     // Plain: 128 positions x up to 256 channels, A = window.
@@ -1230,12 +1291,17 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     const bool w8_ok = hooks.w8 && w8.enabled && e.half_offset && bits != 3;
     auto configure = [&](int tr) -> int {
         p.tr = tr;
+        p.two_taps = Cin == 64 && (bits != 3 || tr);
+        p.kpp = p.two_taps ? 5 : 9;
+        p.ksteps = p.npl * p.kpp;
+        p.xstep = p.two_taps ? 2 * P : P;
+        p.pk = p.two_taps ? 2 * P : 16 * bits;
         p.rb = tr && p.two_taps ? 64 : 128;
         // transposed tiles for <= 64 output channels: the weight rows twice in the
         // A operand (two TMA boxes of the expanded copy), so that all 128 lanes of
         // the accumulator, and all epilogue warps, carry data
         p.dup = tr && Cout <= 64;
-        if (p.dup && !w8_ok) return 0;
+        if (p.dup && !w8_ok && bits != 3) return 0;
         p.w8 = w8_ok && (Cout > 64 || p.dup);
         const int tile_pos = tr ? 256 : W3_BM;
         p.m_tiles = (int)((G + tile_pos - 1) / tile_pos);
@@ -1266,7 +1332,7 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
         if (p.ksteps <= W3_MAX_BST) {
             for (int as = W3_MAX_AS; as >= 2; --as) {
                 const int bp = p.w8 ? 0 : 2;
-                const W3Smem L = w3_layout(p.apx, p.rb, p.BN, bits, p.PB, as, p.ksteps, bp, p.cout_pad);
+                const W3Smem L = w3_layout(p.apx, p.rb, p.BN, p.pk, p.PB, as, p.ksteps, bp, p.cout_pad);
                 if (L.total + 1024 <= 227u * 1024u) {
                     p.b_res = 1; p.b_stages = p.ksteps; p.as_slots = as; p.bp_slots = bp;
                     return 1;
@@ -1279,7 +1345,7 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
             // no packed ring: the operand ring itself hides the latency of the loads
             for (int as = W3_MAX_AS; as >= 1; --as)
                 for (int bst = 6; bst >= 2; --bst) {
-                    const W3Smem L = w3_layout(p.apx, p.rb, p.BN, bits, p.PB, as, bst, 0, p.cout_pad);
+                    const W3Smem L = w3_layout(p.apx, p.rb, p.BN, p.pk, p.PB, as, bst, 0, p.cout_pad);
                     if (L.total + 1024 <= 227u * 1024u) {
                         p.as_slots = as; p.b_stages = bst; p.bp_slots = 0;
                         return 1;
@@ -1289,7 +1355,7 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
         }
         const int tries[6][3] = {{3, 3, 4}, {2, 3, 4}, {2, 2, 4}, {2, 2, 3}, {2, 2, 2}, {1, 2, 2}};
         for (int t = 0; t < 6; ++t) {
-            const W3Smem L = w3_layout(p.apx, p.rb, p.BN, bits, p.PB, tries[t][0], tries[t][1],
+            const W3Smem L = w3_layout(p.apx, p.rb, p.BN, p.pk, p.PB, tries[t][0], tries[t][1],
                                        tries[t][2], p.cout_pad);
             if (L.total + 1024 <= 227u * 1024u) {
                 p.as_slots = tries[t][0]; p.b_stages = tries[t][1]; p.bp_slots = tries[t][2];
@@ -1300,12 +1366,12 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     };
     int found = 0;
     const bool want_tr = hooks.window3 == 3 || hooks.window3 == 1;
-    if (bits != 3 && want_tr) found = configure(1);
+    if (want_tr) found = configure(1);
     if (!found) found = configure(0);
     if (!found) return DSQ_ERR_UNSUPPORTED;
     // (plain tiles convert accumulators by the 2^22 trick)
-    if (!p.tr && !small_acc) epi_kind = DSQ_EPI_GENERAL;
-    p.L = w3_layout(p.apx, p.rb, p.BN, bits, p.PB, p.as_slots, p.b_stages, p.bp_slots, p.cout_pad);
+    if (!p.tr && (!small_acc || bits == 3)) epi_kind = DSQ_EPI_GENERAL;
+    p.L = w3_layout(p.apx, p.rb, p.BN, p.pk, p.PB, p.as_slots, p.b_stages, p.bp_slots, p.cout_pad);
     p.smem_bytes = (int)p.L.total + 1024;
     // grid: a multiple of n_tiles; CTA c takes N tile c % n_tiles and every
     // mstep-th M tile
@@ -1367,7 +1433,7 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     } else {
         cuuint64_t dims[2] = {(cuuint64_t)9 * P, (cuuint64_t)Cout};
         cuuint64_t strides[1] = {(cuuint64_t)9 * P};
-        cuuint32_t box[2] = {(cuuint32_t)(16 * bits), (cuuint32_t)p.BN};
+        cuuint32_t box[2] = {(cuuint32_t)p.pk, (cuuint32_t)p.BN};
         cuuint32_t estr[2] = {1, 1};
         if (enc(&tb, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void *>(w_packed), dims, strides,
                 box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -1392,6 +1458,6 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
             return DSQ_ERR_UNSUPPORTED;
     }
     if (bits == 4) return w3_dispatch<4>(epi_kind, tb, ta, p, stream, hooks.pdl);
-    if (bits == 3) return w3_launch<3, DSQ_EPI_GENERAL>(tb, ta, p, stream, hooks.pdl);
+    if (bits == 3) return w3_dispatch<3>(epi_kind, tb, ta, p, stream, hooks.pdl);
     return w3_dispatch<2>(epi_kind, tb, ta, p, stream, hooks.pdl);
 }

@@ -334,12 +334,14 @@ double estimate_other(const CsParams &p, int bits, int Cin, double macs, int lea
     const int sms = dsq_sm_count() > 0 ? dsq_sm_count() : 148;
     const double ksteps = p.ksize * p.ksize * Cin / 128.0;
     if (p.ksize == 1 && lean) return 2.9 + (double)p.M * p.Ncols / 3.7e6;
-    if (p.ksize == 3 && p.stride == 1 && p.pad == 1 && bits != 3 && (Cin == 64 || Cin % 128 == 0)) {
-        // window kernel: waves of tiles of 256 positions x 128 channels
+    if (p.ksize == 3 && p.stride == 1 && p.pad == 1 && (Cin == 64 || Cin % 128 == 0)) {
+        // window kernel: waves of tiles of 256 positions x 128 channels (3-bit: the expansion
+        // warps set the pace)
         const double tiles = std::ceil((double)p.M / p.H / p.W * (p.H + 2) * (p.W + 2) / 256) *
                              ((p.Ncols + 127) / 128);
         return (Cin == 64 ? 4.3 : Cin <= 256 ? 7.7 : 5.5) +
-               std::ceil(tiles / sms) * ksteps * (Cin == 64 ? 0.4 : 0.27);
+               std::ceil(tiles / sms) * ksteps *
+                   (bits == 3 ? (Cin == 64 ? 0.53 : 0.42) : Cin == 64 ? 0.4 : 0.27);
     }
     return 4.3 + 0.23 * ksteps + macs / 4.5e8;                     // im2col kernel
 }

@@ -197,10 +197,16 @@ __device__ __forceinline__ uint32_t dsq_sat_bytes(int q0, int q1, int q2, int q3
     return r;
 }
 
-// eight such integers of consecutive elements -> their codes, packed (8 * BITS bits)
-template <int BITS>
+// eight such integers of consecutive elements -> their codes, packed (8 * BITS bits;
+// SLOT = 4: a 3-bit code in every four bits)
+template <int BITS, int SLOT = BITS>
 __device__ __forceinline__ uint32_t dsq_pack8(const int (&q)[8])
 {
+    if (BITS == 3 && SLOT == 4) {
+        const uint32_t e = dsq_sat_bytes(q[0], q[2], q[4], q[6]);
+        const uint32_t o = dsq_sat_bytes(q[1], q[3], q[5], q[7]);
+        return ((e >> 5) & 0x07070707u) | ((o >> 1) & 0x70707070u);
+    }
     if (BITS == 4) {
         const uint32_t e = dsq_sat_bytes(q[0], q[2], q[4], q[6]);
         const uint32_t o = dsq_sat_bytes(q[1], q[3], q[5], q[7]);
@@ -268,8 +274,8 @@ __device__ __forceinline__ unsigned long long dsq_code_pair(uint32_t x, int j)
 
 // Raw accumulators of eight consecutive output channels of one position -> their
 // packed codes; sc, bi: the channels' dsq_codes_affine in pairs, res: the
-// position's residual codes of those channels.
-template <int BITS, bool RES, bool LO>
+// position's residual codes of those channels (both in fields of SLOT bits).
+template <int BITS, bool RES, bool LO, int SLOT = BITS>
 __device__ __forceinline__ uint32_t dsq_lean_codes8(const uint32_t (&v)[8],
                                                     const unsigned long long (&sc)[4],
                                                     const unsigned long long (&bi)[4],
@@ -280,11 +286,11 @@ __device__ __forceinline__ uint32_t dsq_lean_codes8(const uint32_t (&v)[8],
     for (int c = 0; c < 4; ++c) {
         unsigned long long y = dsq_fma2(
             dsq_pack2(__int2float_rn((int)v[2 * c]), __int2float_rn((int)v[2 * c + 1])), sc[c], bi[c]);
-        if (RES) y = dsq_add2(y, dsq_fma2(dsq_code_pair<BITS>(res, c), l.res_delta2, l.res_lo2));
+        if (RES) y = dsq_add2(y, dsq_fma2(dsq_code_pair<SLOT>(res, c), l.res_delta2, l.res_lo2));
         if (LO) y = dsq_add2(y, l.neg_lo2);
         dsq_requant2<BITS>(y, l.inv2, q[2 * c], q[2 * c + 1]);
     }
-    return dsq_pack8<BITS>(q);
+    return dsq_pack8<BITS, SLOT>(q);
 }
 
 // Which accumulator column holds output channel ch of a group of 32.  The epilogue

@@ -98,21 +98,28 @@ __device__ __forceinline__ uint32_t expand_word(uint32_t w, int c, uint32_t orv)
     }
 }
 
-// words 4q..4q+3 of a 3-bit row step held in w[12]
+// Chunk q (16 codes) of a 3-bit row step held in w[12], both operands in the same order:
+// of every eight codes the even ones, then the odd ones (11 instructions for eight;
+// consecutive order took 17).
 template <bool SIGNED>
 __device__ __forceinline__ uint4 expand3_chunk(const uint32_t (&w)[12], int q, uint32_t orv)
 {
     uint32_t o[4];
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
-        const int bit = (16 * q + 4 * t) * 3;
+    for (int t = 0; t < 2; ++t) {
+        const int bit = (16 * q + 8 * t) * 3;
         const int wi = bit >> 5, sh = bit & 31;
         const uint32_t hi = wi + 1 < 12 ? w[wi + 1] : 0u;
         const uint32_t x = __funnelshift_r(w[wi], hi, sh);
-        uint32_t b = (x & 7u) | ((x & 0x38u) << 5) | ((x & 0x1C0u) << 10) |
-                     ((x & 0xE00u) << 15);
-        if (SIGNED) b = (b << 5) | orv;
-        o[t] = b;
+        const uint32_t y = (x & 0xFFFu) | ((x << 4) & 0x0FFF0000u);
+        const uint32_t z = (y & 0x003F003Fu) | ((y << 2) & 0x3F003F00u);
+        if (SIGNED) {
+            o[2 * t] = ((z << 5) & 0xE0E0E0E0u) | orv;
+            o[2 * t + 1] = ((z << 2) & 0xE0E0E0E0u) | orv;
+        } else {
+            o[2 * t] = z & 0x07070707u;
+            o[2 * t + 1] = (z >> 3) & 0x07070707u;
+        }
     }
     return make_uint4(o[0], o[1], o[2], o[3]);
 }
