@@ -6,20 +6,20 @@
 // tap.  Here every input pixel of a tile is expanded ONCE:
 //
 //   * Output positions are numbered in a zero-padded, stacked coordinate
-//     g = (n * (H+2) + ho) * (W+2) + wo.  The input pixel under filter tap
-//     (kh, kw) of output g then sits at padded position g + kh*(W+2) + kw,
+//     g = (n * (H+1) + ho) * (W+1) + wo.  The input pixel under filter tap
+//     (kh, kw) of output g then sits at padded position g + kh*(W+1) + kw,
 //     whatever g is: one constant shift per tap.  (Positions with ho >= H or
 //     wo >= W are padding of the numbering; their results are dropped.)
 //   * A tile is 128 consecutive positions g0 .. g0+127.  The padded input
-//     pixels g0 .. g0+129+2(W+2) are fetched by TMA im2col loads whose
-//     bounding box is the image grown by one pixel on every side (the loads
+//     pixels g0 .. g0+129+2(W+1) are fetched by TMA im2col loads whose
+//     bounding box is the image grown by one pixel at its left and top (the loads
 //     traverse W, then H, then N and fill what lies outside the image with
 //     zeros = code 0), into a packed staging buffer.
 //   * Four warps expand the staged codes to int8 rows of 128 bytes (128
 //     channels; wider inputs take several such "planes") in the K-major
 //     128-byte-swizzled layout the tensor core reads.
 //   * For tap (kh, kw) the A operand of tcgen05.mma is that SAME buffer, its
-//     descriptor's start address moved by (kh*(W+2) + kw) rows.  Nine taps x
+//     descriptor's start address moved by (kh*(W+1) + kw) rows.  Nine taps x
 //     Cin/32 instructions of 128 x BN x 32 accumulate one tile in tensor
 //     memory (two accumulator buffers: the epilogue of a tile overlaps the
 //     next tile's instructions).
@@ -40,7 +40,7 @@
 // window to tensor memory (ld.shared + tcgen05.st, A taken from there) was
 // slower than this one at every layer size and is not kept.
 //
-// Wide images (W + 2 > 139) would need a window of more than 416 pixels; they
+// Wide images (W + 1 > 139) would need a window of more than 416 pixels; they
 // are staged as three bands of 136 pixels, one per filter row, instead.
 //
 // Every wait on a barrier is bounded, as in the im2col kernel.
@@ -90,7 +90,7 @@ struct W3Smem {
 
 struct W3Params {
     // geometry
-    int N, H, W, Hp, Wp;               // Hp = H + 2, Wp = W + 2
+    int N, H, W, Hp, Wp;               // Hp = H + 1, Wp = W + 1 (see W3Pos)
     int m_tiles, n_tiles, BN, Ncols;
     int E;                             // int8 bytes per pixel = Cin
     int npl, kpp, ksteps;              // planes of 128 channels, K steps per plane, total
@@ -205,7 +205,12 @@ __device__ __forceinline__ void w3_codes_unit(const uint32_t (&r)[16], const flo
     for (int w = 0; w < BITS / 2; ++w) cw[w] -= 0x4B000000u * FIELDS;
 }
 
-// Position in the padded, stacked numbering: image, padded row, padded column.
+// Position in the padded, stacked numbering: image, padded row, padded column.  One
+// column of zeros serves as the right edge of a row and the left edge of the next, one
+// row of them as the bottom of an image and the top of the next: (H + 1)(W + 1)
+// positions an image, tap (kh, kw) of position g reads position g + kh (W + 1) + kw.
+// (With edges of their own, (H + 2)(W + 2), 28x28 512->512 at batch 32 was 113 tiles a
+// channel tile, four passes of 37 CTAs, instead of 106, three: 49.1 -> 38.8 us.)
 // Moving by a fixed number of positions is an addition of its (host-made)
 // decomposition plus at most one carry per digit: no division in any loop.
 struct W3Pos {
@@ -453,8 +458,8 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
             // The start coordinates of a fill's loads are worked out one fill ahead
             // (the first before anything can be issued), so that between the
             // moment a slot is free and the copies only the issue itself remains.
-            // Loads that start behind the last image hold nothing a valid output
-            // reads: they are left out (and not counted).  An im2col load must
+            // Loads that start behind the last image are left out (and not counted); the
+            // zeros below that image, if they begin there, are written here.  An im2col load must
             // start inside the map's bounding box (0 <= h < Hp, 0 <= w < Wp, n >= 0,
             // which the position arithmetic guarantees): a position outside it is
             // never issued - the roles then run into their wait limit and the
@@ -487,14 +492,26 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                     *ctl.abort_flag = 1;
                     break;
                 }
+                if (nl < nld) {
+                    // positions p.N * Hp * Wp .. + Wp of a load that is left out
+                    for (int i = 0; i < nld; ++i) {
+                        const int behind = (q[i].n - p.N) * img_positions + q[i].h * p.Wp + q[i].w;
+                        if (q[i].n < p.N || behind > p.Wp) continue;
+                        const uint32_t z = smem_u32(smem + L.a_stage) + s * a_stage_bytes +
+                                           (uint32_t)(i * p.a_box * p.PB);
+                        const int bytes = min(p.a_box, p.Wp + 1 - behind) * p.PB;
+                        for (int k = 0; k < bytes; k += 16) sts_128(z + k, 0u, 0u, 0u, 0u);
+                    }
+                    fence_proxy_async_smem();
+                }
                 mbar_arrive_expect_tx(bar_as_full(s), (uint32_t)(nl * p.a_box * p.PB));
                 const uint32_t dst0 = smem_u32(smem + L.a_stage) + s * a_stage_bytes;
 #pragma unroll
                 for (int i = 0; i < 3; ++i) {
                     if (i >= nld) break;
                     if (q[i].n >= p.N) continue;
-                    // bounding box = image grown by one pixel: base positions
-                    // -2 .. W-1 / -2 .. H-1, filter offset (1, 1)
+                    // bounding box = image grown by one pixel at the left and the top:
+                    // base positions -2 .. W-2 / -2 .. H-2, filter offset (1, 1)
                     tma_load_im2col_4d(dst0 + (uint32_t)(i * p.a_box * p.PB), &tmap_a, pl * p.PB,
                                        q[i].w - 2, q[i].h - 2, q[i].n, (uint16_t)1, (uint16_t)1,
                                        bar_as_full(s));
@@ -1258,7 +1275,7 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     if (e.general_offset) epi_kind = DSQ_EPI_GENERAL;
     const int Cin = conv->Cin, Cout = conv->Cout;
     if (!(Cin == 64 || (Cin % 128 == 0 && Cin <= 1024))) return DSQ_ERR_UNSUPPORTED;
-    if (shape->W + 2 > 32000 || shape->H + 2 > 32000) return DSQ_ERR_UNSUPPORTED;
+    if (shape->W + 1 > 32000 || shape->H + 1 > 32000) return DSQ_ERR_UNSUPPORTED;
     // Which form: transposed tiles wherever they fit.  With up to 64 output channels they
     // need the weight rows twice in the A operand (`dup`), from the blob's expanded copy
     // or, at 3 bits, by the expansion warps: 64->64 at 56x56 runs in 18 us against 22.5 us
@@ -1273,8 +1290,8 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     }
     W3Params p = {};
     p.N = shape->N; p.H = shape->H; p.W = shape->W;
-    p.Hp = p.H + 2; p.Wp = p.W + 2;
-    const int64_t G = ((int64_t)p.N - 1) * p.Hp * p.Wp + (int64_t)p.H * p.Wp;
+    p.Hp = p.H + 1; p.Wp = p.W + 1;
+    const int64_t G = ((int64_t)p.N - 1) * p.Hp * p.Wp + (int64_t)(p.H - 1) * p.Wp + p.W;
     if (G > (1ll << 30)) return DSQ_ERR_UNSUPPORTED;
     p.Ncols = Cout;
     p.E = Cin;
@@ -1442,13 +1459,12 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     }
     {
         // im2col map over the NHWC codes: the bounding box of base positions is
-        // [-2, W-1] x [-2, H-1] (lower corner -2, upper corner 0) and every load
-        // uses filter offset (1, 1): pixels -1 .. W / -1 .. H, the image grown by
-        // its zero padding
+        // [-2, W-2] x [-2, H-2] (lower corner -2, upper corner -1) and every load
+        // uses filter offset (1, 1): pixels -1 .. W-1 / -1 .. H-1
         cuuint64_t dims[4] = {(cuuint64_t)P, (cuuint64_t)p.W, (cuuint64_t)p.H, (cuuint64_t)p.N};
         cuuint64_t strides[3] = {(cuuint64_t)P, (cuuint64_t)P * p.W, (cuuint64_t)P * p.W * p.H};
         int lower[2] = {-2, -2};
-        int upper[2] = {0, 0};
+        int upper[2] = {-1, -1};
         cuuint32_t estr[4] = {1, 1, 1, 1};
         if (enc_i2c(&ta, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<void *>(act_codes), dims,
                     strides, lower, upper, (cuuint32_t)p.PB, (cuuint32_t)p.a_box, estr,

@@ -337,7 +337,7 @@ double estimate_other(const CsParams &p, int bits, int Cin, double macs, int lea
     if (p.ksize == 3 && p.stride == 1 && p.pad == 1 && (Cin == 64 || Cin % 128 == 0)) {
         // window kernel: waves of tiles of 256 positions x 128 channels (3-bit: the expansion
         // warps set the pace)
-        const double tiles = std::ceil((double)p.M / p.H / p.W * (p.H + 2) * (p.W + 2) / 256) *
+        const double tiles = std::ceil((double)p.M / p.H / p.W * (p.H + 1) * (p.W + 1) / 256) *
                              ((p.Ncols + 127) / 128);
         return (Cin == 64 ? 4.3 : Cin <= 256 ? 7.7 : 5.5) +
                std::ceil(tiles / sms) * ksteps *
