@@ -179,33 +179,45 @@ dwconv3x3_kernel(const uint8_t *__restrict__ act, const uint8_t *__restrict__ wg
 // and SM, measured); all in all about 10 instructions per element.  The dp4a
 // form this replaces took 30 (byte transposes, funnel shifts and an epilogue of
 // 9) and only existed for 4-bit codes: C = 144, 56x56, batch 64, 4-bit 41.9 us.
+// Loaded words are kept as they came until a row's arithmetic is done (DwhRaw), and
+// the padding behind 2- and 3-bit rows is no unit of work: 112x112, 32 channels, batch 64
+// 2-bit 45.2 -> 22.6 us, 3-bit 42.4 -> 31.4 us (4-bit 19.8).
 // ---------------------------------------------------------------------------
 constexpr int DWH_THREADS = 128, DWH_BLOCKS_PER_SM = 3;
 
 struct DwHalf {
     int N, H, W, C, Ho, Wo, pitch;
-    int units;                // 8-channel units of a row, padding lanes included
+    int units;                // 8-channel units of a row (4-bit: padding lanes included)
+    int spare;                // 2- and 3-bit: bytes of a row behind them
     int strips, rows, chunks; // strips of four columns; output rows of a work item
     int half_offset;
     int early;                // dsq_early_constants
     float inv;
 };
 
-// the unit's packed codes as 4 + 4 fields: field j at bit BITS * j, field j + 4 at
-// bit 16 + BITS * j
+// the words a unit's packed codes lie in (3-bit: 3 bytes at 3 u, one or two aligned
+// words), as loaded: what is done to them waits for the load, so it is left to the place
+// that uses them, a row of arithmetic later
+template <int BITS> struct DwhRaw { uint32_t v[BITS == 3 ? 2 : 1]; };
 template <int BITS>
-__device__ __forceinline__ uint32_t dwh_load(const uint8_t *row, int u, int pitch)
+__device__ __forceinline__ void dwh_load(const uint8_t *row, int u, int pitch, DwhRaw<BITS> &r)
 {
-    if (BITS == 4) return __ldg(reinterpret_cast<const uint32_t *>(row) + u);
-    if (BITS == 2) {
-        const uint32_t x = __ldg(reinterpret_cast<const uint16_t *>(row) + u);
-        return __byte_perm(x, 0u, 0x4140);                 // byte 1 -> byte 2
+    if (BITS == 4) r.v[0] = __ldg(reinterpret_cast<const uint32_t *>(row) + u);
+    if (BITS == 2) r.v[0] = __ldg(reinterpret_cast<const uint16_t *>(row) + u);
+    if (BITS == 3) {
+        const uint32_t *w = reinterpret_cast<const uint32_t *>(row);
+        const int i = (3 * u) >> 2, last = pitch / 4 - 1;
+        r.v[0] = __ldg(w + min(i, last));
+        r.v[BITS == 3] = __ldg(w + min(i + 1, last));
     }
-    // 3 bytes at 3 u: the one or two aligned words they lie in
-    const uint32_t *w = reinterpret_cast<const uint32_t *>(row);
-    const int i = (3 * u) >> 2, last = pitch / 4 - 1;
-    const uint32_t x = __funnelshift_r(__ldg(w + min(i, last)), __ldg(w + min(i + 1, last)),
-                                       8 * ((3 * u) & 3));
+}
+// 4 + 4 fields: field j at bit BITS * j, field j + 4 at bit 16 + BITS * j
+template <int BITS>
+__device__ __forceinline__ uint32_t dwh_split(const DwhRaw<BITS> &r, int u)
+{
+    if (BITS == 4) return r.v[0];
+    if (BITS == 2) return __byte_perm(r.v[0], 0u, 0x4140);   // byte 1 -> byte 2
+    const uint32_t x = __funnelshift_r(r.v[0], r.v[BITS == 3], 8 * ((3 * u) & 3));
     return (x & 0xFFFu) | ((x & 0xFFF000u) << 4);
 }
 
@@ -259,7 +271,9 @@ dwconv3x3_half_kernel(const uint8_t *__restrict__ act, const uint8_t *__restrict
         const __half2 base = __float2half2_rn(1024.0f + HALF);
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
-            const uint32_t x = dwh_load<BITS>(wgt + k * p.pitch, u, p.pitch);
+            DwhRaw<BITS> raw;
+            dwh_load<BITS>(wgt + k * p.pitch, u, p.pitch, raw);
+            const uint32_t x = dwh_split<BITS>(raw, u);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const uint32_t m = (dwh_field<BITS>(x, j) ^ (HALF | (HALF << 16))) | 0x64006400u;
@@ -294,15 +308,15 @@ dwconv3x3_half_kernel(const uint8_t *__restrict__ act, const uint8_t *__restrict
         const int hi0 = ho0 * STRIDE - 1, wi0 = wo0 * STRIDE - 1;
         const uint8_t *base = act + ((int64_t)n * p.H * p.W + wi0) * p.pitch;
         const bool inner = wi0 >= 0 && wi0 + NP <= p.W;
-        uint32_t next[NP];
+        DwhRaw<BITS> next[NP];
         auto load_row = [&](int hi) {
             const bool in = hi >= 0 && hi < p.H;
             const uint8_t *row = base + (int64_t)hi * p.W * p.pitch;
 #pragma unroll
             for (int x = 0; x < NP; ++x) {
-                next[x] = 0u;
+                next[x] = DwhRaw<BITS>{};
                 if (in && (inner || (wi0 + x >= 0 && wi0 + x < p.W)))
-                    next[x] = dwh_load<BITS>(row + x * p.pitch, u, p.pitch);
+                    dwh_load<BITS>(row + x * p.pitch, u, p.pitch, next[x]);
             }
         };
         uint8_t *out = y_codes + (((int64_t)n * p.Ho + ho0) * p.Wo + wo0) * p.pitch;
@@ -332,11 +346,14 @@ dwconv3x3_half_kernel(const uint8_t *__restrict__ act, const uint8_t *__restrict
                 } else if (BITS == 2) {
                     if (live) reinterpret_cast<uint16_t *>(dst)[u] = (uint16_t)cw;
                 } else if (live) {
-                    // (units up to the row pitch: the spare bytes are written as zeros)
-                    const int at = 3 * u;
-                    dst[at] = (uint8_t)cw;
-                    if (at + 1 < p.pitch) dst[at + 1] = (uint8_t)(cw >> 8);
-                    if (at + 2 < p.pitch) dst[at + 2] = (uint8_t)(cw >> 16);
+                    // three bytes: the two at an even address together
+                    const int odd = u & 1;
+                    dst += 3 * u;
+                    *reinterpret_cast<uint16_t *>(dst + odd) = (uint16_t)(cw >> (8 * odd));
+                    dst[odd ? 0 : 2] = (uint8_t)(cw >> (odd ? 0 : 16));
+                    // and the row's spare bytes (a pass over the pixels: 2 % slower)
+                    dst += 3 * (p.units - u);
+                    for (int at = u; at < p.spare; at += p.units) dst[at] = 0;
                 }
             }
             out += (int64_t)p.Wo * p.pitch;
@@ -352,12 +369,14 @@ dwconv3x3_half_kernel(const uint8_t *__restrict__ act, const uint8_t *__restrict
                 const int s = s0 + t;
                 if (s >= n_in) break;
 #pragma unroll
-                for (int x = 0; x < NP; ++x)
+                for (int x = 0; x < NP; ++x) {
+                    const uint32_t codes = dwh_split<BITS>(next[x], u);
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        const uint32_t f = dwh_field<BITS>(next[x], j);
+                        const uint32_t f = dwh_field<BITS>(codes, j);
                         q[x][j] = *reinterpret_cast<const __half2 *>(&f);
                     }
+                }
                 if (s + 1 < n_in) load_row(hi0 + s + 1);
                 if (STRIDE == 1) {
                     // output row s starts, s - 1 goes on, s - 2 is completed
@@ -377,6 +396,15 @@ dwconv3x3_half_kernel(const uint8_t *__restrict__ act, const uint8_t *__restrict
                     if (s >> 1 < rows) taps(acc[(t >> 1) & 1], 0, true);
                 }
             }
+        }
+    }
+    // 2 bits: the rows' spare bytes are zeros, written in a pass of their own over output
+    // pixels (as units of work they were half of the whole on 32-channel rows)
+    if (BITS == 2 && p.spare) {
+        const int64_t pixels = (int64_t)p.N * p.Ho * p.Wo;
+        for (int64_t i = gtid; i < pixels; i += gridDim.x * DWH_THREADS) {
+            uint16_t *dst = reinterpret_cast<uint16_t *>(y_codes + i * p.pitch) + p.units;
+            for (int k = 0; k < p.spare; k += 2) dst[k / 2] = 0;
         }
     }
 }
@@ -413,7 +441,7 @@ extern "C" int dsq_dwconv2d(const void *act_codes, const dsq_nhwc_t *shape,
     // codes to codes, requantiser range starting at 0 (the lean epilogue does not
     // subtract lo); images of at least 2^31 bytes a row keep the general kernel's
     // 64-bit indexing
-    const int units = (pitch + bits - 1) / bits;
+    const int units = bits == 4 ? pitch / 4 : (shape->C + 7) / 8;
     const int strips = (Wo + 3) / 4;
     if (y_codes && !y_f32 && !acc_out && !e.residual && !e.general_offset && e.rq.lo == 0.0f &&
         (int64_t)units * strips * Ho * shape->N < (1ll << 31)) {
@@ -421,6 +449,7 @@ extern "C" int dsq_dwconv2d(const void *act_codes, const dsq_nhwc_t *shape,
         p.N = shape->N; p.H = shape->H; p.W = shape->W; p.C = shape->C;
         p.Ho = Ho; p.Wo = Wo; p.pitch = pitch;
         p.units = units; p.strips = strips;
+        p.spare = pitch - units * bits;
         p.half_offset = e.half_offset;
         p.inv = e.rq.inv;
         p.early = dsq_early_constants();
