@@ -382,6 +382,9 @@ dsq_pw_kernel(const __grid_constant__ CUtensorMap tmap_a, const PwParams p)
         const int j = lane & 3;                       // eight channels 8 j .. of the 32
         unsigned long long sc[4], bi[4];
         int cu_held = -1;
+        // (only the last N tile's columns end near the pitch)
+        const int spare_from = n_tile == p.n_tiles - 1
+                                   ? (n_tile * p.BN + col_units * 32) * BITS / 8 + 4 * j : p.out_pitch;
         bool ok = true;
 #pragma unroll 1
         for (int it = group; ok && it < my_tiles; it += 2) {
@@ -435,29 +438,45 @@ dsq_pw_kernel(const __grid_constant__ CUtensorMap tmap_a, const PwParams p)
                                            q[o + 8], q[o + 9], q[o + 12], q[o + 13]};
                     cw[i] = dsq_lean_codes8<BITS, RES, LO>(v, sc, bi, RES ? res[i] : 0u, lean);
                 }
+                if (BITS == 2) {
+                    // a word is two lanes' half words: even lanes store pixels 0 and 2's, odd
+                    // lanes pixels 1 and 3's
+                    const int odd = j & 1;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int m = mr + 8 * i;
-                    uint32_t word = cw[i];
-                    int at = byte0;
-                    bool live = m < p.M;
-                    if (BITS == 2) {
-                        // two lanes' half words
-                        word |= __shfl_down_sync(0xffffffffu, cw[i], 1) << 16;
-                        live &= (j & 1) == 0;
-                    } else if (BITS == 3) {
-                        // the four lanes' 3 x 4 bytes as three words
-                        const uint32_t nx = __shfl_down_sync(0xffffffffu, cw[i], 1);
-                        word = (cw[i] >> (8 * j)) | (nx << (24 - 8 * j));
-                        at = byte0 + j;
-                        live &= j < 3;
+                    for (int i = 0; i < 4; i += 2) {
+                        const uint32_t got =
+                            __shfl_xor_sync(0xffffffffu, odd ? cw[i] : cw[i + 1], 1);
+                        const uint32_t word = odd ? got | (cw[i + 1] << 16) : cw[i] | (got << 16);
+                        const int m = mr + 8 * (i + odd), at = byte0 - 2 * odd;
+                        if (m < p.M && at < p.out_pitch)
+                            *reinterpret_cast<uint32_t *>(p.e.y_codes + (int64_t)m * p.out_pitch + at) = word;
                     }
-                    uint8_t *row = p.e.y_codes + (int64_t)m * p.out_pitch;
-                    if (live && at < p.out_pitch) *reinterpret_cast<uint32_t *>(row + at) = word;
-                    // (the last unit may end before the row's pitch does)
-                    if (BITS != 4 && m < p.M && j == 0 && cu == col_units - 1 && n_tile == p.n_tiles - 1)
-                        for (int b = byte0 + 4 * BITS; b < p.out_pitch; b += 4)
-                            *reinterpret_cast<uint32_t *>(row + b) = 0u;
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int m = mr + 8 * i;
+                        uint32_t word = cw[i];
+                        int at = byte0;
+                        bool live = m < p.M;
+                        if (BITS == 3) {
+                            // the four lanes' 3 x 4 bytes as three words
+                            const uint32_t nx = __shfl_down_sync(0xffffffffu, cw[i], 1);
+                            word = (cw[i] >> (8 * j)) | (nx << (24 - 8 * j));
+                            at = byte0 + j;
+                            live &= j < 3;
+                        }
+                        uint8_t *row = p.e.y_codes + (int64_t)m * p.out_pitch;
+                        if (live && at < p.out_pitch) *reinterpret_cast<uint32_t *>(row + at) = word;
+                    }
+                }
+                // the last unit may end before the row's pitch does (by at most 12 bytes): a
+                // word per lane (one lane for all of them took 5 to 10 us of 48)
+                if (BITS != 4 && cu == col_units - 1 && spare_from < p.out_pitch) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (mr + 8 * i < p.M)
+                            *reinterpret_cast<uint32_t *>(p.e.y_codes + (int64_t)(mr + 8 * i) * p.out_pitch +
+                                                          spare_from) = 0u;
                 }
                 if (++mt == p.mt) { mt = 0; ++cu; }
             }
