@@ -120,7 +120,6 @@ struct W3Params {
     int early;                         // dsq_early_constants
     unsigned long long wait_ns;
     int skip_b_round;
-    int base_offset_mode;              // probe: put the row phase into the descriptor
     // epilogue
     int shift, out_pitch;
     float r_hi;                        // fmaf(hi - lo, inv, 0.5f) of the requantiser
@@ -1415,7 +1414,6 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     p.wait_ns = hooks.wait_ns;
     p.skip_b_round = hooks.skip_b_round;
     p.early = dsq_early_constants();
-    p.base_offset_mode = hooks.window3 == 2;   // (probe)
     p.e = e;
     p.r_hi = r_hi;
     p.out_pitch = (int)dsq_row_pitch(Cout, bits);
