@@ -11,6 +11,10 @@
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/autograd/python_variable.h>
 
+#include <memory>
+#include <string>
+#include <vector>
+
 #include "../../include/dsq.h"
 #include "dsq_plan.h"
 
@@ -389,74 +393,137 @@ PyObject *wgemm(PyObject *, PyObject *const *a, Py_ssize_t n)
 }
 
 // ---- recorded call sequences (dsq_plan.h) -----------------------------------
-// What a plan was recorded from: the objects a caller could exchange between
-// two passes (tensors, ranges, layers).  A plan runs only while every one of
-// them is still the same object at the same address.
-struct Recorded {
-    dsq_plan *plan = nullptr;
-    std::vector<PyObject *> held;             // strong references
-    std::vector<const void *> data;           // data pointer of a tensor, else null
+// What a plan was recorded from: everything a caller could exchange or change in
+// place between two passes (tensors, ranges, layers).  A plan runs only while all
+// of it is as it was.  The parts are walked in one order, each leaving an entry:
+//   * a device tensor: the object, its address, size and type - its contents are the
+//     kernels' business;
+//   * dicts (keys too), lists, tuples and objects with attributes (a layer): their
+//     kind and size, then what they are made of;
+//   * an object with a buffer (a ctypes structure, a numpy scalar): the object and a
+//     copy of its bytes;
+//   * numbers, strings, None: the object.
+// Anything else could change unseen, host tensors and device scalars (a range read
+// with float()) among them: such a plan runs once and is recorded again.
+struct Part {
+    PyObject *o = nullptr;                    // held; of a container: its type
+    const void *data = nullptr;               // tensor: address
+    int64_t size = 0;                         // tensor: elements; container: members
+    int type = 0;                             // tensor: scalar type, or -1
+    std::string bytes;
+    bool operator==(const Part &p) const
+    {
+        return o == p.o && data == p.data && size == p.size && type == p.type && bytes == p.bytes;
+    }
 };
 
-const void *data_of(PyObject *o)
+struct Recorded {
+    dsq_plan *plan = nullptr;
+    std::vector<Part> parts;
+    bool once = false, ran = false;           // holds something that could change unseen
+    ~Recorded()
+    {
+        dsq_plan_free(plan);
+        for (Part &p : parts) Py_XDECREF(p.o);
+    }
+};
+
+bool is_value(PyObject *o)
 {
-    return THPVariable_Check(o) ? THPVariable_Unpack(o).data_ptr() : nullptr;
+    return o == Py_None || PyFloat_CheckExact(o) || PyUnicode_CheckExact(o) || PyLong_CheckExact(o) ||
+           PyBool_Check(o) || PyBytes_CheckExact(o);
 }
 
-// Calls f(object) for every object `o` is made of: the values of dicts, the
-// items of lists and tuples, recursively; stops when f says so.
-template <class F> bool each_part(PyObject *o, F &f)
+// Calls f(part) for everything `o` is made of, as above; sets *opaque where a change
+// could not be seen; stops when f says so.
+template <class F> bool each_part(PyObject *o, F &f, bool *opaque, int depth = 0)
 {
-    if (PyDict_Check(o)) {
+    Part p;
+    auto container = [&](Py_ssize_t n) {
+        p.o = (PyObject *)Py_TYPE(o);
+        p.size = n;
+        return f(p);
+    };
+    auto attributes = [&](PyObject *dict) {
         Py_ssize_t at = 0;
         PyObject *k, *v;
-        while (PyDict_Next(o, &at, &k, &v))
-            if (!each_part(v, f)) return false;
+        if (!container(PyDict_GET_SIZE(dict))) return false;
+        while (PyDict_Next(dict, &at, &k, &v))
+            if (!each_part(k, f, opaque, depth + 1) || !each_part(v, f, opaque, depth + 1)) return false;
         return true;
+    };
+    p.o = o;
+    if (is_value(o)) return f(p);
+    if (THPVariable_Check(o)) {
+        const at::Tensor &t = THPVariable_Unpack(o);
+        if (!t.is_cuda() || t.dim() == 0 || !t.is_contiguous()) *opaque = true;
+        else p.data = t.data_ptr();
+        p.size = t.numel();
+        p.type = (int)t.scalar_type();
+        return f(p);
     }
+    if (depth > 32) {                         // (an object that holds itself)
+        *opaque = true;
+        return f(p);
+    }
+    if (PyDict_Check(o)) return attributes(o);
     if (PyList_Check(o) || PyTuple_Check(o)) {
         const Py_ssize_t n = PyList_Check(o) ? PyList_GET_SIZE(o) : PyTuple_GET_SIZE(o);
+        if (!container(n)) return false;
         for (Py_ssize_t i = 0; i < n; ++i)
-            if (!each_part(PyList_Check(o) ? PyList_GET_ITEM(o, i) : PyTuple_GET_ITEM(o, i), f))
+            if (!each_part(PyList_Check(o) ? PyList_GET_ITEM(o, i) : PyTuple_GET_ITEM(o, i), f, opaque,
+                           depth + 1))
                 return false;
         return true;
     }
-    return f(o);
+    if (PyObject_CheckBuffer(o)) {
+        Py_buffer b;
+        if (PyObject_GetBuffer(o, &b, PyBUF_SIMPLE) == 0) {
+            p.type = -1;
+            p.bytes.assign(static_cast<const char *>(b.buf), (size_t)b.len);
+            PyBuffer_Release(&b);
+            return f(p);
+        }
+        PyErr_Clear();
+    } else if (PyObject *dict = PyObject_GenericGetDict(o, nullptr)) {
+        const bool ok = attributes(dict);
+        Py_DECREF(dict);
+        // (members in slots are not in the dict)
+        if (ok && PyObject_HasAttrString((PyObject *)Py_TYPE(o), "__slots__")) *opaque = true;
+        return ok;
+    } else {
+        PyErr_Clear();
+    }
+    *opaque = true;
+    return f(p);
 }
 
 void free_recorded(PyObject *capsule)
 {
-    Recorded *r = static_cast<Recorded *>(PyCapsule_GetPointer(capsule, "dsq_plan"));
-    if (!r) return;
-    dsq_plan_free(r->plan);
-    for (PyObject *o : r->held) Py_DECREF(o);
-    delete r;
+    delete static_cast<Recorded *>(PyCapsule_GetPointer(capsule, "dsq_plan"));
 }
 
 // (function, parts) -> plan of the calls that function() makes
 PyObject *plan_record(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
     return guarded(n, 2, [&]() -> PyObject * {
-        check(dsq_plan_begin(), "dsq_plan_begin");
-        PyObject *r = PyObject_CallNoArgs(a[0]);
-        dsq_plan *plan = nullptr;
-        const int st = dsq_plan_end(&plan);
-        if (!r) {
-            dsq_plan_free(plan);
-            throw PyFailed();
-        }
-        Py_DECREF(r);
-        check(st, "dsq_plan_end");
-        Recorded *rec = new Recorded;
-        rec->plan = plan;
-        auto keep = [&](PyObject *o) {
-            rec->held.push_back(Py_NewRef(o));
-            rec->data.push_back(data_of(o));
+        std::unique_ptr<Recorded> rec(new Recorded);
+        // (before the calls: what they change of it makes the plan invalid)
+        auto keep = [&](Part &p) {
+            rec->parts.push_back(p);
+            Py_XINCREF(p.o);
             return true;
         };
-        each_part(a[1], keep);
-        PyObject *c = PyCapsule_New(rec, "dsq_plan", free_recorded);
+        each_part(a[1], keep, &rec->once);
+        check(dsq_plan_begin(), "dsq_plan_begin");
+        PyObject *r = PyObject_CallNoArgs(a[0]);
+        const int st = dsq_plan_end(&rec->plan);
+        if (!r) throw PyFailed();
+        Py_DECREF(r);
+        check(st, "dsq_plan_end");
+        PyObject *c = PyCapsule_New(rec.get(), "dsq_plan", free_recorded);
         if (!c) throw PyFailed();
+        rec.release();
         return c;
     });
 }
@@ -466,16 +533,14 @@ PyObject *plan_record(PyObject *, PyObject *const *a, Py_ssize_t n)
 PyObject *plan_run(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
     return guarded(n, 2, [&]() -> PyObject * {
-        const Recorded *r = static_cast<const Recorded *>(PyCapsule_GetPointer(a[0], "dsq_plan"));
+        Recorded *r = static_cast<Recorded *>(PyCapsule_GetPointer(a[0], "dsq_plan"));
         if (!r) throw PyFailed();
+        if ((r->once && r->ran) || !dsq_plan_valid(r->plan)) Py_RETURN_FALSE;
         size_t i = 0;
-        auto same = [&](PyObject *o) {
-            const bool ok = i < r->held.size() && r->held[i] == o && r->data[i] == data_of(o);
-            ++i;
-            return ok;
-        };
-        if (!dsq_plan_valid(r->plan) || !each_part(a[1], same) || i != r->held.size())
-            Py_RETURN_FALSE;
+        bool opaque = false;
+        auto same = [&](const Part &p) { return i < r->parts.size() && r->parts[i++] == p; };
+        if (!each_part(a[1], same, &opaque) || i != r->parts.size()) Py_RETURN_FALSE;
+        r->ran = true;
         check(enqueue([&](void *s) { return dsq_plan_run(r->plan, s); }), "dsq_plan_run");
         Py_RETURN_TRUE;
     });

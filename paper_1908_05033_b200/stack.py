@@ -69,10 +69,10 @@ class GpuStack:
         self._plan = None
 
     def _parts(self):
-        """Everything the recorded calls were made from: exchange one of these
-        objects and the calls are recorded again."""
+        """Everything _call_layers reads.  Exchange one of these objects, or change a
+        layer's attributes or geometry in place, and the calls are recorded again."""
         return (self.layers, self.codes, self.ranges, self.shapes, self.ws, self.batch, self.bits,
-                self.w_offset, self.st)
+                self.w_offset)
 
     def forward(self, x):
         """x: fp32 NHWC CUDA tensor, or None to run the layers on the input

@@ -44,3 +44,67 @@ def test_replayed_pass(bits):
     x.copy_(x0 * 1.3)
     graph.replay()
     assert torch.equal(out, calls.forward(x0 * 1.3))
+
+
+def _pair(bits=4):
+    """A stack that makes its calls in every pass and one that replays them, of the same
+    layer list."""
+    from paper_1908_05033_b200.stack import GpuStack
+    st = dsq_inputs.tiny_stack(bits=bits)
+    params = dsq_inputs.stack_params(st, workload_id=9)
+    x = T(dsq_inputs.stack_input(st, batch=st.batch, workload_id=9))
+    return GpuStack(st, params, keep_debug=True), GpuStack(st, params), x
+
+
+@pytest.mark.parametrize("passes", [1, 5])       # launched one by one, and as a graph
+def test_changes_in_place(passes):
+    """What a layer is made of may be changed in place between two passes."""
+    calls, replay, x = _pair()
+
+    def same():
+        want = calls.forward(x).clone()
+        assert torch.equal(replay.forward(x), want)
+        return want
+
+    for _ in range(passes):
+        before = same()
+    layer = next(L for L, _ in replay.layers if L.name == "c3")      # (both stacks' layer)
+    layer.out_hi = 0.7
+    assert not torch.equal(before, same())
+    layer.residual = None                        # no shortcut any more
+    same()
+    # geometry of a 1x1 convolution, a ctypes structure: a stride it does not take is refused
+    for net in (calls, replay):
+        next(w for L, w in net.layers if L.name == "pj")["conv"].stride = 3
+    for net in (calls, replay):
+        with pytest.raises(RuntimeError, match="not supported"):
+            net.forward(x)
+        next(w for L, w in net.layers if L.name == "pj")["conv"].stride = 1
+    same()
+
+
+def test_values_read_on_the_host():
+    """A range held as a tensor is read in every pass, and so is a layer of a class whose
+    attributes are not in its dict."""
+    calls, replay, x = _pair()
+    hi = torch.tensor(2.0)
+
+    class Slots:
+        __slots__ = ("name", "kind", "src", "dst", "residual", "out_lo", "out_hi")
+
+        def __init__(self, L):
+            for k in self.__slots__:
+                setattr(self, k, getattr(L, k))
+
+    for net in (calls, replay):
+        i = next(i for i, (L, _) in enumerate(net.layers) if L.name == "c3")
+        net.layers[i] = (Slots(net.layers[i][0]), net.layers[i][1])
+        net.layers[i][0].out_hi = hi
+    slots = [next(L for L, _ in net.layers if L.name == "c3") for net in (calls, replay)]
+    for value in (2.0, 0.7, 1.1, 1.1):
+        hi.fill_(value)
+        assert torch.equal(replay.forward(x), calls.forward(x)), value
+    for value in (0.8, 1.9):
+        for s in slots:
+            s.out_hi = value
+        assert torch.equal(replay.forward(x), calls.forward(x)), value
