@@ -21,6 +21,8 @@ def _delta_f32(bits, lo, hi):
 
 
 class GpuStack:
+    _plan = None          # the recorded pass: of this object and process only
+
     def __init__(self, st, params, batch=None, w_offset=0.5, device="cuda",
                  keep_debug=False):
         self.st, self.bits, self.w_offset = st, st.bits, w_offset
@@ -66,7 +68,10 @@ class GpuStack:
                                         bias=bias)))
         B.check_workspace(self.ws, "dsq_pack_weights")
         self.debug = {}
-        self._plan = None
+
+    def __getstate__(self):
+        """A copied or pickled stack records its own pass."""
+        return {k: v for k, v in self.__dict__.items() if k != "_plan"}
 
     def _parts(self):
         """Everything _call_layers reads.  Exchange one of these objects, or change a

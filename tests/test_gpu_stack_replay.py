@@ -1,6 +1,9 @@
 """A stack's recorded pass: the same codes as the calls it was made from, in the passes
 that launch one by one, from the graph, in a caller's capture, and after something the
 calls were made from has been exchanged."""
+import copy
+import pickle
+
 import pytest
 import torch
 
@@ -108,3 +111,18 @@ def test_values_read_on_the_host():
         for s in slots:
             s.out_hi = value
         assert torch.equal(replay.forward(x), calls.forward(x)), value
+
+
+@pytest.mark.parametrize("how", [copy.copy, copy.deepcopy, lambda net: pickle.loads(pickle.dumps(net))])
+def test_copies(how):
+    """A stack that has recorded its pass can still be copied and pickled; the copy gives
+    the same codes from buffers of its own (a shallow one from the same)."""
+    calls, replay, x = _pair()
+    for passes in (1, 4):
+        for _ in range(passes):
+            replay.forward(x)
+        other = how(replay)
+        for scale in (1.0, 1.3, 0.8, 1.1):
+            want = calls.forward(x * scale).clone()
+            assert torch.equal(other.forward(x * scale), want)
+        assert torch.equal(replay.forward(x * 0.9), calls.forward(x * 0.9))
