@@ -32,18 +32,37 @@ struct DsqLaunchRec {
     alignas(64) unsigned char args[1024];
 };
 
+// While one lives, calls that a stream capture anywhere in the process would forbid
+// (creating and destroying streams, graphs, page-locked memory) are open to this
+// thread and leave that capture alone.  Only around calls that enqueue nothing on a
+// stream of the caller's.
+struct DsqCaptureRelaxed {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    bool changed;
+    DsqCaptureRelaxed() : changed(cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess) {}
+    ~DsqCaptureRelaxed()
+    {
+        if (changed) cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+    DsqCaptureRelaxed(const DsqCaptureRelaxed &) = delete;
+    DsqCaptureRelaxed &operator=(const DsqCaptureRelaxed &) = delete;
+};
+
 struct dsq_plan {
     std::vector<DsqLaunchRec> recs;
     unsigned hooks_generation = 0;      // of the process-wide hooks when recorded
     int device = -1;
     int status = DSQ_OK;                // first failure while recording
-    // the launches as a CUDA graph, made on the third run (dsq_plan_run); guarded
-    mutable std::mutex lock;
-    mutable int runs = 0;
-    mutable cudaGraphExec_t graph = nullptr;
+    // the launches as a CUDA graph (dsq_plan_run); guarded by the lock
+    std::mutex lock;
+    int64_t runs = 0, next_try = GRAPH_AFTER;
+    cudaGraphExec_t graph = nullptr;
+    static constexpr int GRAPH_AFTER = 3;
     ~dsq_plan()
     {
-        if (graph) cudaGraphExecDestroy(graph);
+        if (!graph) return;
+        const DsqCaptureRelaxed relaxed;
+        cudaGraphExecDestroy(graph);
     }
 };
 

@@ -9,6 +9,8 @@ between layers.  The call sequence can be captured in a CUDA graph.
 The layers' calls are the same in every pass, so they are made once, recorded
 as finished launches, and a pass replays them from native code (2 us a launch
 instead of 13 us a call; at small batch the calls took longer than the kernels).
+The third pass makes a CUDA graph of them, which takes about 0.3 ms of host time once
+and whatever memory CUDA keeps for a graph; later passes launch that graph.
 """
 import numpy as np
 import torch

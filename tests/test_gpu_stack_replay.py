@@ -3,6 +3,7 @@ that launch one by one, from the graph, in a caller's capture, and after somethi
 calls were made from has been exchanged."""
 import copy
 import pickle
+import threading
 
 import pytest
 import torch
@@ -126,3 +127,31 @@ def test_copies(how):
             want = calls.forward(x * scale).clone()
             assert torch.equal(other.forward(x * scale), want)
         assert torch.equal(replay.forward(x * 0.9), calls.forward(x * 0.9))
+
+
+def test_graph_made_during_a_capture_in_another_thread():
+    """The third pass makes its graph while another thread captures in the mode that
+    forbids most calls to every thread: the capture stands, and so do the passes."""
+    calls, replay, x = _pair()
+    want = calls.forward(x).clone()
+    replay.forward(x)
+    got = []
+    stream = torch.cuda.Stream()
+
+    def passes():
+        with torch.cuda.stream(stream):
+            got.extend(replay.forward(x) for _ in range(4))
+
+    y = torch.zeros(1000, device="cuda")
+    thread = threading.Thread(target=passes)
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, capture_error_mode="global"):
+        y += 1
+        thread.start()
+        thread.join()
+        y += 1
+    graph.replay()
+    torch.cuda.synchronize()
+    assert float(y[0]) == 2 and len(got) == 4
+    assert torch.equal(got[-1], want)
