@@ -8,6 +8,7 @@
 
 #include <cstring>
 #include <mutex>
+#include <new>
 #include <type_traits>
 #include <vector>
 
@@ -129,7 +130,12 @@ inline int dsq_record_args(dsq_plan *plan, const DsqGrid &g, int n, void *const 
         std::memcpy(r.args + at, argv[i], size[i]);
         at += size[i];
     }
-    plan->recs.push_back(r);
+    try {
+        plan->recs.push_back(r);
+    } catch (const std::bad_alloc &) {        // (no entry point throws)
+        plan->status = DSQ_ERR_SIZE;
+        return DSQ_ERR_SIZE;
+    }
     return DSQ_OK;
 }
 

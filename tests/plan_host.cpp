@@ -3,6 +3,9 @@
 // would refuse, and fails on demand.  Built and driven by test_plan_host.py.
 #include "../paper_1908_05033_b200/csrc/dsq_plan.cu"
 
+#include <cstdlib>
+#include <new>
+
 namespace {
 struct Fake {
     int launches, graph_launches;          // kernels launched singly, graphs launched
@@ -11,6 +14,7 @@ struct Fake {
     int instantiate_calls, fail_instantiate, fail_stream;
     int capture_elsewhere, broken;         // another thread's capture, and whether it was broken
     int caller_capturing, mode_changes;
+    int no_memory;                         // on the host, for the records
 } f;
 cudaStreamCaptureMode g_mode = cudaStreamCaptureModeGlobal;
 cudaStream_t g_private = nullptr;          // the stream being captured
@@ -26,6 +30,16 @@ void kernel(int) { }
 }  // namespace
 
 unsigned dsq_hooks_generation() { return 0; }
+
+// (the records are over-aligned)
+void *operator new(size_t n, std::align_val_t a)
+{
+    void *p = f.no_memory ? nullptr : std::aligned_alloc((size_t)a, (n + (size_t)a - 1) / (size_t)a * (size_t)a);
+    if (!p) throw std::bad_alloc();
+    return p;
+}
+void operator delete(void *p, std::align_val_t) noexcept { std::free(p); }
+void operator delete(void *p, size_t, std::align_val_t) noexcept { std::free(p); }
 
 extern "C" {
 Fake *fake() { return &f; }

@@ -9,7 +9,7 @@ import pytest
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 FIELDS = ("launches graph_launches captured streams graphs execs instantiate_calls fail_instantiate "
-          "fail_stream capture_elsewhere broken caller_capturing mode_changes").split()
+          "fail_stream capture_elsewhere broken caller_capturing mode_changes no_memory").split()
 N = 5                                     # launches of the plan
 
 
@@ -91,3 +91,15 @@ def test_capture_in_another_thread_is_left_alone(lib):
     assert [run(lib, plan) for _ in range(4)] == [False, False, True, True]
     all_given_back(lib, plan)
     assert not f.broken
+
+
+def test_no_memory_for_a_record(lib):
+    """An entry point returns a status, and throws nothing, where its launch cannot be kept."""
+    f = lib.fake().contents
+    plan = C.c_void_p()
+    assert lib.dsq_plan_begin() == 0
+    f.no_memory = 1
+    assert lib.record_launch() == -5
+    f.no_memory = 0
+    assert lib.dsq_plan_end(C.byref(plan)) == -5 and not plan
+    all_given_back(lib, record(lib))
