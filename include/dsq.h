@@ -27,7 +27,8 @@
  *  - All data pointers are DEVICE pointers unless a parameter says "host".
  *    Descriptor structs (dsq_*_t) are read on the host during the call.
  *  - Every buffer is allocated and owned by the caller and must be 16-byte
- *    aligned.  The library allocates no device memory.
+ *    aligned.  The library allocates no device memory (and no other memory that
+ *    a user sees, but for dsq_workspace_status).
  *  - `stream` is a cudaStream_t passed as void* (NULL = the legacy default
  *    stream).  Work is enqueued asynchronously; no entry point synchronises
  *    except dsq_workspace_status.
@@ -133,6 +134,9 @@ size_t dsq_workspace_bytes(void);
 int dsq_workspace_init(void *workspace, size_t ws_bytes, void *stream);
 
 /* Synchronise `stream`, read the status word of the workspace and clear it.
+ * The calling thread keeps four bytes of page-locked host memory for this from
+ * its first call until it ends; where none can be had, or the workspace is not
+ * memory of the current device, the word is copied (slower, same result).
  * Returns DSQ_OK, DSQ_ERR_TIMEOUT (a kernel gave up on a wait; its outputs
  * are undefined) or DSQ_ERR_RANGE (dsq_pack_weights met a bad clip range). */
 int dsq_workspace_status(void *workspace, void *stream);

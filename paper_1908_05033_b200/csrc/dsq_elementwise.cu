@@ -400,25 +400,6 @@ maxpool_chunks_kernel(const uint4 *__restrict__ in, uint4 *__restrict__ out, int
     }
 }
 
-// Hands a workspace's status word to the host and clears it.  Written straight into
-// page-locked host memory: a copy to pageable memory is staged and took about 10 us
-// more of every call that reads the status.
-__global__ void status_kernel(int *ws, volatile int *host)
-{
-    const int st = *(volatile int *)(ws + DSQ_WS_STATUS);
-    if (st) ws[DSQ_WS_STATUS] = ws[DSQ_WS_DETAIL] = 0;
-    *host = st;
-}
-
-// one page-locked word per thread that asks, given back when the thread ends
-struct StatusMailbox {
-    int *word = nullptr;
-    ~StatusMailbox()
-    {
-        if (word) cudaFreeHost(word);
-    }
-};
-
 int grid_for(int64_t work_items, int block, int max_blocks = 148 * 16)
 {
     int64_t g = (work_items + block - 1) / block;
@@ -456,33 +437,6 @@ size_t dsq_weight_bytes(const dsq_conv_t *c, int bits)
     if (c->groups == c->Cin && c->Cin == c->Cout)
         return dsq_packed_bytes((int64_t)c->KH * c->KW, c->Cout, bits);
     return 0;
-}
-
-size_t dsq_workspace_bytes(void) { return DSQ_WS_BYTES; }
-
-int dsq_workspace_init(void *ws, size_t ws_bytes, void *stream)
-{
-    if (!ws) return DSQ_ERR_NULL;
-    if (!dsq_aligned16(ws)) return DSQ_ERR_ALIGN;
-    if (ws_bytes < DSQ_WS_BYTES) return DSQ_ERR_SIZE;
-    DSQ_CUDA_TRY(cudaMemsetAsync(ws, 0, DSQ_WS_BYTES, (cudaStream_t)stream));
-    return DSQ_OK;
-}
-
-int dsq_workspace_status(void *ws, void *stream)
-{
-    if (!ws) return DSQ_ERR_NULL;
-    static thread_local StatusMailbox box;
-    if (!box.word && cudaHostAlloc((void **)&box.word, sizeof(int), cudaHostAllocPortable) != cudaSuccess) {
-        cudaGetLastError();
-        box.word = nullptr;
-        return DSQ_ERR_CUDA;
-    }
-    *box.word = 0;
-    status_kernel<<<1, 1, 0, (cudaStream_t)stream>>>((int *)ws, box.word);
-    DSQ_CUDA_TRY(cudaGetLastError());
-    DSQ_CUDA_TRY(cudaStreamSynchronize((cudaStream_t)stream));
-    return *(volatile int *)box.word;
 }
 
 int dsq_quantize_act(const float *x, const dsq_nhwc_t *shape,

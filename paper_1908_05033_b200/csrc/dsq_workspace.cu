@@ -1,0 +1,87 @@
+// The workspace of the tensor-core kernels: its size, clearing it, reading its status.
+#include "dsq_launch.h"
+
+namespace {
+
+// Hands a workspace's status word to the host and clears it.  Written straight into
+// page-locked host memory: a copy to pageable memory is staged and took 3 us more of
+// every call that reads the status (binary GEMM 3136x512x4608: 41 -> 38 us).
+__global__ void status_kernel(int *ws, volatile int *host)
+{
+    const int st = *(volatile int *)(ws + DSQ_WS_STATUS);
+    if (st) ws[DSQ_WS_STATUS] = ws[DSQ_WS_DETAIL] = 0;
+    *host = st;
+}
+
+// One page-locked word per thread that asks, given back when the thread ends.
+struct StatusMailbox {
+    int *word = nullptr;
+    // (nullptr where there is none to be had)
+    int *get()
+    {
+        if (word) return word;
+        const DsqCaptureRelaxed relaxed;
+        void *p = nullptr;
+        if (cudaHostAlloc(&p, sizeof(int), cudaHostAllocPortable) == cudaSuccess) word = (int *)p;
+        else cudaGetLastError();
+        return word;
+    }
+    ~StatusMailbox()
+    {
+        if (!word) return;
+        const DsqCaptureRelaxed relaxed;
+        cudaFreeHost(word);
+    }
+};
+
+// Whether a kernel of the current device may read `p`: memory of another device may only
+// be copied from.
+bool on_current_device(const void *p)
+{
+    int dev = -1;
+    cudaPointerAttributes a;
+    if (cudaGetDevice(&dev) == cudaSuccess && cudaPointerGetAttributes(&a, p) == cudaSuccess)
+        return a.type == cudaMemoryTypeDevice && a.device == dev;
+    cudaGetLastError();
+    return false;
+}
+
+}  // namespace
+
+extern "C" {
+
+size_t dsq_workspace_bytes(void) { return DSQ_WS_BYTES; }
+
+int dsq_workspace_init(void *ws, size_t ws_bytes, void *stream)
+{
+    if (!ws) return DSQ_ERR_NULL;
+    if (!dsq_aligned16(ws)) return DSQ_ERR_ALIGN;
+    if (ws_bytes < DSQ_WS_BYTES) return DSQ_ERR_SIZE;
+    DSQ_CUDA_TRY(cudaMemsetAsync(ws, 0, DSQ_WS_BYTES, (cudaStream_t)stream));
+    return DSQ_OK;
+}
+
+int dsq_workspace_status(void *ws, void *stream)
+{
+    if (!ws) return DSQ_ERR_NULL;
+    cudaStream_t s = (cudaStream_t)stream;
+    static thread_local StatusMailbox box;
+    int *const word = box.get();
+    if (word && on_current_device(ws)) {
+        *word = 0;
+        int *w = (int *)ws;
+        void *argv[] = {(void *)&w, (void *)&word};
+        const DsqGrid one = {(const void *)status_kernel, dim3(1), dim3(1), 0, 0, 0};
+        const int st = dsq_launch_args(one, argv, s);
+        if (st) return st;
+        DSQ_CUDA_TRY(cudaStreamSynchronize(s));
+        return *(volatile int *)word;
+    }
+    int host[2] = {0, 0};
+    DSQ_CUDA_TRY(cudaMemcpyAsync(host, ws, sizeof(host), cudaMemcpyDeviceToHost, s));
+    DSQ_CUDA_TRY(cudaStreamSynchronize(s));
+    if (host[DSQ_WS_STATUS]) DSQ_CUDA_TRY(cudaMemsetAsync(ws, 0, sizeof(host), s));
+    return host[DSQ_WS_STATUS];
+}
+
+}  // extern "C"
