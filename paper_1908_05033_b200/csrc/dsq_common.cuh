@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <math.h>
+
 #include <atomic>
 
 #include "../../include/dsq.h"
@@ -78,6 +80,16 @@ static inline DsqQ dsq_make_q(const dsq_quant_t &q)
     r.qmax = (1 << q.bits) - 1;
     r.inv = (float)r.qmax / (q.hi - q.lo);
     return r;
+}
+
+// What the lean roundings (nothing clipped at hi first, the code saturated instead) ask
+// of a range: floor(fma(hi - lo, inv, 0.5)) = qmax.  True of every range but those whose
+// width or inv leaves binary32 (hi - lo below 4.4e-38, say, where inv is infinite and
+// 0 * inv a NaN).
+static inline bool dsq_lean_range(const DsqQ &q)
+{
+    const float r = fmaf(q.hi - q.lo, q.inv, 0.5f);
+    return r >= (float)q.qmax && r < (float)(q.qmax + 1);
 }
 
 #ifdef __CUDACC__

@@ -438,13 +438,13 @@ extern "C" int dsq_dwconv2d(const void *act_codes, const dsq_nhwc_t *shape,
     const int Wo = (shape->W + 2 - 3) / conv->stride + 1;
     const int pitch = (int)dsq_row_pitch(shape->C, bits);
     cudaStream_t s = (cudaStream_t)stream;
-    // codes to codes, requantiser range starting at 0 (the lean epilogue does not
-    // subtract lo); images of at least 2^31 bytes a row keep the general kernel's
+    // codes to codes, a requantiser range the lean epilogue takes that starts at 0 (it does
+    // not subtract lo); images of at least 2^31 bytes a row keep the general kernel's
     // 64-bit indexing
     const int units = bits == 4 ? pitch / 4 : (shape->C + 7) / 8;
     const int strips = (Wo + 3) / 4;
     if (y_codes && !y_f32 && !acc_out && !e.residual && !e.general_offset && e.rq.lo == 0.0f &&
-        (int64_t)units * strips * Ho * shape->N < (1ll << 31)) {
+        dsq_lean_range(e.rq) && (int64_t)units * strips * Ho * shape->N < (1ll << 31)) {
         DwHalf p;
         p.N = shape->N; p.H = shape->H; p.W = shape->W; p.C = shape->C;
         p.Ho = Ho; p.Wo = Wo; p.pitch = pitch;

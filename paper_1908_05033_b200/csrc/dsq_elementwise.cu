@@ -466,9 +466,7 @@ int dsq_quantize_act(const float *x, const dsq_nhwc_t *shape,
                           (uint4 *)codes_out, n_lines, dq);
     }
     const int pw = (int)(pitch / 4);
-    // (the lean rounding wants floor(fma(hi - lo, inv, 0.5)) = qmax: every sane range)
-    if (bits < 4 && k % 32 == 0 && ((uintptr_t)x & 31u) == 0 &&
-        (int)floorf(fmaf(dq.hi - dq.lo, dq.inv, 0.5f)) == dq.qmax) {
+    if (bits < 4 && k % 32 == 0 && ((uintptr_t)x & 31u) == 0 && dsq_lean_range(dq)) {
         const int64_t groups = rows * (k / 32);
         return dsq_launch(bits == 3 ? quantize_groups_kernel<3> : quantize_groups_kernel<2>,
                           dim3(grid_for((groups + 3) / 4 * 4, 256, 148 * 32)), dim3(256), 0, s,
