@@ -103,7 +103,10 @@ typedef struct dsq_conv_t {
  *                    code at the same output position (packed NHWC, same
  *                    shape as the output), (l_r, Delta_r) from residual_q
  *   requant.bits>0 : codes = quantise(y; requant)  (ReLU is the clip at lo=0)
- * A non-finite w_offset returns DSQ_ERR_RANGE. */
+ * A non-finite w_offset returns DSQ_ERR_RANGE.  Scales and biases may be any
+ * numbers; a call that writes codes only may move a power of two between
+ * accumulator and scale, so that its last bit is the sequence's for scale = 0
+ * and 2^-118 <= |scale| < 2^100 (and for every scale where hi - lo < 2^-80). */
 typedef struct dsq_epilogue_t {
     const float *scale;          /* [Cout], required */
     const float *bias;           /* [Cout], required */

@@ -1279,13 +1279,11 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     // need the weight rows twice in the A operand (`dup`), from the blob's expanded copy
     // or, at 3 bits, by the expansion warps: 64->64 at 56x56 runs in 18 us against 22.5 us
     // on plain tiles.  Otherwise plain tiles.
-    // the codes epilogues want the requantiser range to start at 0 and
-    // floor(r_hi) = qmax
+    // the codes epilogues want the requantiser range to start at 0, too
     float r_hi = 0.f;
     if (epi_kind != DSQ_EPI_GENERAL) {
         r_hi = fmaf(e.rq.hi - e.rq.lo, e.rq.inv, 0.5f);
-        if (e.rq.lo != 0.0f || (int)floorf(r_hi) != e.rq.qmax)
-            epi_kind = DSQ_EPI_GENERAL;
+        if (e.rq.lo != 0.0f || !dsq_lean_epilogue(e)) epi_kind = DSQ_EPI_GENERAL;
     }
     W3Params p = {};
     p.N = shape->N; p.H = shape->H; p.W = shape->W;

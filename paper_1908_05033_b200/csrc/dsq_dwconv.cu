@@ -444,7 +444,7 @@ extern "C" int dsq_dwconv2d(const void *act_codes, const dsq_nhwc_t *shape,
     const int units = bits == 4 ? pitch / 4 : (shape->C + 7) / 8;
     const int strips = (Wo + 3) / 4;
     if (y_codes && !y_f32 && !acc_out && !e.residual && !e.general_offset && e.rq.lo == 0.0f &&
-        dsq_lean_range(e.rq) && (int64_t)units * strips * Ho * shape->N < (1ll << 31)) {
+        dsq_lean_epilogue(e) && (int64_t)units * strips * Ho * shape->N < (1ll << 31)) {
         DwHalf p;
         p.N = shape->N; p.H = shape->H; p.W = shape->W; p.C = shape->C;
         p.Ho = Ho; p.Wo = Wo; p.pitch = pitch;

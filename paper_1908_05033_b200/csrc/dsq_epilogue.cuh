@@ -66,6 +66,16 @@ static inline int dsq_make_epi(const dsq_epilogue_t *ep, int bits, float *y_f32,
     return DSQ_OK;
 }
 
+// Whether the lean codes epilogues (below) take a layer's requantiser and residual
+// operand: no NaN may arise in them, and they move powers of two between the accumulator
+// and the scale, which rounds scales below 2^-118.  The host cannot see scales, but results
+// that small fill no range wider than 2^-80.
+static inline bool dsq_lean_epilogue(const DsqEpi &e)
+{
+    return dsq_lean_range(e.rq) && e.rq.hi - e.rq.lo >= 0x1p-80f &&
+           (!e.residual || dsq_finite(e.res_delta));
+}
+
 #ifdef __CUDACC__
 // v is acc (half_offset = 0) or 2*acc + S_a (half_offset = 1, with `scale`
 // already multiplied by 0.5f by the caller of this function).

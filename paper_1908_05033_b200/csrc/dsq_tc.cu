@@ -1836,10 +1836,8 @@ int dsq_conv2d(const void *act_codes, const dsq_nhwc_t *shape, const dsq_quant_t
     const int epi = (y_f32 || acc_out || !y_codes || e.general_offset)
                         ? EPI_GENERAL
                         : (e.residual ? EPI_CODES_RES : EPI_CODES);
-    // the lean codes epilogues do not clip before they round: they need
-    // floor(fma(hi - lo, inv, 0.5)) = qmax (true for every sane range)
     const float r_hi = fmaf(e.rq.hi - e.rq.lo, e.rq.inv, 0.5f);
-    const int epi_im2col = epi != EPI_GENERAL && (int)floorf(r_hi) != e.rq.qmax ? EPI_GENERAL : epi;
+    const int epi_im2col = epi != EPI_GENERAL && !dsq_lean_epilogue(e) ? EPI_GENERAL : epi;
     // little work: a latency-bound kernel of its own (the hooks force the others)
     const bool hooked = g_forced_bn.load() || g_forced_ks.load() || g_pair_mode.load() == 2 ||
                         g_window3.load() != 1 || g_skip_b_round.load() >= 0;
