@@ -380,17 +380,17 @@ __device__ __forceinline__ uint32_t max_fields(uint32_t a, uint32_t b)
 // 64-bit index divisions).
 template <int BITS>
 __global__ void __launch_bounds__(256)
-maxpool_chunks_kernel(const uint4 *__restrict__ in, uint4 *__restrict__ out, int total, int H, int W,
+maxpool_chunks_kernel(const uint4 *__restrict__ in, uint4 *__restrict__ out, int total, int W,
                       int chunks)
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int Wo = W / 2, Ho = H / 2;
+    const int Wo = W / 2;
     for (int i = blockIdx.x * 256 + threadIdx.x; i < total; i += gridDim.x * 256) {
         const int pix = i / chunks, c = i - pix * chunks;
-        const int row = pix / Wo, wo = pix - row * Wo;     // row: of all images
-        const int n = row / Ho, ho = row - n * Ho;
-        const uint4 *p = in + ((int64_t)(n * H + 2 * ho) * W + 2 * wo) * chunks + c;
+        // output row `row` of all images lies over input rows 2 row and 2 row + 1 (H is even)
+        const int row = pix / Wo, wo = pix - row * Wo;
+        const uint4 *p = in + (2 * (int64_t)row * W + 2 * wo) * chunks + c;
         const uint4 v00 = __ldg(p), v01 = __ldg(p + chunks), v10 = __ldg(p + (int64_t)W * chunks),
                     v11 = __ldg(p + (int64_t)W * chunks + chunks);
         out[i] = make_uint4(max_fields<BITS>(max_fields<BITS>(v00.x, v01.x), max_fields<BITS>(v10.x, v11.x)),
@@ -550,7 +550,7 @@ int dsq_maxpool2x2(const void *codes_in, const dsq_nhwc_t *shape, int bits,
         return dsq_launch(bits == 4 ? maxpool_chunks_kernel<4> : maxpool_chunks_kernel<2>,
                           dim3(grid_for(items, 256, 148 * 32)), dim3(256), 0, (cudaStream_t)stream,
                           dsq_launch_hooks().pdl, 0, (const uint4 *)codes_in, (uint4 *)codes_out,
-                          (int)items, shape->H, shape->W, (int)(pitch / 16));
+                          (int)items, shape->W, (int)(pitch / 16));
     return dsq_launch(maxpool_kernel, dim3(grid_for(out_rows * pw, 256)), dim3(256), 0,
                       (cudaStream_t)stream, dsq_launch_hooks().pdl, 0, (const uint32_t *)codes_in, (uint32_t *)codes_out,
                       shape->N, shape->H, shape->W, shape->C, pw, bits);

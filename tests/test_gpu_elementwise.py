@@ -113,3 +113,24 @@ def test_maxpool(dsq, bits, shape):
     packed = T(native.pack_rows(q.reshape(-1, shape[3]), bits))
     got = N(dsq.dsq_maxpool2x2(packed, shape, bits)).reshape(ref.shape)
     assert np.array_equal(ref, got)
+
+
+def test_maxpool_many_rows(dsq):
+    """More input rows than 2^31 (69 GB of two-pixel rows): the last images are pooled as
+    they are by themselves."""
+    bits, shape = 4, (1 << 20, 2050, 2, 32)
+    n, h, w, c = shape
+    pitch = dsq.dsq_row_pitch(c, bits)
+    if torch.cuda.mem_get_info()[0] < 1.3 * n * h * w * pitch:
+        pytest.skip("needs 90 GB of device memory")
+    codes = torch.zeros(n, h, w, pitch, dtype=torch.uint8, device="cuda")
+    try:
+        last = torch.randint(0, 256, (3, h, w, pitch), dtype=torch.uint8, device="cuda")
+        codes[-3:] = last
+        out = dsq.dsq_maxpool2x2(codes, shape, bits)
+        assert torch.equal(out[-3:], dsq.dsq_maxpool2x2(last, (3, h, w, c), bits))
+        assert not out[:1000].any()
+    finally:
+        del codes
+        out = None
+        torch.cuda.empty_cache()
