@@ -634,6 +634,16 @@ int resident_clusters()
     return n;
 }
 
+// K split over the two pairs of a cluster where all the tiles' clusters are resident at
+// once (33 of them on 148 SMs) and a part still has twelve K blocks: the exchange costs
+// about as much as eight.  (Four pairs a cluster gained nothing more: 15 such clusters are
+// resident and the exchange doubles.)
+template <bool F16>
+bool takes_split(int64_t tiles, int64_t kblocks)
+{
+    return kblocks >= 24 && tiles <= resident_clusters<F16, 2>();
+}
+
 // Pass 2 over operands that are rows of k_bytes bytes of K (byte maps: the
 // kernel never looks at an element, only the tensor core does).
 template <bool F16>
@@ -656,11 +666,7 @@ int launch_pass2(const void *A, size_t a_pitch, const void *B, size_t b_pitch, s
             (!p.Y_f32 || (reinterpret_cast<uintptr_t>(p.Y_f32) & 31u) == 0);
     const int sms = dsq_sm_count() > 0 ? dsq_sm_count() : 148;
     const int tiles = p.m_tiles * p.n_tiles;
-    // K split over the two pairs of a cluster where all the tiles' clusters are resident
-    // at once (33 of them) and a part still has twelve K blocks: the exchange costs
-    // about as much as eight.  (Four pairs a cluster gained nothing more: 15 such
-    // clusters are resident and the exchange doubles.)
-    if (p.kblocks >= 24 && tiles <= sms / 4 && tiles <= resident_clusters<F16, 2>())
+    if (takes_split<F16>(tiles, p.kblocks))
         return launch_split<F16, 2>(ta, tb, p, tiles, stream);
     return launch_split<F16, 1>(ta, tb, p, std::min(sms / 2, tiles), stream);
 }
@@ -765,9 +771,9 @@ static bool wgemm_prefers_small(int64_t M, int64_t N, int64_t K)
     const int sms = dsq_sm_count() > 0 ? dsq_sm_count() : 148;
     const double blocks = (double)((N + 15) / 16) * (double)((M + 63) / 64);
     const double small = 2.2 + std::ceil(blocks / sms) * (double)((K + 1023) / 1024) * 2.6;
-    const double tiles = (double)((M + G8_BM - 1) / G8_BM) * (double)((N + G8_BN - 1) / G8_BN);
-    const double kb = (double)((K + 63) / 64);
-    const double main_loop = (tiles <= 33 && kb >= 24 ? 0.5 : std::ceil(tiles / (sms / 2))) * kb * 0.27;
+    const int64_t tiles = (M + G8_BM - 1) / G8_BM * ((N + G8_BN - 1) / G8_BN), kb = (K + 63) / 64;
+    const double waves = takes_split<true>(tiles, kb) ? 0.5 : std::ceil((double)tiles / (sms / 2));
+    const double main_loop = waves * kb * 0.27;
     return small < 9.0 + 5.2e-7 * (double)N * (double)K + main_loop;
 }
 
