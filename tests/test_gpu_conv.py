@@ -205,7 +205,8 @@ def dw_case(dsq, N_, H, W, Cc, s, bits, w_off, residual=False, seed=6):
     assert np.array_equal(N(accg), want_acc)
     assert_f32_close(N(yg), y)
     assert np.array_equal(N(codes).reshape(ref_codes.shape), ref_codes)
-    # codes-only call (the form the stacks use; 4-bit takes the dp4a kernel)
+    # codes-only call (the form the stacks use; without residual and offset the
+    # packed-half kernel)
     codes2, _, _ = dsq.dsq_dwconv2d(
         act, (N_, H, W, Cc), (bits, 0.0, 6.0), blob, conv, T(scale), T(bias),
         w_offset=w_off, residual=res_t, residual_q=res_q, requant=(bits, 0.0, 6.0))
@@ -245,10 +246,9 @@ def test_conv3x3_window_kernel(dsq, geom, bits, form, w8):
     channels, weights as the A operand) where the geometry allows, form 4 =
     plain tiles only (128 positions x up to 256 channels).  w8 = 1: weight
     tiles of the wide layers come by TMA from the blob's pre-expanded int8 copy
-    (grid Delta (c + 1/2) only); w8 = 0: the kernel expands the packed rows."""
+    (grid Delta (c + 1/2) only); w8 = 0: the kernel expands the packed rows, as it
+    always does at 3 bits, whose blob has no such copy."""
     n, h, w, ci, co = geom
-    if bits == 3 and (form == 4 or w8 == 0):
-        pytest.skip("3-bit codes take the plain form and packed weights in every setting")
     dsq.dsq_set_conv3_window(form)     # this kernel wherever the geometry allows
     dsq.dsq_set_conv3_expanded_weights(w8)
     try:
