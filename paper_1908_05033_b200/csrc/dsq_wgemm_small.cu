@@ -239,8 +239,12 @@ int launch(const WsParams &p, cudaStream_t s)
 template <int BITS>
 int pick(const WsParams &p, cudaStream_t s)
 {
-    // columns per block: 32 where that still gives every SM a block, else 16
-    const bool wide = p.N >= 32 * dsq_sm_count() * 3 / 4;
+    // Columns per block: 16 while those blocks are one to an SM at most (one fits: its
+    // registers), 32 beyond, where a second wave costs more than the wider block.  4-bit,
+    // K = 4096, us with 16 / 32 columns: N = 2048 (128 blocks of 16) 1 row 3.6 / 5.2, 16 rows
+    // 4.6 / 5.7, 32 rows 7.2 / 8.3; N = 2400 (150) 5.3 / 5.2, 7.0 / 5.9, 12.7 / 8.5; N = 4096
+    // 5.5 / 5.2, 7.2 / 5.9, 13.2 / 8.5.
+    const bool wide = p.N > 16 * (dsq_sm_count() > 0 ? dsq_sm_count() : 148);
     if (p.M <= 16) return wide ? launch<BITS, 1, 4>(p, s) : launch<BITS, 1, 2>(p, s);
     if (p.M <= 32) return wide ? launch<BITS, 2, 4>(p, s) : launch<BITS, 2, 2>(p, s);
     return launch<BITS, 4, 2>(p, s);

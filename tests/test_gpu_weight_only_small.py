@@ -18,7 +18,7 @@ def dsq():
 @pytest.mark.parametrize("bits", [1, 2, 3, 4])
 @pytest.mark.parametrize("size", [(1, 33, 8), (15, 17, 120), (16, 40, 136), (17, 31, 1032),
                                   (33, 70, 264), (64, 65, 2056), (65, 33, 128), (3, 3600, 392),
-                                  (31, 4100, 160)])
+                                  (31, 4100, 160), (5, 2368, 136), (20, 2369, 136)])
 def test_few_rows(dsq, size, bits):
     M, Nn, K = size
     x, q, u, bias = dsq_inputs.weight_only_case(M, Nn, K, bits)
