@@ -5,7 +5,7 @@
 // well under a microsecond of arithmetic.  The tcgen05 kernels took 4 to 14 us for
 // it: 1.5 us before their roles start (23 to 31 warps, tensor memory, barriers), a
 // chain of hand-offs, and one to four CTAs that walk the whole of K alone.  Here
-//   * a block of 4 to 16 warps makes 16 MT pixels x 32 channels, its warps splitting
+//   * a block of 4 to 16 warps makes 16 MT pixels x 8 NT channels, its warps splitting
 //     K (so a layer is a few hundred blocks whose warps load a chunk or two each) and
 //     adding their sums in shared memory;
 //   * every lane takes its packed words straight from global memory to the fragments
@@ -31,14 +31,13 @@
 namespace {
 
 constexpr int CS_MAX_WARPS = 16;
-constexpr int NT = 4;                 // column tiles of eight channels a block: a word of codes a lane
 
 struct CsParams {
     const uint8_t *act, *w;
     int H, W, Ho, Wo, stride, pad, ksize;
     int M, Ncols, P, w_row;           // pixels, channels, bytes of a pixel row, of a weight row
     int upt, chunks;                  // units per tap; chunks of four units
-    int d_tap, d_s;                   // a warp's step of 4 * warps units as taps, units
+    int units, d_tap, d_s;            // all units; a warp's step of 4 * warps units as taps, units
     int shift, out_pitch, lean;
     int early;                        // dsq_early_constants
     uint32_t orv;
@@ -89,7 +88,7 @@ __device__ __forceinline__ uint32_t byte_word(const uint32_t (&v)[Unit<BITS>::WO
     return b;
 }
 
-template <int BITS, int MT>
+template <int BITS, int MT, int NT>
 __global__ void __launch_bounds__((MT == 1 ? CS_MAX_WARPS : 8) * 32)
 conv_small_kernel(const CsParams p)
 {
@@ -290,15 +289,15 @@ conv_small_kernel(const CsParams p)
     }
 }
 
-template <int BITS, int MT>
+template <int BITS, int MT, int NT>
 int launch(const CsParams &p, int warps, cudaStream_t s)
 {
     const size_t smem = (size_t)warps * MT * NT * 32 * 16;
     static std::atomic<unsigned long long> configured{0ull};
-    const int st = dsq_allow_smem((const void *)conv_small_kernel<BITS, MT>, CS_MAX_WARPS * MT * NT * 512,
+    const int st = dsq_allow_smem((const void *)conv_small_kernel<BITS, MT, NT>, CS_MAX_WARPS * MT * NT * 512,
                                   &configured);
     if (st) return st;
-    return dsq_launch(conv_small_kernel<BITS, MT>,
+    return dsq_launch(conv_small_kernel<BITS, MT, NT>,
                       dim3((p.Ncols + 8 * NT - 1) / (8 * NT), (p.M + 16 * MT - 1) / (16 * MT)),
                       dim3(32 * warps), smem, s, dsq_launch_hooks().pdl, 0, p);
 }
@@ -308,7 +307,7 @@ int pick(CsParams &p, int mt, int warps, cudaStream_t s)
 {
     p.d_tap = 4 * warps / p.upt;
     p.d_s = 4 * warps - p.d_tap * p.upt;
-    return mt == 2 ? launch<BITS, 2>(p, warps, s) : launch<BITS, 1>(p, warps, s);
+    return mt == 2 ? launch<BITS, 2, 4>(p, warps, s) : launch<BITS, 1, 4>(p, warps, s);
 }
 
 // Microseconds this kernel takes with a tile and block size, fitted to the layers of the
@@ -366,7 +365,8 @@ int dsq_conv_small(const void *act_codes, const dsq_nhwc_t *shape, int bits, con
     const int taps = conv->KH * conv->KW;
     p.w_row = taps * p.P;
     p.upt = bits == 3 ? (conv->Cin + 31) / 32 : p.P / 16;
-    p.chunks = (taps * p.upt + 3) / 4;
+    p.units = taps * p.upt;
+    p.chunks = (p.units + 3) / 4;
     p.out_pitch = (int)dsq_row_pitch(conv->Cout, bits);
     p.lean = lean;
     p.early = dsq_early_constants();
