@@ -88,6 +88,8 @@ __device__ __forceinline__ uint32_t byte_word(const uint32_t (&v)[Unit<BITS>::WO
     return b;
 }
 
+// (NT is 4 wherever it is launched; as a constant of the file the same source compiles to
+// a kernel that is slower for the ResNet-18-shaped network at batch 1, 67.0 -> 69.0 us)
 template <int BITS, int MT, int NT>
 __global__ void __launch_bounds__((MT == 1 ? CS_MAX_WARPS : 8) * 32)
 conv_small_kernel(const CsParams p)
@@ -327,16 +329,24 @@ double estimate(const CsParams &p, int bits, int mt, int warps)
     return chain > shared ? chain : shared;
 }
 
-// and what the other kernel for the layer takes, likewise: a floor that grows with K
-// (the few CTAs such a layer has walk it alone) plus its work at full rate
+// And what the other kernel for the layer takes, likewise: a floor that grows with K
+// (the few CTAs such a layer has walk it alone) plus its work at full rate.
+// Of 335 measured layers (64 to 1024 channels, 1x1 and 3x3, 2 to 4 bits, batches of 1 to 16)
+// the rule takes the slower kernel for 34, 2 % of time on average: most are 1x1 layers,
+// whose kernel takes 0.5 to 1 us more than said here, and 3-bit ones, where the im2col kernel
+// takes twice as long (64 -> 128 at 56x56, stride 2, batch 6: 14.1 us against 6.5).
 double estimate_other(const CsParams &p, int bits, int Cin, double macs, int lean)
 {
     const int sms = dsq_sm_count() > 0 ? dsq_sm_count() : 148;
     const double ksteps = p.ksize * p.ksize * Cin / 128.0;
     if (p.ksize == 1 && lean) return 2.9 + (double)p.M * p.Ncols / 3.7e6;
     if (p.ksize == 3 && p.stride == 1 && p.pad == 1 && (Cin == 64 || Cin % 128 == 0)) {
-        // window kernel: waves of tiles of 256 positions x 128 channels (3-bit: the expansion
-        // warps set the pace)
+        // Window kernel: waves of tiles of 256 positions x 128 channels (3-bit: the expansion
+        // warps set the pace).  One wave, 4-bit, measured / said here: 64 channels 5.4 / 6.1, 128
+        // 7.6 / 10.1, 256 10.2 / 12.6, 384 12.6 / 12.8, 512 15.2 / 15.2, 1024 25.2 / 24.9 us.  What is too
+        // much at 128 and 256 channels offsets what this kernel's own estimate lacks around
+        // the line there (256 at 14x14, batch 12: 8.7 us, window 10.4, own estimate 9.9): with
+        // 5.5 throughout, 35 of the layers below are on the wrong side instead of 34.
         const double tiles = std::ceil((double)p.M / p.H / p.W * (p.H + 1) * (p.W + 1) / 256) *
                              ((p.Ncols + 127) / 128);
         return (Cin == 64 ? 4.3 : Cin <= 256 ? 7.7 : 5.5) +

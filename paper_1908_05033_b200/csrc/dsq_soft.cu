@@ -216,8 +216,12 @@ int make_soft_params(const dsq_quant_t *q, float alpha, SoftP *out)
     return DSQ_OK;
 }
 
-// blocks per SM: forward two sets of all that fit; backward one set of four, since each ends
-// in three atomic additions to the same three words (12.8M elements: 3 a SM 31.1 us, 4 28.9, 6 32.8)
+// Blocks per SM: whole sets of all that are resident together (forward 8, backward 4: 32 and
+// 57 registers a thread), since every block walks the array at the same step and the last set
+// should not be a partial one.  Backward, us after an L2 flush with 3 / 4 / 5 / 6 / 8 / 16 blocks:
+// 12.8M elements 36.9 / 32.8 / 41.0 / 37.0 / 34.8 / 36.0, 33.5M 77.8 / 71.7 / 88.0 / 81.9 / 72.7 / 73.8, 67M
+// 141 / 133 / 160 / 146 / 133 / 133; below 4M the counts do not differ.  Forward with 4 / 8 / 16 / 32:
+// 12.8M 26.6 / 24.6 / 22.6 / 24.6, 67M 102 / 100 / 96 / 88.
 int soft_grid(int64_t n, int per_sm)
 {
     const int sms = dsq_sm_count() > 0 ? dsq_sm_count() : 148;
