@@ -183,7 +183,8 @@ int dsq_quantize_act(const float *x, const dsq_nhwc_t *shape,
 /* ---- Algorithm 1 step 5 on codes + epilogue ---------------------------- */
 
 /* Dense convolution as an implicit GEMM on the 5th-generation tensor cores
- * (tcgen05.mma kind::i8, int32 accumulation in tensor memory):
+ * (tcgen05.mma kind::i8, int32 accumulation in tensor memory; layers with little
+ * work, one or a few images, with mma.sync from registers):
  * M = N*Ho*Wo output pixels, N = Cout, K = KH*KW*Cin.
  *   act_codes  packed NHWC unsigned codes of `shape`, quantiser act_q.
  *              act_q->lo must be 0 when conv->pad > 0 (padding is code 0).
@@ -277,7 +278,8 @@ int dsq_binary_gemm(const void *A_bits, const void *B_bits, int64_t M, int64_t N
  * fp32 by the tensor core in an order of its own, so Y is within
  * K * 2^-23 * sum_k |X v| * |col_scale| of the exact value.  The weights are
  * expanded to bf16 once into the workspace (dsq_wgemm_workspace_bytes(N, K)),
- * then a TMA-fed bf16 tensor-core GEMM runs. */
+ * then a TMA-fed bf16 tensor-core GEMM runs; few rows (up to 64, or more where
+ * it is faster) are multiplied straight from the packed codes. */
 size_t dsq_wgemm_workspace_bytes(int64_t N, int64_t K);
 int dsq_wgemm_bf16(const void *X_bf16, const void *W_codes, int64_t M, int64_t N,
                    int64_t K, int bits, float w_offset, const float *col_scale,

@@ -1,6 +1,7 @@
 """Single-kernel cases for timing and profiling.
 
     python -m paper_1908_05033_b200.cases gemm --size 4096 --bits 4 --iters 5
+    python -m paper_1908_05033_b200.cases wgemm --m 16 --size 4096 --bits 4
     python -m paper_1908_05033_b200.cases conv --cin 64 --cout 64 --hw 56 --batch 64 --ksize 3
     python -m paper_1908_05033_b200.cases quant --mb 1024 --bits 4
     python -m paper_1908_05033_b200.cases dw --c 192 --hw 56 --batch 64
@@ -41,6 +42,9 @@ def main(argv=None):
     ap = argparse.ArgumentParser()
     ap.add_argument("case", choices=["gemm", "bgemm", "wgemm", "conv", "quant", "dw", "soft"])
     ap.add_argument("--size", type=int, default=4096)
+    ap.add_argument("--m", type=int, default=0, help="rows of a GEMM's result (0: --size)")
+    ap.add_argument("--n", type=int, default=0, help="its columns")
+    ap.add_argument("--k", type=int, default=0, help="its inner extent")
     ap.add_argument("--bits", type=int, default=4)
     ap.add_argument("--iters", type=int, default=5)
     ap.add_argument("--cin", type=int, default=64)
@@ -73,41 +77,39 @@ def main(argv=None):
     B.dsq_set_cta_pairs(a.pairs)
     B.dsq_set_conv3_window(a.window)
     out = {"case": a.case, "bits": bits, "tile_n": a.tile_n}
+    m, n, k = a.m or a.size, a.n or a.size, a.k or a.size
+
+    def packed(rows, bits):
+        return torch.randint(0, 256, (rows, B.dsq_row_pitch(k, bits)), dtype=torch.uint8, device=dev,
+                             generator=gen)
+
     if a.case == "gemm":
-        n = a.size
-        pitch = B.dsq_row_pitch(n, bits)
-        A = torch.randint(0, 256, (n, pitch), dtype=torch.uint8, device=dev, generator=gen)
-        Bm = torch.randint(0, 256, (n, pitch), dtype=torch.uint8, device=dev, generator=gen)
-        Cm = torch.empty((n, n), dtype=torch.int32, device=dev)
+        A, Bm = packed(m, bits), packed(n, bits)
+        Cm = torch.empty((m, n), dtype=torch.int32, device=dev)
         if not a.fused:
-            ws = B.new_gemm_workspace(n, n, n, bits, dev)
-        ms, all_ms = _timeit(lambda: B.dsq_gemm(A, Bm, n, n, n, bits, ws, out_i32=Cm),
+            ws = B.new_gemm_workspace(m, n, k, bits, dev)
+        ms, all_ms = _timeit(lambda: B.dsq_gemm(A, Bm, m, n, k, bits, ws, out_i32=Cm),
                              a.iters, flush)
-        out.update(size=n, ms=ms, tops=2.0 * n ** 3 / (ms * 1e-3) / 1e12, all_ms=all_ms)
+        out.update(size=[m, n, k], ms=ms, tops=2.0 * m * n * k / (ms * 1e-3) / 1e12, all_ms=all_ms)
     elif a.case == "bgemm":
         # binary GEMM: 1-bit rows, values -1 / +1
-        n = a.size
-        pitch = B.dsq_row_pitch(n, 1)
-        A = torch.randint(0, 256, (n, pitch), dtype=torch.uint8, device=dev, generator=gen)
-        Bm = torch.randint(0, 256, (n, pitch), dtype=torch.uint8, device=dev, generator=gen)
-        Cm = torch.empty((n, n), dtype=torch.int32, device=dev)
-        ws = torch.zeros(B.lib.dsq_binary_gemm_workspace_bytes(n, n, n), dtype=torch.uint8, device=dev)
+        A, Bm = packed(m, 1), packed(n, 1)
+        Cm = torch.empty((m, n), dtype=torch.int32, device=dev)
+        ws = torch.zeros(B.lib.dsq_binary_gemm_workspace_bytes(m, n, k), dtype=torch.uint8, device=dev)
         ms, all_ms = _timeit(lambda: B._check(B.lib.dsq_binary_gemm(
-            A.data_ptr(), Bm.data_ptr(), n, n, n, Cm.data_ptr(), None, None, ws.data_ptr(),
+            A.data_ptr(), Bm.data_ptr(), m, n, k, Cm.data_ptr(), None, None, ws.data_ptr(),
             ws.numel(), torch.cuda.current_stream().cuda_stream), "dsq_binary_gemm"), a.iters, flush)
-        out.update(size=n, ms=ms, tops=2.0 * n ** 3 / (ms * 1e-3) / 1e12, all_ms=all_ms)
+        out.update(size=[m, n, k], ms=ms, tops=2.0 * m * n * k / (ms * 1e-3) / 1e12, all_ms=all_ms)
     elif a.case == "wgemm":
-        # weight-only: bf16 activations [size, size] x b-bit weights [size, size]
-        n = a.size
-        X = torch.randn((n, n), device=dev, generator=gen).to(torch.bfloat16)
-        W = torch.randint(0, 256, (n, B.dsq_row_pitch(n, bits)), dtype=torch.uint8, device=dev,
-                          generator=gen)
+        # weight-only: bf16 activations [m, k] x b-bit weights [n, k]
+        X = torch.randn((m, k), device=dev, generator=gen).to(torch.bfloat16)
+        W = packed(n, bits)
         sc = torch.full((n,), 0.01, device=dev)
-        Y = torch.empty((n, n), dtype=torch.float32, device=dev)
-        ws = torch.zeros(B.lib.dsq_wgemm_workspace_bytes(n, n), dtype=torch.uint8, device=dev)
-        ms, all_ms = _timeit(lambda: B.dsq_wgemm_bf16(X, W, n, n, n, bits, sc, ws=ws, out=Y),
+        Y = torch.empty((m, n), dtype=torch.float32, device=dev)
+        ws = torch.zeros(B.lib.dsq_wgemm_workspace_bytes(n, k), dtype=torch.uint8, device=dev)
+        ms, all_ms = _timeit(lambda: B.dsq_wgemm_bf16(X, W, m, n, k, bits, sc, ws=ws, out=Y),
                              a.iters, flush)
-        out.update(size=n, ms=ms, tflops=2.0 * n ** 3 / (ms * 1e-3) / 1e12, all_ms=all_ms)
+        out.update(size=[m, n, k], ms=ms, tflops=2.0 * m * n * k / (ms * 1e-3) / 1e12, all_ms=all_ms)
     elif a.case == "conv":
         shape = (a.batch, a.hw, a.hw, a.cin)
         pitch = B.dsq_row_pitch(a.cin, bits)

@@ -345,7 +345,7 @@ double estimate_other(const CsParams &p, int bits, int Cin, double macs, int lea
         // warps set the pace).  One wave, 4-bit, measured / said here: 64 channels 5.4 / 6.1, 128
         // 7.6 / 10.1, 256 10.2 / 12.6, 384 12.6 / 12.8, 512 15.2 / 15.2, 1024 25.2 / 24.9 us.  What is too
         // much at 128 and 256 channels offsets what this kernel's own estimate lacks around
-        // the line there (256 at 14x14, batch 12: 8.7 us, window 10.4, own estimate 9.9): with
+        // the line there (256 at 14x14, batch 12: 8.6 us, window 10.3, own estimate 10.5): with
         // 5.5 throughout, 35 of the layers below are on the wrong side instead of 34.
         const double tiles = std::ceil((double)p.M / p.H / p.W * (p.H + 1) * (p.W + 1) / 256) *
                              ((p.Ncols + 127) / 128);

@@ -175,10 +175,10 @@ dwconv3x3_kernel(const uint8_t *__restrict__ act, const uint8_t *__restrict__ wg
 // split once and feeds the (up to) three output rows it lies under, whose sums
 // stay in registers.
 //
-// Bound: the fma.f16x2 pipe (4.5 instructions per element at 62 lanes a clock
-// and SM, measured); all in all about 10 instructions per element.  The dp4a
-// form this replaces took 30 (byte transposes, funnel shifts and an epilogue of
-// 9) and only existed for 4-bit codes: C = 144, 56x56, batch 64, 4-bit 41.9 us.
+// Bound: instructions, 16 per element (14.4 M warp instructions for 28.9 M elements, counted;
+// 4.5 of them fma.f16x2, at 62 lanes a clock and SM).  The dp4a form this replaces took 30
+// (byte transposes, funnel shifts and an epilogue of 9) and only existed for 4-bit codes:
+// C = 144, 56x56, batch 64, 4-bit 41.9 -> 22.9 us.
 // Loaded words are kept as they came until a row's arithmetic is done (DwhRaw), and
 // the padding behind 2- and 3-bit rows is no unit of work: 112x112, 32 channels, batch 64
 // 2-bit 45.2 -> 22.6 us, 3-bit 42.4 -> 31.4 us (4-bit 19.8).

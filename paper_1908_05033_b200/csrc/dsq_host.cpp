@@ -4,7 +4,9 @@
 // status turned into DsqError - but on the critical path of every small call:
 // done in Python through ctypes it took 13 us a call (26 us with two calls, 270
 // us for the 20 calls of the ResNet-18-shaped stack, whose kernels at batch 1
-// take 177 us).  Here a call costs its launches and about 2 us.
+// then took 177 us).  Here a call with one launch and one new output takes 6 us of
+// host time, the launch included (quantise and 3x3 convolution of one 56x56x64
+// image: 13 us for the two, 7 us on the GPU), a replayed stack 15 us in all.
 #include <Python.h>
 
 #include <ATen/ops/empty.h>

@@ -72,7 +72,8 @@ __attribute__((visibility("hidden"))) dsq_plan *&dsq_recording_plan();
 
 // Whether a kernel launched now may read a layer's constants (packed weights, scales,
 // biases) before griddepcontrol.wait.  Every kernel of the library waits for the
-// kernels ahead of it before it lets the next one start, so when a kernel starts,
+// kernels ahead of it before it lets the next one start (or is launched without that
+// attribute and starts behind them), so when a kernel starts,
 // everything but its immediate predecessor has completed and is visible.  Behind
 // another launch of the same plan that predecessor is a layer of the network, which
 // writes activations only; elsewhere it may be what wrote the constants.

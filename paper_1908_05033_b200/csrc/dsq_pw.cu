@@ -20,9 +20,9 @@
 //     bulk copy (stride 2: im2col boxes with a traversal stride).
 // Input channels are expanded and multiplied in planes of 128.
 //
-// MobileNetV2-shaped layers, batch 64, 4-bit, against the im2col kernel this
-// takes them from: 112x112 16->96 71.8 us, 32->16 49.4 us; 56x56 24->144 30.4 us,
-// 144->24 + residual 19.9 us.
+// MobileNetV2-shaped layers, batch 64, 4-bit, the im2col kernel that had them before and
+// this one: 112x112 16->96 71.8 -> 28.5 us, 32->16 49.4 -> 14.3; 56x56 24->144 30.4 -> 14.4,
+// 144->24 + residual 19.9 -> 12.2.
 //
 // Every wait on a barrier is bounded, as in the other tensor-core kernels.
 #include "dsq_tc_common.cuh"
@@ -540,7 +540,9 @@ int dsq_pointwise(const void *act_codes, const dsq_nhwc_t *shape, int bits, cons
     // Tiling: the cheapest in a model of the launch in clocks - per tile the slowest
     // of epilogue (25 elements a clock), expansion and instructions (120 clocks
     // each, whatever their N), plus the hand-offs; once per CTA its weights and the
-    // fill of the pipeline.
+    // fill of the pipeline.  Constants fitted for the choice, not rates it reaches: 112x112
+    // 16->96 makes 9 elements a clock and SM in all, 16 would fill the issue slots
+    // (8 instructions an element, counted).
     const int subtiles = (p.M + 127) / 128;
     const int groups = bits == 3 ? (p.K + 31) / 32 : p.P / 16 * (bits == 2 ? 2 : 1);
     double best = 0;

@@ -1,5 +1,4 @@
-// Host-side pieces shared by the two tensor-core translation units
-// (dsq_tc.cu, dsq_conv3.cu).  Internal to the library.
+// Host-side pieces that the kernels' translation units share.  Internal to the library.
 #pragma once
 
 #include <cuda.h>
