@@ -541,8 +541,8 @@ PyObject *plan_record(PyObject *, PyObject *const *a, Py_ssize_t n)
     });
 }
 
-// (plan, parts) -> True when the plan still stands and was run on the current
-// stream; False when it has to be recorded again
+// (plan, parts | None) -> True when the plan still stands and was run on the current
+// stream; False when it has to be recorded again (None: it has just been recorded)
 PyObject *plan_run(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
     return guarded(n, 2, [&]() -> PyObject * {
@@ -559,7 +559,7 @@ PyObject *plan_run(PyObject *, PyObject *const *a, Py_ssize_t n)
             at += (size_t)p.size;
             return std::memcmp(r->bytes.data() + at - (size_t)p.size, p.data, (size_t)p.size) == 0;
         };
-        if (!each_part(a[1], same, &opaque) || i != r->parts.size()) Py_RETURN_FALSE;
+        if (a[1] != Py_None && (!each_part(a[1], same, &opaque) || i != r->parts.size())) Py_RETURN_FALSE;
         r->ran = true;
         check(enqueue([&](void *s) { return dsq_plan_run(r->plan, s); }), "dsq_plan_run");
         Py_RETURN_TRUE;
