@@ -16,12 +16,18 @@
 
 namespace {
 
+// (left: bytes of the row from p on.  A 3-bit row may end inside its last unit, whose
+// other codes are then not channels: 41 channels are 16 bytes, six units 18)
 template <int BITS>
-__device__ __forceinline__ uint32_t load_unit(const uint8_t *p)
+__device__ __forceinline__ uint32_t load_unit(const uint8_t *p, int left)
 {
     if (BITS == 4) return __ldg(reinterpret_cast<const uint32_t *>(p));
-    if (BITS == 3)      // 8 codes = 3 bytes at an odd offset: byte loads
-        return (uint32_t)__ldg(p) | ((uint32_t)__ldg(p + 1) << 8) | ((uint32_t)__ldg(p + 2) << 16);
+    if (BITS == 3) {    // 8 codes = 3 bytes at an odd offset: byte loads
+        uint32_t v = (uint32_t)__ldg(p);
+        if (left > 1) v |= (uint32_t)__ldg(p + 1) << 8;
+        if (left > 2) v |= (uint32_t)__ldg(p + 2) << 16;
+        return v;
+    }
     return __ldg(reinterpret_cast<const uint16_t *>(p));
 }
 
@@ -58,6 +64,7 @@ dwconv3x3_kernel(const uint8_t *__restrict__ act, const uint8_t *__restrict__ wg
         const int n = (int)(t / Ho);
         const int wo0 = sx * OW;
         const int hi0 = ho * STRIDE - 1, wi0 = wo0 * STRIDE - 1;
+        const int left = pitch - u * UB;
 
         uint32_t a[3][IW], wv[9];
 #pragma unroll
@@ -69,11 +76,11 @@ dwconv3x3_kernel(const uint8_t *__restrict__ act, const uint8_t *__restrict__ wg
                 a[r][x] = 0u;
                 if (hi >= 0 && hi < H && wi >= 0 && wi < W)
                     a[r][x] = load_unit<BITS>(
-                        act + (((int64_t)n * H + hi) * W + wi) * pitch + u * UB);
+                        act + (((int64_t)n * H + hi) * W + wi) * pitch + u * UB, left);
             }
         }
 #pragma unroll
-        for (int k = 0; k < 9; ++k) wv[k] = load_unit<BITS>(wgt + k * pitch + u * UB);
+        for (int k = 0; k < 9; ++k) wv[k] = load_unit<BITS>(wgt + k * pitch + u * UB, left);
 
         const int64_t pix0 = ((int64_t)n * Ho + ho) * Wo + wo0;
         uint32_t res[OW], cw[OW];
@@ -82,7 +89,7 @@ dwconv3x3_kernel(const uint8_t *__restrict__ act, const uint8_t *__restrict__ wg
             cw[o] = 0u;
             res[o] = 0u;
             if (e.residual && wo0 + o < Wo)
-                res[o] = load_unit<BITS>(e.residual + (pix0 + o) * pitch + u * UB);
+                res[o] = load_unit<BITS>(e.residual + (pix0 + o) * pitch + u * UB, left);
         }
 #pragma unroll
         for (int f = 0; f < 8; ++f) {
@@ -147,8 +154,9 @@ dwconv3x3_kernel(const uint8_t *__restrict__ act, const uint8_t *__restrict__ wg
                 uint8_t *dst = e.y_codes + (pix0 + o) * pitch + u * UB;
                 if (BITS == 4) *reinterpret_cast<uint32_t *>(dst) = cw[o];
                 else if (BITS == 3) {
-                    dst[0] = (uint8_t)cw[o]; dst[1] = (uint8_t)(cw[o] >> 8);
-                    dst[2] = (uint8_t)(cw[o] >> 16);
+                    dst[0] = (uint8_t)cw[o];
+                    if (left > 1) dst[1] = (uint8_t)(cw[o] >> 8);
+                    if (left > 2) dst[2] = (uint8_t)(cw[o] >> 16);
                     // the row's spare bytes behind the last unit are zero
                     if (u == units - 1)
                         for (int b = 3 * units; b < pitch; ++b) dst[b - u * UB] = 0;
@@ -439,12 +447,13 @@ extern "C" int dsq_dwconv2d(const void *act_codes, const dsq_nhwc_t *shape,
     const int pitch = (int)dsq_row_pitch(shape->C, bits);
     cudaStream_t s = (cudaStream_t)stream;
     // codes to codes, a requantiser range the lean epilogue takes that starts at 0 (it does
-    // not subtract lo); images of at least 2^31 bytes a row keep the general kernel's
+    // not subtract lo), rows that do not end inside a unit (3-bit rows of 41 or 84 channels
+    // do); images of at least 2^31 bytes a row keep the general kernel's
     // 64-bit indexing
     const int units = bits == 4 ? pitch / 4 : (shape->C + 7) / 8;
     const int strips = (Wo + 3) / 4;
     if (y_codes && !y_f32 && !acc_out && !e.residual && !e.general_offset && e.rq.lo == 0.0f &&
-        dsq_lean_epilogue(e) && (int64_t)units * strips * Ho * shape->N < (1ll << 31)) {
+        dsq_lean_epilogue(e) && units * bits <= pitch && (int64_t)units * strips * Ho * shape->N < (1ll << 31)) {
         DwHalf p;
         p.N = shape->N; p.H = shape->H; p.W = shape->W; p.C = shape->C;
         p.Ho = Ho; p.Wo = Wo; p.pitch = pitch;
