@@ -118,6 +118,7 @@ struct W3Params {
     int ld_dn[3], ld_dh[3], ld_dw[3];
     int smem_bytes;
     int early;                         // dsq_early_constants
+    uint32_t zero;                     // 0 (see w3_release_slot)
     unsigned long long wait_ns;
     int skip_b_round;
     // epilogue
@@ -223,6 +224,19 @@ __device__ __forceinline__ W3Pos w3_add(W3Pos a, int dn, int dh, int dw, int Hp,
     if (a.w >= Wp) { a.w -= Wp; ++a.h; }
     if (a.h >= Hp) { a.h -= Hp; ++a.n; }
     return a;
+}
+
+// Gives a packed slot back to the TMA producer when every lane of the warp HOLDS what it
+// read from it: `seen` is made of a word of each of the lane's loads, and the arrival
+// depends on a vote over it that only the kernel's parameter (zero) makes constant.
+// Loads merely written before the arrival are not enough: a warp that had arrived could
+// still read its rows after the slot had been filled again (seen on images more than 139
+// columns wide, whose windows take longest to expand: the weights of tap t + 4 in place
+// of tap t's, in one warp's rows of a CTA's second window).
+__device__ __forceinline__ void w3_release_slot(uint32_t bar, uint32_t seen, uint32_t zero, int lane)
+{
+    const bool never = __any_sync(0xffffffffu, (seen & zero) != 0u);
+    if (lane == 0 && !never) mbar_arrive(bar);
 }
 
 // Transposed tiles (template parameter TR).  An instruction whose A operand
@@ -682,29 +696,30 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
         for (uint32_t g = group; ok && g < n_b_fills; g += 2) {
             if (!(ok = wait_bar_warp(bar_bp_full(sp), php, ctl, 6))) break;
             if (warp == W3_WARP_B0) W3_STAMP(10, g >> 1);
-            const uint4 *src = reinterpret_cast<const uint4 *>(smem + L.b_packed + sp * b_packed_bytes);
+            const uint32_t src = smem_u32(smem + L.b_packed + sp * b_packed_bytes);
+            uint32_t seen = 0u;
             uint8_t *rowp = smem + L.b_tiles + st * b_stage_bytes + row0 * 128;
             bool waited = p.b_res != 0;
             if (BITS == 3 && TR) {
                 // one thread per operand row: 48 packed bytes of a tap and plane, or the
                 // 24 bytes of each of two taps (rows 64 .. 127 repeat 0 .. 63: dup)
                 const int row = tid;
-                const uint4 *r4 = reinterpret_cast<const uint4 *>(
-                    smem + L.b_packed + sp * b_packed_bytes + (p.dup ? row & 63 : row) * p.pk);
+                const uint32_t r4 = src + (uint32_t)((p.dup ? row & 63 : row) * p.pk);
                 uint32_t w[12], w1[12];
 #pragma unroll
                 for (int l = 0; l < 3; ++l) {
-                    const uint4 v = r4[l];
+                    const uint4 v = lds_128(r4 + 16 * l);
+                    seen |= v.x;
                     w[4 * l] = v.x; w[4 * l + 1] = v.y; w[4 * l + 2] = v.z; w[4 * l + 3] = v.w;
                 }
                 if (p.two_taps) {
-                    const uint4 v = r4[3];
+                    const uint4 v = lds_128(r4 + 48);
+                    seen |= v.x;
 #pragma unroll
                     for (int l = 0; l < 4; ++l) w1[l] = w[8 + l];
                     w1[4] = v.x; w1[5] = v.y;
                 }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar_bp_empty(sp));
+                w3_release_slot(bar_bp_empty(sp), seen, p.zero, lane);
                 if (!waited && !(ok = wait_bar_warp(bar_b_empty(st), phu ^ 1u, ctl, 7))) break;
                 uint8_t *rp = smem + L.b_tiles + st * b_stage_bytes + row * 128;
                 const int sw3 = row & 7;
@@ -721,17 +736,16 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
 #pragma unroll
                 for (int i = 0; i < 2; ++i)
                     if (tid + i * BT < BN) {
-                        const uint4 *r4 = reinterpret_cast<const uint4 *>(
-                            smem + L.b_packed + sp * b_packed_bytes + (tid + i * BT) * 48);
+                        const uint32_t r4 = src + (uint32_t)((tid + i * BT) * 48);
 #pragma unroll
                         for (int l = 0; l < 3; ++l) {
-                            const uint4 v = r4[l];
+                            const uint4 v = lds_128(r4 + 16 * l);
+                            seen |= v.x;
                             w[i][4 * l] = v.x; w[i][4 * l + 1] = v.y;
                             w[i][4 * l + 2] = v.z; w[i][4 * l + 3] = v.w;
                         }
                     }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar_bp_empty(sp));
+                w3_release_slot(bar_bp_empty(sp), seen, p.zero, lane);
                 if (!waited && !(ok = wait_bar_warp(bar_b_empty(st), phu ^ 1u, ctl, 7))) break;
 #pragma unroll
                 for (int i = 0; i < 2; ++i)
@@ -750,13 +764,12 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                 uint4 v[HALF_IT];
 #pragma unroll
                 for (int i = 0; i < HALF_IT; ++i)
-                    if (r0 + row0 + i * ROWS_PER_IT < BN)
-                        v[i] = src[(r0 + row0 + i * ROWS_PER_IT) * CH + j];
-                if (r0 + 128 >= BN) {
-                    // the packed slot is free as soon as every lane holds its chunks
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar_bp_empty(sp));
-                }
+                    if (r0 + row0 + i * ROWS_PER_IT < BN) {
+                        v[i] = lds_128(src + 16u * ((r0 + row0 + i * ROWS_PER_IT) * CH + j));
+                        seen |= v[i].x;
+                    }
+                // the packed slot is free as soon as every lane holds its chunks
+                if (r0 + 128 >= BN) w3_release_slot(bar_bp_empty(sp), seen, p.zero, lane);
                 if (!waited) {
                     if (!(ok = wait_bar_warp(bar_b_empty(st), phu ^ 1u, ctl, 7))) break;
                     waited = true;
