@@ -141,7 +141,8 @@ int dsq_workspace_init(void *workspace, size_t ws_bytes, void *stream);
  * its first call until it ends; where none can be had, or the workspace is not
  * memory of the current device, the word is copied (slower, same result).
  * Returns DSQ_OK, DSQ_ERR_TIMEOUT (a kernel gave up on a wait; its outputs
- * are undefined) or DSQ_ERR_RANGE (dsq_pack_weights met a bad clip range). */
+ * are undefined), DSQ_ERR_RANGE (dsq_pack_weights met a bad clip range) or
+ * DSQ_ERR_UNSUPPORTED (a weight blob of another library version). */
 int dsq_workspace_status(void *workspace, void *stream);
 
 /* ---- Algorithm 1 steps 1, 3 for weights (offline) ---------------------- */
@@ -162,7 +163,11 @@ int dsq_workspace_status(void *workspace, void *stream);
  *              rows already expanded to the 8-bit operand bytes of the grid
  *              Delta (c + 1/2), which dsq_conv2d then copies to the tensor
  *              core's shared-memory operand without expanding them again
- *              (dsq_weight_bytes includes that copy).
+ *              (dsq_weight_bytes includes that copy).  At 2 bits with 64, 128
+ *              or a multiple of 256 channels the copy holds 4-bit
+ *              floating-point operands and is marked as such: dsq_conv2d
+ *              records DSQ_ERR_UNSUPPORTED in the workspace when it meets such
+ *              a blob without the mark (packed by an earlier library).
  * A clip range with hi <= lo or a non-finite bound cannot be seen from the
  * host: the kernel writes code 0 for that channel and records DSQ_ERR_RANGE
  * in the workspace. */

@@ -44,6 +44,8 @@
 // are staged as three bands of 136 pixels, one per filter row, instead.
 //
 // Every wait on a barrier is bounded, as in the im2col kernel.
+#include <algorithm>
+
 #include "dsq_tc_common.cuh"
 #include "dsq_tc_host.h"
 
@@ -76,32 +78,40 @@ constexpr int W3_B_GROUP_WARPS = W3_NUM_B_WARPS / 2;   // two B groups take alte
 constexpr int W3_EPQ = W3_NUM_E_WARPS / 4;   // epilogue warps per tensor-memory lane quarter
 constexpr int W3_MAX_COUT = 1024;            // scale / bias of the layer stay in shared memory
 constexpr int W3_THREADS = W3_NUM_WARPS * 32;
-constexpr int W3_A_SLOTS = 2;          // expanded windows
+constexpr int W3_A_SLOTS = 2;          // expanded windows, at most
 constexpr int W3_MAX_BP = 4;           // packed B ring slots
 constexpr int W3_MAX_AS = 3;           // packed A staging slots
 constexpr int W3_MAX_BST = 10;         // expanded B stages (resident: all K steps)
 constexpr int W3_BAND_PX = 136;        // pixels of a band (three-band staging)
+constexpr int W3_F4_BAND_PX = 248;
 constexpr int W3_MAX_WINDOW_PX = 416;
+constexpr int W3_MAX_LOADS = 3;        // im2col loads of a window
+// 4-bit floating-point operands (see F4 below)
+constexpr uint32_t W3_F4_MARK = 0x34463271u;   // behind the blob's copy of the weights
+constexpr int W3_F4_TP = 240;          // positions of a tile
+constexpr int W3_F4_SF = 2 * W3_F4_TP; // tensor-memory columns of the block scales: 480 .. 511
 
 // byte offsets of the kernel's shared-memory regions (w3_layout)
 struct W3Smem {
-    uint32_t a_slots, b_tiles, a_stage, b_packed, epi, lut, a_tab, bars, tmem_slot, abort_flag, total;
+    uint32_t a_slots, b_tiles, a_stage, b_packed, epi, lut, bars, tmem_slot, abort_flag, total;
 };
 
 struct W3Params {
     // geometry
     int N, H, W, Hp, Wp;               // Hp = H + 1, Wp = W + 1 (see W3Pos)
     int m_tiles, n_tiles, BN, Ncols;
-    int E;                             // int8 bytes per pixel = Cin
-    int npl, kpp, ksteps;              // planes of 128 channels, K steps per plane, total
+    int E;                             // operand bytes per pixel: Cin (F4: Cin / 2)
+    int npl, kpp, ksteps;              // planes of 128 (F4: 256) channels, K steps per plane, total
     int PB, cpp;                       // packed bytes per pixel and plane; 16-byte chunks of it
-    int two_taps;                      // 64-channel rows (3-bit: transposed tiles): a K step is two filter taps
+    int tps;                           // filter taps of a K step: 2 with 64-channel rows (3-bit: transposed
+                                       // tiles only); F4: 4 with 64 channels, 2 with 128
     int pk;                            // packed bytes of a K step in a weight row
     int rb;                            // bytes of a window row: 128, or 64 (transposed tiles over 64
                                        // channels: half the shared memory, which is what leaves room
-                                       // for resident weights beside the window of a wide image)
+                                       // for resident weights beside the window of a wide image);
+                                       // F4: 32, 64 or 128 for 64, 128 or more channels
     int xstep;                         // bytes between two K steps of a plane in a weight row
-    int apx;                           // pixels of an A slot
+    int apx, a_slots;                  // pixels of an A slot, slots
     int a_box, a_nload, nbands, band_px;
     int tap_stride;                    // slot rows between two filter rows
     int as_slots, bp_slots, b_stages, b_res;
@@ -111,11 +121,12 @@ struct W3Params {
                                        // 0..63 and their epilogue warps take the other half of the columns
     int cout_pad;                      // Cout rounded up to the N tiling
     int tr;                            // transposed tiles (kernel form TR)
+    int f4;                            // 4-bit floating-point operands (kernel form F4)
     int mstep;                         // M tiles between two tiles of a CTA
-    int t_dn, t_dh, t_dw;              // mstep * 128 positions as images, padded rows, columns
+    int t_dn, t_dh, t_dw;              // the positions of mstep tiles as images, padded rows, columns
     // start of every load of a fill, from the tile's start: images, padded rows
     // (< Hp), padded columns (< Wp)
-    int ld_dn[3], ld_dh[3], ld_dw[3];
+    int ld_dn[W3_MAX_LOADS], ld_dh[W3_MAX_LOADS], ld_dw[W3_MAX_LOADS];
     int smem_bytes;
     int early;                         // dsq_early_constants
     uint32_t zero;                     // 0 (see w3_release_slot)
@@ -126,30 +137,34 @@ struct W3Params {
     float r_hi;                        // fmaf(hi - lo, inv, 0.5f) of the requantiser
     DsqEpi e;
     uint32_t orv;
+    const uint32_t *mark;              // F4: W3_F4_MARK, if the blob's copy is of that form
     const uint8_t *act;                // input codes and pixel pitch (general weight offset: S_a)
     int P;
+    // window offsets (16-byte units) of the four instructions of every K step of a plane
+    // (MMA_NONE: left out); in the parameters, so that the issuing warp keeps them, and what
+    // it makes of them, in uniform registers
+    uint4 x_off[9];
     W3Smem L;                          // shared-memory layout (host-made: w3_layout)
     int *ws;
 };
 
 
-__host__ __device__ inline W3Smem w3_layout(int apx, int rb, int BN, int pk, int PB, int as_slots,
+__host__ __device__ inline W3Smem w3_layout(int apx, int a_slots, int rb, int BN, int pk, int PB, int as_slots,
                                             int b_stages, int bp_slots, int cout_pad)
 {
     W3Smem L;
     uint32_t o = 0;
-    L.a_slots = o;  o += W3_A_SLOTS * apx * rb;            // apx is a multiple of 8
+    L.a_slots = o;  o += a_slots * apx * rb;            // apx is a multiple of 8
     o = (o + 1023u) & ~1023u;
     L.b_tiles = o;  o += b_stages * BN * 128;              // BN is a multiple of 8
     L.a_stage = o;  o += as_slots * apx * PB;
     L.b_packed = o; o += bp_slots * BN * pk;
     L.epi = o;      o += 2 * cout_pad * 4;                  // scale[cout_pad], bias[cout_pad]
     L.lut = o;      o += 16 * 4;
-    L.a_tab = o;    o += 9 * 16;                            // four A offsets per K step of a plane
     o = (o + 127u) & ~127u;
     // barriers: a_full/a_empty[2], as_full/as_empty[3], bp_full/bp_empty[4],
-    // b_full/b_empty[W3_MAX_BST], acc_full/acc_empty[2], drain
-    L.bars = o;     o += 8 * (2 * W3_A_SLOTS + 2 * W3_MAX_AS + 2 * W3_MAX_BP + 2 * W3_MAX_BST + 4 + 1);
+    // b_full/b_empty[W3_MAX_BST], acc_full/acc_empty[2], drain, scales
+    L.bars = o;     o += 8 * (2 * W3_A_SLOTS + 2 * W3_MAX_AS + 2 * W3_MAX_BP + 2 * W3_MAX_BST + 4 + 2);
     L.tmem_slot = o; o += 8;
     L.abort_flag = o; o += 8;
     L.total = o;
@@ -268,14 +283,29 @@ __device__ __forceinline__ uint32_t w3_transpose_fields(uint32_t x, int lane)
     return x;
 }
 
-template <int BITS, int EPI, bool TR>
+//
+// F4: 2-bit codes (weight grid Delta (c + 1/2)) as 4-bit floating-point operands.  E2M1
+// holds the codes 0 .. 3 and the weights 2 c + 1 exactly, and every partial sum is a whole
+// number far below 2^24, so the f32 accumulators hold the int32 sums bit for bit
+// (checked up to 2^23.9 on the hardware, in every order that the sums may be taken).  An
+// instruction covers K = 64 in the clocks in which kind::i8 covers 32, from the same 32
+// bytes a row; the window and the weights take half of the shared memory.  The block
+// scales (all 2, so that the accumulators come as 2 acc + S_a) need tensor memory
+// beside the two accumulators, so a tile is 240 positions instead of 256.
+//
+// int8 -> F4, batch 32: 64->64 at 224x224 82 -> 60 us, 128->128 at 112x112 44.7 -> 26.3,
+// 256->256 at 56x56 41.3 -> 25.6, 512->512 at 28x28 38.9 -> 27.6 (four passes of 240
+// positions for three of 256), at 14x14 16.3 -> 11.0.  What bounds it now: shared-memory
+// bandwidth (an instruction reads 11.5 KB in 120 clocks) and, with 64 channels, the epilogue.
+template <int BITS, int EPI, bool TR, bool F4 = false>
 __global__ void __launch_bounds__(W3_THREADS, 1)
 dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                 const __grid_constant__ CUtensorMap tmap_a, const W3Params p)
 {
     constexpr int CH = Chunks<BITS>::CH;       // packed 16-byte chunks per 128 codes
     constexpr int OUT = Chunks<BITS>::OUT;     // int8 chunks per packed chunk
-    constexpr int TP = TR ? 256 : W3_BM;       // positions of a tile
+    constexpr int TP = F4 ? W3_F4_TP : TR ? 256 : W3_BM;       // positions of a tile
+    static_assert(!F4 || (TR && BITS == 2), "F4: 2-bit codes, transposed tiles");
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     if ((threadIdx.x >> 5) == 1) W3_STAMP(13, 0);
     uint8_t *smem = reinterpret_cast<uint8_t *>(
@@ -321,6 +351,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
     auto bar_acc_full = [&](int s) { return bars + 8u * (O_ACC + s); };
     auto bar_acc_empty = [&](int s) { return bars + 8u * (O_ACC + 2 + s); };
     const uint32_t bar_drain = bars + 8u * (O_ACC + 4);
+    const uint32_t bar_scales = bars + 8u * (O_ACC + 5);
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(smem + L.tmem_slot);
     Ctl ctl{reinterpret_cast<volatile int *>(smem + L.abort_flag), p.ws, p.wait_ns};
 
@@ -347,6 +378,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
             mbar_init(bar_acc_empty(s), W3_NUM_E_WARPS);
         }
         mbar_init(bar_drain, 1);
+        if (F4) mbar_init(bar_scales, 4);
         *ctl.abort_flag = 0;
         W3_STAMP(13, 10);
         mbar_init_fence();
@@ -357,19 +389,6 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
         tmem_alloc(smem_u32((const void *)tmem_slot), 512);
         tmem_relinquish();
         W3_STAMP(13, 6);
-        // A descriptor offsets (16-byte units from the start of a slot) of the
-        // four instructions of every K step of a plane; 0xFFFFFFFF = no
-        // instruction (the half-empty last K step of a 64-channel input)
-        uint32_t *tab = reinterpret_cast<uint32_t *>(smem + L.a_tab);
-        for (int i = lane; i < 4 * p.kpp; i += 32) {
-            const int kk = i >> 2, j = i & 3;
-            const int tap = p.two_taps ? 2 * kk + (j >> 1) : kk;
-            const int within = p.two_taps ? 32 * (j & 1) : 32 * j;
-            const int kh = tap / 3, kw = tap - 3 * kh;
-            tab[i] = tap < 9 && within < p.E
-                         ? (uint32_t)((kh * p.tap_stride + kw) * (p.rb >> 4) + (within >> 4))
-                         : 0xFFFFFFFFu;
-        }
     }
     if (warp == W3_WARP_TMA_B && lane == 0) tma_prefetch_desc(&tmap_b);
     if (warp == W3_WARP_TMA_A && lane == 0) tma_prefetch_desc(&tmap_a);
@@ -415,8 +434,16 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
             const int BST = p.b_stages;
             const int y = n_tile * BN;
             int s = 0, x = 0;
+            bool ok = true;
+            // (a blob packed by a library that kept its copy in another form)
+            if (F4 && n_b_fills > 0 && __ldg(p.mark) != W3_F4_MARK) {
+                if (atomicCAS(p.ws + DSQ_WS_STATUS, 0, (int)DSQ_ERR_UNSUPPORTED) == 0)
+                    p.ws[DSQ_WS_DETAIL] = 17;
+                *ctl.abort_flag = 1;
+                ok = false;
+            }
 #pragma unroll 1
-            for (uint32_t g = 0; g < n_b_fills; ++g) {
+            for (uint32_t g = 0; ok && g < n_b_fills; ++g) {
                 if (!wait_bar(bar_b_empty(s), ph ^ 1u, ctl, 1)) break;
                 if ((int)g == p.skip_b_round) break;
                 mbar_arrive_expect_tx(bar_b_full(s), b_stage_bytes);
@@ -478,14 +505,14 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
             // never issued - the roles then run into their wait limit and the
             // kernel reports the failure.
             W3Pos base = a_base0;
-            W3Pos q[3];
+            W3Pos q[W3_MAX_LOADS];
             int nl = 0;
             bool bad = false;
             auto prepare = [&]() {
                 nl = 0;
                 bad = false;
 #pragma unroll
-                for (int i = 0; i < 3; ++i) {
+                for (int i = 0; i < W3_MAX_LOADS; ++i) {
                     if (i >= nld) break;
                     q[i] = w3_add(base, p.ld_dn[i], p.ld_dh[i], p.ld_dw[i], p.Hp, p.Wp);
                     if (q[i].n < p.N) {
@@ -507,7 +534,9 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                 }
                 if (nl < nld) {
                     // positions p.N * Hp * Wp .. + Wp of a load that is left out
-                    for (int i = 0; i < nld; ++i) {
+#pragma unroll
+                    for (int i = 0; i < W3_MAX_LOADS; ++i) {
+                        if (i >= nld) break;
                         const int behind = (q[i].n - p.N) * img_positions + q[i].h * p.Wp + q[i].w;
                         if (q[i].n < p.N || behind > p.Wp) continue;
                         const uint32_t z = smem_u32(smem + L.a_stage) + s * a_stage_bytes +
@@ -520,7 +549,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                 mbar_arrive_expect_tx(bar_as_full(s), (uint32_t)(nl * p.a_box * p.PB));
                 const uint32_t dst0 = smem_u32(smem + L.a_stage) + s * a_stage_bytes;
 #pragma unroll
-                for (int i = 0; i < 3; ++i) {
+                for (int i = 0; i < W3_MAX_LOADS; ++i) {
                     if (i >= nld) break;
                     if (q[i].n >= p.N) continue;
                     // bounding box = image grown by one pixel at the left and the top:
@@ -544,52 +573,55 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
     } else if (warp == W3_WARP_MMA) {
         // ---------------- MMA issuer (whole warp, uniform; one lane issues) --------
         // (TR: A = 128 weight rows, signed; B = 256 window rows, unsigned)
-        const uint32_t idesc = TR ? idesc_i8(256, true, false, 128) : idesc_i8(BN, false, true, W3_BM);
+        const uint32_t idesc = F4   ? idesc_mxf4(W3_F4_TP)
+                               : TR ? idesc_i8(256, true, false, 128)
+                                    : idesc_i8(BN, false, true, W3_BM);
         const uint64_t desc0 = smem_desc_sw128(0u);
         const uint32_t desc_hi = (uint32_t)(desc0 >> 32), desc_lo = (uint32_t)desc0;
-        const uint32_t win_hi = p.rb == 64 ? (uint32_t)(smem_desc_sw64(0u) >> 32) : desc_hi;
+        const uint32_t win_hi = p.rb == 64         ? (uint32_t)(smem_desc_sw64(0u) >> 32)
+                                : F4 && p.rb == 32 ? (uint32_t)(smem_desc_sw32(0u) >> 32)
+                                                   : desc_hi;
         const uint32_t a_lo_base = desc_lo + (smem_u32(smem + L.a_slots) >> 4);
         const uint32_t b_lo_base = desc_lo + (smem_u32(smem + L.b_tiles) >> 4);
-        const uint4 *tab = reinterpret_cast<const uint4 *>(smem + L.a_tab);
         const int BST = p.b_stages;
         int aslot = 0, st = 0;
         uint32_t aph = 0, bph = 0;
-        bool ok = true;
+        bool ok = !F4 || wait_bar_warp(bar_scales, 0u, ctl, 14);
 #pragma unroll 1
         for (int it = 0; ok && it < my_tiles; ++it) {
             const int as = it & 1;
             if (!(ok = wait_bar_warp(bar_acc_empty(as), ((it >> 1) & 1) ^ 1u, ctl, 3))) break;
             W3_STAMP(4, it);
             tc_fence_after_sync();
-            const uint32_t d_tmem = tmem_base + as * (TR ? 256 : BN);
+            const uint32_t d_tmem = tmem_base + as * (TR ? TP : BN);
             uint32_t first = 0u;                    // 0: the tile's first instruction overwrites
 #pragma unroll 1
             for (int pl = 0; ok && pl < p.npl; ++pl) {
                 if (!(ok = wait_bar_warp(bar_a_full(aslot), aph, ctl, 4))) break;
                 if (pl == 0) W3_STAMP(5, it);
                 tc_fence_after_sync();
-                const uint32_t a_lo = a_lo_base + aslot * (a_slot_bytes >> 4);
+                const uint32_t x_lo = a_lo_base + aslot * (a_slot_bytes >> 4);
                 if (p.b_res) st = pl * p.kpp;
 #pragma unroll 1
                 for (int kk = 0; kk < p.kpp; ++kk) {
-                    const uint4 t = tab[kk];
                     if (!p.b_res || it == 0) {
                         if (!(ok = wait_bar_warp(bar_b_full(st), bph, ctl, 10))) break;
                         tc_fence_after_sync();
                     }
-                    // (a slot lies below 256 KB, so the sums stay inside the
-                    // 14-bit address field; 0xFFFFFFFF marks no instruction)
-                    if (TR)
-                        mma_i8_ss_x4b_elect(d_tmem, b_lo_base + st * (b_stage_bytes >> 4), desc_hi,
-                                            a_lo + t.x, t.y == 0xFFFFFFFFu ? t.y : a_lo + t.y,
-                                            t.z == 0xFFFFFFFFu ? t.z : a_lo + t.z,
-                                            t.w == 0xFFFFFFFFu ? t.w : a_lo + t.w, win_hi, idesc,
-                                            first);
+                    // (slots and stages lie below 256 KB, so the sums stay inside the
+                    // 14-bit address field)
+                    const uint32_t w_lo = b_lo_base + st * (b_stage_bytes >> 4);
+                    const uint4 t = p.x_off[kk];
+                    const uint32_t x0 = x_lo + t.x, x1 = t.y == MMA_NONE ? t.y : x_lo + t.y,
+                                   x2 = t.z == MMA_NONE ? t.z : x_lo + t.z,
+                                   x3 = t.w == MMA_NONE ? t.w : x_lo + t.w;
+                    if (F4)
+                        mma_f4_ss_x4b_elect(d_tmem, w_lo, desc_hi, x0, x1, x2, x3, win_hi, idesc,
+                                            tmem_base + W3_F4_SF, tmem_base + W3_F4_SF + 16, first);
+                    else if (TR)
+                        mma_i8_ss_x4b_elect(d_tmem, w_lo, desc_hi, x0, x1, x2, x3, win_hi, idesc, first);
                     else
-                    mma_i8_ss_x4_elect(d_tmem, a_lo + t.x, t.y == 0xFFFFFFFFu ? t.y : a_lo + t.y,
-                                       t.z == 0xFFFFFFFFu ? t.z : a_lo + t.z,
-                                       t.w == 0xFFFFFFFFu ? t.w : a_lo + t.w, desc_hi,
-                                       b_lo_base + st * (b_stage_bytes >> 4), desc_hi, idesc, first);
+                        mma_i8_ss_x4_elect(d_tmem, x0, x1, x2, x3, desc_hi, w_lo, desc_hi, idesc, first);
                     first = 1u;
                     if (!p.b_res) {
                         mma_commit_elect(bar_b_empty(st));
@@ -599,7 +631,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                     }
                 }
                 if (ok) mma_commit_elect(bar_a_empty(aslot));
-                if (++aslot == W3_A_SLOTS) { aslot = 0; aph ^= 1u; }
+                if (++aslot == p.a_slots) { aslot = 0; aph ^= 1u; }
             }
             if (ok) mma_commit_elect(bar_acc_full(as));
             W3_STAMP(6, it);
@@ -657,9 +689,17 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
             for (int t = tid; t < n_tasks; t += W3_NUM_A_WARPS * 32) {
                 const int px = t >> lcpp, ch = t & (p.cpp - 1);
                 const uint4 v = lds_128(src + 16u * t);
-                // (16-byte chunks XOR-ed with address bits 7..9, of 64-byte rows bits 7..8)
+                // (16-byte chunks XOR-ed with address bits 7..9, of 64-byte rows bits 7..8, of
+                // 32-byte rows bit 7)
                 const uint32_t row = dst + (uint32_t)(px * p.rb);
-                const int sw = p.rb == 64 ? (px >> 1) & 3 : px & 7;
+                const int sw = p.rb == 64 ? (px >> 1) & 3 : F4 && p.rb == 32 ? (px >> 2) & 1 : px & 7;
+                if constexpr (F4) {
+#pragma unroll
+                    for (int c = 0; c < 2; ++c)
+                        sts_128(row + (uint32_t)(((ch * 2 + c) ^ sw) << 4),
+                                expand_word_f4<false>(v.x, c), expand_word_f4<false>(v.y, c),
+                                expand_word_f4<false>(v.z, c), expand_word_f4<false>(v.w, c));
+                } else
 #pragma unroll
                 for (int c = 0; c < OUT; ++c)
                     sts_128(row + (uint32_t)(((ch * OUT + c) ^ sw) << 4),
@@ -674,7 +714,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
             }
             if (warp == W3_WARP_A0) W3_STAMP(3, g);
             if (++ss == AS) { ss = 0; phs ^= 1u; }
-            if (++slot == W3_A_SLOTS) { slot = 0; pha ^= 1u; }
+            if (++slot == p.a_slots) { slot = 0; pha ^= 1u; }
         }
     } else if (warp < W3_WARP_E0) {
         // ---------------- B: expand packed weight rows --------------------------------
@@ -691,7 +731,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
         // own fills: g = group, group + 2, ...
         int sp = group % BP, st = p.b_res ? group : group % BST;
         uint32_t php = (uint32_t)(group / BP) & 1u, phu = p.b_res ? 0u : (uint32_t)(group / BST) & 1u;
-        bool ok = !p.w8;                           // (w8: nothing to expand)
+        bool ok = !F4 && !p.w8;                    // (w8: nothing to expand)
 #pragma unroll 1
         for (uint32_t g = group; ok && g < n_b_fills; g += 2) {
             if (!(ok = wait_bar_warp(bar_bp_full(sp), php, ctl, 6))) break;
@@ -712,7 +752,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                     seen |= v.x;
                     w[4 * l] = v.x; w[4 * l + 1] = v.y; w[4 * l + 2] = v.z; w[4 * l + 3] = v.w;
                 }
-                if (p.two_taps) {
+                if (p.tps == 2) {
                     const uint4 v = lds_128(r4 + 48);
                     seen |= v.x;
 #pragma unroll
@@ -726,7 +766,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                     uint4 c;
-                    if (q >= 4 && p.two_taps) c = expand3_chunk<true>(w1, q & 3, p.orv);
+                    if (q >= 4 && p.tps == 2) c = expand3_chunk<true>(w1, q & 3, p.orv);
                     else c = expand3_chunk<true>(w, q, p.orv);
                     *reinterpret_cast<uint4 *>(rp + ((q ^ sw3) << 4)) = c;
                 }
@@ -805,6 +845,17 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
         // ---------------- epilogue: four warps per tensor-memory lane quarter -----------
         const int quarter = warp & 3;
         const int k = (warp - W3_WARP_E0) >> 2;              // which of the quarter's warps
+        if (F4 && k == 0) {
+            // every block scale is 2 (UE8M0 128), whatever place the tensor core reads it from
+            uint32_t two[32];
+#pragma unroll
+            for (int i = 0; i < 32; ++i) two[i] = 0x80808080u;
+            tmem_st_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + W3_F4_SF, two);
+            tmem_st_wait();
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_scales);
+        }
         if constexpr (TR) {
             // thread = output channel (tensor-memory lane), columns = positions;
             // warp k of a quarter takes columns 64 k .. 64 k + 63 in units of 16
@@ -816,7 +867,8 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
             // (dup: lanes 64..127 repeat channels 0..63; quarters 2, 3 take columns 128..255)
             const int chq = p.dup ? (quarter & 1) * 32 : quarter * 32;
             const int colbase = p.dup ? 128 * (quarter >> 1) + 32 * k : 64 * k;
-            const int units = p.dup ? 2 : 4;
+            // (F4: 15 units of columns, the last warp has one less)
+            const int units = (p.dup ? 2 : 4) - (F4 && k == 3 && (!p.dup || quarter >= 2));
             const int ch = n_tile * 128 + chq + lane;
             // a warp has work while its first code word lies inside the output row:
             // channels past Cout are padding lanes of the packed row and get zeros
@@ -895,7 +947,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                 if (!(ok = wait_bar_warp(bar_acc_full(as), (it >> 1) & 1u, ctl, 8))) break;
                 if (warp == W3_WARP_E0) W3_STAMP(8, it);
                 tc_fence_after_sync();
-                const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + as * 256;
+                const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + as * TP;
 #pragma unroll 1
                 for (int u = 0; warp_live && u < units; ++u) {
                     const int col0 = colbase + 16 * u;
@@ -930,7 +982,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
 #pragma unroll
                             for (int j = 0; j < 8; ++j) v[j] = r[8 * h + j];
                             const uint32_t rw = SB == 4 ? resT[h < CWU ? h : 0] : resT[0] >> (16 * h);
-                            const uint32_t x = dsq_lean_codes8<BITS, EPI == DSQ_EPI_CODES_RES, false, SB>(
+                            const uint32_t x = dsq_lean_codes8<BITS, EPI == DSQ_EPI_CODES_RES, false, SB, F4>(
                                 v, sc4, bi4, rw, lean);
                             if (SB == 4) cw[h < CWU ? h : 0] = x;
                             else cw[0] |= x << (16 * h);
@@ -940,7 +992,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                         for (int j = 0; j < 16; ++j) {
                             // column 16 u + j of the warp: held by lane 8 u + j / 2
                             const int mj = __shfl_sync(0xffffffffu, (j & 1) ? m1 : m0, 8 * u + (j >> 1));
-                            const int vi = (int)r[j] >> p.shift;
+                            const int vi = F4 ? __float2int_rn(__uint_as_float(r[j])) : (int)r[j] >> p.shift;
                             if (mj >= 0 && ch < p.Ncols) {
                                 if (e.acc_out) e.acc_out[(int64_t)mj * p.Ncols + ch] = vi;
                                 float y;
@@ -1160,7 +1212,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
     }
 }
 
-template <int BITS, int EPI, bool TR = false>
+template <int BITS, int EPI, bool TR = false, bool F4 = false>
 int w3_launch(const CUtensorMap &tb, const CUtensorMap &ta, const W3Params &p, cudaStream_t s,
               int pdl)
 {
@@ -1169,14 +1221,14 @@ int w3_launch(const CUtensorMap &tb, const CUtensorMap &ta, const W3Params &p, c
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return DSQ_ERR_CUDA;
     const unsigned long long dev_bit = dev < 64 ? 1ull << dev : 0ull;
     if (!(configured.load(std::memory_order_acquire) & dev_bit)) {
-        if (cudaFuncSetAttribute(dsq_win3_kernel<BITS, EPI, TR>,
+        if (cudaFuncSetAttribute(dsq_win3_kernel<BITS, EPI, TR, F4>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  227 * 1024) != cudaSuccess)
             return DSQ_ERR_CUDA;
         configured.fetch_or(dev_bit, std::memory_order_release);
     }
     const int grid = p.mstep * p.n_tiles;
-    return dsq_launch(dsq_win3_kernel<BITS, EPI, TR>, dim3(grid), dim3(W3_THREADS),
+    return dsq_launch(dsq_win3_kernel<BITS, EPI, TR, F4>, dim3(grid), dim3(W3_THREADS),
                       (size_t)p.smem_bytes, s, pdl, 0, tb, ta, p);
 }
 
@@ -1184,6 +1236,14 @@ template <int BITS>
 int w3_dispatch(int epi, const CUtensorMap &tb, const CUtensorMap &ta, const W3Params &p,
                 cudaStream_t s, int pdl)
 {
+    if constexpr (BITS == 2)
+        if (p.f4) {
+            switch (epi) {
+            case DSQ_EPI_CODES: return w3_launch<BITS, DSQ_EPI_CODES, true, true>(tb, ta, p, s, pdl);
+            case DSQ_EPI_CODES_RES: return w3_launch<BITS, DSQ_EPI_CODES_RES, true, true>(tb, ta, p, s, pdl);
+            default: return w3_launch<BITS, DSQ_EPI_GENERAL, true, true>(tb, ta, p, s, pdl);
+            }
+        }
     if (p.tr) {
         switch (epi) {
         case DSQ_EPI_CODES: return w3_launch<BITS, DSQ_EPI_CODES, true>(tb, ta, p, s, pdl);
@@ -1208,28 +1268,37 @@ int w3_dispatch(int epi, const CUtensorMap &tb, const CUtensorMap &ta, const W3P
 // ---------------------------------------------------------------------------
 namespace {
 
-// One thread per (row, K step, packed 16-byte chunk): the chunk's OUT int8
+// One thread per (row, K step, packed 16-byte chunk): the chunk's OUT operand
 // chunks, in the operand's logical order (TMA applies the 128-byte swizzle when
-// it copies a tile).  Same expansion as the kernel's own (expand_word), for the
-// grid Delta (c + 1/2); bytes past the end of a weight row read as packed
-// zeros, as the kernel's TMA loads of the packed rows do.
-template <int BITS>
+// it copies a tile).  Same expansion as the kernel's own (expand_word, the window's
+// expand_word_f4), for the grid Delta (c + 1/2); bytes past the end of a weight row
+// read as packed zeros, as the kernel's TMA loads of the packed rows do.
+// F4: `mark` gets W3_F4_MARK.
+template <int BITS, bool F4>
 __global__ void __launch_bounds__(256)
 w8_build_kernel(const uint8_t *__restrict__ packed, uint8_t *__restrict__ out, int Cout,
-                int row_bytes, int ksteps, int kpp, int xstep)
+                int row_bytes, int ksteps, int kpp, int xstep, uint32_t *__restrict__ mark)
 {
-    constexpr int CH = Chunks<BITS>::CH, OUT = Chunks<BITS>::OUT;
+    constexpr int OUT = F4 ? 2 : Chunks<BITS>::OUT, CH = 8 / OUT;
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int j = (int)(idx % CH);
     const int ks = (int)((idx / CH) % ksteps);
     const int64_t row = idx / ((int64_t)CH * ksteps);
     if (row >= Cout) return;
     const int pl = ks / kpp, kk = ks - pl * kpp;
-    const int x = kk * xstep + pl * 16 * BITS + 16 * j;        // byte offset in the packed row
+    const int x = kk * xstep + (pl * CH + j) * 16;             // byte offset in the packed row
     uint4 v = make_uint4(0u, 0u, 0u, 0u);
     if (x < row_bytes) v = *reinterpret_cast<const uint4 *>(packed + row * row_bytes + x);
     const uint32_t orv = 0x01010101u << (7 - BITS);
     uint8_t *dst = out + (row * ksteps + ks) * 128;
+    if (F4 && idx == 0) *mark = W3_F4_MARK;
+    if constexpr (F4) {
+#pragma unroll
+        for (int c = 0; c < OUT; ++c)
+            *reinterpret_cast<uint4 *>(dst + 16 * (j * OUT + c)) =
+                make_uint4(expand_word_f4<true>(v.x, c), expand_word_f4<true>(v.y, c),
+                           expand_word_f4<true>(v.z, c), expand_word_f4<true>(v.w, c));
+    } else
 #pragma unroll
     for (int c = 0; c < OUT; ++c)
         *reinterpret_cast<uint4 *>(dst + 16 * (j * OUT + c)) =
@@ -1239,40 +1308,59 @@ w8_build_kernel(const uint8_t *__restrict__ packed, uint8_t *__restrict__ out, i
 
 }  // namespace
 
+// planes of a pixel's channels, K steps of a plane and taps of a K step, the latter two of
+// rows that are not 128 bytes long
+static inline void w3_steps(int Cin, int f4, int *npl, int *kpp, int *tps)
+{
+    const int full = f4 ? 256 : 128;               // channels of a 128-byte row
+    *npl = Cin < full ? 1 : Cin / full;
+    *tps = Cin < full ? full / Cin : 1;
+    *kpp = (9 + *tps - 1) / *tps;
+}
+
 DsqW8Info dsq_w8_info(const dsq_conv_t *conv, int bits)
 {
-    DsqW8Info w = {0, 0, 0, 0};
+    DsqW8Info w = {0, 0, 0, 0, 0};
     if (!conv || conv->groups != 1 || conv->KH != 3 || conv->KW != 3 || conv->stride != 1 ||
         conv->pad != 1 || (bits != 2 && bits != 4))
         return w;
     const int Cin = conv->Cin;
     if (!(Cin == 64 || (Cin % 128 == 0 && Cin <= 1024))) return w;
-    const int npl = Cin == 64 ? 1 : Cin / 128;
+    int npl, kpp, tps;
+    w3_steps(Cin, 0, &npl, &kpp, &tps);
     w.enabled = 1;
-    w.ksteps = npl * (Cin == 64 ? 5 : 9);
+    w.ksteps = npl * kpp;
     const size_t packed = (size_t)conv->Cout * 9 * dsq_row_pitch(Cin, bits);
     w.offset = (packed + 1023) / 1024 * 1024;
     w.bytes = (size_t)conv->Cout * w.ksteps * 128;
+    w.f4 = bits == 2 && (Cin == 64 || Cin == 128 || Cin % 256 == 0);
+    if (w.f4) {
+        w3_steps(Cin, 1, &npl, &kpp, &tps);
+        w.ksteps = npl * kpp;
+    }
     return w;
 }
+
+// where an F4 copy is marked: the last 16 bytes of its room (the copy fills half)
+static inline size_t w3_mark_offset(const DsqW8Info &w) { return w.offset + w.bytes - 16; }
 
 int dsq_w8_build(void *blob, const dsq_conv_t *conv, int bits, cudaStream_t stream)
 {
     const DsqW8Info w = dsq_w8_info(conv, bits);
     if (!w.enabled) return DSQ_OK;
-    const int Cin = conv->Cin;
-    const int P = (int)dsq_row_pitch(Cin, bits);
-    const int kpp = Cin == 64 ? 5 : 9;
-    const int xstep = Cin == 64 ? 16 * bits : P;
-    const int64_t threads = (int64_t)conv->Cout * w.ksteps * bits;       // CH = bits
+    const int P = (int)dsq_row_pitch(conv->Cin, bits);
+    int npl, kpp, tps;
+    w3_steps(conv->Cin, w.f4, &npl, &kpp, &tps);
+    const int ch = w.f4 || bits == 4 ? 4 : 2;                            // packed chunks of a K step
+    const int64_t threads = (int64_t)conv->Cout * w.ksteps * ch;
     const unsigned blocks = (unsigned)((threads + 255) / 256);
     const uint8_t *packed = (const uint8_t *)blob;
     uint8_t *out = (uint8_t *)blob + w.offset;
-    if (bits == 4)
-        return dsq_launch(w8_build_kernel<4>, dim3(blocks), dim3(256), 0, stream, 0, 0, packed, out,
-                          conv->Cout, 9 * P, w.ksteps, kpp, xstep);
-    return dsq_launch(w8_build_kernel<2>, dim3(blocks), dim3(256), 0, stream, 0, 0, packed, out,
-                      conv->Cout, 9 * P, w.ksteps, kpp, xstep);
+    return dsq_launch(w.f4        ? w8_build_kernel<2, true>
+                      : bits == 4 ? w8_build_kernel<4, false>
+                                  : w8_build_kernel<2, false>,
+                      dim3(blocks), dim3(256), 0, stream, 0, 0, packed, out, conv->Cout, 9 * P, w.ksteps,
+                      kpp, tps * P, (uint32_t *)((uint8_t *)blob + w3_mark_offset(w)));
 }
 
 int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
@@ -1305,62 +1393,67 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     const int64_t G = ((int64_t)p.N - 1) * p.Hp * p.Wp + (int64_t)(p.H - 1) * p.Wp + p.W;
     if (G > (1ll << 30)) return DSQ_ERR_UNSUPPORTED;
     p.Ncols = Cout;
-    p.E = Cin;
-    p.npl = Cin == 64 ? 1 : Cin / 128;
     const int P = (int)dsq_row_pitch(Cin, bits);           // packed bytes per pixel
-    p.PB = Cin == 64 ? P : 16 * bits;
-    p.cpp = p.PB / 16;
     // Tiling, window and shared memory for one of the two kernel forms.
     // Transposed (tr): tiles of 256 positions x 128 output channels, A = weights.
     // Plain: 128 positions x up to 256 channels, A = window.
     const DsqW8Info w8 = dsq_w8_info(conv, bits);
     // (plain tiles with up to 64 output channels keep the expanded weights resident in
     // shared memory for the whole CTA anyway: nothing to gain, measured slightly slower)
-    const bool w8_ok = hooks.w8 && w8.enabled && e.half_offset && bits != 3;
-    auto configure = [&](int tr) -> int {
+    const bool w8_any = hooks.w8 && w8.enabled && e.half_offset;
+    // f4: 4-bit floating-point operands (2-bit codes; transposed tiles over the blob's copy)
+    auto configure = [&](int tr, int f4) -> int {
+        const bool w8_ok = w8_any && f4 == w8.f4;
+        if (f4 && !w8_ok) return 0;
         p.tr = tr;
-        p.two_taps = Cin == 64 && (bits != 3 || tr);
-        p.kpp = p.two_taps ? 5 : 9;
+        p.f4 = f4;
+        w3_steps(Cin, f4, &p.npl, &p.kpp, &p.tps);
+        if (bits == 3 && !tr) { p.tps = 1; p.kpp = 9; }
+        p.E = f4 ? Cin / 2 : Cin;
+        p.PB = std::min(P, (f4 ? 32 : 16) * bits);
+        p.cpp = p.PB / 16;
         p.ksteps = p.npl * p.kpp;
-        p.xstep = p.two_taps ? 2 * P : P;
-        p.pk = p.two_taps ? 2 * P : 16 * bits;
-        p.rb = tr && p.two_taps ? 64 : 128;
+        p.xstep = p.tps * P;
+        p.pk = p.tps > 1 ? p.tps * P : 16 * bits;
+        p.rb = tr ? 128 / p.tps : 128;
         // transposed tiles for <= 64 output channels: the weight rows twice in the
         // A operand (two TMA boxes of the expanded copy), so that all 128 lanes of
         // the accumulator, and all epilogue warps, carry data
         p.dup = tr && Cout <= 64;
         if (p.dup && !w8_ok && bits != 3) return 0;
         p.w8 = w8_ok && (Cout > 64 || p.dup);
-        const int tile_pos = tr ? 256 : W3_BM;
+        const int tile_pos = f4 ? W3_F4_TP : tr ? 256 : W3_BM;
         p.m_tiles = (int)((G + tile_pos - 1) / tile_pos);
         p.BN = tr ? 128 : (Cout >= 256 ? 256 : ((Cout + 63) / 64) * 64);
         p.n_tiles = (Cout + p.BN - 1) / p.BN;
         p.cout_pad = p.n_tiles * p.BN;
         if (p.cout_pad > W3_MAX_COUT) return 0;
         const int need = tile_pos + 2 + 2 * p.Wp;
-        if (need <= (tr ? 768 : W3_MAX_WINDOW_PX)) {
+        const int band = f4 ? W3_F4_BAND_PX : W3_BAND_PX;
+        if (need <= (f4 ? 3 * W3_F4_BAND_PX : tr ? 768 : W3_MAX_WINDOW_PX)) {
             p.nbands = 1;
             p.a_nload = (need + 255) / 256;
             p.a_box = (((need + p.a_nload - 1) / p.a_nload) + 7) / 8 * 8;
             p.band_px = p.a_nload * p.a_box;
             p.apx = p.band_px;
             p.tap_stride = p.Wp;
-        } else if (!tr) {
+        } else if (!tr || f4) {
             p.nbands = 3;
             p.a_nload = 1;
-            p.a_box = W3_BAND_PX;
-            p.band_px = W3_BAND_PX;
-            p.apx = 3 * W3_BAND_PX;
-            p.tap_stride = W3_BAND_PX;
+            p.a_box = band;
+            p.band_px = band;
+            p.apx = 3 * band;
+            p.tap_stride = band;
         } else {
             return 0;
         }
+        p.a_slots = W3_A_SLOTS;
         // shared memory: resident B where one N tile's K steps all fit, else rings
         p.b_res = 0;
         if (p.ksteps <= W3_MAX_BST) {
             for (int as = W3_MAX_AS; as >= 2; --as) {
                 const int bp = p.w8 ? 0 : 2;
-                const W3Smem L = w3_layout(p.apx, p.rb, p.BN, p.pk, p.PB, as, p.ksteps, bp, p.cout_pad);
+                const W3Smem L = w3_layout(p.apx, p.a_slots, p.rb, p.BN, p.pk, p.PB, as, p.ksteps, bp, p.cout_pad);
                 if (L.total + 1024 <= 227u * 1024u) {
                     p.b_res = 1; p.b_stages = p.ksteps; p.as_slots = as; p.bp_slots = bp;
                     return 1;
@@ -1371,9 +1464,11 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
         // what hides the latency of the weight loads, so it goes first
         if (p.w8) {
             // no packed ring: the operand ring itself hides the latency of the loads
+            // (one window slot: 256 channels as 4-bit operands in three bands)
+            for (p.a_slots = W3_A_SLOTS; p.a_slots >= (f4 ? 1 : 2); --p.a_slots)
             for (int as = W3_MAX_AS; as >= 1; --as)
                 for (int bst = 6; bst >= 2; --bst) {
-                    const W3Smem L = w3_layout(p.apx, p.rb, p.BN, p.pk, p.PB, as, bst, 0, p.cout_pad);
+                    const W3Smem L = w3_layout(p.apx, p.a_slots, p.rb, p.BN, p.pk, p.PB, as, bst, 0, p.cout_pad);
                     if (L.total + 1024 <= 227u * 1024u) {
                         p.as_slots = as; p.b_stages = bst; p.bp_slots = 0;
                         return 1;
@@ -1383,7 +1478,7 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
         }
         const int tries[6][3] = {{3, 3, 4}, {2, 3, 4}, {2, 2, 4}, {2, 2, 3}, {2, 2, 2}, {1, 2, 2}};
         for (int t = 0; t < 6; ++t) {
-            const W3Smem L = w3_layout(p.apx, p.rb, p.BN, p.pk, p.PB, tries[t][0], tries[t][1],
+            const W3Smem L = w3_layout(p.apx, p.a_slots, p.rb, p.BN, p.pk, p.PB, tries[t][0], tries[t][1],
                                        tries[t][2], p.cout_pad);
             if (L.total + 1024 <= 227u * 1024u) {
                 p.as_slots = tries[t][0]; p.b_stages = tries[t][1]; p.bp_slots = tries[t][2];
@@ -1394,12 +1489,12 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     };
     int found = 0;
     const bool want_tr = hooks.window3 == 3 || hooks.window3 == 1;
-    if (want_tr) found = configure(1);
-    if (!found) found = configure(0);
+    if (want_tr) found = configure(1, 1) || configure(1, 0);
+    if (!found) found = configure(0, 0);
     if (!found) return DSQ_ERR_UNSUPPORTED;
     // (plain tiles convert accumulators by the 2^22 trick)
     if (!p.tr && (!small_acc || bits == 3)) epi_kind = DSQ_EPI_GENERAL;
-    p.L = w3_layout(p.apx, p.rb, p.BN, p.pk, p.PB, p.as_slots, p.b_stages, p.bp_slots, p.cout_pad);
+    p.L = w3_layout(p.apx, p.a_slots, p.rb, p.BN, p.pk, p.PB, p.as_slots, p.b_stages, p.bp_slots, p.cout_pad);
     p.smem_bytes = (int)p.L.total + 1024;
     // grid: a multiple of n_tiles; CTA c takes N tile c % n_tiles and every
     // mstep-th M tile
@@ -1409,7 +1504,7 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     if (p.mstep > p.m_tiles) p.mstep = p.m_tiles;
     if (p.mstep < 1) return DSQ_ERR_UNSUPPORTED;
     {
-        const int64_t d = (int64_t)p.mstep * (p.tr ? 256 : W3_BM), img = (int64_t)p.Hp * p.Wp;
+        const int64_t d = (int64_t)p.mstep * (p.f4 ? W3_F4_TP : p.tr ? 256 : W3_BM), img = (int64_t)p.Hp * p.Wp;
         p.t_dn = (int)(d / img);
         p.t_dh = (int)((d % img) / p.Wp);
         p.t_dw = (int)((d % img) % p.Wp);
@@ -1423,13 +1518,22 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
                 p.ld_dw[b * p.a_nload + i] = (int)((off % img) % p.Wp);
             }
     }
+    for (int i = 0; i < 4 * p.kpp; ++i) {
+        const int tap = p.tps * (i >> 2) + ((i & 3) * p.tps >> 2), within = 32 * (i & (4 / p.tps - 1));
+        (&p.x_off[i >> 2].x)[i & 3] =
+            tap < 9 && within < p.E
+                ? (uint32_t)((tap / 3 * p.tap_stride + tap % 3) * (p.rb >> 4) + (within >> 4))
+                : MMA_NONE;
+    }
     p.wait_ns = hooks.wait_ns;
     p.skip_b_round = hooks.skip_b_round;
     p.early = dsq_early_constants();
     p.e = e;
     p.r_hi = r_hi;
     p.out_pitch = (int)dsq_row_pitch(Cout, bits);
-    if (e.half_offset) {
+    if (p.f4) {
+        p.mark = (const uint32_t *)((const uint8_t *)w_packed + w3_mark_offset(w8));
+    } else if (e.half_offset) {
         p.shift = 7 - bits;
         p.orv = 0x01010101u << (7 - bits);
     } else {

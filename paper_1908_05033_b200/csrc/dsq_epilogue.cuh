@@ -284,8 +284,9 @@ __device__ __forceinline__ unsigned long long dsq_code_pair(uint32_t x, int j)
 
 // Raw accumulators of eight consecutive output channels of one position -> their
 // packed codes; sc, bi: the channels' dsq_codes_affine in pairs, res: the
-// position's residual codes of those channels (both in fields of SLOT bits).
-template <int BITS, bool RES, bool LO, int SLOT = BITS>
+// position's residual codes of those channels (both in fields of SLOT bits).  FACC: the
+// accumulators are whole numbers in binary32.
+template <int BITS, bool RES, bool LO, int SLOT = BITS, bool FACC = false>
 __device__ __forceinline__ uint32_t dsq_lean_codes8(const uint32_t (&v)[8],
                                                     const unsigned long long (&sc)[4],
                                                     const unsigned long long (&bi)[4],
@@ -295,7 +296,9 @@ __device__ __forceinline__ uint32_t dsq_lean_codes8(const uint32_t (&v)[8],
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
         unsigned long long y = dsq_fma2(
-            dsq_pack2(__int2float_rn((int)v[2 * c]), __int2float_rn((int)v[2 * c + 1])), sc[c], bi[c]);
+            FACC ? dsq_pack2(__uint_as_float(v[2 * c]), __uint_as_float(v[2 * c + 1]))
+                 : dsq_pack2(__int2float_rn((int)v[2 * c]), __int2float_rn((int)v[2 * c + 1])),
+            sc[c], bi[c]);
         if (RES) y = dsq_add2(y, dsq_fma2(dsq_code_pair<SLOT>(res, c), l.res_delta2, l.res_lo2));
         if (LO) y = dsq_add2(y, l.neg_lo2);
         dsq_requant2<BITS>(y, l.inv2, q[2 * c], q[2 * c + 1]);

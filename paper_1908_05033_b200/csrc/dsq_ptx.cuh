@@ -389,6 +389,9 @@ __device__ __forceinline__ void mma_i8_ts_x4(uint32_t d_tmem, uint32_t a_tmem, u
 }
 #undef DSQ_MMA_X4_BODY
 
+// an instruction to leave out of the blocks of four below
+constexpr uint32_t MMA_NONE = 0xFFFFFFFFu;
+
 // One tcgen05.mma kind::i8 with BOTH operands read through shared-memory
 // descriptors (given as their two 32-bit halves), issued by one elected lane
 // of a converged warp; all lanes call with warp-uniform arguments.
@@ -409,7 +412,7 @@ __device__ __forceinline__ void mma_i8_ss_elect(uint32_t d_tmem, uint32_t a_lo, 
 // Four such instructions in one block (one K step of 128 bytes): the B
 // descriptor advances 32 bytes (2 units of 16 bytes in its low word) per
 // instruction, the low words of the four A descriptors are given one by one
-// (0xFFFFFFFF = leave this instruction out); the first instruction takes the
+// (MMA_NONE: left out); the first instruction takes the
 // caller's accumulate flag, the others accumulate.  a_lo0 must be valid.
 __device__ __forceinline__ void mma_i8_ss_x4_elect(uint32_t d_tmem, uint32_t a_lo0, uint32_t a_lo1,
                                                    uint32_t a_lo2, uint32_t a_lo3, uint32_t a_hi,
@@ -440,7 +443,7 @@ __device__ __forceinline__ void mma_i8_ss_x4_elect(uint32_t d_tmem, uint32_t a_l
 
 // Same with the roles swapped: the A descriptor advances 32 bytes per
 // instruction, the four B descriptors' low words are given one by one
-// (0xFFFFFFFF = leave this instruction out).
+// (MMA_NONE: left out).
 __device__ __forceinline__ void mma_i8_ss_x4b_elect(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi,
                                                     uint32_t b_lo0, uint32_t b_lo1, uint32_t b_lo2,
                                                     uint32_t b_lo3, uint32_t b_hi, uint32_t idesc,
@@ -466,6 +469,39 @@ __device__ __forceinline__ void mma_i8_ss_x4b_elect(uint32_t d_tmem, uint32_t a_
         "r"(a_lo), "r"(a_hi), "r"(b_lo0), "r"(b_lo1), "r"(b_lo2), "r"(b_lo3), "r"(b_hi), "r"(idesc),
         "r"(accumulate_first)
         : "memory");
+}
+
+// The same for 4-bit floating-point operands (kind::mxf4: E2M1 values, two a byte, K = 64
+// = the same 32 bytes per instruction; f32 accumulate).  Every 32 values of a row share a
+// power-of-two scale read from tensor memory (sf_a, sf_b).
+__device__ __forceinline__ void mma_f4_ss_x4b_elect(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi,
+                                                    uint32_t b_lo0, uint32_t b_lo1, uint32_t b_lo2,
+                                                    uint32_t b_lo3, uint32_t b_hi, uint32_t idesc,
+                                                    uint32_t sf_a, uint32_t sf_b,
+                                                    uint32_t accumulate_first)
+{
+#define DSQ_MXF4 " tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], "
+    asm volatile(
+        "{\n\t.reg .pred p0, p1, pe, v1, v2, v3;\n\t"
+        ".reg .b64 da0, da1, da2, da3, db0, db1, db2, db3;\n\t.reg .b32 l1, l2, l3;\n\t"
+        "setp.ne.b32 p0, %9, 0;\n\tsetp.eq.b32 p1, %9, %9;\n\t"
+        "add.u32 l1, %1, 2;\n\tadd.u32 l2, %1, 4;\n\tadd.u32 l3, %1, 6;\n\t"
+        "mov.b64 da0, {%1, %2};\n\tmov.b64 da1, {l1, %2};\n\t"
+        "mov.b64 da2, {l2, %2};\n\tmov.b64 da3, {l3, %2};\n\t"
+        "mov.b64 db0, {%3, %7};\n\tmov.b64 db1, {%4, %7};\n\t"
+        "mov.b64 db2, {%5, %7};\n\tmov.b64 db3, {%6, %7};\n\t"
+        "elect.sync _|pe, 0xffffffff;\n\t"
+        "setp.ne.b32 v1, %4, 0xFFFFFFFF;\n\tsetp.ne.b32 v2, %5, 0xFFFFFFFF;\n\t"
+        "setp.ne.b32 v3, %6, 0xFFFFFFFF;\n\t"
+        "and.pred v1, v1, pe;\n\tand.pred v2, v2, pe;\n\tand.pred v3, v3, pe;\n\t"
+        "@pe" DSQ_MXF4 "da0, db0, %8, [%10], [%11], p0;\n\t"
+        "@v1" DSQ_MXF4 "da1, db1, %8, [%10], [%11], p1;\n\t"
+        "@v2" DSQ_MXF4 "da2, db2, %8, [%10], [%11], p1;\n\t"
+        "@v3" DSQ_MXF4 "da3, db3, %8, [%10], [%11], p1;\n\t}" ::"r"(d_tmem),
+        "r"(a_lo), "r"(a_hi), "r"(b_lo0), "r"(b_lo1), "r"(b_lo2), "r"(b_lo3), "r"(b_hi), "r"(idesc),
+        "r"(accumulate_first), "r"(sf_a), "r"(sf_b)
+        : "memory");
+#undef DSQ_MXF4
 }
 
 // One 128-byte K step of a CTA pair's tile with both operands in shared
@@ -657,6 +693,18 @@ __device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t smem_addr)
     return d;
 }
 
+// The same with the 32-byte swizzle: rows of 32 bytes, 8-row groups 256 bytes apart.
+__device__ __forceinline__ uint64_t smem_desc_sw32(uint32_t smem_addr)
+{
+    uint64_t d = 0;
+    d |= (uint64_t)((smem_addr >> 4) & 0x3FFF);
+    d |= (uint64_t)1 << 16;
+    d |= (uint64_t)(256 >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)6 << 61;                       // SWIZZLE_32B
+    return d;
+}
+
 // Instruction descriptor for kind::i8: s32 accumulator, K-major A and B.
 __host__ __device__ inline uint32_t idesc_i8(int n, bool a_signed, bool b_signed, int m = 128)
 {
@@ -666,6 +714,18 @@ __host__ __device__ inline uint32_t idesc_i8(int n, bool a_signed, bool b_signed
     d |= (b_signed ? 1u : 0u) << 10;           // B
     d |= (uint32_t)(n >> 3) << 17;             // N / 8
     d |= (uint32_t)(m >> 4) << 24;             // M / 16 (256: both CTAs of a pair)
+    return d;
+}
+
+// Instruction descriptor for kind::mxf4: E2M1 operands, UE8M0 scales, f32 accumulator.
+__host__ __device__ inline uint32_t idesc_mxf4(int n, int m = 128)
+{
+    uint32_t d = 0;
+    d |= 1u << 7;                              // A: E2M1
+    d |= 1u << 10;                             // B: E2M1
+    d |= (uint32_t)(n >> 3) << 17;             // N / 8
+    d |= 1u << 23;                             // scales: UE8M0
+    d |= (uint32_t)(m >> 4) << 24;             // M / 16
     return d;
 }
 

@@ -98,6 +98,19 @@ __device__ __forceinline__ uint32_t expand_word(uint32_t w, int c, uint32_t orv)
     }
 }
 
+// packed -> 4-bit floating point (E2M1, steps of 1/2 from 0 to 2), for 2-bit codes: two
+// words of eight values a word, the even codes (c = 0) and the odd ones (c = 1).  An
+// unsigned code q IS the pattern of q / 2; a signed one becomes (2 code + 1) / 2.  Products
+// are multiples of 1/4, which two block scales of 2 make whole numbers, and every partial
+// sum is a whole number below 2^24: the f32 accumulator holds the integer sum exactly.
+template <bool SIGNED>
+__device__ __forceinline__ uint32_t expand_word_f4(uint32_t w, int c)
+{
+    const uint32_t x = (c == 0 ? w : (w >> 2)) & 0x33333333u;
+    if (!SIGNED) return x;
+    return ((x & 0x22222222u) << 2) | (((x ^ (x >> 1)) & 0x11111111u) << 1) | 0x11111111u;
+}
+
 // Chunk q (16 codes) of a 3-bit row step held in w[12], both operands in the same order:
 // of every eight codes the even ones, then the odd ones (11 instructions for eight;
 // consecutive order took 17).

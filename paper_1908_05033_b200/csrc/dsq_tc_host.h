@@ -101,7 +101,10 @@ DSQ_HIDDEN int dsq_wgemm_small(const void *X, const void *W, int64_t M, int64_t 
 // order the window kernel consumes them (Cout rows of ksteps x 128 bytes).
 // The kernel then copies weight tiles by TMA straight into the swizzled operand
 // ring, with no expansion warps.  enabled = 0: this geometry has no such copy.
-struct DsqW8Info { int enabled; size_t offset; int ksteps; size_t bytes; };
+// f4: 2-bit rows of 64, 128 or k * 256 channels are kept as 4-bit floating-point
+// operands (expand_word_f4) instead, 256 codes to a K step of 128 bytes; they fill half
+// of the room.
+struct DsqW8Info { int enabled; size_t offset; int ksteps; size_t bytes; int f4; };
 DSQ_HIDDEN DsqW8Info dsq_w8_info(const dsq_conv_t *conv, int bits);
 // builds the expanded copy from the packed rows at the start of `blob`
 DSQ_HIDDEN int dsq_w8_build(void *blob, const dsq_conv_t *conv, int bits, cudaStream_t stream);
