@@ -88,7 +88,7 @@ constexpr int W3_MAX_WINDOW_PX = 416;
 constexpr int W3_MAX_LOADS = 3;        // im2col loads of a window
 // 4-bit floating-point operands (see F4 below)
 constexpr uint32_t W3_F4_MARK = 0x34463271u;   // behind the blob's copy of the weights
-constexpr int W3_F4_TP = 240;          // positions of a tile
+constexpr int W3_F4_TP = 240;          // positions of a tile, at most
 constexpr int W3_F4_SF = 2 * W3_F4_TP; // tensor-memory columns of the block scales: 480 .. 511
 
 // byte offsets of the kernel's shared-memory regions (w3_layout)
@@ -121,6 +121,7 @@ struct W3Params {
                                        // 0..63 and their epilogue warps take the other half of the columns
     int cout_pad;                      // Cout rounded up to the N tiling
     int tr;                            // transposed tiles (kernel form TR)
+    int tp;                            // positions of a tile: 128; TR: a multiple of 16 (w3_tile)
     int f4;                            // 4-bit floating-point operands (kernel form F4)
     int mstep;                         // M tiles between two tiles of a CTA
     int t_dn, t_dh, t_dw;              // the positions of mstep tiles as images, padded rows, columns
@@ -304,7 +305,8 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
 {
     constexpr int CH = Chunks<BITS>::CH;       // packed 16-byte chunks per 128 codes
     constexpr int OUT = Chunks<BITS>::OUT;     // int8 chunks per packed chunk
-    constexpr int TP = F4 ? W3_F4_TP : TR ? 256 : W3_BM;       // positions of a tile
+    constexpr int ACC = F4 ? W3_F4_TP : 256;   // TR: tensor-memory columns of an accumulator
+    const int TP = TR ? p.tp : W3_BM;          // positions of a tile
     static_assert(!F4 || (TR && BITS == 2), "F4: 2-bit codes, transposed tiles");
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     if ((threadIdx.x >> 5) == 1) W3_STAMP(13, 0);
@@ -573,8 +575,8 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
     } else if (warp == W3_WARP_MMA) {
         // ---------------- MMA issuer (whole warp, uniform; one lane issues) --------
         // (TR: A = 128 weight rows, signed; B = 256 window rows, unsigned)
-        const uint32_t idesc = F4   ? idesc_mxf4(W3_F4_TP)
-                               : TR ? idesc_i8(256, true, false, 128)
+        const uint32_t idesc = F4   ? idesc_mxf4(TP)
+                               : TR ? idesc_i8(TP, true, false, 128)
                                     : idesc_i8(BN, false, true, W3_BM);
         const uint64_t desc0 = smem_desc_sw128(0u);
         const uint32_t desc_hi = (uint32_t)(desc0 >> 32), desc_lo = (uint32_t)desc0;
@@ -593,7 +595,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
             if (!(ok = wait_bar_warp(bar_acc_empty(as), ((it >> 1) & 1) ^ 1u, ctl, 3))) break;
             W3_STAMP(4, it);
             tc_fence_after_sync();
-            const uint32_t d_tmem = tmem_base + as * (TR ? TP : BN);
+            const uint32_t d_tmem = tmem_base + as * (TR ? ACC : BN);
             uint32_t first = 0u;                    // 0: the tile's first instruction overwrites
 #pragma unroll 1
             for (int pl = 0; ok && pl < p.npl; ++pl) {
@@ -858,17 +860,19 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
         }
         if constexpr (TR) {
             // thread = output channel (tensor-memory lane), columns = positions;
-            // warp k of a quarter takes columns 64 k .. 64 k + 63 in units of 16
+            // warp k of a quarter takes a k-th part of the columns (up to 64) in units of 16
             constexpr int SB = BITS == 3 ? 4 : BITS;         // bits of a field
             constexpr int E = 32 / SB;                       // positions per code word
             constexpr int CWU = 16 / E;                      // code words per unit: 2 (1 at 2 bits)
             constexpr uint32_t MASK = (1u << SB) - 1u;
             const DsqEpi &e = p.e;
-            // (dup: lanes 64..127 repeat channels 0..63; quarters 2, 3 take columns 128..255)
+            // (dup: lanes 64..127 repeat channels 0..63; quarters 2, 3 take the second half
+            // of the columns)
             const int chq = p.dup ? (quarter & 1) * 32 : quarter * 32;
-            const int colbase = p.dup ? 128 * (quarter >> 1) + 32 * k : 64 * k;
-            // (F4: 15 units of columns, the last warp has one less)
-            const int units = (p.dup ? 2 : 4) - (F4 && k == 3 && (!p.dup || quarter >= 2));
+            const int half0 = p.dup ? (TP / 16 + 1) / 2 : TP / 16;   // units of 16 columns
+            const int all = p.dup && quarter >= 2 ? TP / 16 - half0 : half0;
+            const int each = (all + 3) / 4, unit0 = (p.dup && quarter >= 2 ? half0 : 0) + k * each;
+            const int units = max(0, min(each, all - k * each)), colbase = 16 * unit0;
             const int ch = n_tile * 128 + chq + lane;
             // a warp has work while its first code word lies inside the output row:
             // channels past Cout are padding lanes of the packed row and get zeros
@@ -894,7 +898,6 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
             uint32_t *y32 = reinterpret_cast<uint32_t *>(e.y_codes);
             // output pixel (or -1) of the warp's columns: lane L follows columns
             // colbase + 2 L and colbase + 2 L + 1; the others get them by shuffle
-            // (dup: a warp has 32 columns and only asks lanes 0..15)
             W3Pos pos0, pos1;
             {
                 const int g0 = m_first * TP + colbase + 2 * lane;
@@ -947,7 +950,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                 if (!(ok = wait_bar_warp(bar_acc_full(as), (it >> 1) & 1u, ctl, 8))) break;
                 if (warp == W3_WARP_E0) W3_STAMP(8, it);
                 tc_fence_after_sync();
-                const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + as * TP;
+                const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + as * ACC;
 #pragma unroll 1
                 for (int u = 0; warp_live && u < units; ++u) {
                     const int col0 = colbase + 16 * u;
@@ -1363,6 +1366,22 @@ int dsq_w8_build(void *blob, const dsq_conv_t *conv, int bits, cudaStream_t stre
                       kpp, tps * P, (uint32_t *)((uint8_t *)blob + w3_mark_offset(w)));
 }
 
+// Positions of a transposed tile, at most `most`: what fills as many passes of the `mstep`
+// CTAs of an N tile as the largest tile would take, so that the last pass is no emptier than
+// the others.  (4-bit, batch 64, largest / this: 28x28 128->128 11.6 / 10.8 us, 14x14 256->256
+// 11.3 / 10.5, 7x7 512->512 15.6 / 14.2; 2-bit 28x28 512->512 at batch 32 27.9 / 26.9.)  No
+// fewer than 112: the instructions get shorter, the weights' K steps do not (28x28 128->128 at
+// batch 16: 96 to 144 positions alike).  With more than four passes the last one weighs little, and
+// larger tiles have less overhead each (64->64 at 56x56, six passes: 256 positions 15.4, 240
+// 15.8).
+static int w3_tile(int64_t positions, int mstep, int most)
+{
+    const int64_t passes = (positions + (int64_t)most * mstep - 1) / ((int64_t)most * mstep);
+    if (passes > 4) return most;
+    const int64_t each = (positions + passes * mstep - 1) / (passes * mstep);
+    return (int)std::min<int64_t>(most, std::max<int64_t>(112, (each + 15) / 16 * 16));
+}
+
 int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
                      const void *w_packed, const dsq_conv_t *conv, const DsqEpi &e,
                      int epi_kind, int small_acc, void *workspace, cudaStream_t stream)
@@ -1387,6 +1406,8 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
         r_hi = fmaf(e.rq.hi - e.rq.lo, e.rq.inv, 0.5f);
         if (e.rq.lo != 0.0f || !dsq_lean_epilogue(e)) epi_kind = DSQ_EPI_GENERAL;
     }
+    const int sms = dsq_sm_count();
+    if (sms <= 0) return DSQ_ERR_CUDA;
     W3Params p = {};
     p.N = shape->N; p.H = shape->H; p.W = shape->W;
     p.Hp = p.H + 1; p.Wp = p.W + 1;
@@ -1422,10 +1443,12 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
         p.dup = tr && Cout <= 64;
         if (p.dup && !w8_ok && bits != 3) return 0;
         p.w8 = w8_ok && (Cout > 64 || p.dup);
-        const int tile_pos = f4 ? W3_F4_TP : tr ? 256 : W3_BM;
-        p.m_tiles = (int)((G + tile_pos - 1) / tile_pos);
         p.BN = tr ? 128 : (Cout >= 256 ? 256 : ((Cout + 63) / 64) * 64);
         p.n_tiles = (Cout + p.BN - 1) / p.BN;
+        p.mstep = std::max(sms / p.n_tiles, 1);
+        const int tile_pos = tr ? w3_tile(G, p.mstep, f4 ? W3_F4_TP : 256) : W3_BM;
+        p.tp = tile_pos;
+        p.m_tiles = (int)((G + tile_pos - 1) / tile_pos);
         p.cout_pad = p.n_tiles * p.BN;
         if (p.cout_pad > W3_MAX_COUT) return 0;
         const int need = tile_pos + 2 + 2 * p.Wp;
@@ -1498,13 +1521,10 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     p.smem_bytes = (int)p.L.total + 1024;
     // grid: a multiple of n_tiles; CTA c takes N tile c % n_tiles and every
     // mstep-th M tile
-    const int sms = dsq_sm_count();
-    if (sms <= 0) return DSQ_ERR_CUDA;
-    p.mstep = sms / p.n_tiles;
+    if (p.n_tiles > sms) return DSQ_ERR_UNSUPPORTED;
     if (p.mstep > p.m_tiles) p.mstep = p.m_tiles;
-    if (p.mstep < 1) return DSQ_ERR_UNSUPPORTED;
     {
-        const int64_t d = (int64_t)p.mstep * (p.f4 ? W3_F4_TP : p.tr ? 256 : W3_BM), img = (int64_t)p.Hp * p.Wp;
+        const int64_t d = (int64_t)p.mstep * p.tp, img = (int64_t)p.Hp * p.Wp;
         p.t_dn = (int)(d / img);
         p.t_dh = (int)((d % img) / p.Wp);
         p.t_dw = (int)((d % img) % p.Wp);

@@ -32,6 +32,15 @@ def test_shapes(dsq, geom):
     conv_case(dsq, *geom, 3, 1, 1, 2, 0.5, residual=geom[0] % 2 == 1, seed=sum(geom))
 
 
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("geom", [(149, 10, 10, 64, 64), (70, 12, 13, 128, 128), (37, 13, 12, 256, 256), (64, 7, 7, 512, 512),
+                                  (90, 14, 14, 128, 40)])
+def test_tiles_of_fewer_positions(dsq, geom, bits):
+    """One pass of 112 .. 240 positions a tile (columns of a tile that the warps of a
+    tensor-memory quarter share unevenly) and two passes."""
+    conv_case(dsq, *geom, 3, 1, 1, bits, 0.5, residual=geom[3] != 128, seed=sum(geom))
+
+
 @pytest.mark.parametrize("cin", [64, 128, 256, 1024])
 @pytest.mark.parametrize("sign", [1.0, -1.0])
 def test_largest_sums(dsq, cin, sign):
