@@ -85,7 +85,6 @@ constexpr int W3_MAX_BST = 10;         // expanded B stages (resident: all K ste
 constexpr int W3_BAND_PX = 136;        // pixels of a band (three-band staging)
 constexpr int W3_F4_BAND_PX = 248;
 constexpr int W3_MAX_WINDOW_PX = 416;
-constexpr int W3_MAX_LOADS = 3;        // im2col loads of a window
 // 4-bit floating-point operands (see F4 below)
 constexpr uint32_t W3_F4_MARK = 0x34463271u;   // behind the blob's copy of the weights
 constexpr int W3_F4_TP = 240;          // positions of a tile, at most
@@ -98,7 +97,9 @@ struct W3Smem {
 
 struct W3Params {
     // geometry
-    int N, H, W, Hp, Wp;               // Hp = H + 1, Wp = W + 1 (see W3Pos)
+    int N, H, W, Ho, Wo, Hp, Wp;       // input and output; Hp, Wp: positions of an image (see W3Pos)
+    int stride;
+    int sh, sw;                        // input rows and columns between two positions: 1 or 2
     int m_tiles, n_tiles, BN, Ncols;
     int E;                             // operand bytes per pixel: Cin (F4: Cin / 2)
     int npl, kpp, ksteps;              // planes of 128 (F4: 256) channels, K steps per plane, total
@@ -112,25 +113,23 @@ struct W3Params {
                                        // F4: 32, 64 or 128 for 64, 128 or more channels
     int xstep;                         // bytes between two K steps of a plane in a weight row
     int apx, a_slots;                  // pixels of an A slot, slots
+    // A window is nbands bands of band_px positions, each fetched by a_nload loads of a_box;
+    // band b starts band_pos[b] positions behind the tile's first and takes the input pixels
+    // of filter tap band_tap[b] (column | row << 8) of a filter whose corner is at (-2, -2)
     int a_box, a_nload, nbands, band_px;
-    int tap_stride;                    // slot rows between two filter rows
+    int band_pos[4], band_tap[4];
     int as_slots, bp_slots, b_stages, b_res;
     int w8;                            // weight K steps come expanded, by TMA, into the operand ring
-    int dup;                           // transposed tiles, <= 64 output channels: the 128 A rows hold the
-                                       // weight rows twice; lanes 64..127 of the accumulator repeat lanes
-                                       // 0..63 and their epilogue warps take the other half of the columns
+    int pair;                          // transposed tiles, <= 64 output channels: two image rows a position
     int cout_pad;                      // Cout rounded up to the N tiling
     int tr;                            // transposed tiles (kernel form TR)
     int tp;                            // positions of a tile: 128; TR: a multiple of 16 (w3_tile)
     int f4;                            // 4-bit floating-point operands (kernel form F4)
     int mstep;                         // M tiles between two tiles of a CTA
     int t_dn, t_dh, t_dw;              // the positions of mstep tiles as images, padded rows, columns
-    // start of every load of a fill, from the tile's start: images, padded rows
-    // (< Hp), padded columns (< Wp)
-    int ld_dn[W3_MAX_LOADS], ld_dh[W3_MAX_LOADS], ld_dw[W3_MAX_LOADS];
     int smem_bytes;
-    int early;                         // dsq_early_constants
     uint32_t zero;                     // 0 (see w3_release_slot)
+    int early;                         // dsq_early_constants
     unsigned long long wait_ns;
     int skip_b_round;
     // epilogue
@@ -144,7 +143,7 @@ struct W3Params {
     // window offsets (16-byte units) of the four instructions of every K step of a plane
     // (MMA_NONE: left out); in the parameters, so that the issuing warp keeps them, and what
     // it makes of them, in uniform registers
-    uint4 x_off[9];
+    uint4 x_off[12];
     W3Smem L;                          // shared-memory layout (host-made: w3_layout)
     int *ws;
 };
@@ -255,6 +254,14 @@ __device__ __forceinline__ void w3_release_slot(uint32_t bar, uint32_t seen, uin
     if (lane == 0 && !never) mbar_arrive(bar);
 }
 
+// word c of a packed word's operand words
+template <int BITS, bool SIGNED, bool F4>
+__device__ __forceinline__ uint32_t w3_operand(uint32_t w, int c, uint32_t orv)
+{
+    if constexpr (F4) return expand_word_f4<SIGNED>(w, c);
+    else return expand_word<BITS, SIGNED>(w, c, orv);
+}
+
 // Transposed tiles (template parameter TR).  An instruction whose A operand
 // comes through a shared-memory descriptor takes ~130 clocks whatever its N, so
 // it should carry N = 256.  With the roles swapped - A = 128 weight rows of the K
@@ -285,6 +292,21 @@ __device__ __forceinline__ uint32_t w3_transpose_fields(uint32_t x, int lane)
 }
 
 //
+// Pairs of image rows (p.pair).  With up to 64 output channels half of the 128 A rows
+// would be idle.  The lower 64 rows then are the same channels of the NEXT image row: a
+// position stands for two output rows, the four input rows under them lie in two bands of
+// the window (rows -1, 1, .. and 0, 2, .., fetched by im2col loads that step over every other row), and of twelve
+// taps (four rows) the upper 64 weight rows have the first nine, the lower ones the last
+// nine, zeros elsewhere.  12 taps for two output rows instead of 18, and every input row
+// is expanded 1.0 + 1/tile times instead of once per tile of its neighbours' too.
+// 64->64, one row a position / pairs: 224x224 2-bit, batch 32 60 / 45 us, 56x56 4-bit, batch 64 15.3 / 12.2,
+// 3-bit 18.3 / 17.3.
+//
+// Stride 2: positions are output pixels; the window is four bands (even and odd rows and
+// columns of the image), and a tap is a band and a shift in it.  Batch 64, im2col kernel /
+// this, us: 56x56 64->128 4-bit 12.7 / 10.5, 3-bit 36 / 13, 2-bit 12.2 / 8.2; 28x28 128->256
+// 11.9 / 10.3, 21.8 / 12.7, 11.2 / 8.6; 14x14 256->512 10.8 / 12.2, 22 / 14.2, 10.1 / 10.0.
+//
 // F4: 2-bit codes (weight grid Delta (c + 1/2)) as 4-bit floating-point operands.  E2M1
 // holds the codes 0 .. 3 and the weights 2 c + 1 exactly, and every partial sum is a whole
 // number far below 2^24, so the f32 accumulators hold the int32 sums bit for bit
@@ -298,13 +320,17 @@ __device__ __forceinline__ uint32_t w3_transpose_fields(uint32_t x, int lane)
 // 256->256 at 56x56 41.3 -> 25.6, 512->512 at 28x28 38.9 -> 27.6 (four passes of 240
 // positions for three of 256), at 14x14 16.3 -> 11.0.  What bounds it now: shared-memory
 // bandwidth (an instruction reads 11.5 KB in 120 clocks) and, with 64 channels, the epilogue.
-template <int BITS, int EPI, bool TR, bool F4 = false>
+//
+// PAIR3: pairs of image rows at 3 bits, whose weights' expansion masks the taps outside the
+// filter (in the common form the masks cost the wide layers 6 %: these instructions bound
+// them).
+template <int BITS, int EPI, bool TR, bool F4 = false, bool PAIR3 = false>
 __global__ void __launch_bounds__(W3_THREADS, 1)
 dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                 const __grid_constant__ CUtensorMap tmap_a, const W3Params p)
 {
-    constexpr int CH = Chunks<BITS>::CH;       // packed 16-byte chunks per 128 codes
-    constexpr int OUT = Chunks<BITS>::OUT;     // int8 chunks per packed chunk
+    constexpr int CH = F4 ? 4 : Chunks<BITS>::CH;      // packed 16-byte chunks per 128 operand bytes
+    constexpr int OUT = F4 ? 2 : Chunks<BITS>::OUT;    // operand chunks per packed chunk
     constexpr int ACC = F4 ? W3_F4_TP : 256;   // TR: tensor-memory columns of an accumulator
     const int TP = TR ? p.tp : W3_BM;          // positions of a tile
     static_assert(!F4 || (TR && BITS == 2), "F4: 2-bit codes, transposed tiles");
@@ -399,16 +425,19 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
         const int q = threadIdx.x - 64;
         reinterpret_cast<float *>(smem + L.lut)[q] = __fmaf_rn((float)q, p.e.res_delta, p.e.res_lo);
     }
-    // the window producer's first position (two divisions on one lane), worked out
+    // the window producer's first positions, a lane per load (two divisions), worked out
     // here, where the warp would otherwise only wait for the slower warps at the
     // barrier: it is on the critical path of a launch
-    W3Pos a_base0 = {0, 0, 0};
-    if (warp == W3_WARP_TMA_A && lane == 0) {
-        const int g0 = m_first * TP;
-        a_base0.n = g0 / img_positions;
-        const int rem = g0 - a_base0.n * img_positions;
-        a_base0.h = rem / p.Wp;
-        a_base0.w = rem - a_base0.h * p.Wp;
+    W3Pos ld_pos = {0, 0, 0};
+    int ld_tap = 0;
+    if (warp == W3_WARP_TMA_A && lane < p.nbands * p.a_nload) {
+        const int band = lane / p.a_nload;
+        const int g0 = m_first * TP + p.band_pos[band] + (lane - band * p.a_nload) * p.a_box;
+        ld_tap = p.band_tap[band];
+        ld_pos.n = g0 / img_positions;
+        const int rem = g0 - ld_pos.n * img_positions;
+        ld_pos.h = rem / p.Wp;
+        ld_pos.w = rem - ld_pos.h * p.Wp;
     }
     if (warp == W3_WARP_MMA) W3_STAMP(13, 7);
     if (warp == W3_WARP_E0) W3_STAMP(13, 8);
@@ -435,7 +464,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
             uint32_t issued = 0, ph = 0;
             const int BST = p.b_stages;
             const int y = n_tile * BN;
-            int s = 0, x = 0;
+            int s = 0, x = 0, kk = 0, pl = 0;
             bool ok = true;
             // (a blob packed by a library that kept its copy in another form)
             if (F4 && n_b_fills > 0 && __ldg(p.mark) != W3_F4_MARK) {
@@ -449,11 +478,19 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                 if (!wait_bar(bar_b_empty(s), ph ^ 1u, ctl, 1)) break;
                 if ((int)g == p.skip_b_round) break;
                 mbar_arrive_expect_tx(bar_b_full(s), b_stage_bytes);
-                tma_load_2d(smem_u32(smem + L.b_tiles + s * b_stage_bytes), &tmap_b, x, y,
-                            bar_b_full(s));
-                if (p.dup)     // the map's box is 64 rows: the same rows again behind them
-                    tma_load_2d(smem_u32(smem + L.b_tiles + s * b_stage_bytes + 64 * 128), &tmap_b,
-                                x, y, bar_b_full(s));
+                const uint32_t dst = smem_u32(smem + L.b_tiles + s * b_stage_bytes);
+                if (p.pair) {
+                    // a K step's taps for the upper 64 rows, those a filter row before them for
+                    // the lower ones; zeros before a plane's first and behind its last tap
+                    tma_load_3d(dst, &tmap_b, 128 * kk, pl, 0, bar_b_full(s));
+                    tma_load_3d(dst + 64 * 128, &tmap_b, 128 * kk - 3 * p.rb, pl, 0, bar_b_full(s));
+                    if (++kk == p.kpp) {
+                        kk = 0;
+                        if (++pl == p.npl) pl = 0;
+                    }
+                } else {
+                    tma_load_2d(dst, &tmap_b, x, y, bar_b_full(s));
+                }
                 ++issued;
                 x += 128;
                 if (x == p.ksteps * 128) x = 0;
@@ -474,15 +511,17 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                 if (!wait_bar(bar_bp_empty(s), ph ^ 1u, ctl, 1)) break;
                 if ((int)g == p.skip_b_round) break;
                 mbar_arrive_expect_tx(bar_bp_full(s), b_packed_bytes);
-                tma_load_2d(smem_u32(smem + L.b_packed + s * b_packed_bytes), &tmap_b, xk + xpl, y,
-                            bar_bp_full(s));
+                const uint32_t dst = smem_u32(smem + L.b_packed + s * b_packed_bytes);
+                tma_load_2d(dst, &tmap_b, xk + xpl, y, bar_bp_full(s));
+                if (p.pair)
+                    tma_load_2d(dst + 64 * p.pk, &tmap_b, xk + xpl - 3 * p.P, y, bar_bp_full(s));
                 ++issued;
                 W3_STAMP(12, g);
                 xk += xstep;
                 if (++kk == p.kpp) {
                     kk = 0; xk = 0;
-                    xpl += 16 * BITS;
-                    if (xpl == p.npl * 16 * BITS) xpl = 0;
+                    xpl += p.pk;
+                    if (xpl == p.npl * p.pk) xpl = 0;
                 }
                 if (++s == BP) { s = 0; ph ^= 1u; }
             }
@@ -491,87 +530,59 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
         }
     } else if (warp == W3_WARP_TMA_A) {
         // ---------------- producer: packed window of a tile and plane ------------
-        if (lane != 0) grid_dependency_wait();
-        if (lane == 0) {
-            uint32_t issued = 0, ph = 0;
-            const int AS = p.as_slots;
-            const int nld = p.nbands * p.a_nload;
-            int s = 0, pl = 0;
-            // The start coordinates of a fill's loads are worked out one fill ahead
-            // (the first before anything can be issued), so that between the
-            // moment a slot is free and the copies only the issue itself remains.
-            // Loads that start behind the last image are left out (and not counted); the
-            // zeros below that image, if they begin there, are written here.  An im2col load must
-            // start inside the map's bounding box (0 <= h < Hp, 0 <= w < Wp, n >= 0,
-            // which the position arithmetic guarantees): a position outside it is
-            // never issued - the roles then run into their wait limit and the
-            // kernel reports the failure.
-            W3Pos base = a_base0;
-            W3Pos q[W3_MAX_LOADS];
-            int nl = 0;
-            bool bad = false;
-            auto prepare = [&]() {
-                nl = 0;
-                bad = false;
-#pragma unroll
-                for (int i = 0; i < W3_MAX_LOADS; ++i) {
-                    if (i >= nld) break;
-                    q[i] = w3_add(base, p.ld_dn[i], p.ld_dh[i], p.ld_dw[i], p.Hp, p.Wp);
-                    if (q[i].n < p.N) {
-                        ++nl;
-                        bad |= q[i].n < 0 || q[i].h < 0 || q[i].h >= p.Hp || q[i].w < 0 || q[i].w >= p.Wp;
-                    }
-                }
-            };
-            prepare();
-            grid_dependency_wait();
+        // Lane i issues load i of a fill.  Loads that start behind the last image are left
+        // out (and not counted); the zeros below that image, if they begin there, are
+        // written here.  An im2col load must start inside the map's bounding box
+        // (0 <= h < Hp, 0 <= w < Wp, n >= 0, which the position arithmetic guarantees): a
+        // position outside it is never issued - the roles then run into their wait limit
+        // and the kernel reports the failure.
+        uint32_t issued = 0, ph = 0;
+        const int AS = p.as_slots;
+        const bool mine = lane < p.nbands * p.a_nload;
+        const uint32_t box_bytes = (uint32_t)(p.a_box * p.PB);
+        int s = 0, pl = 0;
+        grid_dependency_wait();
 #pragma unroll 1
-            for (uint32_t g = 0; g < n_a_fills; ++g) {
-                if (!wait_bar(bar_as_empty(s), ph ^ 1u, ctl, 11)) break;
-                if (bad) {
+        for (uint32_t g = 0; g < n_a_fills; ++g) {
+            if (!wait_bar_warp(bar_as_empty(s), ph ^ 1u, ctl, 11)) break;
+            const W3Pos q = ld_pos;
+            const bool live = mine && q.n < p.N;
+            if (__any_sync(0xffffffffu, live && (q.n < 0 || q.h < 0 || q.h >= p.Hp || q.w < 0 || q.w >= p.Wp))) {
+                if (lane == 0) {
                     if (atomicCAS(p.ws + DSQ_WS_STATUS, 0, (int)DSQ_ERR_SHAPE) == 0)
                         p.ws[DSQ_WS_DETAIL] = 16;
                     *ctl.abort_flag = 1;
-                    break;
                 }
-                if (nl < nld) {
-                    // positions p.N * Hp * Wp .. + Wp of a load that is left out
-#pragma unroll
-                    for (int i = 0; i < W3_MAX_LOADS; ++i) {
-                        if (i >= nld) break;
-                        const int behind = (q[i].n - p.N) * img_positions + q[i].h * p.Wp + q[i].w;
-                        if (q[i].n < p.N || behind > p.Wp) continue;
-                        const uint32_t z = smem_u32(smem + L.a_stage) + s * a_stage_bytes +
-                                           (uint32_t)(i * p.a_box * p.PB);
-                        const int bytes = min(p.a_box, p.Wp + 1 - behind) * p.PB;
-                        for (int k = 0; k < bytes; k += 16) sts_128(z + k, 0u, 0u, 0u, 0u);
-                    }
+                break;
+            }
+            const uint32_t dst = smem_u32(smem + L.a_stage) + s * a_stage_bytes + lane * box_bytes;
+            if (mine && !live) {
+                // positions p.N * Hp * Wp .. + Wp of a load that is left out
+                const int behind = (q.n - p.N) * img_positions + q.h * p.Wp + q.w;
+                if (behind <= p.Wp) {
+                    const int bytes = min(p.a_box, p.Wp + 1 - behind) * p.PB;
+                    for (int k = 0; k < bytes; k += 16) sts_128(dst + k, 0u, 0u, 0u, 0u);
                     fence_proxy_async_smem();
                 }
-                mbar_arrive_expect_tx(bar_as_full(s), (uint32_t)(nl * p.a_box * p.PB));
-                const uint32_t dst0 = smem_u32(smem + L.a_stage) + s * a_stage_bytes;
-#pragma unroll
-                for (int i = 0; i < W3_MAX_LOADS; ++i) {
-                    if (i >= nld) break;
-                    if (q[i].n >= p.N) continue;
-                    // bounding box = image grown by one pixel at the left and the top:
-                    // base positions -2 .. W-2 / -2 .. H-2, filter offset (1, 1)
-                    tma_load_im2col_4d(dst0 + (uint32_t)(i * p.a_box * p.PB), &tmap_a, pl * p.PB,
-                                       q[i].w - 2, q[i].h - 2, q[i].n, (uint16_t)1, (uint16_t)1,
-                                       bar_as_full(s));
-                }
-                ++issued;
-                W3_STAMP(0, g);
-                if (++pl == p.npl) {
-                    pl = 0;
-                    base = w3_add(base, p.t_dn, p.t_dh, p.t_dw, p.Hp, p.Wp);
-                    prepare();
-                }
-                if (++s == AS) { s = 0; ph ^= 1u; }
             }
+            const uint32_t bytes = (uint32_t)__popc(__ballot_sync(0xffffffffu, live)) * box_bytes;
+            if (lane == 0) mbar_arrive_expect_tx(bar_as_full(s), bytes);
+            __syncwarp();
+            if (live)
+                tma_load_im2col_4d(dst, &tmap_a, pl * p.PB, q.w * p.sw - 2, q.h * p.sh - 2, q.n,
+                                   (uint16_t)(ld_tap & 255), (uint16_t)(ld_tap >> 8), bar_as_full(s));
+            ++issued;
+            W3_STAMP(0, g);
+            if (++pl == p.npl) {
+                pl = 0;
+                ld_pos = w3_add(ld_pos, p.t_dn, p.t_dh, p.t_dw, p.Hp, p.Wp);
+            }
+            if (++s == AS) { s = 0; ph ^= 1u; }
+        }
+        if (lane == 0)
             for (uint32_t k = (issued > (uint32_t)AS ? issued - AS : 0); k < issued; ++k)
                 wait_bar_drain(bar_as_full(k % AS), (k / AS) & 1u);
-        }
+        __syncwarp();
     } else if (warp == W3_WARP_MMA) {
         // ---------------- MMA issuer (whole warp, uniform; one lane issues) --------
         // (TR: A = 128 weight rows, signed; B = 256 window rows, unsigned)
@@ -695,18 +706,11 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                 // 32-byte rows bit 7)
                 const uint32_t row = dst + (uint32_t)(px * p.rb);
                 const int sw = p.rb == 64 ? (px >> 1) & 3 : F4 && p.rb == 32 ? (px >> 2) & 1 : px & 7;
-                if constexpr (F4) {
-#pragma unroll
-                    for (int c = 0; c < 2; ++c)
-                        sts_128(row + (uint32_t)(((ch * 2 + c) ^ sw) << 4),
-                                expand_word_f4<false>(v.x, c), expand_word_f4<false>(v.y, c),
-                                expand_word_f4<false>(v.z, c), expand_word_f4<false>(v.w, c));
-                } else
 #pragma unroll
                 for (int c = 0; c < OUT; ++c)
                     sts_128(row + (uint32_t)(((ch * OUT + c) ^ sw) << 4),
-                            expand_word<BITS, false>(v.x, c, 0u), expand_word<BITS, false>(v.y, c, 0u),
-                            expand_word<BITS, false>(v.z, c, 0u), expand_word<BITS, false>(v.w, c, 0u));
+                            w3_operand<BITS, false, F4>(v.x, c, 0u), w3_operand<BITS, false, F4>(v.y, c, 0u),
+                            w3_operand<BITS, false, F4>(v.z, c, 0u), w3_operand<BITS, false, F4>(v.w, c, 0u));
             }
             fence_proxy_async_smem();
             __syncwarp();
@@ -733,7 +737,8 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
         // own fills: g = group, group + 2, ...
         int sp = group % BP, st = p.b_res ? group : group % BST;
         uint32_t php = (uint32_t)(group / BP) & 1u, phu = p.b_res ? 0u : (uint32_t)(group / BST) & 1u;
-        bool ok = !F4 && !p.w8;                    // (w8: nothing to expand)
+        int kk = group;                            // PAIR3: K step within its plane
+        bool ok = !p.w8;                           // (w8: nothing to expand)
 #pragma unroll 1
         for (uint32_t g = group; ok && g < n_b_fills; g += 2) {
             if (!(ok = wait_bar_warp(bar_bp_full(sp), php, ctl, 6))) break;
@@ -744,9 +749,11 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
             bool waited = p.b_res != 0;
             if (BITS == 3 && TR) {
                 // one thread per operand row: 48 packed bytes of a tap and plane, or the
-                // 24 bytes of each of two taps (rows 64 .. 127 repeat 0 .. 63: dup)
+                // 24 bytes of each of two taps.  pair: rows 64 .. 127 are the taps a filter row
+                // before; outside the filter the packed bytes are zeros (TMA), and so are
+                // the operand's
                 const int row = tid;
-                const uint32_t r4 = src + (uint32_t)((p.dup ? row & 63 : row) * p.pk);
+                const uint32_t r4 = src + (uint32_t)(row * p.pk);
                 uint32_t w[12], w1[12];
 #pragma unroll
                 for (int l = 0; l < 3; ++l) {
@@ -765,11 +772,19 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                 if (!waited && !(ok = wait_bar_warp(bar_b_empty(st), phu ^ 1u, ctl, 7))) break;
                 uint8_t *rp = smem + L.b_tiles + st * b_stage_bytes + row * 128;
                 const int sw3 = row & 7;
+                uint32_t orv0 = p.orv, orv1 = p.orv;
+                if (PAIR3) {
+                    const int tap = kk * p.tps - (row >= 64 ? 3 : 0);
+                    if ((unsigned)tap >= 9u) orv0 = 0u;
+                    if ((unsigned)(tap + 1) >= 9u) orv1 = 0u;
+                    kk += 2;
+                    while (kk >= p.kpp) kk -= p.kpp;
+                }
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                     uint4 c;
-                    if (q >= 4 && p.tps == 2) c = expand3_chunk<true>(w1, q & 3, p.orv);
-                    else c = expand3_chunk<true>(w, q, p.orv);
+                    if (q >= 4 && p.tps == 2) c = expand3_chunk<true>(w1, q & 3, orv1);
+                    else c = expand3_chunk<true>(w, q, orv0);
                     *reinterpret_cast<uint4 *>(rp + ((q ^ sw3) << 4)) = c;
                 }
             } else if (BITS == 3) {
@@ -823,10 +838,10 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                         for (int c = 0; c < OUT; ++c)
                             *reinterpret_cast<uint4 *>(rowp + (r0 + i * ROWS_PER_IT) * 128 +
                                                        (((j * OUT + c) ^ sw) << 4)) =
-                                make_uint4(expand_word<BITS, true>(v[i].x, c, p.orv),
-                                           expand_word<BITS, true>(v[i].y, c, p.orv),
-                                           expand_word<BITS, true>(v[i].z, c, p.orv),
-                                           expand_word<BITS, true>(v[i].w, c, p.orv));
+                                make_uint4(w3_operand<BITS, true, F4>(v[i].x, c, p.orv),
+                                           w3_operand<BITS, true, F4>(v[i].y, c, p.orv),
+                                           w3_operand<BITS, true, F4>(v[i].z, c, p.orv),
+                                           w3_operand<BITS, true, F4>(v[i].w, c, p.orv));
                     }
             }
             if (!ok) break;
@@ -866,13 +881,11 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
             constexpr int CWU = 16 / E;                      // code words per unit: 2 (1 at 2 bits)
             constexpr uint32_t MASK = (1u << SB) - 1u;
             const DsqEpi &e = p.e;
-            // (dup: lanes 64..127 repeat channels 0..63; quarters 2, 3 take the second half
-            // of the columns)
-            const int chq = p.dup ? (quarter & 1) * 32 : quarter * 32;
-            const int half0 = p.dup ? (TP / 16 + 1) / 2 : TP / 16;   // units of 16 columns
-            const int all = p.dup && quarter >= 2 ? TP / 16 - half0 : half0;
-            const int each = (all + 3) / 4, unit0 = (p.dup && quarter >= 2 ? half0 : 0) + k * each;
-            const int units = max(0, min(each, all - k * each)), colbase = 16 * unit0;
+            // (pair: lanes 64..127 are channels 0..63 of the second of two image rows)
+            const int chq = p.pair ? (quarter & 1) * 32 : quarter * 32;
+            const int row1 = p.pair ? quarter >> 1 : 0;
+            const int each = (TP / 16 + 3) / 4;              // units of 16 columns a warp
+            const int units = max(0, min(each, TP / 16 - k * each)), colbase = 16 * k * each;
             const int ch = n_tile * 128 + chq + lane;
             // a warp has work while its first code word lies inside the output row:
             // channels past Cout are padding lanes of the packed row and get zeros
@@ -911,10 +924,11 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
 #pragma unroll 1
             for (int it = 0; ok && it < my_tiles; ++it) {
                 const int as = it & 1;
-                const int m0 = (pos0.n < p.N && pos0.h < p.H && pos0.w < p.W)
-                                   ? (pos0.n * p.H + pos0.h) * p.W + pos0.w : -1;
-                const int m1 = (pos1.n < p.N && pos1.h < p.H && pos1.w < p.W)
-                                   ? (pos1.n * p.H + pos1.h) * p.W + pos1.w : -1;
+                const int h0 = p.pair ? 2 * pos0.h + row1 : pos0.h, h1 = p.pair ? 2 * pos1.h + row1 : pos1.h;
+                const int m0 = (pos0.n < p.N && h0 < p.Ho && pos0.w < p.Wo)
+                                   ? (pos0.n * p.Ho + h0) * p.Wo + pos0.w : -1;
+                const int m1 = (pos1.n < p.N && h1 < p.Ho && pos1.w < p.Wo)
+                                   ? (pos1.n * p.Ho + h1) * p.Wo + pos1.w : -1;
                 pos0 = w3_add(pos0, p.t_dn, p.t_dh, p.t_dw, p.Hp, p.Wp);
                 pos1 = w3_add(pos1, p.t_dn, p.t_dh, p.t_dw, p.Hp, p.Wp);
                 // Word w of a unit covers E positions; lane i of a channel group owns
@@ -1002,9 +1016,9 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                                 if (e.general_offset) {
                                     // S_a of the position (recomputed by every channel's
                                     // thread: this form is not a fast path)
-                                    const int wo = mj % p.W, t2 = mj / p.W;
-                                    const int s_a = dsq_window_sa<BITS>(p.act, t2 / p.H, t2 % p.H, wo,
-                                                                        p.H, p.W, 3, 1, 1, p.P);
+                                    const int wo = mj % p.Wo, t2 = mj / p.Wo;
+                                    const int s_a = dsq_window_sa<BITS>(p.act, t2 / p.Ho, t2 % p.Ho, wo,
+                                                                        p.H, p.W, 3, p.stride, 1, p.P);
                                     y = dsq_epi_y_offset(vi, s_a, e.w_offset, sc, bi);
                                 } else {
                                     y = dsq_epi_y(vi, sc, bi);
@@ -1039,7 +1053,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                                 uint32_t *row = y32 + (int64_t)mp[w] * pw;
                                 if (grp < 3) {
                                     if (mp[w] >= 0 && wi < pw) row[wi] = word;
-                                } else if (p.dup && mp[w] >= 0 && wi == 6) {
+                                } else if (p.pair && mp[w] >= 0 && wi == 6) {
                                     for (int i = wi; i < pw; ++i) row[i] = 0u;
                                 }
                             } else if (mp[w] >= 0 && 4 * cg < p.out_pitch) y32[(int64_t)mp[w] * pw + cg] = word;
@@ -1215,7 +1229,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
     }
 }
 
-template <int BITS, int EPI, bool TR = false, bool F4 = false>
+template <int BITS, int EPI, bool TR = false, bool F4 = false, bool PAIR3 = false>
 int w3_launch(const CUtensorMap &tb, const CUtensorMap &ta, const W3Params &p, cudaStream_t s,
               int pdl)
 {
@@ -1224,14 +1238,14 @@ int w3_launch(const CUtensorMap &tb, const CUtensorMap &ta, const W3Params &p, c
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return DSQ_ERR_CUDA;
     const unsigned long long dev_bit = dev < 64 ? 1ull << dev : 0ull;
     if (!(configured.load(std::memory_order_acquire) & dev_bit)) {
-        if (cudaFuncSetAttribute(dsq_win3_kernel<BITS, EPI, TR, F4>,
+        if (cudaFuncSetAttribute(dsq_win3_kernel<BITS, EPI, TR, F4, PAIR3>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  227 * 1024) != cudaSuccess)
             return DSQ_ERR_CUDA;
         configured.fetch_or(dev_bit, std::memory_order_release);
     }
     const int grid = p.mstep * p.n_tiles;
-    return dsq_launch(dsq_win3_kernel<BITS, EPI, TR, F4>, dim3(grid), dim3(W3_THREADS),
+    return dsq_launch(dsq_win3_kernel<BITS, EPI, TR, F4, PAIR3>, dim3(grid), dim3(W3_THREADS),
                       (size_t)p.smem_bytes, s, pdl, 0, tb, ta, p);
 }
 
@@ -1245,6 +1259,14 @@ int w3_dispatch(int epi, const CUtensorMap &tb, const CUtensorMap &ta, const W3P
             case DSQ_EPI_CODES: return w3_launch<BITS, DSQ_EPI_CODES, true, true>(tb, ta, p, s, pdl);
             case DSQ_EPI_CODES_RES: return w3_launch<BITS, DSQ_EPI_CODES_RES, true, true>(tb, ta, p, s, pdl);
             default: return w3_launch<BITS, DSQ_EPI_GENERAL, true, true>(tb, ta, p, s, pdl);
+            }
+        }
+    if constexpr (BITS == 3)
+        if (p.tr && p.pair) {
+            switch (epi) {
+            case DSQ_EPI_CODES: return w3_launch<BITS, DSQ_EPI_CODES, true, false, true>(tb, ta, p, s, pdl);
+            case DSQ_EPI_CODES_RES: return w3_launch<BITS, DSQ_EPI_CODES_RES, true, false, true>(tb, ta, p, s, pdl);
+            default: return w3_launch<BITS, DSQ_EPI_GENERAL, true, false, true>(tb, ta, p, s, pdl);
             }
         }
     if (p.tr) {
@@ -1382,24 +1404,79 @@ static int w3_tile(int64_t positions, int mstep, int most)
     return (int)std::min<int64_t>(most, std::max<int64_t>(112, (each + 15) / 16 * 16));
 }
 
+// Positions of the numbering up to the last pixel, channel tiles, CTAs a channel tile.
+struct W3Work {
+    int64_t positions;
+    int Hp, Wp, n_tiles, mstep;
+};
+static W3Work w3_work(const dsq_nhwc_t *shape, const dsq_conv_t *conv, int pair, int bn, int sms)
+{
+    W3Work w;
+    const int Ho = (shape->H - 1) / conv->stride + 1, Wo = (shape->W - 1) / conv->stride + 1;
+    const bool two = pair || conv->stride == 2;
+    w.Hp = two ? shape->H / 2 + 1 : shape->H + 1;
+    w.Wp = conv->stride == 2 ? shape->W / 2 + 1 : shape->W + 1;
+    w.positions = ((int64_t)shape->N - 1) * w.Hp * w.Wp + (int64_t)((Ho - 1) / (pair ? 2 : 1)) * w.Wp + Wo;
+    w.n_tiles = (conv->Cout + bn - 1) / bn;
+    w.mstep = std::max(sms / w.n_tiles, 1);
+    return w;
+}
+
+static bool w3_takes_f4(const dsq_conv_t *conv, int bits, int half_offset)
+{
+    return bits == 2 && half_offset && (conv->Cin <= 128 || conv->Cin % 256 == 0);
+}
+
+// 4-bit operands at stride 2, where the blob has no expanded weights: the im2col kernel is
+// the faster one unless a CTA expands its weights once - they stay resident, or one pass
+// of large tiles does (28x28 128->256 at batch 64 10.3 us against 11.9, at batch 16, tiles of 112, 7.7
+// against 7.5; 112x112 128->128 18.8 against 17.3; 14x14 256->512 12.2 against 10.8).
+static bool w3_takes_stride2(int Cin, int tile, int64_t passes)
+{
+    return Cin == 64 || (Cin == 128 && passes == 1 && tile >= 160);
+}
+
+// Microseconds the window kernel takes for a layer of few tiles, or a negative number
+// where it does not take it: start-up and the last epilogue, and for every pass of the
+// CTAs its K steps.  Fitted to 666 layers of 64 to 512 channels at batches of 1 to 32: 5 % off
+// in the mean, 17 % at most.
+double dsq_conv3_estimate(const dsq_nhwc_t *shape, int bits, const dsq_conv_t *conv, int half_offset)
+{
+    const int Cin = conv->Cin, sms = dsq_sm_count() > 0 ? dsq_sm_count() : 148;
+    if (conv->KH != 3 || conv->pad != 1 || !(Cin == 64 || (Cin % 128 == 0 && Cin <= 1024))) return -1.0;
+    const int f4 = w3_takes_f4(conv, bits, half_offset), pair = conv->stride == 1 && conv->Cout <= 64;
+    int npl, kpp, tps;
+    w3_steps(Cin, f4, &npl, &kpp, &tps);
+    if (pair) kpp = (12 + tps - 1) / tps;
+    const W3Work w = w3_work(shape, conv, pair, 128, sms);
+    const int tile = w3_tile(w.positions, w.mstep, f4 ? W3_F4_TP : 256);
+    const int64_t passes = (w.positions + (int64_t)tile * w.mstep - 1) / ((int64_t)tile * w.mstep);
+    const double steps = (double)passes * npl * kpp, t = tile / 256.0;
+    if (conv->stride == 1)
+        return f4 ? 3.7 + steps * (1.41 * t - 0.36) : bits == 3 ? 4.5 + steps * (t - 0.07) : 3.8 + steps * (0.754 * t - 0.076);
+    if (bits != 3 && !f4 && !w3_takes_stride2(Cin, tile, passes)) return -1.0;
+    return f4 ? 3.4 + steps * (2.24 * t - 0.49) : bits == 3 ? 4.8 + steps * (1.59 * t - 0.27) : 3.6 + steps * (1.39 * t - 0.215);
+}
+
 int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
                      const void *w_packed, const dsq_conv_t *conv, const DsqEpi &e,
                      int epi_kind, int small_acc, void *workspace, cudaStream_t stream)
 {
     const DsqLaunchHooks hooks = dsq_launch_hooks();
     if (!hooks.window3) return DSQ_ERR_UNSUPPORTED;
-    if (conv->KH != 3 || conv->KW != 3 || conv->stride != 1 || conv->pad != 1)
+    const int stride = conv->stride;
+    if (conv->KH != 3 || conv->KW != 3 || conv->pad != 1 || (stride != 1 && stride != 2))
         return DSQ_ERR_UNSUPPORTED;
     if (bits < 2 || bits > 4) return DSQ_ERR_UNSUPPORTED;
     if (e.general_offset) epi_kind = DSQ_EPI_GENERAL;
     const int Cin = conv->Cin, Cout = conv->Cout;
     if (!(Cin == 64 || (Cin % 128 == 0 && Cin <= 1024))) return DSQ_ERR_UNSUPPORTED;
     if (shape->W + 1 > 32000 || shape->H + 1 > 32000) return DSQ_ERR_UNSUPPORTED;
-    // Which form: transposed tiles wherever they fit.  With up to 64 output channels they
-    // need the weight rows twice in the A operand (`dup`), from the blob's expanded copy
-    // or, at 3 bits, by the expansion warps.  Otherwise plain tiles.  Batch 64, transposed /
-    // plain, us: 64->64 at 56x56 4-bit 15.4 / 21.1, 3-bit 18.3 / 63.8; 128->128 at 28x28 11.5 / 12.1,
-    // 15.5 / 23.6; 256->256 at 14x14 11.4 / 11.7, 14.2 / 23.5; 512->512 at 7x7 15.6 / 16.0, 20.0 / 31.0.
+    // Which form: transposed tiles wherever they fit, else, at stride 1, plain tiles.  Up to
+    // 64 output channels want pairs of image rows (`pair`), for which the weights come from the
+    // blob's expanded copy or, at 3 bits, from the expansion warps.  Batch 64, transposed /
+    // plain, us: 64->64 at 56x56 4-bit 12.2 / 21.1, 3-bit 17.3 / 63.8; 128->128 at 28x28 10.0 / 12.1,
+    // 14.0 / 23.6; 256->256 at 14x14 10.4 / 11.7, 13.3 / 23.5; 512->512 at 7x7 14.0 / 16.0, 19.1 / 31.0.
     // the codes epilogues want the requantiser range to start at 0, too
     float r_hi = 0.f;
     if (epi_kind != DSQ_EPI_GENERAL) {
@@ -1410,9 +1487,8 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     if (sms <= 0) return DSQ_ERR_CUDA;
     W3Params p = {};
     p.N = shape->N; p.H = shape->H; p.W = shape->W;
-    p.Hp = p.H + 1; p.Wp = p.W + 1;
-    const int64_t G = ((int64_t)p.N - 1) * p.Hp * p.Wp + (int64_t)(p.H - 1) * p.Wp + p.W;
-    if (G > (1ll << 30)) return DSQ_ERR_UNSUPPORTED;
+    p.stride = stride;
+    p.Ho = (p.H - 1) / stride + 1; p.Wo = (p.W - 1) / stride + 1;
     p.Ncols = Cout;
     const int P = (int)dsq_row_pitch(Cin, bits);           // packed bytes per pixel
     // Tiling, window and shared memory for one of the two kernel forms.
@@ -1422,59 +1498,80 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     // (plain tiles with up to 64 output channels keep the expanded weights resident in
     // shared memory for the whole CTA anyway: nothing to gain, measured slightly slower)
     const bool w8_any = hooks.w8 && w8.enabled && e.half_offset;
-    // f4: 4-bit floating-point operands (2-bit codes; transposed tiles over the blob's copy)
-    auto configure = [&](int tr, int f4) -> int {
+    // f4: 4-bit floating-point operands (2-bit codes; transposed tiles; at stride 1 over the
+    // blob's copy).  most: the largest tile to consider; false where the form does not take
+    // the problem or no tile of that size fits.
+    auto configure = [&](int tr, int f4, int most) -> int {
         const bool w8_ok = w8_any && f4 == w8.f4;
-        if (f4 && !w8_ok) return 0;
+        if (f4 && !(stride == 1 ? w8_ok : hooks.w8 && w3_takes_f4(conv, bits, e.half_offset))) return 0;
+        if (stride != 1 && !tr) return 0;
         p.tr = tr;
         p.f4 = f4;
         w3_steps(Cin, f4, &p.npl, &p.kpp, &p.tps);
         if (bits == 3 && !tr) { p.tps = 1; p.kpp = 9; }
+        p.pair = tr && stride == 1 && Cout <= 64;
+        if (p.pair && !w8_ok && bits != 3) return 0;
+        const int taps = p.pair ? 12 : 9;
+        p.kpp = (taps + p.tps - 1) / p.tps;
+        p.w8 = w8_ok && (Cout > 64 || p.pair);
         p.E = f4 ? Cin / 2 : Cin;
         p.PB = std::min(P, (f4 ? 32 : 16) * bits);
         p.cpp = p.PB / 16;
         p.ksteps = p.npl * p.kpp;
         p.xstep = p.tps * P;
-        p.pk = p.tps > 1 ? p.tps * P : 16 * bits;
+        p.pk = p.tps > 1 ? p.tps * P : (f4 ? 32 : 16) * bits;
         p.rb = tr ? 128 / p.tps : 128;
-        // transposed tiles for <= 64 output channels: the weight rows twice in the
-        // A operand (two TMA boxes of the expanded copy), so that all 128 lanes of
-        // the accumulator, and all epilogue warps, carry data
-        p.dup = tr && Cout <= 64;
-        if (p.dup && !w8_ok && bits != 3) return 0;
-        p.w8 = w8_ok && (Cout > 64 || p.dup);
         p.BN = tr ? 128 : (Cout >= 256 ? 256 : ((Cout + 63) / 64) * 64);
-        p.n_tiles = (Cout + p.BN - 1) / p.BN;
-        p.mstep = std::max(sms / p.n_tiles, 1);
-        const int tile_pos = tr ? w3_tile(G, p.mstep, f4 ? W3_F4_TP : 256) : W3_BM;
-        p.tp = tile_pos;
-        p.m_tiles = (int)((G + tile_pos - 1) / tile_pos);
+        // positions (see W3Pos) and what a window is made of
+        const W3Work work = w3_work(shape, conv, p.pair, p.BN, sms);
+        p.n_tiles = work.n_tiles;
         p.cout_pad = p.n_tiles * p.BN;
-        if (p.cout_pad > W3_MAX_COUT) return 0;
-        const int need = tile_pos + 2 + 2 * p.Wp;
-        const int band = f4 ? W3_F4_BAND_PX : W3_BAND_PX;
-        if (need <= (f4 ? 3 * W3_F4_BAND_PX : tr ? 768 : W3_MAX_WINDOW_PX)) {
-            p.nbands = 1;
-            p.a_nload = (need + 255) / 256;
-            p.a_box = (((need + p.a_nload - 1) / p.a_nload) + 7) / 8 * 8;
-            p.band_px = p.a_nload * p.a_box;
-            p.apx = p.band_px;
-            p.tap_stride = p.Wp;
-        } else if (!tr || f4) {
-            p.nbands = 3;
-            p.a_nload = 1;
-            p.a_box = band;
-            p.band_px = band;
-            p.apx = 3 * band;
-            p.tap_stride = band;
-        } else {
+        if (p.cout_pad > W3_MAX_COUT || p.n_tiles > sms || work.positions > (1ll << 30)) return 0;
+        p.sh = p.pair ? 2 : stride; p.sw = stride;
+        p.Hp = work.Hp;
+        p.Wp = work.Wp;
+        p.mstep = work.mstep;
+        p.tp = tr ? w3_tile(work.positions, p.mstep, most) : W3_BM;
+        p.m_tiles = (int)((work.positions + p.tp - 1) / p.tp);
+        if (stride == 2 && bits != 3 && !f4 && hooks.window3 == 1 &&
+            !w3_takes_stride2(Cin, p.tp, (p.m_tiles + p.mstep - 1) / p.mstep))
             return 0;
+        if (p.mstep > p.m_tiles) p.mstep = p.m_tiles;
+        p.nbands = p.sh * p.sw;
+        int need = p.tp + (p.sh == 2 ? 1 : 2) * p.Wp + (p.sw == 2 ? 1 : 2);
+        if (p.nbands == 1 && (!tr || f4) && need > (f4 ? 3 * W3_F4_BAND_PX : W3_MAX_WINDOW_PX)) {
+            p.nbands = 3;
+            need = f4 ? W3_F4_BAND_PX : W3_BAND_PX;
+        }
+        p.a_nload = (need + 255) / 256;
+        if (p.nbands * p.a_nload > 32 || (p.nbands == 1 && tr && !f4 && need - p.tp + 256 > 768)) return 0;
+        p.a_box = (((need + p.a_nload - 1) / p.a_nload) + 7) / 8 * 8;
+        p.band_px = p.a_nload * p.a_box;
+        p.apx = p.nbands * p.band_px;
+        for (int b = 0; b < p.nbands; ++b) {
+            // filter taps with the corner at (-2, -2): 1 = pixels -1, 0 .. (or -1, 1, ..), 2 = 0, 2 ..
+            p.band_pos[b] = p.nbands == 3 ? b * p.Wp : 0;
+            const int row = p.sh == 2 ? 1 + b / p.sw : 1, col = p.sw == 2 ? 1 + b % 2 : 1;
+            p.band_tap[b] = col | row << 8;
+        }
+        // window rows of the taps' operands, four instructions of 32 bytes a K step
+        for (int i = 0; i < 4 * p.kpp; ++i) {
+            const int tap = p.tps * (i >> 2) + ((i & 3) * p.tps >> 2), within = 32 * (i & (4 / p.tps - 1));
+            const int kh = tap / 3, kw = tap % 3;
+            int row;
+            if (p.nbands == 3) row = kh * p.band_px + kw;
+            else {
+                const int b = (p.sh == 2 ? (kh & 1) * p.sw : 0) + (p.sw == 2 ? kw & 1 : 0);
+                row = b * p.band_px + kh / p.sh * p.Wp + kw / p.sw;
+            }
+            (&p.x_off[i >> 2].x)[i & 3] =
+                tap < taps && within < p.E ? (uint32_t)(row * (p.rb >> 4) + (within >> 4)) : MMA_NONE;
         }
         p.a_slots = W3_A_SLOTS;
         // shared memory: resident B where one N tile's K steps all fit, else rings
         p.b_res = 0;
         if (p.ksteps <= W3_MAX_BST) {
-            for (int as = W3_MAX_AS; as >= 2; --as) {
+            for (int as = W3_MAX_AS; as >= 1; --as) {
                 const int bp = p.w8 ? 0 : 2;
                 const W3Smem L = w3_layout(p.apx, p.a_slots, p.rb, p.BN, p.pk, p.PB, as, p.ksteps, bp, p.cout_pad);
                 if (L.total + 1024 <= 227u * 1024u) {
@@ -1499,8 +1596,11 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
                 }
             return 0;
         }
-        const int tries[6][3] = {{3, 3, 4}, {2, 3, 4}, {2, 2, 4}, {2, 2, 3}, {2, 2, 2}, {1, 2, 2}};
-        for (int t = 0; t < 6; ++t) {
+        // (packed slots: a multiple of the two groups, so that a slot's rounds are one
+        // group's - a parity cannot tell a round from the one two before it)
+        const int tries[5][3] = {{3, 3, 4}, {2, 3, 4}, {2, 2, 4}, {2, 2, 2}, {1, 2, 2}};
+        for (p.a_slots = W3_A_SLOTS; p.a_slots >= (stride == 2 ? 1 : 2); --p.a_slots)
+        for (int t = 0; t < 5; ++t) {
             const W3Smem L = w3_layout(p.apx, p.a_slots, p.rb, p.BN, p.pk, p.PB, tries[t][0], tries[t][1],
                                        tries[t][2], p.cout_pad);
             if (L.total + 1024 <= 227u * 1024u) {
@@ -1512,38 +1612,20 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     };
     int found = 0;
     const bool want_tr = hooks.window3 == 3 || hooks.window3 == 1;
-    if (want_tr) found = configure(1, 1) || configure(1, 0);
-    if (!found) found = configure(0, 0);
+    for (int f4 = 1; want_tr && !found && f4 >= 0; --f4)
+        for (int most = f4 ? W3_F4_TP : 256; !found && most >= 112; most -= 16) found = configure(1, f4, most);
+    if (!found) found = configure(0, 0, 0);
     if (!found) return DSQ_ERR_UNSUPPORTED;
     // (plain tiles convert accumulators by the 2^22 trick)
     if (!p.tr && (!small_acc || bits == 3)) epi_kind = DSQ_EPI_GENERAL;
     p.L = w3_layout(p.apx, p.a_slots, p.rb, p.BN, p.pk, p.PB, p.as_slots, p.b_stages, p.bp_slots, p.cout_pad);
     p.smem_bytes = (int)p.L.total + 1024;
-    // grid: a multiple of n_tiles; CTA c takes N tile c % n_tiles and every
-    // mstep-th M tile
-    if (p.n_tiles > sms) return DSQ_ERR_UNSUPPORTED;
-    if (p.mstep > p.m_tiles) p.mstep = p.m_tiles;
     {
+        // (grid: a multiple of n_tiles; CTA c takes N tile c % n_tiles and every mstep-th M tile)
         const int64_t d = (int64_t)p.mstep * p.tp, img = (int64_t)p.Hp * p.Wp;
         p.t_dn = (int)(d / img);
         p.t_dh = (int)((d % img) / p.Wp);
         p.t_dw = (int)((d % img) % p.Wp);
-        for (int b = 0; b < p.nbands; ++b)
-            for (int i = 0; i < p.a_nload; ++i) {
-                // (every digit below its base, so that one carry per digit is
-                // enough when the kernel adds them to a position)
-                const int off = p.nbands > 1 ? b * p.Wp : i * p.a_box;
-                p.ld_dn[b * p.a_nload + i] = (int)(off / img);
-                p.ld_dh[b * p.a_nload + i] = (int)((off % img) / p.Wp);
-                p.ld_dw[b * p.a_nload + i] = (int)((off % img) % p.Wp);
-            }
-    }
-    for (int i = 0; i < 4 * p.kpp; ++i) {
-        const int tap = p.tps * (i >> 2) + ((i & 3) * p.tps >> 2), within = 32 * (i & (4 / p.tps - 1));
-        (&p.x_off[i >> 2].x)[i & 3] =
-            tap < 9 && within < p.E
-                ? (uint32_t)((tap / 3 * p.tap_stride + tap % 3) * (p.rb >> 4) + (within >> 4))
-                : MMA_NONE;
     }
     p.wait_ns = hooks.wait_ns;
     p.skip_b_round = hooks.skip_b_round;
@@ -1551,8 +1633,11 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     p.e = e;
     p.r_hi = r_hi;
     p.out_pitch = (int)dsq_row_pitch(Cout, bits);
-    if (p.f4) {
+    if (p.f4 && p.w8) {
         p.mark = (const uint32_t *)((const uint8_t *)w_packed + w3_mark_offset(w8));
+    }
+    if (p.f4) {
+        p.shift = 0;
     } else if (e.half_offset) {
         p.shift = 7 - bits;
         p.orv = 0x01010101u << (7 - bits);
@@ -1571,12 +1656,15 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     CUtensorMap tb, ta;
     if (p.w8) {
         // the blob's expanded copy: Cout rows of ksteps x 128 bytes; one box = BN
-        // rows x one K step, swizzled on the way in
-        cuuint64_t dims[2] = {(cuuint64_t)p.ksteps * 128, (cuuint64_t)Cout};
-        cuuint64_t strides[1] = {(cuuint64_t)p.ksteps * 128};
-        cuuint32_t box[2] = {128u, (cuuint32_t)(p.dup ? 64 : p.BN)};
-        cuuint32_t estr[2] = {1, 1};
-        if (enc(&tb, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2,
+        // rows x one K step, swizzled on the way in.  pair: 64 rows, and a plane's nine taps
+        // are a dimension of their own, so that taps before and behind them are zeros
+        const int steps = w8.ksteps / p.npl * 128;              // bytes of a row's plane
+        cuuint64_t dims[3] = {(cuuint64_t)(p.pair ? 9 * p.rb : w8.ksteps * 128),
+                              (cuuint64_t)(p.pair ? p.npl : Cout), (cuuint64_t)Cout};
+        cuuint64_t strides[2] = {(cuuint64_t)(p.pair ? steps : w8.ksteps * 128), (cuuint64_t)w8.ksteps * 128};
+        cuuint32_t box[3] = {128u, (cuuint32_t)(p.pair ? 1 : p.BN), 64u};
+        cuuint32_t estr[3] = {1, 1, 1};
+        if (enc(&tb, CU_TENSOR_MAP_DATA_TYPE_UINT8, p.pair ? 3 : 2,
                 const_cast<uint8_t *>((const uint8_t *)w_packed + w8.offset), dims, strides, box,
                 estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -1584,7 +1672,7 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     } else {
         cuuint64_t dims[2] = {(cuuint64_t)9 * P, (cuuint64_t)Cout};
         cuuint64_t strides[1] = {(cuuint64_t)9 * P};
-        cuuint32_t box[2] = {(cuuint32_t)p.pk, (cuuint32_t)p.BN};
+        cuuint32_t box[2] = {(cuuint32_t)p.pk, (cuuint32_t)(p.pair ? 64 : p.BN)};
         cuuint32_t estr[2] = {1, 1};
         if (enc(&tb, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void *>(w_packed), dims, strides,
                 box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -1593,13 +1681,13 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     }
     {
         // im2col map over the NHWC codes: the bounding box of base positions is
-        // [-2, W-2] x [-2, H-2] (lower corner -2, upper corner -1) and every load
-        // uses filter offset (1, 1): pixels -1 .. W-1 / -1 .. H-1
+        // [-2, W-2] x [-2, H-2] (lower corner -2, upper corner -1), taken in steps of
+        // sw and sh; the loads' filter offsets make pixels -1, .. or 0, .. of them
         cuuint64_t dims[4] = {(cuuint64_t)P, (cuuint64_t)p.W, (cuuint64_t)p.H, (cuuint64_t)p.N};
         cuuint64_t strides[3] = {(cuuint64_t)P, (cuuint64_t)P * p.W, (cuuint64_t)P * p.W * p.H};
         int lower[2] = {-2, -2};
         int upper[2] = {-1, -1};
-        cuuint32_t estr[4] = {1, 1, 1, 1};
+        cuuint32_t estr[4] = {1, (cuuint32_t)p.sw, (cuuint32_t)p.sh, 1};
         if (enc_i2c(&ta, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<void *>(act_codes), dims,
                     strides, lower, upper, (cuuint32_t)p.PB, (cuuint32_t)p.a_box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,

@@ -222,7 +222,18 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *m,
         : "memory");
 }
 
-// Same for a CTA pair (cta_group::2): the copy lands in THIS CTA's shared
+// 3-D tiled load
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *m, int x, int y, int z,
+                                            uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
+        "l"(m), "r"(x), "r"(y), "r"(z), "r"(bar)
+        : "memory");
+}
+
+// The 2-D load for a CTA pair (cta_group::2): the copy lands in THIS CTA's shared
 // memory, its bytes are counted on an mbarrier of either CTA of the pair
 // (`bar` is a shared::cluster address, e.g. the leader's barrier through
 // map_to_cta).  No multicast: every CTA fetches its own tile.
