@@ -329,31 +329,19 @@ double estimate(const CsParams &p, int bits, int mt, int warps)
     return chain > shared ? chain : shared;
 }
 
-// And what the other kernel for the layer takes, likewise: a floor that grows with K
-// (the few CTAs such a layer has walk it alone) plus its work at full rate.
-// Of 335 measured layers (64 to 1024 channels, 1x1 and 3x3, 2 to 4 bits, batches of 1 to 16)
-// the rule takes the slower kernel for 34, 2 % of time on average: most are 1x1 layers,
-// whose kernel takes 0.5 to 1 us more than said here, and 3-bit ones, where the im2col kernel
-// takes twice as long (64 -> 128 at 56x56, stride 2, batch 6: 14.1 us against 6.5).
-double estimate_other(const CsParams &p, int bits, int Cin, double macs, int lean)
+// And what the other kernel for the layer takes, likewise: the window kernel as it says
+// itself; the im2col kernel a floor that grows with K (the few CTAs such a layer has walk
+// it alone) plus its work at full rate.
+// Of 666 measured 3x3 layers (64 to 512 channels, strides 1 and 2, 2 to 4 bits, batches of 1 to 32)
+// the rule takes the slower kernel for 5 %, 0.8 % of time on average.
+double estimate_other(const CsParams &p, const dsq_nhwc_t *shape, const dsq_conv_t *conv, int bits, int half_offset,
+                      int lean)
 {
-    const int sms = dsq_sm_count() > 0 ? dsq_sm_count() : 148;
-    const double ksteps = p.ksize * p.ksize * Cin / 128.0;
+    const double ksteps = p.ksize * p.ksize * conv->Cin / 128.0;
     if (p.ksize == 1 && lean) return 2.9 + (double)p.M * p.Ncols / 3.7e6;
-    if (p.ksize == 3 && p.stride == 1 && p.pad == 1 && (Cin == 64 || Cin % 128 == 0)) {
-        // Window kernel: waves of tiles of 256 positions x 128 channels (3-bit: the expansion
-        // warps set the pace).  One wave, 4-bit, measured / said here: 64 channels 5.4 / 6.1, 128
-        // 7.6 / 10.1, 256 10.2 / 12.6, 384 12.6 / 12.8, 512 15.2 / 15.2, 1024 25.2 / 24.9 us.  What is too
-        // much at 128 and 256 channels offsets what this kernel's own estimate lacks around
-        // the line there (256 at 14x14, batch 12: 8.6 us, window 10.3, own estimate 10.5): with
-        // 5.5 throughout, 35 of the layers below are on the wrong side instead of 34.
-        const double tiles = std::ceil((double)p.M / p.H / p.W * (p.H + 1) * (p.W + 1) / 256) *
-                             ((p.Ncols + 127) / 128);
-        return (Cin == 64 ? 4.3 : Cin <= 256 ? 7.7 : 5.5) +
-               std::ceil(tiles / sms) * ksteps *
-                   (bits == 3 ? (Cin == 64 ? 0.53 : 0.42) : Cin == 64 ? 0.4 : 0.27);
-    }
-    return 4.3 + 0.23 * ksteps + macs / 4.5e8;                     // im2col kernel
+    const double window = dsq_conv3_estimate(shape, bits, conv, half_offset);
+    if (window > 0.0) return window;
+    return 4.3 + 0.23 * ksteps + (double)p.M * p.Ncols * p.ksize * p.ksize * conv->Cin / 4.5e8;
 }
 
 }  // namespace
@@ -392,8 +380,7 @@ int dsq_conv_small(const void *act_codes, const dsq_nhwc_t *shape, int bits, con
             const double t = estimate(p, bits, m, w);
             if (t < best) { best = t; mt = m; warps = w; }
         }
-    const double macs = (double)p.M * p.Ncols * taps * conv->Cin;
-    if (best > estimate_other(p, bits, conv->Cin, macs, lean)) return DSQ_ERR_UNSUPPORTED;
+    if (best > estimate_other(p, shape, conv, bits, e.half_offset, lean)) return DSQ_ERR_UNSUPPORTED;
     switch (bits) {
     case 2: return pick<2>(p, mt, warps, stream);
     case 3: return pick<3>(p, mt, warps, stream);
