@@ -8,16 +8,15 @@
 // Here every row is expanded ONCE:
 //   pass 1  expand_rows_kernel: packed codes -> int8 rows in a scratch area
 //           the caller provides (M*Kp + N*Kp bytes, Kp = K rounded up to 16;
-//           HBM / L2-bound, a few microseconds);
-//   pass 2  gemm8_kernel: an 8-bit integer GEMM whose operands go from that
-//           scratch straight into swizzled shared memory by TMA - no thread
-//           touches an operand byte.  CTA pairs on 256 x 256 tiles
-//           (tcgen05.mma cta_group::2, kind::i8, both operands through
-//           shared-memory descriptors: at N = 256 a descriptor-fed instruction
-//           runs at the pipe's full rate), a ring of seven 32 KB stages per CTA,
-//           and TWO 256-column accumulators in tensor memory, so the epilogue
-//           of a tile (eight warps per CTA) overlaps the next tile's
-//           instructions.
+//           HBM / L2-bound, a few microseconds); codes of 1 and 2 bits -> 4-bit
+//           floating point (expand_rows_f4_kernel), half of that;
+//   pass 2  gemm8_kernel: a GEMM whose operands go from that scratch straight into
+//           swizzled shared memory by TMA - no thread touches an operand byte.
+//           CTA pairs on tiles of 256 rows and 64 to 256 columns (tcgen05.mma
+//           cta_group::2, kind::i8 or kind::mxf4, both operands through
+//           shared-memory descriptors), a ring of seven or more stages per CTA,
+//           and TWO accumulators in tensor memory, so the epilogue of a tile (eight
+//           warps per CTA) overlaps the next tile's instructions.
 // The scratch for 4096^3 is 33.5 MB and stays in the 126 MB L2 between the
 // passes.
 //
@@ -35,24 +34,31 @@
 
 namespace {
 
-constexpr int G8_ROWS = 128;                 // operand rows per CTA and stage (A and B alike)
-constexpr int G8_BN = 256;                   // tile width (both CTAs' B halves)
+enum G8Kind { G8_I8, G8_BF16, G8_F4 };       // operands: int8, bf16, 4-bit floating point
+constexpr int G8_ROWS = 128;                 // A rows per CTA and stage
 constexpr int G8_BM = 256;                   // tile height of a pair
 constexpr int G8_KB = 128;                   // bytes of K per stage
-constexpr int G8_STAGES = 7;
-constexpr int G8_OP_BYTES = G8_ROWS * G8_KB;             // 16 KB
-constexpr int G8_STAGE_BYTES = 2 * G8_OP_BYTES;          // A then B
+constexpr int G8_OP_BYTES = G8_ROWS * G8_KB;             // A of a stage: 16 KB
+constexpr int G8_MAX_STAGES = 12;
+// tensor-memory columns of an accumulator, which are the widest tile; behind the two
+// accumulators of 4-bit operands lie the block scales
+template <int KIND> constexpr int g8_acc() { return KIND == G8_F4 ? 240 : 256; }
+constexpr int G8_F4_SF = 480;
 constexpr int G8_WARP_TMA = 0, G8_WARP_MMA = 1, G8_WARP_TMEM = 2, G8_WARP_E0 = 4;
 constexpr int G8_E_WARPS = 8;                // per CTA: two per tensor-memory lane quarter
 constexpr int G8_THREADS = 32 * (G8_WARP_E0 + G8_E_WARPS);
-constexpr int G8_BARS = 2 * G8_STAGES + 4 + 1;
-constexpr int G8_SMEM = G8_STAGES * G8_STAGE_BYTES + 1024 /* alignment */ + 256 /* barriers */;
+constexpr int G8_BARS = 2 * G8_MAX_STAGES + 4 + 1;
+constexpr int G8_SMEM = 227 * 1024;
+constexpr int G8_TAIL = 8 * G8_BARS + 24;    // barriers, tensor-memory slot, abort flag
+constexpr int G8_STAGING = G8_E_WARPS * 32 * 33 * 4;     // a 32 x 32 block per epilogue warp
 
 struct G8Params {
     int M, N;
     int m_tiles, n_tiles, kblocks;
+    int BN;                  // tile width (both CTAs' B halves): a multiple of 32
+    int stages, stage_bytes; // A (16 KB), then BN / 2 rows of B
     int vec;                 // N is a multiple of 8: 32-byte stores
-    uint32_t idesc;          // instruction descriptor (operand types, M = 256, N = 256)
+    uint32_t idesc;          // instruction descriptor (operand types, M = 256, N = BN)
     // integer problems: C = acc, D = (float)acc * row_scale[m]
     int32_t *C_i32;
     const float *row_scale;
@@ -174,6 +180,52 @@ expand_rows_kernel(const uint8_t *__restrict__ A, const uint8_t *__restrict__ B,
     }
 }
 
+// Integer operands of 1 and 2 bits as 4-bit floating point (E2M1 in steps of 1/2, as
+// expand_word_f4; block scales of 2 make the products whole numbers): a chunk of 16 output
+// bytes is 32 values, in the order in which a shift and a mask find them (the same for
+// both operands).  A 2-bit signed code -2 .. 1 is 1010, 1001, 0000, 0001, an unsigned one
+// its own pattern; a bit is 0001 (+1) or 1001 (-1), past K 0.
+template <int BITS>
+__global__ void __launch_bounds__(EX_THREADS)
+expand_rows_f4_kernel(const uint8_t *__restrict__ A, const uint8_t *__restrict__ B, int M, int N, int K,
+                      int pitch_in, int pitch_out, uint8_t *__restrict__ A4, uint8_t *__restrict__ B4)
+{
+    grid_launch_dependents();
+    const int c = blockIdx.x * EX_THREADS + threadIdx.x;
+    if (16 * c >= pitch_out) return;
+    for (int r0 = blockIdx.y * EX_ROWS; r0 < M + N; r0 += gridDim.y * EX_ROWS) {
+        uint2 v[EX_ROWS];
+#pragma unroll
+        for (int i = 0; i < EX_ROWS; ++i) {
+            const int r = min(r0 + i, M + N - 1);
+            const uint8_t *row = r < M ? A + (int64_t)r * pitch_in : B + (int64_t)(r - M) * pitch_in;
+            if (BITS == 2) v[i] = __ldg(reinterpret_cast<const uint2 *>(row) + c);
+            else v[i].x = __ldg(reinterpret_cast<const uint32_t *>(row) + c);
+        }
+#pragma unroll
+        for (int i = 0; i < EX_ROWS; ++i) {
+            const int r = r0 + i;
+            if (r >= M + N) break;
+            uint32_t o[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if (BITS == 2) {
+                    const uint32_t x = ((j < 2 ? v[i].x : v[i].y) >> (2 * (j & 1))) & 0x33333333u;
+                    const uint32_t hi = x & 0x22222222u, lo = x & 0x11111111u;
+                    o[j] = r < M ? (hi << 2) | (hi & ~(lo << 1)) | lo : x;
+                } else {
+                    const int left = K - 32 * c;
+                    const uint32_t in = left >= 32 ? 0xFFFFFFFFu : (1u << left) - 1u;
+                    const uint32_t on = (in >> j) & 0x11111111u;
+                    o[j] = ((on & ~(v[i].x >> j)) << 3) | on;
+                }
+            }
+            uint8_t *dst = r < M ? A4 + (int64_t)r * pitch_out : B4 + (int64_t)(r - M) * pitch_out;
+            *reinterpret_cast<uint4 *>(dst + 16 * c) = make_uint4(o[0], o[1], o[2], o[3]);
+        }
+    }
+}
+
 // Weight codes -> bf16: value 2 c + 1 (grid Delta (c + 1/2), `odd`) or c, c the
 // signed BITS-bit code; K is a multiple of 8, a chunk of 8 values lies inside the
 // row.  By bit operations: the field (code ^ half) in the low mantissa bits of
@@ -240,82 +292,108 @@ inline dim3 expand_grid(int64_t chunks, int64_t rows)
 // ---------------------------------------------------------------------------
 // pass 2: int8 GEMM, CTA pairs
 // ---------------------------------------------------------------------------
-// 32 lanes x 32 columns in the 16x256b shape: r[2 e], r[2 e + 1] are two adjacent
-// columns 8 ((e >> 1) & 3) + 2 (lane & 3) of row lane / 4 + 8 (e & 1) + 16 (e >> 3).
-// A store instruction then covers eight rows x 32 contiguous bytes.
-__device__ __forceinline__ void g8_load_pairs(uint32_t taddr, uint32_t (&r)[32])
+// Outputs of a 32 x 32 block of accumulators: r[j] is row m + lane, column n + j; columns
+// from `limit` on belong to another tile or lie outside.
+// vec: N is a multiple of 8, so every group of eight columns of a row is a full 32-byte
+// sector, inside or outside the matrix as a whole, and a lane stores its row.  Otherwise the
+// block is turned round in shared memory (`stage`, rows of 33 words: no bank conflicts either
+// way) and a warp stores one row after the other, 128 contiguous bytes at a time.
+// (With two adjacent columns a lane, 4-byte stores for odd N, 2500x1111x1777 3-bit took 22 us,
+// 16 of them in the epilogue; so, and with tiles of 160 columns: 12.5.)
+template <int KIND>
+__device__ __forceinline__ void g8_store_block(const G8Params &p, int m, int n, int limit, int lane,
+                                               uint32_t stage, const uint32_t (&r)[32])
 {
-    uint32_t lo[16], hi[16];
-    tmem_ld_16x256b_x4(taddr, lo);
-    tmem_ld_16x256b_x4(taddr + (16u << 16), hi);
+    constexpr bool FACC = KIND != G8_I8;                  // f32 accumulators
+    const int row = m + lane;
+    // scaled and, of F4, integer results of an accumulator
+    auto whole = [](uint32_t x) { return FACC ? (uint32_t)__float2int_rn(__uint_as_float(x)) : x; };
+    auto scaled = [](uint32_t x, float rs) {
+        return __float_as_uint(__fmul_rn(FACC ? __uint_as_float(x) : (float)(int)x, rs));
+    };
+    const float rs = KIND != G8_BF16 && p.D_f32 && row < p.M ? __ldg(p.row_scale + row) : 0.0f;
+    if (p.vec) {
+        if (row >= p.M) return;
+        const int64_t at = (int64_t)row * p.N + n;
 #pragma unroll
-    for (int i = 0; i < 16; ++i) { r[i] = lo[i]; r[16 + i] = hi[i]; }
-}
-
-// outputs of such a block; m, n: this lane's first row and column
-template <bool F16>
-__device__ __forceinline__ void g8_store_pairs(const G8Params &p, int m, int n, const uint32_t (&r)[32])
-{
-    const bool even = (p.N & 1) == 0;      // (bases are 16-byte aligned: pairs at even offsets)
-    float cs[8], cb[8];
-    if (F16) {
+        for (int j = 0; j < 32; j += 8) {
+            if (n + j >= limit) break;
+            uint32_t f[8];
+            if (KIND == G8_BF16) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int c = min(n + 8 * (i >> 1) + (i & 1), p.N - 1);
-            cs[i] = __ldg(p.col_scale + c);
-            cb[i] = p.col_bias ? __ldg(p.col_bias + c) : 0.0f;
-        }
-    }
-#pragma unroll
-    for (int e = 0; e < 16; ++e) {
-        const int row = m + 8 * (e & 1) + 16 * (e >> 3), b = (e >> 1) & 3, c = n + 8 * b;
-        if (row >= p.M || c >= p.N) continue;
-        const int64_t at = (int64_t)row * p.N + c;
-        const bool two = c + 1 < p.N;
-        auto put = [&](void *base, uint32_t x, uint32_t y) {
-            uint32_t *dst = reinterpret_cast<uint32_t *>(base) + at;
-            if (even) *reinterpret_cast<uint2 *>(dst) = make_uint2(x, y);
-            else {
-                dst[0] = x;
-                if (two) dst[1] = y;
+                for (int t = 0; t < 8; ++t)
+                    f[t] = __float_as_uint(
+                        __fmaf_rn(__uint_as_float(r[j + t]), __ldg(p.col_scale + n + j + t),
+                                  p.col_bias ? __ldg(p.col_bias + n + j + t) : 0.0f));
+                stg_256(p.Y_f32 + at + j, f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7]);
+                continue;
             }
-        };
-        if (F16) {
-            put(p.Y_f32, __float_as_uint(__fmaf_rn(__uint_as_float(r[2 * e]), cs[2 * b], cb[2 * b])),
-                __float_as_uint(__fmaf_rn(__uint_as_float(r[2 * e + 1]), cs[2 * b + 1], cb[2 * b + 1])));
-            continue;
+            if (p.C_i32) {
+#pragma unroll
+                for (int t = 0; t < 8; ++t) f[t] = whole(r[j + t]);
+                stg_256(p.C_i32 + at + j, f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7]);
+            }
+            if (p.D_f32) {
+#pragma unroll
+                for (int t = 0; t < 8; ++t) f[t] = scaled(r[j + t], rs);
+                stg_256(p.D_f32 + at + j, f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7]);
+            }
         }
-        if (p.C_i32) put(p.C_i32, r[2 * e], r[2 * e + 1]);
-        if (p.D_f32) {
-            const float rs = __ldg(p.row_scale + row);
-            put(p.D_f32, __float_as_uint(__fmul_rn((float)(int)r[2 * e], rs)),
-                __float_as_uint(__fmul_rn((float)(int)r[2 * e + 1], rs)));
+        return;
+    }
+    const int col = n + lane;
+    const int rows = min(32, p.M - m);
+    float cs = 0.0f, cb = 0.0f;
+    if (KIND == G8_BF16 && col < limit) {
+        cs = __ldg(p.col_scale + col);
+        cb = p.col_bias ? __ldg(p.col_bias + col) : 0.0f;
+    }
+#pragma unroll 1
+    for (int which = 0; which < 2; ++which) {
+        uint32_t *const out = KIND == G8_BF16 ? (uint32_t *)(which ? nullptr : p.Y_f32)
+                                              : which ? (uint32_t *)p.D_f32 : (uint32_t *)p.C_i32;
+        if (!out) continue;
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 32; ++j)
+            sts_32(stage + 4u * (uint32_t)(lane * 33 + j),
+                   KIND == G8_BF16 ? r[j] : which ? scaled(r[j], rs) : whole(r[j]));
+        __syncwarp();
+        if (col < limit) {
+            uint32_t *dst = out + (int64_t)m * p.N + col;
+#pragma unroll 8
+            for (int i = 0; i < rows; ++i, dst += p.N) {
+                const uint32_t v = lds_32(stage + 4u * (uint32_t)(i * 33 + lane));
+                *dst = KIND == G8_BF16 ? __float_as_uint(__fmaf_rn(__uint_as_float(v), cs, cb)) : v;
+            }
         }
     }
 }
 
-// F16 = false: 8-bit integer operands, s32 accumulators (kind::i8);
-// F16 = true: bf16 operands, f32 accumulators (kind::f16).  A stage row is 128
-// bytes of K either way (128 or 64 elements), four instructions per stage.
+// KIND: 8-bit integer operands with s32 accumulators (kind::i8), bf16 operands or 4-bit
+// floating-point ones with f32 accumulators (kind::f16, kind::mxf4).  A stage row is 128
+// bytes of K (128, 64 or 256 elements), four instructions per stage.
 //
 // S > 1: few tiles and a long K.  A cluster is S pairs on ONE tile, pair s taking the
 // s-th part of K; when all are done, pair s gets the other pairs' partial sums of
-// columns s * 256 / S .. through distributed shared memory (into the stage ring,
+// columns s * BN / S .. through distributed shared memory (into the stage ring,
 // which nothing reads any more), adds them to its own in a fixed order and writes
 // those columns.  One tile per cluster.
-template <bool F16, int S>
+template <int KIND, int S>
 __global__ void __launch_bounds__(G8_THREADS, 1)
 gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
              const __grid_constant__ CUtensorMap tmap_b, const G8Params p)
 {
     extern __shared__ uint8_t smem_raw[];
+    constexpr int ACC = g8_acc<KIND>();
     uint8_t *smem = reinterpret_cast<uint8_t *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023u) & ~(uintptr_t)1023u);
-    uint8_t *tail = smem + G8_STAGES * G8_STAGE_BYTES;
+    uint8_t *tail = smem + p.stages * p.stage_bytes;
     const uint32_t bars = smem_u32(tail);
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(tail + 8 * G8_BARS);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tail + 8 * G8_BARS + 8);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t staging = smem_u32(tail + G8_TAIL) + (uint32_t)((warp - G8_WARP_E0) * 32 * 33 * 4);
     const uint32_t crank = cluster_ctarank();
     const uint32_t rank = crank & 1u, split = crank >> 1;       // in the pair; which part of K
     const uint32_t leader = crank & ~1u;
@@ -323,20 +401,20 @@ gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
     Ctl ctl{abort_flag, p.ws, p.wait_ns};
 
     // full: operand bytes of BOTH CTAs' stage s have landed (counted on the
-    //       leader's barrier only: the leader's producer expects 64 KB, both
-    //       producers' copies complete on it);
+    //       leader's barrier only: the leader's producer expects both stages' bytes,
+    //       both producers' copies complete on it);
     // empty: the pair's instructions on stage s are done (tcgen05.commit,
     //       signalled in both CTAs);
     // acc_full[b]: the tile in accumulator b is complete (both CTAs);
     // acc_empty[b]: (leader) all epilogue warps of both CTAs have read it.
     auto bar_full = [&](int s) { return bars + 8u * s; };
-    auto bar_empty = [&](int s) { return bars + 8u * (G8_STAGES + s); };
-    auto bar_acc_full = [&](int b) { return bars + 8u * (2 * G8_STAGES + b); };
-    auto bar_acc_empty = [&](int b) { return bars + 8u * (2 * G8_STAGES + 2 + b); };
-    const uint32_t bar_drain = bars + 8u * (2 * G8_STAGES + 4);
+    auto bar_empty = [&](int s) { return bars + 8u * (G8_MAX_STAGES + s); };
+    auto bar_acc_full = [&](int b) { return bars + 8u * (2 * G8_MAX_STAGES + b); };
+    auto bar_acc_empty = [&](int b) { return bars + 8u * (2 * G8_MAX_STAGES + 2 + b); };
+    const uint32_t bar_drain = bars + 8u * (2 * G8_MAX_STAGES + 4);
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < G8_STAGES; ++s) {
+        for (int s = 0; s < p.stages; ++s) {
             mbar_init(bar_full(s), 1);
             mbar_init(bar_empty(s), 1);
         }
@@ -358,10 +436,22 @@ gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
     }
     tc_fence_before_sync();
     __syncthreads();
-    // the peer's barriers must be initialised before anything signals them
-    cluster_sync_all();
     tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_slot;
+    if (KIND == G8_F4 && warp >= G8_WARP_E0 && warp < G8_WARP_E0 + 4) {
+        // every block scale is 2 (UE8M0 128), whatever place the tensor core reads it from
+        uint32_t two[32];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) two[i] = 0x80808080u;
+        tmem_st_32x32(tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + G8_F4_SF, two);
+        tmem_st_wait();
+        tc_fence_before_sync();
+    }
+    __syncwarp();
+    // the peer's barriers must be initialised (and its scales written) before anything
+    // signals (reads) them
+    cluster_sync_all();
+    tc_fence_after_sync();
 
     const int pair = blockIdx.x / (2 * S), npairs = gridDim.x / (2 * S);
     const int kb0 = S == 1 ? 0 : (int)split * p.kblocks / S;
@@ -372,19 +462,20 @@ gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
     if (warp == G8_WARP_TMA) {
         // ---------------- TMA producer (one thread per CTA) -----------------
         if (lane == 0) {
-            uint32_t g = 0;
+            int s = 0;
+            uint32_t ph = 0;
             bool ok = true;
             for (int tile = pair; ok && tile < total_tiles; tile += npairs) {
                 const int m0 = (tile / p.n_tiles) * G8_BM + (int)rank * G8_ROWS;
-                const int n0 = (tile % p.n_tiles) * G8_BN + (int)rank * G8_ROWS;
-                for (int kb = kb0; kb < kb1; ++kb, ++g) {
-                    const int s = g % G8_STAGES;
-                    if (!(ok = wait_bar(bar_empty(s), ((g / G8_STAGES) & 1u) ^ 1u, ctl, 21))) break;
+                const int n0 = (tile % p.n_tiles) * p.BN + (int)rank * (p.BN / 2);
+                for (int kb = kb0; kb < kb1; ++kb) {
+                    if (!(ok = wait_bar(bar_empty(s), ph ^ 1u, ctl, 21))) break;
                     const uint32_t full0 = map_to_cta(bar_full(s), leader);
-                    if (rank == 0) mbar_arrive_expect_tx(bar_full(s), 2 * G8_STAGE_BYTES);
-                    const uint32_t dst = smem_u32(smem + s * G8_STAGE_BYTES);
+                    if (rank == 0) mbar_arrive_expect_tx(bar_full(s), 2 * (uint32_t)p.stage_bytes);
+                    const uint32_t dst = smem_u32(smem + s * p.stage_bytes);
                     tma_load_2d_pair(dst, &tmap_a, kb * G8_KB, m0, full0);
                     tma_load_2d_pair(dst + G8_OP_BYTES, &tmap_b, kb * G8_KB, n0, full0);
+                    if (++s == p.stages) { s = 0; ph ^= 1u; }
                 }
             }
             if (!ok) {
@@ -397,31 +488,32 @@ gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
         // ---------------- MMA issuer (leader CTA; whole warp, elected lane) ---
         if (rank == 0) {
             const uint32_t idesc = p.idesc;
-            uint32_t g = 0, it = 0;
+            const uint64_t desc = smem_desc_sw128(smem_u32(smem));
+            const uint32_t hi = (uint32_t)(desc >> 32);
+            uint32_t it = 0, ph = 0;
+            int s = 0;
             bool ok = true;
             for (int tile = pair; ok && tile < total_tiles; tile += npairs, ++it) {
                 const int b = it & 1;
                 if (!(ok = wait_bar_warp<true>(bar_acc_empty(b), ((it >> 1) & 1u) ^ 1u, ctl, 22)))
                     break;
                 tc_fence_after_sync();
-                const uint32_t d_tmem = tmem_base + b * G8_BN;
-                for (int kb = kb0; kb < kb1; ++kb, ++g) {
-                    const int s = g % G8_STAGES;
-                    if (!(ok = wait_bar_warp<true>(bar_full(s), (g / G8_STAGES) & 1u, ctl, 23)))
-                        break;
+                const uint32_t d_tmem = tmem_base + b * ACC;
+                for (int kb = kb0; kb < kb1; ++kb) {
+                    if (!(ok = wait_bar_warp<true>(bar_full(s), ph, ctl, 23))) break;
                     tc_fence_after_sync();
-                    const uint64_t ad = smem_desc_sw128(smem_u32(smem + s * G8_STAGE_BYTES));
-                    const uint64_t bd =
-                        smem_desc_sw128(smem_u32(smem + s * G8_STAGE_BYTES + G8_OP_BYTES));
-                    if (F16)
-                        mma_f16_ss_pair_x4_elect(d_tmem, (uint32_t)ad, (uint32_t)(ad >> 32),
-                                                 (uint32_t)bd, (uint32_t)(bd >> 32), idesc,
-                                                 (uint32_t)(kb - kb0));
+                    // (a stage lies below 256 KB: the address field does not overflow)
+                    const uint32_t ad = (uint32_t)desc + (uint32_t)s * (uint32_t)(p.stage_bytes >> 4);
+                    const uint32_t bd = ad + (G8_OP_BYTES >> 4);
+                    if (KIND == G8_BF16)
+                        mma_f16_ss_pair_x4_elect(d_tmem, ad, hi, bd, hi, idesc, (uint32_t)(kb - kb0));
+                    else if (KIND == G8_F4)
+                        mma_f4_ss_pair_x4_elect(d_tmem, ad, hi, bd, hi, idesc, tmem_base + G8_F4_SF,
+                                                tmem_base + G8_F4_SF + 16, (uint32_t)(kb - kb0));
                     else
-                        mma_i8_ss_pair_x4_elect(d_tmem, (uint32_t)ad, (uint32_t)(ad >> 32),
-                                                (uint32_t)bd, (uint32_t)(bd >> 32), idesc,
-                                                (uint32_t)(kb - kb0));
+                        mma_i8_ss_pair_x4_elect(d_tmem, ad, hi, bd, hi, idesc, (uint32_t)(kb - kb0));
                     mma_commit_pair_elect(bar_empty(s), pair_mask);
+                    if (++s == p.stages) { s = 0; ph ^= 1u; }
                 }
                 if (ok) mma_commit_pair_elect(bar_acc_full(b), pair_mask);
             }
@@ -438,124 +530,91 @@ gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
     } else if (warp >= G8_WARP_E0) {
         // ---------------- epilogue: eight warps per CTA ----------------------
         const int quarter = warp & 3;                      // tensor-memory lane quarter
-        const int half = (warp - G8_WARP_E0) >> 2;         // columns [128 half, 128 half + 128)
+        const int half = (warp - G8_WARP_E0) >> 2;         // every other block of 32 columns
+        const int blocks = p.BN / 32;
         uint32_t it = 0;
         bool ok = true;
         for (int tile = pair; ok && tile < total_tiles; tile += npairs, ++it) {
             const int b = it & 1;
-            const int m = (tile / p.n_tiles) * G8_BM + (int)rank * G8_ROWS + quarter * 32 + lane;
-            const int n0 = (tile % p.n_tiles) * G8_BN + half * 128;
+            const int m = (tile / p.n_tiles) * G8_BM + (int)rank * G8_ROWS + quarter * 32;
+            const int n0 = (tile % p.n_tiles) * p.BN, limit = min(p.N, n0 + p.BN);
             if (!(ok = wait_bar_warp(bar_acc_full(b), (it >> 1) & 1u, ctl, 24))) break;
             tc_fence_after_sync();
-            const float rs = (!F16 && p.D_f32 && m < p.M) ? __ldg(p.row_scale + m) : 0.0f;
-            const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + b * G8_BN + half * 128;
+            const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + b * ACC;
+            auto release = [&]() {
+                // the accumulator is in registers: hand it back
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) {
+                    if (rank != 0) mbar_arrive_cluster(map_to_cta(bar_acc_empty(b), leader));
+                    else mbar_arrive(bar_acc_empty(b));
+                }
+            };
 #pragma unroll 1
-            for (int c0 = 0; c0 < 128; c0 += 32) {
+            for (int c = half; c < blocks; c += 2) {
                 uint32_t r[32];
-                if (p.vec) tmem_ld_32x32(taddr + c0, r);
-                else g8_load_pairs(taddr + c0, r);
+                tmem_ld_32x32(taddr + 32 * c, r);
                 tmem_ld_wait();
-                if (c0 == 96) {
-                    // the accumulator is in registers: hand it back
-                    tc_fence_before_sync();
-                    __syncwarp();
-                    if (lane == 0) {
-                        if (rank != 0) mbar_arrive_cluster(map_to_cta(bar_acc_empty(b), leader));
-                        else mbar_arrive(bar_acc_empty(b));
-                    }
-                }
-                const int n = n0 + c0;
-                if (!p.vec) {
-                    g8_store_pairs<F16>(p, m - lane + (lane >> 2), n + 2 * (lane & 3), r);
-                    continue;
-                }
-                // N is a multiple of 8: every group of eight columns of a row is a full
-                // 32-byte sector, inside or outside the matrix as a whole
-                if (m >= p.M || n >= p.N) continue;
-                const int64_t at = (int64_t)m * p.N + n;
-#pragma unroll
-                for (int j = 0; j < 32; j += 8) {
-                    if (n + j >= p.N) break;
-                    uint32_t f[8];
-                    if (F16) {
-#pragma unroll
-                        for (int t = 0; t < 8; ++t)
-                            f[t] = __float_as_uint(
-                                __fmaf_rn(__uint_as_float(r[j + t]), __ldg(p.col_scale + n + j + t),
-                                          p.col_bias ? __ldg(p.col_bias + n + j + t) : 0.0f));
-                        stg_256(p.Y_f32 + at + j, f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7]);
-                        continue;
-                    }
-                    if (p.C_i32)
-                        stg_256(p.C_i32 + at + j, r[j], r[j + 1], r[j + 2], r[j + 3], r[j + 4], r[j + 5],
-                                r[j + 6], r[j + 7]);
-                    if (p.D_f32) {
-#pragma unroll
-                        for (int t = 0; t < 8; ++t)
-                            f[t] = __float_as_uint(__fmul_rn((float)(int)r[j + t], rs));
-                        stg_256(p.D_f32 + at + j, f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7]);
-                    }
-                }
+                if (c + 2 >= blocks) release();
+                if (m < p.M && n0 + 32 * c < limit)
+                    g8_store_block<KIND>(p, m, n0 + 32 * c, limit, lane, staging, r);
             }
         }
     }
 
     if (S > 1) {
         // ---------------- exchange of the partial sums --------------------------
-        constexpr int COLS = G8_BN / S;                    // columns a pair writes
-        constexpr uint32_t BLOCK = 128u * COLS * 4u;       // one pair's sums of them, 128 rows
-        // [row][COLS] words, 16-byte units XOR-ed with the row: conflict-free for a
-        // lane per row and for eight rows per load
-        auto unit = [](int row, int u) { return (uint32_t)(row * (COLS * 4) + ((u ^ (row & 7)) << 4)); };
+        const int cols = p.BN / S;                         // columns a pair writes: a multiple of 32
+        const uint32_t block = 128u * (uint32_t)cols * 4u; // one pair's sums of them, 128 rows
+        // [row][cols] words, 16-byte units XOR-ed with the row: conflict-free for a
+        // lane per row
+        auto unit = [&](int row, int u) { return (uint32_t)(row * (cols * 4) + ((u ^ (row & 7)) << 4)); };
         const int quarter = warp & 3, k = (warp - G8_WARP_E0) >> 2;
         const uint32_t ring = smem_u32(smem);
         const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16);
+        const int row = quarter * 32 + lane;
         tc_fence_after_sync();
         __syncwarp();
         cluster_sync_all();                                // every pair's instructions are done
         if (warp >= G8_WARP_E0) {
-            const int row = quarter * 32 + lane;
 #pragma unroll 1
-            for (int c0 = 32 * k; c0 < G8_BN; c0 += 64) {
-                const uint32_t d = (uint32_t)c0 / COLS;    // the pair these columns belong to
+            for (int c0 = 32 * k; c0 < p.BN; c0 += 64) {
+                const uint32_t d = (uint32_t)(c0 / cols);  // the pair these columns belong to
                 if (d == split) continue;
                 uint32_t r[32];
                 tmem_ld_32x32(taddr + c0, r);
                 tmem_ld_wait();
-                const uint32_t dst = map_to_cta(ring, 2 * d + rank) + (split - (split > d)) * BLOCK;
+                const uint32_t dst = map_to_cta(ring, 2 * d + rank) + (split - (split > d)) * block;
 #pragma unroll
                 for (int v = 0; v < 8; ++v)
-                    st_cluster_128(dst + unit(row, (c0 % COLS) / 4 + v), r[4 * v], r[4 * v + 1],
+                    st_cluster_128(dst + unit(row, (c0 % cols) / 4 + v), r[4 * v], r[4 * v + 1],
                                    r[4 * v + 2], r[4 * v + 3]);
             }
         }
         __syncwarp();
         cluster_sync_all();
         if (warp >= G8_WARP_E0 && pair < total_tiles) {
-            const int row = quarter * 32 + (lane >> 2), j = lane & 3;
-            const int m = (pair / p.n_tiles) * G8_BM + (int)rank * G8_ROWS + row;
-            const int n0 = (pair % p.n_tiles) * G8_BN + (int)split * COLS;
+            const int m = (pair / p.n_tiles) * G8_BM + (int)rank * G8_ROWS + quarter * 32;
+            const int n0 = (pair % p.n_tiles) * p.BN + (int)split * cols, limit = min(p.N, n0 + cols);
 #pragma unroll 1
-            for (int c0 = 32 * k; c0 < COLS; c0 += 64) {
+            for (int c0 = 32 * k; c0 < cols; c0 += 64) {
                 uint32_t r[32];
-                g8_load_pairs(taddr + split * COLS + c0, r);
+                tmem_ld_32x32(taddr + split * cols + c0, r);
                 tmem_ld_wait();
 #pragma unroll
                 for (int o = 0; o < S - 1; ++o)
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        // r[2 e], r[2 e + 1]: row + 8 (e & 1) + 16 (e >> 3), columns of block (e >> 1) & 3
-                        const int rr = row + 8 * (e & 1) + 16 * (e >> 3), cc = c0 + 8 * ((e >> 1) & 3) + 2 * j;
-                        const uint2 v = lds_64(ring + o * BLOCK + unit(rr, cc >> 2) + 4 * (cc & 3));
-                        if (F16) {
-                            r[2 * e] = __float_as_uint(__uint_as_float(r[2 * e]) + __uint_as_float(v.x));
-                            r[2 * e + 1] = __float_as_uint(__uint_as_float(r[2 * e + 1]) + __uint_as_float(v.y));
-                        } else {
-                            r[2 * e] += v.x;
-                            r[2 * e + 1] += v.y;
-                        }
+                    for (int v = 0; v < 8; ++v) {
+                        const uint4 x = lds_128(ring + o * block + unit(row, c0 / 4 + v));
+                        const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+                        for (int t = 0; t < 4; ++t)
+                            r[4 * v + t] = KIND == G8_I8 ? r[4 * v + t] + w[t]
+                                                         : __float_as_uint(__uint_as_float(r[4 * v + t]) +
+                                                                           __uint_as_float(w[t]));
                     }
-                g8_store_pairs<F16>(p, m, n0 + c0 + 2 * j, r);
+                if (m < p.M && n0 + c0 < limit)
+                    g8_store_block<KIND>(p, m, n0 + c0, limit, lane, staging, r);
             }
         }
     }
@@ -573,14 +632,14 @@ gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
     }
 }
 
-int make_rows128_tmap(CUtensorMap *map, const void *base, uint64_t k_bytes, uint64_t rows,
-                      uint64_t pitch)
+int make_rows_tmap(CUtensorMap *map, const void *base, uint64_t k_bytes, uint64_t rows,
+                   uint64_t pitch, int box_rows)
 {
     DsqEncodeTiledFn fn = dsq_encode_tiled_fn();
     if (!fn) return DSQ_ERR_CUDA;
     cuuint64_t dims[2] = {k_bytes, rows};
     cuuint64_t strides[1] = {pitch};
-    cuuint32_t box[2] = {G8_KB, G8_ROWS};
+    cuuint32_t box[2] = {G8_KB, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
     CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void *>(base), dims, strides,
                     box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -590,22 +649,22 @@ int make_rows128_tmap(CUtensorMap *map, const void *base, uint64_t k_bytes, uint
 
 inline size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-template <bool F16, int S>
+template <int KIND, int S>
 int launch_split(const CUtensorMap &ta, const CUtensorMap &tb, const G8Params &p, int clusters,
                  cudaStream_t stream)
 {
     static std::atomic<unsigned long long> configured{0};
-    const int st = dsq_allow_smem((const void *)gemm8_kernel<F16, S>, G8_SMEM, &configured);
+    const int st = dsq_allow_smem((const void *)gemm8_kernel<KIND, S>, G8_SMEM, &configured);
     if (st) return st;
     // (dependent launch: set-up overlaps the tail of pass 1; the kernel waits for it
     // itself before the first copy)
-    return dsq_launch(gemm8_kernel<F16, S>, dim3(2 * S * clusters), dim3(G8_THREADS), (size_t)G8_SMEM,
+    return dsq_launch(gemm8_kernel<KIND, S>, dim3(2 * S * clusters), dim3(G8_THREADS), (size_t)G8_SMEM,
                       stream, dsq_launch_hooks().pdl, 2 * S, ta, tb, p);
 }
 
 // Clusters of S pairs that fit on the GPU at once (a cluster lives inside one group
 // of SMs, so this is less than SMs / 2 S).
-template <bool F16, int S>
+template <int KIND, int S>
 int resident_clusters()
 {
     static std::atomic<int> cached[DSQ_MAX_DEVICES];
@@ -613,7 +672,7 @@ int resident_clusters()
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= DSQ_MAX_DEVICES) return 0;
     int n = cached[dev].load(std::memory_order_relaxed);
     if (n) return n;
-    if (cudaFuncSetAttribute(gemm8_kernel<F16, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, G8_SMEM) !=
+    if (cudaFuncSetAttribute(gemm8_kernel<KIND, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, G8_SMEM) !=
         cudaSuccess)
         return 0;
     cudaLaunchConfig_t cfg = {};
@@ -626,7 +685,7 @@ int resident_clusters()
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&n, gemm8_kernel<F16, S>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, gemm8_kernel<KIND, S>, &cfg) != cudaSuccess) {
         cudaGetLastError();
         n = 0;
     }
@@ -634,41 +693,70 @@ int resident_clusters()
     return n;
 }
 
-// K split over the two pairs of a cluster where all the tiles' clusters are resident at
-// once (33 of them on 148 SMs) and a part still has twelve K blocks: the exchange costs
-// about as much as eight.  (Four pairs a cluster gained nothing more: 15 such clusters are
-// resident and the exchange doubles.)
-template <bool F16>
-bool takes_split(int64_t tiles, int64_t kblocks)
+// Tile width, and whether K is split over the two pairs of a cluster, for a problem of
+// kblocks K blocks.  A K block of a tile takes 2.5 BN clocks (at 1.9 GHz; the tensor cores), and
+// of narrow tiles 330 + 0.72 BN (what a block costs whatever its width): fitted to 4096^3 4-bit at 96 to
+// 256 columns, 76.7 59.0 54.1 50.2 55.4 52.6 us.  So the width that fills the pairs' waves is
+// taken: 4096^3 4.8 waves of 192 columns instead of 3.5 of 256, 2500x1111x1777 70 tiles of 160
+// instead of 50 of 256, 3136x512x4608 at 1 bit 52 of 128 instead of 26 (and no split).  Split: only
+// with all the clusters resident at once and twelve K blocks a part; the exchange costs about
+// as much as eight.  (Four pairs a cluster gained nothing more: 15 such clusters are resident and
+// the exchange doubles.)
+struct G8Tile {
+    int bn, split;
+    double clocks;
+};
+template <int KIND>
+G8Tile pick_tile(int64_t M, int64_t N, int64_t kblocks)
 {
-    return kblocks >= 24 && tiles <= resident_clusters<F16, 2>();
+    const int pairs = std::max((dsq_sm_count() > 0 ? dsq_sm_count() : 148) / 2, 1);
+    const int64_t m_tiles = (M + G8_BM - 1) / G8_BM;
+    G8Tile best = {0, 0, 0.0};
+    for (int split = 1; split <= 2; ++split)
+        for (int bn = g8_acc<KIND>() / 32 * 32; bn >= 64; bn -= 32) {      // (pairs take N in steps of 32)
+            if (split == 2 && (bn % 64 != 0 || kblocks < 24)) continue;
+            const int64_t tiles = m_tiles * ((N + bn - 1) / bn);
+            if (split == 2 && tiles > resident_clusters<KIND, 2>()) continue;
+            const int64_t waves = split == 2 ? 1 : (tiles + pairs - 1) / pairs;
+            const double block = std::max(2.5 * bn, 330.0 + 0.72 * bn);
+            const double clocks = (double)waves * ((double)((kblocks + split - 1) / split) * block + 400.0) +
+                                  (split == 2 ? 4000 + 20 * bn : 20 * bn);
+            if (best.bn == 0 || clocks < best.clocks) best = G8Tile{bn, split, clocks};
+        }
+    return best;
 }
 
 // Pass 2 over operands that are rows of k_bytes bytes of K (byte maps: the
 // kernel never looks at an element, only the tensor core does).
-template <bool F16>
+template <int KIND>
 int launch_pass2(const void *A, size_t a_pitch, const void *B, size_t b_pitch, size_t k_bytes,
-                 int64_t M, int64_t N, G8Params p, cudaStream_t stream)
+                 int64_t M, int64_t N, bool a_signed, bool b_signed, G8Params p, cudaStream_t stream)
 {
     p.M = (int)M; p.N = (int)N;
-    p.m_tiles = (int)((M + G8_BM - 1) / G8_BM);
-    p.n_tiles = (int)((N + G8_BN - 1) / G8_BN);
     p.kblocks = (int)((k_bytes + G8_KB - 1) / G8_KB);
-    p.wait_ns = dsq_launch_hooks().wait_ns;
-    CUtensorMap ta, tb;
-    int st = make_rows128_tmap(&ta, A, k_bytes, (uint64_t)M, a_pitch);
-    if (st) return st;
-    st = make_rows128_tmap(&tb, B, k_bytes, (uint64_t)N, b_pitch);
-    if (st) return st;
-
+    const G8Tile tile = pick_tile<KIND>(M, N, p.kblocks);
+    p.BN = tile.bn;
+    p.m_tiles = (int)((M + G8_BM - 1) / G8_BM);
+    p.n_tiles = (int)((N + p.BN - 1) / p.BN);
+    p.idesc = KIND == G8_F4     ? idesc_mxf4(p.BN, G8_BM)
+              : KIND == G8_BF16 ? idesc_bf16(p.BN, G8_BM)
+                                : idesc_i8(p.BN, a_signed, b_signed, G8_BM);
     p.vec = N % 8 == 0 && (!p.C_i32 || (reinterpret_cast<uintptr_t>(p.C_i32) & 31u) == 0) &&
             (!p.D_f32 || (reinterpret_cast<uintptr_t>(p.D_f32) & 31u) == 0) &&
             (!p.Y_f32 || (reinterpret_cast<uintptr_t>(p.Y_f32) & 31u) == 0);
+    p.stage_bytes = G8_OP_BYTES + p.BN / 2 * G8_KB;
+    p.stages = std::min(G8_MAX_STAGES,
+                        (G8_SMEM - 1024 - G8_TAIL - (p.vec ? 0 : G8_STAGING)) / p.stage_bytes);
+    p.wait_ns = dsq_launch_hooks().wait_ns;
+    CUtensorMap ta, tb;
+    int st = make_rows_tmap(&ta, A, k_bytes, (uint64_t)M, a_pitch, G8_ROWS);
+    if (st) return st;
+    st = make_rows_tmap(&tb, B, k_bytes, (uint64_t)N, b_pitch, p.BN / 2);
+    if (st) return st;
     const int sms = dsq_sm_count() > 0 ? dsq_sm_count() : 148;
     const int tiles = p.m_tiles * p.n_tiles;
-    if (takes_split<F16>(tiles, p.kblocks))
-        return launch_split<F16, 2>(ta, tb, p, tiles, stream);
-    return launch_split<F16, 1>(ta, tb, p, std::min(sms / 2, tiles), stream);
+    if (tile.split == 2) return launch_split<KIND, 2>(ta, tb, p, tiles, stream);
+    return launch_split<KIND, 1>(ta, tb, p, std::min(sms / 2, tiles), stream);
 }
 
 // first 1024-byte boundary behind the status words of a caller workspace
@@ -680,27 +768,63 @@ inline uint8_t *scratch_of(void *workspace)
 
 }  // namespace
 
+static bool f4_exact(int64_t K, int bits) { return bits < 3 && K * (bits == 2 ? 6 : 1) < (1 << 23); }
+
 // Scratch the two-pass path needs behind the status words (0: the problem is
-// one the fused kernel keeps).
+// one the fused kernel keeps): where it is expected to be the faster one.  Both estimates
+// (microseconds) are fits to 228 measured problems of 2 to 4 bits and 128 to 6144 a side, 7 and 10 % off in the
+// mean; the rule takes the slower path for 21 of them, 1.3 % of time on average.  Two passes:
+// their launches, the tiles of the second, the bytes of the first, the outputs (turned round
+// in shared memory where rows are not whole sectors).  The fused kernel: its rounds of K,
+// the expansion of each row once per tile (3-bit rows one K step a round), the outputs (one
+// word at a time where rows are no multiple of 16 bytes).  Fused / two passes, us: 4-bit 1024^3
+// 6.7 / 8.8, 2048^3 16.0 / 15.6 (either), 3072x3072x1024 20.6 / 18.1, 2500x1111x1777 29 / 12.5; 3-bit 1024^3 10.1 / 8.8, 2048^3 22 / 16;
+// 2-bit 2048^3 16.1 / 13.9.
 size_t dsq_gemm8_scratch_bytes(int64_t M, int64_t N, int64_t K, int bits, int force)
 {
-    // Measured, fused / two passes in us: 4-bit 1500x1500x6000 (1.4e10) 22 / 31,
-    // 2048x2048x4096 (1.7e10) 22 / 21, 3072^3 33 / 26, 4096^3 75 / 52.  3-bit rows,
-    // which the fused kernel takes one K step a round: 1024^3 10.6 / 12, 128x6144x6144
-    // (4.8e9) 41 / 26, 2048^3 24 / 15.  Where N is not a multiple of 4 the fused
-    // kernel stores words: 4-bit 1023^2 outputs 11 / 16, 2500x1111 29 / 20.
-    const double work = (double)M * (double)N * (double)K;
-    const bool large = work >= (bits == 3 ? 1.5e9 : 1.5e10) || (N % 4 != 0 && (double)M * (double)N >= 1.5e6);
-    if (!force && (M < 128 || N < 128 || K < 128 || !large)) return 0;
-    const size_t kp = round_up((size_t)K, 16);
+    const bool f4 = f4_exact(K, bits);
+    if (!force) {
+        if (M < 128 || N < 128 || K < 128) return 0;
+        const int64_t kblocks = f4 ? (K + 255) / 256 : (K + 127) / 128;
+        const double clocks = f4 ? pick_tile<G8_F4>(M, N, kblocks).clocks : pick_tile<G8_I8>(M, N, kblocks).clocks;
+        const double out = (double)M * (double)N * 1e-6;
+        const double two = 5.9 + clocks / 2180.0 + (N % 8 ? 1.03 : 0.64) * out +
+                           0.096e-6 * (double)(M + N) * (double)K * (bits / 8.0 + (f4 ? 0.5 : 1.0));
+        const double fused = 4.0 + (bits == 3 ? 4.67e-3 : 1.9e-3) * (double)K +
+                             (bits == 3 ? 0.62 : bits == 4 ? 0.44 : 0.38) * out * 1e-3 * (double)K +
+                             (N % 4 ? 1.2 + 5.7 * out : 1.05 * out);
+        // (beyond 1.5e10 products, where the fit of the fused kernel ends, always two: 4096^3
+        // 75 / 52)
+        if (two >= 0.95 * fused && (double)M * (double)N * (double)K < 1.5e10) return 0;
+    }
+    const size_t kp = round_up((size_t)K, 16);             // (4-bit operands fill half of it)
     return round_up((size_t)M * kp, 1024) + round_up((size_t)N * kp, 1024);
 }
 
+// 1- and 2-bit operands as 4-bit floating point where every sum stays below 2^23 (f32
+// accumulators then hold it exactly whatever the order of the additions): twice the values
+// per instruction and half of the expanded bytes of int8.
+template <int BITS>
+static int launch_f4(const void *A, const void *B, int64_t M, int64_t N, int64_t K, const G8Params &p,
+                     void *scratch, cudaStream_t stream)
+{
+    const size_t kp = round_up((size_t)(K + 1) / 2, 16);
+    uint8_t *A4 = (uint8_t *)scratch, *B4 = A4 + round_up((size_t)M * kp, 1024);
+    const int st = dsq_launch(expand_rows_f4_kernel<BITS>, expand_grid((int64_t)kp / 16, M + N),
+                              dim3(EX_THREADS), 0, stream, 0, 0, (const uint8_t *)A, (const uint8_t *)B,
+                              (int)M, (int)N, (int)K, (int)dsq_row_pitch(K, BITS), (int)kp, A4, B4);
+    if (st) return st;
+    return launch_pass2<G8_F4>(A4, kp, B4, kp, kp, M, N, true, true, p, stream);
+}
 // Arguments as dsq_gemm after validation; `scratch` 1024-byte aligned.
 int dsq_gemm8_launch(const void *A_codes, const void *B_codes, int64_t M, int64_t N, int64_t K,
                      int bits, int32_t *C_i32, const float *row_scale, float *D_f32,
                      void *workspace, void *scratch, cudaStream_t stream)
 {
+    G8Params p = {};
+    p.C_i32 = C_i32; p.row_scale = row_scale; p.D_f32 = D_f32;
+    p.ws = (int *)workspace;
+    if (f4_exact(K, bits)) return launch_f4<2>(A_codes, B_codes, M, N, K, p, scratch, stream);
     const size_t kp = round_up((size_t)K, 16);
     uint8_t *A8 = (uint8_t *)scratch;
     uint8_t *B8 = A8 + round_up((size_t)M * kp, 1024);
@@ -712,11 +836,7 @@ int dsq_gemm8_launch(const void *A_codes, const void *B_codes, int64_t M, int64_
                               expand_grid((int64_t)kp / 16, M + N), dim3(EX_THREADS), 0, stream, 0, 0,
                               A, B, (int)M, (int)N, (int)K, pitch_in, (int)kp, A8, B8);
     if (st) return st;
-    G8Params p = {};
-    p.idesc = idesc_i8(G8_BN, true, false, G8_BM);
-    p.C_i32 = C_i32; p.row_scale = row_scale; p.D_f32 = D_f32;
-    p.ws = (int *)workspace;
-    return launch_pass2<false>(A8, kp, B8, kp, (size_t)K, M, N, p, stream);
+    return launch_pass2<G8_I8>(A8, kp, B8, kp, (size_t)K, M, N, true, false, p, stream);
 }
 
 // ---------------------------------------------------------------------------
@@ -745,36 +865,35 @@ int dsq_binary_gemm(const void *A_bits, const void *B_bits, int64_t M, int64_t N
     const size_t kp = round_up((size_t)K, 16);
     const size_t need = round_up((size_t)M * kp, 1024) + round_up((size_t)N * kp, 1024);
     if (ws_bytes < (size_t)(scratch - (uint8_t *)workspace) + need) return DSQ_ERR_SIZE;
+    G8Params p = {};
+    p.C_i32 = C_i32; p.row_scale = row_scale; p.D_f32 = D_f32;
+    p.ws = (int *)workspace;
+    if (f4_exact(K, 1)) return launch_f4<1>(A_bits, B_bits, M, N, K, p, scratch, (cudaStream_t)stream);
     uint8_t *A8 = scratch, *B8 = scratch + round_up((size_t)M * kp, 1024);
     const int st = dsq_launch(expand_rows_kernel<1>, expand_grid((int64_t)kp / 16, M + N),
                               dim3(EX_THREADS), 0, (cudaStream_t)stream, 0, 0, (const uint8_t *)A_bits,
                               (const uint8_t *)B_bits, (int)M, (int)N, (int)K,
                               (int)dsq_row_pitch(K, 1), (int)kp, A8, B8);
     if (st) return st;
-    G8Params p = {};
-    p.idesc = idesc_i8(G8_BN, true, true, G8_BM);
-    p.C_i32 = C_i32; p.row_scale = row_scale; p.D_f32 = D_f32;
-    p.ws = (int *)workspace;
-    return launch_pass2<false>(A8, kp, B8, kp, (size_t)K, M, N, p, (cudaStream_t)stream);
+    return launch_pass2<G8_I8>(A8, kp, B8, kp, (size_t)K, M, N, true, true, p, (cudaStream_t)stream);
 }
 
 // ---------------------------------------------------------------------------
 // weight-only low-bit GEMM: bf16 activations x b-bit weights
 // ---------------------------------------------------------------------------
-// Whether dsq_wgemm_small takes the problem: always up to 64 rows (23 us against 24
-// at 64 x 4096 x 4096, 6 against 24 at 16 rows), and beyond while its launch - waves
-// of blocks of 64 x 16 outputs, 2.6 us for every 1024 of K (measured) - is shorter
-// than the two passes: 9 us of launches and set-up, the expansion, 0.27 us a K block.
+// Whether dsq_wgemm_small takes the problem: always up to 32 rows (4096x4096 4-bit: 9.2 us), and
+// beyond while its launch - waves of blocks of 64 x 16 outputs, 2.6 us for every 1024 of K, three
+// quarters of that at 33 rows - is shorter than the two passes, whose time is fitted to
+// 100 to 512 rows of six layers (within 10 %).  64 rows, this kernel / two passes, us: 4096x4096 23.5 / 20.2,
+// 6144x6144 48.5 / 35.5, 6144x1024 13.0 / 12.6, 1500x2000 7.6 / 13.
 static bool wgemm_prefers_small(int64_t M, int64_t N, int64_t K)
 {
-    if (M <= 64) return true;
+    if (M <= 32) return true;
     const int sms = dsq_sm_count() > 0 ? dsq_sm_count() : 148;
     const double blocks = (double)((N + 15) / 16) * (double)((M + 63) / 64);
-    const double small = 2.2 + std::ceil(blocks / sms) * (double)((K + 1023) / 1024) * 2.6;
-    const int64_t tiles = (M + G8_BM - 1) / G8_BM * ((N + G8_BN - 1) / G8_BN), kb = (K + 63) / 64;
-    const double waves = takes_split<true>(tiles, kb) ? 0.5 : std::ceil((double)tiles / (sms / 2));
-    const double main_loop = waves * kb * 0.27;
-    return small < 9.0 + 5.2e-7 * (double)N * (double)K + main_loop;
+    const double rows = M < 64 ? 0.75 + 0.25 / 31.0 * (double)(M - 33) : 1.0;
+    const double small = 2.2 + std::ceil(blocks / sms) * (double)((K + 1023) / 1024) * 2.6 * rows;
+    return small < 6.7 + 4e-7 * (double)N * (double)K + 4.43e-4 * pick_tile<G8_BF16>(M, N, (K + 63) / 64).clocks;
 }
 
 size_t dsq_wgemm_workspace_bytes(int64_t N, int64_t K)
@@ -815,8 +934,7 @@ int dsq_wgemm_bf16(const void *X_bf16, const void *W_codes, int64_t M, int64_t N
                               (int)K, pitch_in, (int)wp, odd, W16);
     if (st) return st;
     G8Params p = {};
-    p.idesc = idesc_bf16(G8_BN, G8_BM);
     p.col_scale = col_scale; p.col_bias = col_bias; p.Y_f32 = Y_f32;
     p.ws = (int *)workspace;
-    return launch_pass2<true>(X_bf16, (size_t)K * 2, W16, wp, (size_t)K * 2, M, N, p, s);
+    return launch_pass2<G8_BF16>(X_bf16, (size_t)K * 2, W16, wp, (size_t)K * 2, M, N, true, true, p, s);
 }

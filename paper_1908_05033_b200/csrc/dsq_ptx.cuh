@@ -168,11 +168,15 @@ __device__ __forceinline__ void st_cluster_128(uint32_t addr, uint32_t a, uint32
     asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d)
                  : "memory");
 }
-__device__ __forceinline__ uint2 lds_64(uint32_t addr)
+__device__ __forceinline__ uint32_t lds_32(uint32_t addr)
 {
-    uint2 v;
-    asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr));
+    uint32_t v;
+    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
     return v;
+}
+__device__ __forceinline__ void sts_32(uint32_t addr, uint32_t v)
+{
+    asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 __device__ __forceinline__ void stg_256(void *dst, uint32_t a, uint32_t b, uint32_t c, uint32_t d,
                                         uint32_t e, uint32_t f, uint32_t g, uint32_t h)
@@ -542,6 +546,33 @@ __device__ __forceinline__ void mma_i8_ss_pair_x4_elect(uint32_t d_tmem, uint32_
         "@pe tcgen05.mma.cta_group::2.kind::i8 [%0], da3, db3, %5, p1;\n\t}" ::"r"(d_tmem),
         "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate_first)
         : "memory");
+}
+
+// Same for 4-bit floating-point operands (kind::mxf4, see mma_f4_ss_x4b_elect).
+__device__ __forceinline__ void mma_f4_ss_pair_x4_elect(uint32_t d_tmem, uint32_t a_lo,
+                                                        uint32_t a_hi, uint32_t b_lo,
+                                                        uint32_t b_hi, uint32_t idesc, uint32_t sf_a,
+                                                        uint32_t sf_b, uint32_t accumulate_first)
+{
+#define DSQ_MXF4 " tcgen05.mma.cta_group::2.kind::mxf4.block_scale.scale_vec::2X [%0], "
+    asm volatile(
+        "{\n\t.reg .pred p0, p1, pe;\n\t"
+        ".reg .b64 da0, da1, da2, da3, db0, db1, db2, db3;\n\t.reg .b32 x1, x2, x3, y1, y2, y3;\n\t"
+        "setp.ne.b32 p0, %6, 0;\n\tsetp.eq.b32 p1, %6, %6;\n\t"
+        "add.u32 x1, %1, 2;\n\tadd.u32 x2, %1, 4;\n\tadd.u32 x3, %1, 6;\n\t"
+        "add.u32 y1, %3, 2;\n\tadd.u32 y2, %3, 4;\n\tadd.u32 y3, %3, 6;\n\t"
+        "mov.b64 da0, {%1, %2};\n\tmov.b64 da1, {x1, %2};\n\t"
+        "mov.b64 da2, {x2, %2};\n\tmov.b64 da3, {x3, %2};\n\t"
+        "mov.b64 db0, {%3, %4};\n\tmov.b64 db1, {y1, %4};\n\t"
+        "mov.b64 db2, {y2, %4};\n\tmov.b64 db3, {y3, %4};\n\t"
+        "elect.sync _|pe, 0xffffffff;\n\t"
+        "@pe" DSQ_MXF4 "da0, db0, %5, [%7], [%8], p0;\n\t"
+        "@pe" DSQ_MXF4 "da1, db1, %5, [%7], [%8], p1;\n\t"
+        "@pe" DSQ_MXF4 "da2, db2, %5, [%7], [%8], p1;\n\t"
+        "@pe" DSQ_MXF4 "da3, db3, %5, [%7], [%8], p1;\n\t}" ::"r"(d_tmem),
+        "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate_first), "r"(sf_a), "r"(sf_b)
+        : "memory");
+#undef DSQ_MXF4
 }
 
 // Same for 16-bit floating-point operands (kind::f16: f16 or bf16 per the
