@@ -598,7 +598,8 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
         const uint32_t b_lo_base = desc_lo + (smem_u32(smem + L.b_tiles) >> 4);
         const int BST = p.b_stages;
         int aslot = 0, st = 0;
-        uint32_t aph = 0, bph = 0;
+        uint32_t aph = 0, bph = 0, ready = 0u;
+        uint4 tn = p.x_off[0];
         bool ok = !F4 || wait_bar_warp(bar_scales, 0u, ctl, 14);
 #pragma unroll 1
         for (int it = 0; ok && it < my_tiles; ++it) {
@@ -614,17 +615,10 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                 if (pl == 0) W3_STAMP(5, it);
                 tc_fence_after_sync();
                 const uint32_t x_lo = a_lo_base + aslot * (a_slot_bytes >> 4);
-                if (p.b_res) st = pl * p.kpp;
-#pragma unroll 1
-                for (int kk = 0; kk < p.kpp; ++kk) {
-                    if (!p.b_res || it == 0) {
-                        if (!(ok = wait_bar_warp(bar_b_full(st), bph, ctl, 10))) break;
-                        tc_fence_after_sync();
-                    }
-                    // (slots and stages lie below 256 KB, so the sums stay inside the
-                    // 14-bit address field)
-                    const uint32_t w_lo = b_lo_base + st * (b_stage_bytes >> 4);
-                    const uint4 t = p.x_off[kk];
+                // (slots and stages lie below 256 KB, so the sums stay inside the
+                // 14-bit address field)
+                auto issue = [&](uint4 t, int stage) {
+                    const uint32_t w_lo = b_lo_base + stage * (b_stage_bytes >> 4);
                     const uint32_t x0 = x_lo + t.x, x1 = t.y == MMA_NONE ? t.y : x_lo + t.y,
                                    x2 = t.z == MMA_NONE ? t.z : x_lo + t.z,
                                    x3 = t.w == MMA_NONE ? t.w : x_lo + t.w;
@@ -636,11 +630,34 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                     else
                         mma_i8_ss_x4_elect(d_tmem, x0, x1, x2, x3, desc_hi, w_lo, desc_hi, idesc, first);
                     first = 1u;
-                    if (!p.b_res) {
-                        mma_commit_elect(bar_b_empty(st));
+                };
+                if (p.b_res) {
+                    st = pl * p.kpp;
+#pragma unroll 1
+                    for (int kk = 0; kk < p.kpp; ++kk, ++st) {
+                        if (it == 0) {
+                            if (!(ok = wait_bar_warp(bar_b_full(st), bph, ctl, 10))) break;
+                            tc_fence_after_sync();
+                        }
+                        issue(p.x_off[kk], st);
+                    }
+                } else {
+                    // what the next K step needs is asked for before this one is issued, so that
+                    // its latency passes meanwhile (4-bit 7x7 512->512 14.0 -> 12.2 us, 2-bit 28x28
+                    // 512->512 at batch 32 26.7 -> 24.5)
+#pragma unroll 1
+                    for (int kk = 0; kk < p.kpp; ++kk) {
+                        if (!__all_sync(0xffffffffu, ready) &&
+                            !(ok = wait_bar_warp(bar_b_full(st), bph, ctl, 10)))
+                            break;
+                        tc_fence_after_sync();
+                        const uint4 t = tn;
+                        const int stage = st;
+                        tn = p.x_off[kk + 1 == p.kpp ? 0 : kk + 1];
                         if (++st == BST) { st = 0; bph ^= 1u; }
-                    } else {
-                        ++st;
+                        ready = mbar_test_wait(bar_b_full(st), bph);
+                        issue(t, stage);
+                        mma_commit_elect(bar_b_empty(stage));
                     }
                 }
                 if (ok) mma_commit_elect(bar_a_empty(aslot));
@@ -1391,7 +1408,7 @@ int dsq_w8_build(void *blob, const dsq_conv_t *conv, int bits, cudaStream_t stre
 // Positions of a transposed tile, at most `most`: what fills as many passes of the `mstep`
 // CTAs of an N tile as the largest tile would take, so that the last pass is no emptier than
 // the others.  (4-bit, batch 64, largest / this: 28x28 128->128 11.6 / 10.8 us, 14x14 256->256
-// 11.3 / 10.5, 7x7 512->512 15.6 / 14.2; 2-bit 28x28 512->512 at batch 32 27.9 / 26.9.)  No
+// 11.3 / 10.5, 7x7 512->512 15.6 / 14.2 (12.2 since); 2-bit 28x28 512->512 at batch 32 27.9 / 26.9.)  No
 // fewer than 112: the instructions get shorter, the weights' K steps do not (28x28 128->128 at
 // batch 16: 96 to 144 positions alike).  With more than four passes the last one weighs little, and
 // larger tiles have less overhead each (64->64 at 56x56, six passes: 256 positions 15.4, 240
@@ -1476,7 +1493,7 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
     // 64 output channels want pairs of image rows (`pair`), for which the weights come from the
     // blob's expanded copy or, at 3 bits, from the expansion warps.  Batch 64, transposed /
     // plain, us: 64->64 at 56x56 4-bit 12.2 / 21.1, 3-bit 17.3 / 63.8; 128->128 at 28x28 10.0 / 12.1,
-    // 14.0 / 23.6; 256->256 at 14x14 10.4 / 11.7, 13.3 / 23.5; 512->512 at 7x7 14.0 / 16.0, 19.1 / 31.0.
+    // 14.0 / 23.6; 256->256 at 14x14 10.4 / 11.7, 13.3 / 23.5; 512->512 at 7x7 12.2 / 16.0, 19.1 / 31.0.
     // the codes epilogues want the requantiser range to start at 0, too
     float r_hi = 0.f;
     if (epi_kind != DSQ_EPI_GENERAL) {

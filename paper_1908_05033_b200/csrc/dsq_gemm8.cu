@@ -493,6 +493,8 @@ gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
             uint32_t it = 0, ph = 0;
             int s = 0;
             bool ok = true;
+            // (a stage is asked for while the one before it is being issued)
+            uint32_t ready = mbar_test_wait<true>(bar_full(0), 0u);
             for (int tile = pair; ok && tile < total_tiles; tile += npairs, ++it) {
                 const int b = it & 1;
                 if (!(ok = wait_bar_warp<true>(bar_acc_empty(b), ((it >> 1) & 1u) ^ 1u, ctl, 22)))
@@ -500,11 +502,16 @@ gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
                 tc_fence_after_sync();
                 const uint32_t d_tmem = tmem_base + b * ACC;
                 for (int kb = kb0; kb < kb1; ++kb) {
-                    if (!(ok = wait_bar_warp<true>(bar_full(s), ph, ctl, 23))) break;
+                    if (!__all_sync(0xffffffffu, ready) &&
+                        !(ok = wait_bar_warp<true>(bar_full(s), ph, ctl, 23)))
+                        break;
                     tc_fence_after_sync();
+                    const uint32_t bar_used = bar_empty(s);
                     // (a stage lies below 256 KB: the address field does not overflow)
                     const uint32_t ad = (uint32_t)desc + (uint32_t)s * (uint32_t)(p.stage_bytes >> 4);
                     const uint32_t bd = ad + (G8_OP_BYTES >> 4);
+                    if (++s == p.stages) { s = 0; ph ^= 1u; }
+                    ready = mbar_test_wait<true>(bar_full(s), ph);
                     if (KIND == G8_BF16)
                         mma_f16_ss_pair_x4_elect(d_tmem, ad, hi, bd, hi, idesc, (uint32_t)(kb - kb0));
                     else if (KIND == G8_F4)
@@ -512,8 +519,7 @@ gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
                                                 tmem_base + G8_F4_SF + 16, (uint32_t)(kb - kb0));
                     else
                         mma_i8_ss_pair_x4_elect(d_tmem, ad, hi, bd, hi, idesc, (uint32_t)(kb - kb0));
-                    mma_commit_pair_elect(bar_empty(s), pair_mask);
-                    if (++s == p.stages) { s = 0; ph ^= 1u; }
+                    mma_commit_pair_elect(bar_used, pair_mask);
                 }
                 if (ok) mma_commit_pair_elect(bar_acc_full(b), pair_mask);
             }
