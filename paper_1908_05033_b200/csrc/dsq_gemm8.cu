@@ -458,6 +458,7 @@ gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
     const int kb1 = S == 1 ? p.kblocks : ((int)split + 1) * p.kblocks / S;
     const int total_tiles = p.m_tiles * p.n_tiles;
     grid_dependency_wait();
+    grid_launch_dependents();
 
     if (warp == G8_WARP_TMA) {
         // ---------------- TMA producer (one thread per CTA) -----------------

@@ -1,13 +1,20 @@
 // The workspace of the tensor-core kernels: its size, clearing it, reading its status.
+#include <chrono>
+
 #include "dsq_launch.h"
 
 namespace {
 
 // Hands a workspace's status word to the host and clears it.  Written straight into
 // page-locked host memory: a copy to pageable memory is staged and took 3 us more of
-// every call that reads the status (binary GEMM 3136x512x4608: 41 -> 38 us).
+// every call that reads the status (binary GEMM 3136x512x4608: 41 -> 38 us).  Launched
+// dependently: it starts beside the kernel whose status it reads and waits for it.
+constexpr int STATUS_PENDING = 1;        // (statuses are 0 or negative)
 __global__ void status_kernel(int *ws, volatile int *host)
 {
+#ifdef __CUDA_ARCH__
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+#endif
     const int st = *(volatile int *)(ws + DSQ_WS_STATUS);
     if (st) ws[DSQ_WS_STATUS] = ws[DSQ_WS_DETAIL] = 0;
     *host = st;
@@ -68,12 +75,18 @@ int dsq_workspace_status(void *ws, void *stream)
     static thread_local StatusMailbox box;
     int *const word = box.get();
     if (word && on_current_device(ws)) {
-        *word = 0;
+        *(volatile int *)word = STATUS_PENDING;
         int *w = (int *)ws;
         void *argv[] = {(void *)&w, (void *)&word};
-        const DsqGrid one = {(const void *)status_kernel, dim3(1), dim3(1), 0, 0, 0};
+        const DsqGrid one = {(const void *)status_kernel, dim3(1), dim3(1), 0, 1, 0};
         const int st = dsq_launch_args(one, argv, s);
         if (st) return st;
+        // The word is watched for a while first: the stream's own wait, entered when its work
+        // is as good as done, returns sooner than one that was asleep for it.
+        const auto t0 = std::chrono::steady_clock::now();
+        bool pending = true;
+        while (pending && std::chrono::steady_clock::now() - t0 < std::chrono::microseconds(200))
+            for (int i = 0; i < 64 && pending; ++i) pending = *(volatile int *)word == STATUS_PENDING;
         DSQ_CUDA_TRY(cudaStreamSynchronize(s));
         return *(volatile int *)word;
     }
