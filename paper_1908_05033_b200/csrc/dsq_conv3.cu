@@ -362,6 +362,10 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
     const uint32_t b_stage_bytes = (uint32_t)BN * 128u;
     const uint32_t b_packed_bytes = (uint32_t)BN * p.pk;
     const int img_positions = p.Hp * p.Wp;
+    // F4: where the weights come expanded, their expansion warps work on the window, too (2-bit
+    // 64->64 at 56x56 with residual 14.4 -> 13.7 us, 14x14 256->256 8.1 -> 7.9; the int8 form's epilogue
+    // loses more to them than the first window gains: 15.9 -> 16.6)
+    const int a_warps = F4 && p.w8 ? W3_NUM_A_WARPS + W3_NUM_B_WARPS : W3_NUM_A_WARPS;
 
     const uint32_t bars = smem_u32(smem + L.bars);
     auto bar_a_full = [&](int s) { return bars + 8u * s; };
@@ -386,12 +390,12 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
     if (warp == 0) W3_STAMP(13, 9);
     if (threadIdx.x == 0) {
         for (int s = 0; s < W3_A_SLOTS; ++s) {
-            mbar_init(bar_a_full(s), W3_NUM_A_WARPS);
+            mbar_init(bar_a_full(s), a_warps);
             mbar_init(bar_a_empty(s), 1);            // tcgen05.commit
         }
         for (int s = 0; s < W3_MAX_AS; ++s) {
             mbar_init(bar_as_full(s), 1);            // TMA producer (+ bytes)
-            mbar_init(bar_as_empty(s), W3_NUM_A_WARPS);
+            mbar_init(bar_as_empty(s), a_warps);
         }
         for (int s = 0; s < W3_MAX_BP; ++s) {
             mbar_init(bar_bp_full(s), 1);            // TMA producer (+ bytes)
@@ -672,7 +676,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
             mma_commit_elect(bar_drain);
             wait_bar_drain(bar_drain, 0u);
         }
-    } else if (warp < W3_WARP_B0) {
+    } else if (warp < W3_WARP_A0 + a_warps) {
         // ---------------- A: expand the staged window -------------------------------
         const int tid = threadIdx.x - W3_WARP_A0 * 32;
         const int n_tasks = p.apx * p.cpp;
@@ -697,7 +701,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                 const int nq = p.E >= 128 ? 8 : 4;
                 const bool half_rows = p.rb == 64;
 #pragma unroll 1
-                for (int px = tid; px < p.apx; px += W3_NUM_A_WARPS * 32) {
+                for (int px = tid; px < p.apx; px += a_warps * 32) {
                     uint32_t w[12];
 #pragma unroll
                     for (int l = 0; l < 3; ++l) {
@@ -716,7 +720,7 @@ dsq_win3_kernel(const __grid_constant__ CUtensorMap tmap_b,
                 }
             } else
 #pragma unroll 4
-            for (int t = tid; t < n_tasks; t += W3_NUM_A_WARPS * 32) {
+            for (int t = tid; t < n_tasks; t += a_warps * 32) {
                 const int px = t >> lcpp, ch = t & (p.cpp - 1);
                 const uint4 v = lds_128(src + 16u * t);
                 // (16-byte chunks XOR-ed with address bits 7..9, of 64-byte rows bits 7..8, of
