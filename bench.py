@@ -38,8 +38,8 @@ import dsq_inputs  # noqa: E402
 # DRAM traffic of the tensor-core convolution kernels per launch in this
 # workload, from one ncu capture (profiles/bench_launch_list.txt); valid only
 # for the kernel sources it was taken on (checked by hash)
-TRAFFIC = {"bytes_per_launch": 4974255,
-           "sources_sha256": "fa0c9b9798b02688645fc2cf06a825ef0b003e68606dce4f9ed710cf0d260424"}
+TRAFFIC = {"bytes_per_launch": 4973514,
+           "sources_sha256": "cdc731f6e88726472cb7e48f29e745cf6707dbd81037eb02f5844df7e8158ce6"}
 
 WORKLOAD = "resnet18-shaped stack, 4-bit W/A, batch 64, 56x56x64 stem output, 19 convs"
 METRIC = "4-bit ResNet-18 conv-stack throughput (effective low-bit conv TOPS alongside)"

@@ -1,4 +1,4 @@
-// 3x3, stride 1, pad 1 low-bit convolution on the tensor cores, with the A
+// 3x3, pad 1 low-bit convolution (strides 1 and 2) on the tensor cores, with the A
 // operand read from an expanded WINDOW of the input in shared memory
 // (Algorithm 1 step 5 on codes, plus the fused epilogue of steps 4, 1, 3).
 //
@@ -33,12 +33,14 @@
 //     of the whole layer sit in shared memory, the residual words of a tile
 //     are fetched before its accumulators are waited for.
 //
-// Measured: with the A operand read through a shared-memory descriptor an
-// instruction takes about 110-130 clocks whatever its N (the tensor core
-// fetches A at roughly 32 bytes a clock), so only 256-wide N tiles run the
-// tensor pipe at its full rate; a variant that copied each K step of the
-// window to tensor memory (ld.shared + tcgen05.st, A taken from there) was
-// slower than this one at every layer size and is not kept.
+// Measured: alone on an SM, instructions issued four at a time run for N / 2 clocks each
+// (40 at least; both operands through shared-memory descriptors).  In this kernel a block of
+// four takes 480 to 700: the issuing warp shares its scheduler with epilogue warps, and the
+// operands' reads (12 KB an instruction of 256 columns) share the shared-memory port with the
+// expansion.  So instructions should be wide and few.  (Two issuing warps on alternate tiles,
+// single instructions in a tight loop: no faster, slower.  A variant that copied each K step
+// of the window to tensor memory - ld.shared + tcgen05.st, A taken from there - was
+// slower than this one at every layer size.)
 //
 // Wide images (W + 1 > 139) would need a window of more than 416 pixels; they
 // are staged as three bands of 136 pixels, one per filter row, instead.
@@ -262,9 +264,8 @@ __device__ __forceinline__ uint32_t w3_operand(uint32_t w, int c, uint32_t orv)
     else return expand_word<BITS, SIGNED>(w, c, orv);
 }
 
-// Transposed tiles (template parameter TR).  An instruction whose A operand
-// comes through a shared-memory descriptor takes ~130 clocks whatever its N, so
-// it should carry N = 256.  With the roles swapped - A = 128 weight rows of the K
+// Transposed tiles (template parameter TR).  An instruction should carry as many columns
+// as there are (see above).  With the roles swapped - A = 128 weight rows of the K
 // step, B = 256 rows of the window - every instruction is 128 x 256 x 32 even
 // for 64 or 128 output channels.  The accumulator then has output CHANNELS on
 // the tensor-memory lanes and POSITIONS in the columns: an epilogue thread owns

@@ -33,15 +33,15 @@ int dsq_set_dependent_launch(int on);
  * restores the default). */
 int dsq_set_wait_limit_ns(long long ns);
 
-/* 3x3 stride-1 convolutions on an expanded shared-memory window
+/* 3x3 convolutions on an expanded shared-memory window
  * (dsq_conv3.cu): 1 = where it is the faster kernel (default), 0 = never (the
  * im2col kernel takes them), 3 = wherever the geometry allows (transposed
  * tiles where those fit), 4 (and 2) = as 3 but plain tiles only. */
 int dsq_set_conv3_window(int mode);
 
 /* Window kernel: 1 = weight tiles come by TMA from the blob's pre-expanded
- * int8 copy where it exists (default), 0 = always expand the packed rows in
- * the kernel. */
+ * copy where it exists and 2-bit layers take 4-bit floating-point operands
+ * (default), 0 = always expand the packed rows in the kernel, to int8. */
 int dsq_set_conv3_expanded_weights(int on);
 
 /* dsq_gemm with a workspace large enough for the expanded operands: 1 = take
