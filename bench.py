@@ -473,7 +473,7 @@ def run_ours(args):
     int8_peak = 2.0 * bf16_peak                 # int8 : bf16 nominal ratio 2
     achieved = 2.0 * macs_step / (conv_in_step_ms * 1e-3) / 1e12
     roofline = {
-        "kernel": f"dsq_win3_kernel (3x3 stride 1) + dsq_tc_kernel (strided 3x3) + dsq_pw_kernel (1x1) "
+        "kernel": f"dsq_win3_kernel (3x3) + dsq_tc_kernel (last strided 3x3) + dsq_pw_kernel (1x1) "
                   f"behind dsq_conv2d, {n_conv} launches per step",
         "bound": "tensor", "achieved": achieved, "peak": int8_peak, "unit": "TOP/s",
         "frac": achieved / int8_peak,
