@@ -703,9 +703,10 @@ int resident_clusters()
 // Tile width, and whether K is split over the two pairs of a cluster, for a problem of
 // kblocks K blocks.  A K block of a tile takes 2.5 BN clocks (at 1.9 GHz; the tensor cores), and
 // of narrow tiles 330 + 0.72 BN (what a block costs whatever its width): fitted to 4096^3 4-bit at 96 to
-// 256 columns, 76.7 59.0 54.1 50.2 55.4 52.6 us.  So the width that fills the pairs' waves is
-// taken: 4096^3 4.8 waves of 192 columns instead of 3.5 of 256, 2500x1111x1777 70 tiles of 160
-// instead of 50 of 256, 3136x512x4608 at 1 bit 52 of 128 instead of 26 (and no split).  Split: only
+// 256 columns in a graph, 76.7 59.0 54.1 50.2 55.4 52.6 us; the widest tiles a tenth less, for they read
+// their operands least often (among other passes, with inputs that are not in the L2, 58.4 us with 256
+// columns, 59.4 with 192).  So the width that fills the pairs' waves is taken: 2500x1111x1777 70
+// tiles of 160 instead of 50 of 256, 3136x512x4608 at 1 bit 52 of 128 instead of 26 (and no split).  Split: only
 // with all the clusters resident at once and twelve K blocks a part; the exchange costs about
 // as much as eight.  (Four pairs a cluster gained nothing more: 15 such clusters are resident and
 // the exchange doubles.)
@@ -725,7 +726,7 @@ G8Tile pick_tile(int64_t M, int64_t N, int64_t kblocks)
             const int64_t tiles = m_tiles * ((N + bn - 1) / bn);
             if (split == 2 && tiles > resident_clusters<KIND, 2>()) continue;
             const int64_t waves = split == 2 ? 1 : (tiles + pairs - 1) / pairs;
-            const double block = std::max(2.5 * bn, 330.0 + 0.72 * bn);
+            const double block = std::max(2.5 * bn, 330.0 + 0.72 * bn) * (bn == 256 ? 0.9 : 1.0);
             const double clocks = (double)waves * ((double)((kblocks + split - 1) / split) * block + 400.0) +
                                   (split == 2 ? 4000 + 20 * bn : 20 * bn);
             if (best.bn == 0 || clocks < best.clocks) best = G8Tile{bn, split, clocks};
