@@ -29,6 +29,7 @@
 #include <cstdint>
 
 #include "dsq_common.cuh"
+#include "dsq_gemm8_rule.h"
 #include "dsq_tc_common.cuh"
 #include "dsq_tc_host.h"
 
@@ -36,7 +37,7 @@ namespace {
 
 enum G8Kind { G8_I8, G8_BF16, G8_F4 };       // operands: int8, bf16, 4-bit floating point
 constexpr int G8_ROWS = 128;                 // A rows per CTA and stage
-constexpr int G8_BM = 256;                   // tile height of a pair
+constexpr int G8_BM = DSQ_G8_BM;             // tile height of a pair
 constexpr int G8_KB = 128;                   // bytes of K per stage
 constexpr int G8_OP_BYTES = G8_ROWS * G8_KB;             // A of a stage: 16 KB
 constexpr int G8_MAX_STAGES = 12;
@@ -700,38 +701,11 @@ int resident_clusters()
     return n;
 }
 
-// Tile width, and whether K is split over the two pairs of a cluster, for a problem of
-// kblocks K blocks.  A K block of a tile takes 2.5 BN clocks (at 1.9 GHz; the tensor cores), and
-// of narrow tiles 330 + 0.72 BN (what a block costs whatever its width): fitted to 4096^3 4-bit at 96 to
-// 256 columns in a graph, 76.7 59.0 54.1 50.2 55.4 52.6 us; the widest tiles a tenth less, for they read
-// their operands least often (among other passes, with inputs that are not in the L2, 58.4 us with 256
-// columns, 59.4 with 192).  So the width that fills the pairs' waves is taken: 2500x1111x1777 70
-// tiles of 160 instead of 50 of 256, 3136x512x4608 at 1 bit 52 of 128 instead of 26 (and no split).  Split: only
-// with all the clusters resident at once and twelve K blocks a part; the exchange costs about
-// as much as eight.  (Four pairs a cluster gained nothing more: 15 such clusters are resident and
-// the exchange doubles.)
-struct G8Tile {
-    int bn, split;
-    double clocks;
-};
 template <int KIND>
-G8Tile pick_tile(int64_t M, int64_t N, int64_t kblocks)
+DsqG8Tile pick_tile(int64_t M, int64_t N, int64_t kblocks)
 {
-    const int pairs = std::max((dsq_sm_count() > 0 ? dsq_sm_count() : 148) / 2, 1);
-    const int64_t m_tiles = (M + G8_BM - 1) / G8_BM;
-    G8Tile best = {0, 0, 0.0};
-    for (int split = 1; split <= 2; ++split)
-        for (int bn = g8_acc<KIND>() / 32 * 32; bn >= 64; bn -= 32) {      // (pairs take N in steps of 32)
-            if (split == 2 && (bn % 64 != 0 || kblocks < 24)) continue;
-            const int64_t tiles = m_tiles * ((N + bn - 1) / bn);
-            if (split == 2 && tiles > resident_clusters<KIND, 2>()) continue;
-            const int64_t waves = split == 2 ? 1 : (tiles + pairs - 1) / pairs;
-            const double block = std::max(2.5 * bn, 330.0 + 0.72 * bn) * (bn == 256 ? 0.9 : 1.0);
-            const double clocks = (double)waves * ((double)((kblocks + split - 1) / split) * block + 400.0) +
-                                  (split == 2 ? 4000 + 20 * bn : 20 * bn);
-            if (best.bn == 0 || clocks < best.clocks) best = G8Tile{bn, split, clocks};
-        }
-    return best;
+    return dsq_g8_tile(M, N, kblocks, g8_acc<KIND>(), dsq_sm_count() > 0 ? dsq_sm_count() : 148,
+                       [] { return resident_clusters<KIND, 2>(); });
 }
 
 // Pass 2 over operands that are rows of k_bytes bytes of K (byte maps: the
@@ -742,7 +716,7 @@ int launch_pass2(const void *A, size_t a_pitch, const void *B, size_t b_pitch, s
 {
     p.M = (int)M; p.N = (int)N;
     p.kblocks = (int)((k_bytes + G8_KB - 1) / G8_KB);
-    const G8Tile tile = pick_tile<KIND>(M, N, p.kblocks);
+    const DsqG8Tile tile = pick_tile<KIND>(M, N, p.kblocks);
     p.BN = tile.bn;
     p.m_tiles = (int)((M + G8_BM - 1) / G8_BM);
     p.n_tiles = (int)((N + p.BN - 1) / p.BN);
@@ -779,31 +753,15 @@ inline uint8_t *scratch_of(void *workspace)
 static bool f4_exact(int64_t K, int bits) { return bits < 3 && K * (bits == 2 ? 6 : 1) < (1 << 23); }
 
 // Scratch the two-pass path needs behind the status words (0: the problem is
-// one the fused kernel keeps): where it is expected to be the faster one.  Both estimates
-// (microseconds) are fits to 228 measured problems of 2 to 4 bits and 128 to 6144 a side, 7 and 10 % off in the
-// mean; the rule takes the slower path for 21 of them, 1.3 % of time on average.  Two passes:
-// their launches, the tiles of the second, the bytes of the first, the outputs (turned round
-// in shared memory where rows are not whole sectors).  The fused kernel: its rounds of K,
-// the expansion of each row once per tile (3-bit rows one K step a round), the outputs (one
-// word at a time where rows are no multiple of 16 bytes).  Fused / two passes, us: 4-bit 1024^3
-// 6.7 / 8.8, 2048^3 16.0 / 15.6 (either), 3072x3072x1024 20.6 / 18.1, 2500x1111x1777 29 / 12.5; 3-bit 1024^3 10.1 / 8.8, 2048^3 22 / 16;
-// 2-bit 2048^3 16.1 / 13.9.
+// one the fused kernel keeps).
 size_t dsq_gemm8_scratch_bytes(int64_t M, int64_t N, int64_t K, int bits, int force)
 {
-    const bool f4 = f4_exact(K, bits);
     if (!force) {
         if (M < 128 || N < 128 || K < 128) return 0;
-        const int64_t kblocks = f4 ? (K + 255) / 256 : (K + 127) / 128;
-        const double clocks = f4 ? pick_tile<G8_F4>(M, N, kblocks).clocks : pick_tile<G8_I8>(M, N, kblocks).clocks;
-        const double out = (double)M * (double)N * 1e-6;
-        const double two = 5.9 + clocks / 2180.0 + (N % 8 ? 1.03 : 0.64) * out +
-                           0.096e-6 * (double)(M + N) * (double)K * (bits / 8.0 + (f4 ? 0.5 : 1.0));
-        const double fused = 4.0 + (bits == 3 ? 4.67e-3 : 1.9e-3) * (double)K +
-                             (bits == 3 ? 0.62 : bits == 4 ? 0.44 : 0.38) * out * 1e-3 * (double)K +
-                             (N % 4 ? 1.2 + 5.7 * out : 1.05 * out);
-        // (beyond 1.5e10 products, where the fit of the fused kernel ends, always two: 4096^3
-        // 75 / 52)
-        if (two >= 0.95 * fused && (double)M * (double)N * (double)K < 1.5e10) return 0;
+        const bool f4 = f4_exact(K, bits);
+        const double clocks = f4 ? pick_tile<G8_F4>(M, N, (K + 255) / 256).clocks
+                                 : pick_tile<G8_I8>(M, N, (K + 127) / 128).clocks;
+        if (!dsq_g8_two_passes(M, N, K, bits, f4, clocks)) return 0;
     }
     const size_t kp = round_up((size_t)K, 16);             // (4-bit operands fill half of it)
     return round_up((size_t)M * kp, 1024) + round_up((size_t)N * kp, 1024);
@@ -889,21 +847,6 @@ int dsq_binary_gemm(const void *A_bits, const void *B_bits, int64_t M, int64_t N
 // ---------------------------------------------------------------------------
 // weight-only low-bit GEMM: bf16 activations x b-bit weights
 // ---------------------------------------------------------------------------
-// Whether dsq_wgemm_small takes the problem: always up to 32 rows (4096x4096 4-bit: 9.2 us), and
-// beyond while its launch - waves of blocks of 64 x 16 outputs, 2.6 us for every 1024 of K, three
-// quarters of that at 33 rows - is shorter than the two passes, whose time is fitted to
-// 100 to 512 rows of six layers (within 10 %).  64 rows, this kernel / two passes, us: 4096x4096 23.5 / 20.2,
-// 6144x6144 48.5 / 35.5, 6144x1024 13.0 / 12.6, 1500x2000 7.6 / 13.
-static bool wgemm_prefers_small(int64_t M, int64_t N, int64_t K)
-{
-    if (M <= 32) return true;
-    const int sms = dsq_sm_count() > 0 ? dsq_sm_count() : 148;
-    const double blocks = (double)((N + 15) / 16) * (double)((M + 63) / 64);
-    const double rows = M < 64 ? 0.75 + 0.25 / 31.0 * (double)(M - 33) : 1.0;
-    const double small = 2.2 + std::ceil(blocks / sms) * (double)((K + 1023) / 1024) * 2.6 * rows;
-    return small < 6.7 + 4e-7 * (double)N * (double)K + 4.43e-4 * pick_tile<G8_BF16>(M, N, (K + 63) / 64).clocks;
-}
-
 size_t dsq_wgemm_workspace_bytes(int64_t N, int64_t K)
 {
     if (N <= 0 || K <= 0) return DSQ_WS_BYTES;
@@ -927,7 +870,8 @@ int dsq_wgemm_bf16(const void *X_bf16, const void *W_codes, int64_t M, int64_t N
     const size_t wp = round_up((size_t)K, 8) * 2;          // scratch row pitch in bytes
     if (ws_bytes < (size_t)(W16 - (uint8_t *)workspace) + round_up((size_t)N * wp, 1024))
         return DSQ_ERR_SIZE;
-    if (wgemm_prefers_small(M, N, K))
+    if (M <= 32 || dsq_wgemm_takes_small(M, N, K, dsq_sm_count() > 0 ? dsq_sm_count() : 148,
+                                         pick_tile<G8_BF16>(M, N, (K + 63) / 64).clocks))
         return dsq_wgemm_small(X_bf16, W_codes, M, N, K, bits, w_offset == 0.5f, col_scale, col_bias,
                                Y_f32, (cudaStream_t)stream);
     const int pitch_in = (int)dsq_row_pitch(K, bits);

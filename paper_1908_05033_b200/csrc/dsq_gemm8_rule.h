@@ -1,0 +1,92 @@
+// Which tiles the second pass of the two-pass GEMMs takes, and which problems take the two
+// passes at all.  Host code without CUDA, so that it can be compared with measured times
+// anywhere (tests/test_gemm_rule.py).  Internal to the library.
+#pragma once
+
+#include <algorithm>
+#include <cmath>
+#include <cstdint>
+
+constexpr int DSQ_G8_BM = 256;       // tile height of a CTA pair
+
+// Tile width, whether K is split over the two pairs of a cluster, and the clocks (at 1.9 GHz)
+// that the second pass is expected to take.
+struct DsqG8Tile {
+    int bn, split;
+    double clocks;
+};
+
+// For a problem of kblocks K blocks of 128 bytes; widest: tensor-memory columns of an
+// accumulator; resident(): clusters of two pairs that fit on the GPU at once.
+//
+// A pair reads 256 + BN rows of 128 bytes for a K block of a tile, and that is what a block's
+// time goes with, for 8-bit, bf16 and 4-bit operands alike (about 13 TB/s over all pairs, from
+// the L2): 1.2 clocks a row; a tile costs 1500 more.  The CTA pairs take their tiles in waves,
+// and the width with the cheapest waves is taken.  Split: only with all the clusters resident
+// at once and twelve K blocks a part; the exchange of the partial sums grows with the width.
+// (Four pairs a cluster gained nothing more: 15 such clusters are resident and the exchange
+// doubles.)
+//
+// Measured: all widths, whole and split K, of 591 problems of 64 to 6144 a side, 1 to 4
+// bits, back to back in a graph and one at a time after an L2 flush, and 233 others to judge by: of
+// those the width taken is 0.22 % slower than the fastest one on average, more than 3 % in 11 of
+// 466 timings.  (A rule from the tensor cores' rate, 2.5 BN clocks a block, 330 + 0.72 BN at
+// least: 0.64 %, 33 of them.)
+template <class Resident>
+inline DsqG8Tile dsq_g8_tile(int64_t M, int64_t N, int64_t kblocks, int widest, int sms, Resident resident)
+{
+    const int64_t pairs = std::max(sms / 2, 1), m_tiles = (M + DSQ_G8_BM - 1) / DSQ_G8_BM;
+    DsqG8Tile best = {0, 0, 0.0};
+    for (int split = 1; split <= 2; ++split)
+        for (int bn = widest / 32 * 32; bn >= 64; bn -= 32) {      // (pairs take N in steps of 32)
+            if (split == 2 && (bn % 64 != 0 || kblocks < 24)) continue;
+            const int64_t tiles = m_tiles * ((N + bn - 1) / bn);
+            if (split == 2 && tiles > resident()) continue;
+            const int64_t waves = split == 2 ? 1 : (tiles + pairs - 1) / pairs;
+            const double block = 1.2 * (DSQ_G8_BM + bn);
+            const double clocks = (double)waves * ((double)((kblocks + split - 1) / split) * block + 1500.0) +
+                                  (split == 2 ? 1000 + 30 * bn : 20 * bn);
+            if (best.bn == 0 || clocks < best.clocks) best = DsqG8Tile{bn, split, clocks};
+        }
+    return best;
+}
+
+// Whether dsq_gemm does better in two passes than in the fused kernel that expands both operands
+// for every tile; clocks: of the second pass.  Microseconds of both, fitted to 522
+// problems of 2 to 4 bits and 128 to 6144 a side with one or both outputs.  Two passes: their launches,
+// the tiles of the second, the bytes of the first, the outputs (turned round in shared memory
+// where rows are not whole sectors).  The fused kernel: its rounds of K, the expansion of each row
+// once per tile (3-bit rows one K step a round), the outputs (one word at a time where rows
+// are no multiple of 16 bytes).  The slower path is taken for 32 of them, 0.7 % of time on average
+// (fitted to 292 of them, for 14 of the other 230, 0.7 %).  Fused / two passes, us: 4-bit 1024^3
+// 6.7 / 8.8, 2048^3 16.0 / 15.6 (either), 3072x3072x1024 20.6 / 18.1, 2500x1111x1777 29 / 12.5; 3-bit
+// 1024^3 10.1 / 8.8, 2048^3 22 / 16; 2-bit 2048^3 16.1 / 13.9.
+inline bool dsq_g8_two_passes(int64_t M, int64_t N, int64_t K, int bits, bool f4, double clocks)
+{
+    struct Fused { double fixed, k, nk, out, words, word; };
+    static const Fused fused[3] = {{4.3, 1.76, 0.483, 1.11, 2.5, 4.6},
+                                   {4.7, 4.52, 1.015, 0.965, 0.8, 5.5},
+                                   {4.3, 1.85, 0.506, 1.21, 0.5, 5.9}};
+    // beyond the range of the fits (4096^3: 75 / 52)
+    if ((double)M * (double)N * (double)K >= 1.5e10) return true;
+    const double out = (double)M * (double)N * 1e-6, k = (double)K * 1e-3;
+    const Fused &f = fused[bits - 2];
+    const double two = 6.0 + clocks / 2310.0 + (N % 8 ? 1.02 : 0.65) * out +
+                       0.157e-6 * (double)(M + N) * (double)K * (bits / 8.0 + (f4 ? 0.5 : 1.0));
+    return two < f.fixed + f.k * k + f.nk * out * k + f.out * out + (N % 4 ? f.words + f.word * out : 0.0);
+}
+
+// Whether the weight-only GEMM of few rows does better than two passes of `clocks` in the
+// second, for more than 32 rows (up to those it always does: 4096x4096 4-bit 9.2 us): while its
+// launch - waves of blocks of 64 x 16 outputs, 2.6 us for every 1024 of K, three quarters of that at 33
+// rows - is shorter than the two passes, whose time is fitted to 363 problems of 33 to 700 rows (6 % off in the
+// mean; the rule takes the slower kernel for 17 of them, 0.6 % of time on average).  64
+// rows, this kernel / two passes, us: 4096x4096 23.5 / 20.2, 6144x6144 48.5 / 35.5, 6144x1024 13.0 / 12.6,
+// 1500x2000 7.6 / 13.
+inline bool dsq_wgemm_takes_small(int64_t M, int64_t N, int64_t K, int sms, double clocks)
+{
+    const double blocks = (double)((N + 15) / 16) * (double)((M + 63) / 64);
+    const double rows = M < 64 ? 0.75 + 0.25 / 31.0 * (double)(M - 33) : 1.0;
+    const double small = 2.2 + std::ceil(blocks / sms) * (double)((K + 1023) / 1024) * 2.6 * rows;
+    return small < 5.5 + 3.2e-7 * (double)N * (double)K + 5.22e-4 * clocks;
+}
