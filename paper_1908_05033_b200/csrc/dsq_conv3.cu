@@ -49,6 +49,7 @@
 #include <algorithm>
 
 #include "dsq_tc_common.cuh"
+#include "dsq_conv_rule.h"
 #include "dsq_tc_host.h"
 
 // Cycle stamps of the roles of CTA 0 (profiling builds only: -DDSQ_W3_STAMPS).
@@ -72,13 +73,11 @@ extern "C" int dsq_w3_read_stamps(long long *out)
 
 namespace {
 
-constexpr int W3_BM = 128;
 constexpr int W3_WARP_TMA_B = 0, W3_WARP_MMA = 1, W3_WARP_TMA_A = 2, W3_WARP_A0 = 3,
               W3_NUM_A_WARPS = 4, W3_WARP_B0 = 7, W3_NUM_B_WARPS = 8, W3_WARP_E0 = 15,
               W3_NUM_E_WARPS = 16, W3_NUM_WARPS = 31;
 constexpr int W3_B_GROUP_WARPS = W3_NUM_B_WARPS / 2;   // two B groups take alternate K steps
 constexpr int W3_EPQ = W3_NUM_E_WARPS / 4;   // epilogue warps per tensor-memory lane quarter
-constexpr int W3_MAX_COUT = 1024;            // scale / bias of the layer stay in shared memory
 constexpr int W3_THREADS = W3_NUM_WARPS * 32;
 constexpr int W3_A_SLOTS = 2;          // expanded windows, at most
 constexpr int W3_MAX_BP = 4;           // packed B ring slots
@@ -89,7 +88,6 @@ constexpr int W3_F4_BAND_PX = 248;
 constexpr int W3_MAX_WINDOW_PX = 416;
 // 4-bit floating-point operands (see F4 below)
 constexpr uint32_t W3_F4_MARK = 0x34463271u;   // behind the blob's copy of the weights
-constexpr int W3_F4_TP = 240;          // positions of a tile, at most
 constexpr int W3_F4_SF = 2 * W3_F4_TP; // tensor-memory columns of the block scales: 480 .. 511
 
 // byte offsets of the kernel's shared-memory regions (w3_layout)
@@ -1355,16 +1353,6 @@ w8_build_kernel(const uint8_t *__restrict__ packed, uint8_t *__restrict__ out, i
 
 }  // namespace
 
-// planes of a pixel's channels, K steps of a plane and taps of a K step, the latter two of
-// rows that are not 128 bytes long
-static inline void w3_steps(int Cin, int f4, int *npl, int *kpp, int *tps)
-{
-    const int full = f4 ? 256 : 128;               // channels of a 128-byte row
-    *npl = Cin < full ? 1 : Cin / full;
-    *tps = Cin < full ? full / Cin : 1;
-    *kpp = (9 + *tps - 1) / *tps;
-}
-
 DsqW8Info dsq_w8_info(const dsq_conv_t *conv, int bits)
 {
     DsqW8Info w = {0, 0, 0, 0, 0};
@@ -1408,76 +1396,6 @@ int dsq_w8_build(void *blob, const dsq_conv_t *conv, int bits, cudaStream_t stre
                                   : w8_build_kernel<2, false>,
                       dim3(blocks), dim3(256), 0, stream, 0, 0, packed, out, conv->Cout, 9 * P, w.ksteps,
                       kpp, tps * P, (uint32_t *)((uint8_t *)blob + w3_mark_offset(w)));
-}
-
-// Positions of a transposed tile, at most `most`: what fills as many passes of the `mstep`
-// CTAs of an N tile as the largest tile would take, so that the last pass is no emptier than
-// the others.  (4-bit, batch 64, largest / this: 28x28 128->128 11.6 / 10.8 us, 14x14 256->256
-// 11.3 / 10.5, 7x7 512->512 15.6 / 14.2 (12.2 since); 2-bit 28x28 512->512 at batch 32 27.9 / 26.9.)  No
-// fewer than 112: the instructions get shorter, the weights' K steps do not (28x28 128->128 at
-// batch 16: 96 to 144 positions alike).  With more than four passes the last one weighs little, and
-// larger tiles have less overhead each (64->64 at 56x56, six passes: 256 positions 15.4, 240
-// 15.8).
-static int w3_tile(int64_t positions, int mstep, int most)
-{
-    const int64_t passes = (positions + (int64_t)most * mstep - 1) / ((int64_t)most * mstep);
-    if (passes > 4) return most;
-    const int64_t each = (positions + passes * mstep - 1) / (passes * mstep);
-    return (int)std::min<int64_t>(most, std::max<int64_t>(112, (each + 15) / 16 * 16));
-}
-
-// Positions of the numbering up to the last pixel, channel tiles, CTAs a channel tile.
-struct W3Work {
-    int64_t positions;
-    int Hp, Wp, n_tiles, mstep;
-};
-static W3Work w3_work(const dsq_nhwc_t *shape, const dsq_conv_t *conv, int pair, int bn, int sms)
-{
-    W3Work w;
-    const int Ho = (shape->H - 1) / conv->stride + 1, Wo = (shape->W - 1) / conv->stride + 1;
-    const bool two = pair || conv->stride == 2;
-    w.Hp = two ? shape->H / 2 + 1 : shape->H + 1;
-    w.Wp = conv->stride == 2 ? shape->W / 2 + 1 : shape->W + 1;
-    w.positions = ((int64_t)shape->N - 1) * w.Hp * w.Wp + (int64_t)((Ho - 1) / (pair ? 2 : 1)) * w.Wp + Wo;
-    w.n_tiles = (conv->Cout + bn - 1) / bn;
-    w.mstep = std::max(sms / w.n_tiles, 1);
-    return w;
-}
-
-static bool w3_takes_f4(const dsq_conv_t *conv, int bits, int half_offset)
-{
-    return bits == 2 && half_offset && (conv->Cin <= 128 || conv->Cin % 256 == 0);
-}
-
-// 4-bit operands at stride 2, where the blob has no expanded weights: the im2col kernel is
-// the faster one unless a CTA expands its weights once - they stay resident, or one pass
-// of large tiles does (28x28 128->256 at batch 64 10.3 us against 11.9, at batch 16, tiles of 112, 7.7
-// against 7.5; 112x112 128->128 18.8 against 17.3; 14x14 256->512 12.2 against 10.8).
-static bool w3_takes_stride2(int Cin, int tile, int64_t passes)
-{
-    return Cin == 64 || (Cin == 128 && passes == 1 && tile >= 160);
-}
-
-// Microseconds the window kernel takes for a layer of few tiles, or a negative number
-// where it does not take it: start-up and the last epilogue, and for every pass of the
-// CTAs its K steps.  Fitted to 666 layers of 64 to 512 channels at batches of 1 to 32: 5 % off
-// in the mean, 17 % at most.
-double dsq_conv3_estimate(const dsq_nhwc_t *shape, int bits, const dsq_conv_t *conv, int half_offset)
-{
-    const int Cin = conv->Cin, sms = dsq_sm_count() > 0 ? dsq_sm_count() : 148;
-    if (conv->KH != 3 || conv->pad != 1 || !(Cin == 64 || (Cin % 128 == 0 && Cin <= 1024))) return -1.0;
-    const int f4 = w3_takes_f4(conv, bits, half_offset), pair = conv->stride == 1 && conv->Cout <= 64;
-    int npl, kpp, tps;
-    w3_steps(Cin, f4, &npl, &kpp, &tps);
-    if (pair) kpp = (12 + tps - 1) / tps;
-    const W3Work w = w3_work(shape, conv, pair, 128, sms);
-    const int tile = w3_tile(w.positions, w.mstep, f4 ? W3_F4_TP : 256);
-    const int64_t passes = (w.positions + (int64_t)tile * w.mstep - 1) / ((int64_t)tile * w.mstep);
-    const double steps = (double)passes * npl * kpp, t = tile / 256.0;
-    if (conv->stride == 1)
-        return f4 ? 3.7 + steps * (1.41 * t - 0.36) : bits == 3 ? 4.5 + steps * (t - 0.07) : 3.8 + steps * (0.754 * t - 0.076);
-    if (bits != 3 && !f4 && !w3_takes_stride2(Cin, tile, passes)) return -1.0;
-    return f4 ? 3.4 + steps * (2.24 * t - 0.49) : bits == 3 ? 4.8 + steps * (1.59 * t - 0.27) : 3.6 + steps * (1.39 * t - 0.215);
 }
 
 int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
@@ -1543,7 +1461,7 @@ int dsq_conv3_window(const void *act_codes, const dsq_nhwc_t *shape, int bits,
         p.xstep = p.tps * P;
         p.pk = p.tps > 1 ? p.tps * P : (f4 ? 32 : 16) * bits;
         p.rb = tr ? 128 / p.tps : 128;
-        p.BN = tr ? 128 : (Cout >= 256 ? 256 : ((Cout + 63) / 64) * 64);
+        p.BN = tr ? 128 : w3_plain_bn(Cout);
         // positions (see W3Pos) and what a window is made of
         const W3Work work = w3_work(shape, conv, p.pair, p.BN, sms);
         p.n_tiles = work.n_tiles;

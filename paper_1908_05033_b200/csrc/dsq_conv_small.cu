@@ -23,8 +23,7 @@
 // K is a list of units: 16 bytes of one filter tap of a pixel row (32 codes of 4 bits,
 // 64 of 2; 12 bytes = 32 codes at 3 bits), four units - lanes j = 0 .. 3 - a chunk.
 // The order of K inside a unit is free as long as both operands agree.
-#include <cmath>
-
+#include "dsq_conv_rule.h"
 #include "dsq_tc_common.cuh"
 #include "dsq_tc_host.h"
 
@@ -312,38 +311,6 @@ int pick(CsParams &p, int mt, int warps, cudaStream_t s)
     return mt == 2 ? launch<BITS, 2, 4>(p, warps, s) : launch<BITS, 1, 4>(p, warps, s);
 }
 
-// Microseconds this kernel takes with a tile and block size, fitted to the layers of the
-// ResNet-18- and MobileNetV2-shaped networks at batches of 1, 2 and 4: the longer of
-// a block's chain (0.55 us for every chunk a warp walks) and what the blocks of an SM
-// take together (most of it per warp, whatever it has to do).
-double estimate(const CsParams &p, int bits, int mt, int warps)
-{
-    const int sms = dsq_sm_count() > 0 ? dsq_sm_count() : 148;
-    const double blocks = (double)((p.M + 16 * mt - 1) / (16 * mt)) * ((p.Ncols + 31) / 32);
-    // (a 2-bit unit is twice the arithmetic, 3-bit fields take twice the instructions)
-    const double f = bits == 4 ? 1.0 : 2.0;
-    const double fixed = mt == 1 ? (warps == 4 ? 0.44 : warps == 8 ? 1.1 : 2.5) : (warps == 4 ? 0.7 : 1.35);
-    const double per_block = fixed + f * (mt == 1 ? 0.06 : 0.09) * p.chunks;
-    const double chain = 1.5 + 0.05 * warps + 0.55 * (bits == 4 ? 1.0 : 1.3) * ((p.chunks + warps - 1) / warps);
-    const double shared = 1.2 + blocks / sms * per_block;
-    return chain > shared ? chain : shared;
-}
-
-// And what the other kernel for the layer takes, likewise: the window kernel as it says
-// itself; the im2col kernel a floor that grows with K (the few CTAs such a layer has walk
-// it alone) plus its work at full rate.
-// Of 666 measured 3x3 layers (64 to 512 channels, strides 1 and 2, 2 to 4 bits, batches of 1 to 32)
-// the rule takes the slower kernel for 5 %, 0.8 % of time on average.
-double estimate_other(const CsParams &p, const dsq_nhwc_t *shape, const dsq_conv_t *conv, int bits, int half_offset,
-                      int lean)
-{
-    const double ksteps = p.ksize * p.ksize * conv->Cin / 128.0;
-    if (p.ksize == 1 && lean) return 2.9 + (double)p.M * p.Ncols / 3.7e6;
-    const double window = dsq_conv3_estimate(shape, bits, conv, half_offset);
-    if (window > 0.0) return window;
-    return 4.3 + 0.23 * ksteps + (double)p.M * p.Ncols * p.ksize * p.ksize * conv->Cin / 4.5e8;
-}
-
 }  // namespace
 
 int dsq_conv_small(const void *act_codes, const dsq_nhwc_t *shape, int bits, const void *w_packed,
@@ -373,17 +340,13 @@ int dsq_conv_small(const void *act_codes, const dsq_nhwc_t *shape, int bits, con
     p.e = e;
     if ((p.M + 15) / 16 > 65535 || (int64_t)shape->N * shape->H * shape->W >= (1ll << 30))
         return DSQ_ERR_UNSUPPORTED;
-    int mt = 1, warps = 4;
-    double best = estimate(p, bits, 1, 4);
-    for (int m = 1; m <= 2; ++m)
-        for (int w = 4; w <= (m == 1 ? 16 : 8); w *= 2) {
-            const double t = estimate(p, bits, m, w);
-            if (t < best) { best = t; mt = m; warps = w; }
-        }
-    if (best > estimate_other(p, shape, conv, bits, e.half_offset, lean)) return DSQ_ERR_UNSUPPORTED;
+    const int sms = dsq_sm_count() > 0 ? dsq_sm_count() : 148;
+    const DsqSmallTile best = dsq_small_tile(p.M, p.Ncols, p.chunks, bits, sms);
+    if (best.us > dsq_small_other(shape, bits, conv, p.M, e.half_offset && dsq_launch_hooks().w8, lean, sms))
+        return DSQ_ERR_UNSUPPORTED;
     switch (bits) {
-    case 2: return pick<2>(p, mt, warps, stream);
-    case 3: return pick<3>(p, mt, warps, stream);
-    default: return pick<4>(p, mt, warps, stream);
+    case 2: return pick<2>(p, best.mt, best.warps, stream);
+    case 3: return pick<3>(p, best.mt, best.warps, stream);
+    default: return pick<4>(p, best.mt, best.warps, stream);
     }
 }

@@ -57,10 +57,6 @@ DSQ_HIDDEN int dsq_pointwise(const void *act_codes, const dsq_nhwc_t *shape, int
 
 // Dense convolution with little work (dsq_conv_small.cu).  Arguments as dsq_pointwise,
 // any outputs; lean: codes only, with a requantiser the lean epilogue takes.
-// Time of the window kernel for a 3x3 layer, negative where it does not take it
-// (dsq_conv3.cu).
-DSQ_HIDDEN double dsq_conv3_estimate(const dsq_nhwc_t *shape, int bits, const dsq_conv_t *conv, int half_offset);
-
 DSQ_HIDDEN int dsq_conv_small(const void *act_codes, const dsq_nhwc_t *shape, int bits,
                               const void *w_packed, const dsq_conv_t *conv, const DsqEpi &e,
                               int lean, cudaStream_t stream);
