@@ -167,7 +167,11 @@ int dsq_workspace_status(void *workspace, void *stream);
  *              or a multiple of 256 channels the copy holds 4-bit
  *              floating-point operands and is marked as such: dsq_conv2d
  *              records DSQ_ERR_UNSUPPORTED in the workspace when it meets such
- *              a blob without the mark (packed by an earlier library).
+ *              a blob without the mark (packed by an earlier library); the
+ *              call itself returns DSQ_OK and its outputs are undefined.  Keep
+ *              dsq_version() with a stored blob and, where it differs, pack
+ *              again: the packed rows at its start are the same format in
+ *              every version, and dsq_unpack reads them.
  * A clip range with hi <= lo or a non-finite bound cannot be seen from the
  * host: the kernel writes code 0 for that channel and records DSQ_ERR_RANGE
  * in the workspace. */
@@ -385,6 +389,7 @@ int dsq_probe_i8_mma_rate(int iters, float *ms_out, double *macs_out,
 
 /* ---- misc --------------------------------------------------------------- */
 const char *dsq_status_string(int status);
+/* Raised whenever blobs that dsq_pack_weights wrote before may be refused. */
 int dsq_version(void);
 
 #ifdef __cplusplus

@@ -11,7 +11,9 @@
 
 #include "../../include/dsq.h"
 
-#define DSQ_VERSION 100
+// raised whenever blobs of dsq_pack_weights from before may be refused (101: 2-bit ones, whose
+// expanded copy was int8)
+#define DSQ_VERSION 101
 
 // Workspace layout (device memory owned by the caller).
 //   word 0 : status (0 = ok, else a dsq_status code written by a kernel)

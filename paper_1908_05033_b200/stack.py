@@ -24,6 +24,7 @@ def _delta_f32(bits, lo, hi):
 
 class GpuStack:
     _plan = None          # the recorded pass: of this object and process only
+    _packed_by = None     # version of the library that packed the weight blobs
 
     def __init__(self, st, params, batch=None, w_offset=0.5, device="cuda",
                  keep_debug=False):
@@ -69,11 +70,34 @@ class GpuStack:
             self.layers.append((L, dict(blob=blob, conv=conv, scale=scale,
                                         bias=bias)))
         B.check_workspace(self.ws, "dsq_pack_weights")
+        self._packed_by = B.dsq_version()
         self.debug = {}
 
     def __getstate__(self):
         """A copied or pickled stack records its own pass."""
         return {k: v for k, v in self.__dict__.items() if k != "_plan"}
+
+    def __setstate__(self, state):
+        """A stack stored by another version of the library packs its weights again."""
+        self.__dict__.update(state)
+        if self._packed_by != B.dsq_version() and self.ws.is_cuda:
+            with torch.cuda.device(self.ws.device):
+                self._pack_again()
+
+    def _pack_again(self):
+        """The packed rows at the start of a blob are a public format, the expanded copy behind
+        them is its version's own: new blobs from the codes of the rows (a code q is
+        what q on the range [0, 2^b - 1] quantises to)."""
+        for L, w in self.layers:
+            if w is None or L.kind == "dw":               # (no copy behind these rows)
+                continue
+            c = w["conv"]
+            rows, pitch = c.Cout * c.KH * c.KW, B.dsq_row_pitch(c.Cin, self.bits)
+            codes = B.dsq_unpack(w["blob"][:rows * pitch].view(rows, pitch), rows, c.Cin, self.bits, True)
+            q = codes.view(c.Cout, c.KH, c.KW, c.Cin).float() + 2 ** (self.bits - 1)
+            w["blob"], _ = B.dsq_pack_weights(q, self.bits, 0.0, 2 ** self.bits - 1, self.ws, stride=c.stride,
+                                              pad=c.pad)
+        self._packed_by = B.dsq_version()
 
     def _parts(self):
         """Everything _call_layers reads.  Exchange one of these objects, or change a
