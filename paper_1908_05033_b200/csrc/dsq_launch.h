@@ -14,6 +14,20 @@
 
 #include "dsq_common.cuh"
 
+#define DSQ_HIDDEN __attribute__((visibility("hidden")))
+
+// current values of the process-wide hooks (csrc/dsq_hooks.h)
+struct DsqLaunchHooks {
+    int pdl;                    // programmatic dependent launch on / off
+    unsigned long long wait_ns; // limit of the device-side waits
+    int skip_b_round;           // test hook, -1 = off
+    int window3;                // dsq_set_conv3_window
+    int w8;                     // dsq_set_conv3_expanded_weights
+};
+DSQ_HIDDEN DsqLaunchHooks dsq_launch_hooks();
+// a number that changes whenever a hook is set
+DSQ_HIDDEN unsigned dsq_hooks_generation();
+
 // how a kernel is launched
 struct DsqGrid {
     const void *func;
@@ -68,7 +82,7 @@ struct dsq_plan {
 };
 
 // the plan the calling thread records into, or nullptr
-__attribute__((visibility("hidden"))) dsq_plan *&dsq_recording_plan();
+DSQ_HIDDEN dsq_plan *&dsq_recording_plan();
 
 // Whether a kernel launched now may read a layer's constants (packed weights, scales,
 // biases) before griddepcontrol.wait.  Every kernel of the library waits for the

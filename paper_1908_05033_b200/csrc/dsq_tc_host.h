@@ -7,20 +7,6 @@
 #include "dsq_epilogue.cuh"
 #include "dsq_launch.h"
 
-#define DSQ_HIDDEN __attribute__((visibility("hidden")))
-
-// current values of the process-wide hooks (csrc/dsq_hooks.h)
-struct DsqLaunchHooks {
-    int pdl;                    // programmatic dependent launch on / off
-    unsigned long long wait_ns; // limit of the device-side waits
-    int skip_b_round;           // test hook, -1 = off
-    int window3;                // dsq_set_conv3_window
-    int w8;                     // dsq_set_conv3_expanded_weights
-};
-DSQ_HIDDEN DsqLaunchHooks dsq_launch_hooks();
-// a number that changes whenever a hook is set
-DSQ_HIDDEN unsigned dsq_hooks_generation();
-
 typedef CUresult (*DsqEncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
                                      const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
                                      const cuuint32_t *, CUtensorMapInterleave,

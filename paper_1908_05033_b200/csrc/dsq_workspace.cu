@@ -53,6 +53,18 @@ bool on_current_device(const void *p)
     return false;
 }
 
+// Whether CUDA's own waits spin on the current device (the default while cores are free).
+bool waits_spin()
+{
+    unsigned flags = 0;
+    if (cudaGetDeviceFlags(&flags) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    flags &= cudaDeviceScheduleMask;
+    return flags != cudaDeviceScheduleYield && flags != cudaDeviceScheduleBlockingSync;
+}
+
 }  // namespace
 
 extern "C" {
@@ -78,13 +90,14 @@ int dsq_workspace_status(void *ws, void *stream)
         *(volatile int *)word = STATUS_PENDING;
         int *w = (int *)ws;
         void *argv[] = {(void *)&w, (void *)&word};
-        const DsqGrid one = {(const void *)status_kernel, dim3(1), dim3(1), 0, 1, 0};
+        const DsqGrid one = {(const void *)status_kernel, dim3(1), dim3(1), 0, dsq_launch_hooks().pdl, 0};
         const int st = dsq_launch_args(one, argv, s);
         if (st) return st;
         // The word is watched for a while first: the stream's own wait, entered when its work
-        // is as good as done, returns sooner than one that was asleep for it.
+        // is as good as done, returns sooner than one that was asleep for it.  Not in a program
+        // that has CUDA's waits yield or block: it wants its cores back.
         const auto t0 = std::chrono::steady_clock::now();
-        bool pending = true;
+        bool pending = waits_spin();
         while (pending && std::chrono::steady_clock::now() - t0 < std::chrono::microseconds(200))
             for (int i = 0; i < 64 && pending; ++i) pending = *(volatile int *)word == STATUS_PENDING;
         DSQ_CUDA_TRY(cudaStreamSynchronize(s));

@@ -8,7 +8,7 @@ import pytest
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 FIELDS = ("host_allocs host_frees kernels copies syncs fail_host_alloc device_of_ws capture_elsewhere "
-          "broken").split()
+          "broken pdl dependent schedule late waited").split()
 
 
 class Fake(C.Structure):
@@ -44,3 +44,25 @@ def test_status(built, change, by_kernel):
     assert f.syncs == 9 and not f.broken
     # one word a thread, given back when the thread ends
     assert f.host_allocs == f.host_frees == (0 if "fail_host_alloc" in change else 3)
+
+
+@pytest.mark.parametrize("pdl", [0, 1])
+def test_dependent_launch_hook(built, pdl):
+    C.memset(built.fake(), 0, C.sizeof(Fake))
+    f = built.fake().contents
+    f.pdl = pdl
+    assert built.status_of_new_thread((C.c_int * 64)(), 3) == 0
+    assert (f.kernels, f.dependent) == (3, 3 * pdl)
+
+
+@pytest.mark.parametrize("schedule,watched", [(0, True), (1, True), (2, False), (4, False)])
+def test_watch_follows_the_schedule_flags(built, schedule, watched):
+    """cudaDeviceScheduleAuto, Spin, Yield, BlockingSync: the word is watched (up to 200 us) only
+    where CUDA's own wait would spin, too."""
+    C.memset(built.fake(), 0, C.sizeof(Fake))
+    f = built.fake().contents
+    f.schedule, f.late = schedule, 1
+    ws = (C.c_int * 64)()
+    ws[0] = -10
+    assert built.status_of_new_thread(ws, 20) == -10 and f.syncs == 20
+    assert (f.waited >= 200) == watched       # the shortest of the twenty

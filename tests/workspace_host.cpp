@@ -2,6 +2,7 @@
 // and driven by test_workspace_host.py.
 #include "../paper_1908_05033_b200/csrc/dsq_workspace.cu"
 
+#include <chrono>
 #include <cstring>
 #include <thread>
 #include <utility>
@@ -10,7 +11,11 @@ namespace {
 struct Fake {
     int host_allocs, host_frees, kernels, copies, syncs;
     int fail_host_alloc, device_of_ws, capture_elsewhere, broken;
+    int pdl, dependent;          // the hook; launches with the attribute
+    int schedule, late, waited;  // device flags; the kernel runs in the stream's wait; us before it
 } f;
+int *g_late[2];
+std::chrono::steady_clock::time_point g_launched;
 thread_local cudaStreamCaptureMode g_mode = cudaStreamCaptureModeGlobal;
 int g_word[64];
 
@@ -26,6 +31,13 @@ dsq_plan *&dsq_recording_plan()
 {
     static dsq_plan *none = nullptr;
     return none;
+}
+
+DsqLaunchHooks dsq_launch_hooks()
+{
+    DsqLaunchHooks h = {};
+    h.pdl = f.pdl;
+    return h;
 }
 
 extern "C" {
@@ -66,10 +78,15 @@ cudaError_t cudaPointerGetAttributes(cudaPointerAttributes *a, const void *)
     a->device = f.device_of_ws;
     return cudaSuccess;
 }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *, const void *k, void **args)
+cudaError_t cudaGetDeviceFlags(unsigned *flags) { *flags = (unsigned)f.schedule; return cudaSuccess; }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *cfg, const void *k, void **args)
 {
     ++f.kernels;
-    status_kernel(*(int **)args[0], *(volatile int **)args[1]);
+    f.dependent += cfg->numAttrs != 0;
+    g_late[0] = *(int **)args[0];
+    g_late[1] = *(int **)args[1];
+    g_launched = std::chrono::steady_clock::now();
+    if (!f.late) status_kernel(g_late[0], g_late[1]);
     return cudaSuccess;
 }
 cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cudaStream_t)
@@ -83,6 +100,15 @@ cudaError_t cudaMemsetAsync(void *d, int v, size_t n, cudaStream_t)
     std::memset(d, v, n);
     return cudaSuccess;
 }
-cudaError_t cudaStreamSynchronize(cudaStream_t) { ++f.syncs; return cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t)
+{
+    ++f.syncs;
+    if (f.late) {
+        const auto us = std::chrono::duration_cast<std::chrono::microseconds>(std::chrono::steady_clock::now() - g_launched);
+        if (!f.waited || us.count() < f.waited) f.waited = (int)us.count();
+        status_kernel(g_late[0], g_late[1]);
+    }
+    return cudaSuccess;
+}
 cudaError_t cudaGraphExecDestroy(cudaGraphExec_t) { return cudaSuccess; }
 }
