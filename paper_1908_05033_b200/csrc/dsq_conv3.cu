@@ -308,9 +308,9 @@ __device__ __forceinline__ uint32_t w3_transpose_fields(uint32_t x, int lane)
 //
 // F4: 2-bit codes (weight grid Delta (c + 1/2)) as 4-bit floating-point operands.  E2M1
 // holds the codes 0 .. 3 and the weights 2 c + 1 exactly, and every partial sum is a whole
-// number far below 2^24, so the f32 accumulators hold the int32 sums bit for bit
-// (checked up to 2^23.9 on the hardware, in every order that the sums may be taken).  An
-// instruction covers K = 64 in the clocks in which kind::i8 covers 32, from the same 32
+// number of at most 9 * 9 * 1024, so the f32 accumulators hold the int32 sums bit for bit
+// (the adder is exact up to 2^23, large steps of both signs among least ones included:
+// tests/test_gpu_gemm_exact_sums.py).  An instruction covers K = 64 in the clocks in which kind::i8 covers 32, from the same 32
 // bytes a row; the window and the weights take half of the shared memory.  The block
 // scales (all 2, so that the accumulators come as 2 acc + S_a) need tensor memory
 // beside the two accumulators, so a tile is 240 positions instead of 256.
