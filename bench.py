@@ -38,8 +38,8 @@ import dsq_inputs  # noqa: E402
 # DRAM traffic of the tensor-core convolution kernels per launch in this
 # workload, from one ncu capture (profiles/bench_launch_list.txt); valid only
 # for the kernel sources it was taken on (checked by hash)
-TRAFFIC = {"bytes_per_launch": 4973514,
-           "sources_sha256": "cdc731f6e88726472cb7e48f29e745cf6707dbd81037eb02f5844df7e8158ce6"}
+TRAFFIC = {"bytes_per_launch": 4974080,
+           "sources_sha256": "0c3e258fd843fddfc5ce755674c0538fae56b8274c6cc061966ba289bf4f1a5a"}
 
 WORKLOAD = "resnet18-shaped stack, 4-bit W/A, batch 64, 56x56x64 stem output, 19 convs"
 METRIC = "4-bit ResNet-18 conv-stack throughput (effective low-bit conv TOPS alongside)"
@@ -52,7 +52,7 @@ INT8_NOMINAL_TOPS = 4500.0
 def kernel_sources_sha256():
     import hashlib
     h = hashlib.sha256()
-    for f in ("dsq_tc.cu", "dsq_conv3.cu", "dsq_pw.cu", "dsq_conv_small.cu", "dsq_tc_common.cuh",
+    for f in ("dsq_tc.cu", "dsq_conv3.cu", "dsq_conv_rule.h", "dsq_pw.cu", "dsq_conv_small.cu", "dsq_tc_common.cuh",
               "dsq_ptx.cuh", "dsq_epilogue.cuh", "dsq_common.cuh"):
         h.update(open(os.path.join(ROOT, "paper_1908_05033_b200", "csrc", f), "rb").read())
     return h.hexdigest()

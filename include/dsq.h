@@ -160,7 +160,7 @@ int dsq_workspace_status(void *workspace, void *stream);
  *              For dense 3x3 stride-1 pad-1 convolutions at 2 or 4 bits with
  *              64 or a multiple of 128 input channels the buffer is larger:
  *              behind the packed rows (1024-byte aligned) it holds the same
- *              rows already expanded to the 8-bit operand bytes of the grid
+ *              rows already expanded to the operand bytes of the grid
  *              Delta (c + 1/2), which dsq_conv2d then copies to the tensor
  *              core's shared-memory operand without expanding them again
  *              (dsq_weight_bytes includes that copy).  At 2 bits with 64, 128
@@ -261,9 +261,10 @@ size_t dsq_gemm_workspace_bytes(int64_t M, int64_t N, int64_t K, int bits);
  *           dsq_row_pitch(K, 1); bits past K are ignored)
  *   B_bits  packed rows [N][K], same format
  *   C_i32, row_scale, D_f32 as in dsq_gemm.
- * On this GPU the +-1 values go through the 8-bit integer tensor-core path:
- * every row is expanded to int8 once into the workspace, then the same
- * TMA-fed 8-bit GEMM as dsq_gemm's two-pass path runs.  `workspace` must hold
+ * On this GPU the +-1 values go through the tensor cores: every row is expanded
+ * once into the workspace, to 4-bit floating point while K is below 2^23 and to
+ * int8 from there on, then the same TMA-fed GEMM as dsq_gemm's two-pass path
+ * runs.  `workspace` must hold
  * dsq_binary_gemm_workspace_bytes(M, N, K) bytes (DSQ_ERR_SIZE otherwise),
  * its first dsq_workspace_bytes() bytes cleared with dsq_workspace_init. */
 size_t dsq_binary_gemm_workspace_bytes(int64_t M, int64_t N, int64_t K);
@@ -288,8 +289,9 @@ int dsq_binary_gemm(const void *A_bits, const void *B_bits, int64_t M, int64_t N
  * fp32 by the tensor core in an order of its own, so Y is within
  * K * 2^-23 * sum_k |X v| * |col_scale| of the exact value.  The weights are
  * expanded to bf16 once into the workspace (dsq_wgemm_workspace_bytes(N, K)),
- * then a TMA-fed bf16 tensor-core GEMM runs; few rows (up to 64, or more where
- * it is faster) are multiplied straight from the packed codes. */
+ * then a TMA-fed bf16 tensor-core GEMM runs; few rows (up to 32, and more where
+ * it is faster) are multiplied straight from the packed codes and leave the
+ * scratch alone. */
 size_t dsq_wgemm_workspace_bytes(int64_t N, int64_t K);
 int dsq_wgemm_bf16(const void *X_bf16, const void *W_codes, int64_t M, int64_t N,
                    int64_t K, int bits, float w_offset, const float *col_scale,

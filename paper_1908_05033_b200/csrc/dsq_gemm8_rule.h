@@ -20,7 +20,7 @@ struct DsqG8Tile {
 // accumulator; resident(): clusters of two pairs that fit on the GPU at once.
 //
 // A pair reads 256 + BN rows of 128 bytes for a K block of a tile, and that is what a block's
-// time goes with, for 8-bit, bf16 and 4-bit operands alike (about 13 TB/s over all pairs, from
+// time goes with, for 8-bit, bf16 and 4-bit operands alike (about 15 TB/s over all pairs, from
 // the L2): 1.2 clocks a row; a tile costs 1500 more.  The CTA pairs take their tiles in waves,
 // and the width with the cheapest waves is taken.  Split: only with all the clusters resident
 // at once and twelve K blocks a part; the exchange of the partial sums grows with the width.

@@ -1846,7 +1846,7 @@ int dsq_conv2d(const void *act_codes, const dsq_nhwc_t *shape, const dsq_quant_t
                             (cudaStream_t)stream);
         if (st != DSQ_ERR_UNSUPPORTED) return st;
     }
-    // 3x3 stride-1 convolutions: every input pixel expanded once (dsq_conv3.cu)
+    // 3x3 convolutions (strides 1 and 2): every input pixel expanded once (dsq_conv3.cu)
     st = dsq_conv3_window(act_codes, shape, bits, w_packed, conv, e, epi, small_acc, workspace,
                           (cudaStream_t)stream);
     if (st != DSQ_ERR_UNSUPPORTED) return st;

@@ -25,7 +25,7 @@ DSQ_HIDDEN DsqEncodeIm2colFn dsq_encode_im2col_fn();
 // residual operand; any outputs
 enum { DSQ_EPI_CODES = 1, DSQ_EPI_CODES_RES = 2, DSQ_EPI_GENERAL = 3 };
 
-// 3x3, stride 1, pad 1 convolution on an expanded shared-memory window
+// 3x3, pad 1 convolution (strides 1 and 2) on an expanded shared-memory window
 // (dsq_conv3.cu).  Arguments are those of dsq_conv2d after validation.
 // Returns DSQ_ERR_UNSUPPORTED without launching anything when the geometry is
 // not one it handles; the caller then takes the im2col kernel.
@@ -61,8 +61,8 @@ static inline int dsq_allow_smem(const void *func, int bytes, std::atomic<unsign
     return DSQ_OK;
 }
 
-// Two-pass GEMM (dsq_gemm8.cu): every packed row is expanded to int8 once
-// into caller-provided scratch, then an 8-bit GEMM reads it by TMA.
+// Two-pass GEMM (dsq_gemm8.cu): every packed row is expanded once, to int8 or 4-bit
+// floating point, into caller-provided scratch, then a GEMM reads it by TMA.
 // dsq_gemm8_scratch_bytes: scratch the path needs (0: not a problem it takes;
 // force: whatever the size).
 // dsq_gemm8_launch: arguments as dsq_gemm after validation, `scratch`
