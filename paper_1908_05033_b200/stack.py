@@ -97,6 +97,8 @@ class GpuStack:
             q = codes.view(c.Cout, c.KH, c.KW, c.Cin).float() + 2 ** (self.bits - 1)
             w["blob"], _ = B.dsq_pack_weights(q, self.bits, 0.0, 2 ** self.bits - 1, self.ws, stride=c.stride,
                                               pad=c.pad)
+        # (usable on every stream at once, as a new stack is)
+        torch.cuda.current_stream().synchronize()
         self._packed_by = B.dsq_version()
 
     def _parts(self):

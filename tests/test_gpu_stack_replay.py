@@ -158,30 +158,35 @@ def test_graph_made_during_a_capture_in_another_thread():
 
 
 @pytest.mark.parametrize("bits", [2, 3, 4])
-def test_stack_stored_by_another_version(bits):
+@pytest.mark.parametrize("make", [lambda bits: dsq_inputs.resnet18_stack(batch=2, bits=bits, hw=14),
+                                  lambda bits: dsq_inputs.tiny_stack(bits=bits)], ids=["resnet18", "every_kind"])
+def test_stack_stored_by_another_version(make, bits):
     """Its blobs have the same packed rows, and behind them what this version cannot read."""
     import paper_1908_05033_b200 as dsq
     from paper_1908_05033_b200.stack import GpuStack
-    st = dsq_inputs.resnet18_stack(batch=2, bits=bits, hw=14)
+    st = make(bits)
     net = GpuStack(st, dsq_inputs.stack_params(st, workload_id=5))
-    x = torch.randn(2, *st.in_shape, device="cuda").clamp_(0.0, st.in_cap)
+    x = torch.randn(st.batch, *st.in_shape, device="cuda").clamp_(0.0, st.in_cap)
+    weights = [w for _, w in net.layers if w is not None]
+    taps = [w["conv"].KH * w["conv"].KW * (1 if w["conv"].groups > 1 else w["conv"].Cout) for w in weights]
+    rows = [t * dsq.dsq_row_pitch(w["conv"].Cin, bits) for t, w in zip(taps, weights)]
     dsq.dsq_set_conv3_window(3)                  # (the kernel that reads the copy)
     try:
         want = net.forward(x).clone()
         state = pickle.loads(pickle.dumps(net)).__getstate__()
         state.pop("_packed_by")
-        rows = [w["conv"].Cout * w["conv"].KH * w["conv"].KW * dsq.dsq_row_pitch(w["conv"].Cin, bits)
-                for _, w in state["layers"]]
-        for n, (_, w) in zip(rows, state["layers"]):
+        state["codes"][st.out].zero_()
+        for n, (_, w) in zip(rows, [e for e in state["layers"] if e[1] is not None]):
             w["blob"][n:] = 0x41
         old = GpuStack.__new__(GpuStack)
         old.__setstate__(pickle.loads(pickle.dumps(state)))
         assert torch.equal(old.forward(x), want)
         old.check()
-        for n, (_, a), (_, b) in zip(rows, old.layers, net.layers):
-            assert torch.equal(a["blob"][:n], b["blob"][:n])
+        again = [w for _, w in old.layers if w is not None]
+        assert all(torch.equal(a["blob"][:n], b["blob"][:n]) for n, a, b in zip(rows, again, weights))
         # of this version: the blobs as they are
         other = pickle.loads(pickle.dumps(old))
-        assert all(torch.equal(a["blob"], b["blob"]) for (_, a), (_, b) in zip(other.layers, old.layers))
+        assert all(a is None or torch.equal(a["blob"], b["blob"])
+                   for (_, a), (_, b) in zip(other.layers, old.layers))
     finally:
         dsq.dsq_set_conv3_window(1)
