@@ -310,10 +310,10 @@ __device__ __forceinline__ uint32_t w3_transpose_fields(uint32_t x, int lane)
 // holds the codes 0 .. 3 and the weights 2 c + 1 exactly, and every partial sum is a whole
 // number of at most 9 * 9 * 1024, so the f32 accumulators hold the int32 sums bit for bit
 // (the adder is exact up to 2^23, large steps of both signs among least ones included:
-// tests/test_gpu_gemm_exact_sums.py).  An instruction covers K = 64 in the clocks in which kind::i8 covers 32, from the same 32
-// bytes a row; the window and the weights take half of the shared memory.  The block
-// scales (all 2, so that the accumulators come as 2 acc + S_a) need tensor memory
-// beside the two accumulators, so a tile is 240 positions instead of 256.
+// tests/test_gpu_gemm_exact_sums.py).  An instruction covers K = 64 in the clocks in which
+// kind::i8 covers 32, from the same 32 bytes a row; the window and the weights take half of
+// the shared memory.  The block scales (all 2, so that the accumulators come as 2 acc + S_a)
+// need tensor memory beside the two accumulators, so a tile is 240 positions instead of 256.
 //
 // int8 -> F4, batch 32: 64->64 at 224x224 82 -> 60 us, 128->128 at 112x112 44.7 -> 26.3,
 // 256->256 at 56x56 41.3 -> 25.6, 512->512 at 28x28 38.9 -> 27.6 (four passes of 240
