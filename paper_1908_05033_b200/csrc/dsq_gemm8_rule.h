@@ -28,10 +28,10 @@ struct DsqG8Tile {
 // doubles.)
 //
 // Measured: all widths, whole and split K, of 591 problems of 64 to 6144 a side, 1 to 4
-// bits, back to back in a graph and one at a time after an L2 flush, and 233 others to judge by: of
-// those the width taken is 0.22 % slower than the fastest one on average, more than 3 % in 11 of
-// 466 timings.  (A rule from the tensor cores' rate, 2.5 BN clocks a block, 330 + 0.72 BN at
-// least: 0.64 %, 33 of them.)
+// bits, back to back in a graph and one at a time after an L2 flush, and of 233 more that it was
+// not fitted to: of those the width taken is 0.22 % slower than the fastest one on average, more
+// than 3 % in 11 of 466 timings.  (A rule from the tensor cores' rate, 2.5 BN clocks a block,
+// 330 + 0.72 BN at least: 0.64 %, 33 of them.)
 template <class Resident>
 inline DsqG8Tile dsq_g8_tile(int64_t M, int64_t N, int64_t kblocks, int widest, int sms, Resident resident)
 {
