@@ -49,9 +49,12 @@ constexpr int G8_WARP_TMA = 0, G8_WARP_MMA = 1, G8_WARP_TMEM = 2, G8_WARP_E0 = 4
 constexpr int G8_E_WARPS = 8;                // per CTA: two per tensor-memory lane quarter
 constexpr int G8_THREADS = 32 * (G8_WARP_E0 + G8_E_WARPS);
 constexpr int G8_BARS = 2 * G8_MAX_STAGES + 4 + 1;
-constexpr int G8_SMEM = 227 * 1024;
+// A block of the next expansion has room beside a CTA: 1 KB of an SM's 228 is the system's for
+// each, and 40 registers for each of 256 threads are left.
+constexpr int G8_SMEM = 226 * 1024, G8_REGS = 128;
 constexpr int G8_TAIL = 8 * G8_BARS + 24;    // barriers, tensor-memory slot, abort flag
-constexpr int G8_STAGING = G8_E_WARPS * 32 * 33 * 4;     // a 32 x 32 block per epilogue warp
+constexpr int G8_STAGING = G8_E_WARPS * 32 * 32 * 4;     // a 32 x 32 block per epilogue warp
+static_assert(G8_TAIL % 128 == 0, "the staging blocks are 128-byte aligned");
 
 struct G8Params {
     int M, N;
@@ -89,6 +92,10 @@ __device__ __forceinline__ uint32_t sign_extend_bytes(uint32_t x)
 // 512 contiguous bytes (with 64 bytes a thread every store touched half sectors all
 // over, and the L2 took each sector twice); a thread does the same chunk of four
 // rows, their loads first.
+//
+// Launched dependently, as every kernel behind another of the library is: the first blocks
+// are on the SMs, beside the kernel ahead, when that ends (2500x1111x1777, 3-bit, among other
+// passes 14.35 -> 13.1 us, 2048x4096x4096 weight-only 69.2 -> 68.5; 4096^3 is bound by power).
 constexpr int EX_ROWS = 4, EX_THREADS = 256;
 
 // `BITS`-bit codes at bit 0 of a word, ascending -> one code per byte, four a word
@@ -145,6 +152,7 @@ __global__ void __launch_bounds__(EX_THREADS)
 expand_rows_kernel(const uint8_t *__restrict__ A, const uint8_t *__restrict__ B, int M, int N, int K,
                    int pitch_in, int pitch_out, uint8_t *__restrict__ A8, uint8_t *__restrict__ B8)
 {
+    grid_dependency_wait();
     // lets the second pass (queued behind with programmatic dependent launch) set
     // itself up while this grid runs; it waits for this grid before its first copy
     grid_launch_dependents();
@@ -191,6 +199,7 @@ __global__ void __launch_bounds__(EX_THREADS)
 expand_rows_f4_kernel(const uint8_t *__restrict__ A, const uint8_t *__restrict__ B, int M, int N, int K,
                       int pitch_in, int pitch_out, uint8_t *__restrict__ A4, uint8_t *__restrict__ B4)
 {
+    grid_dependency_wait();
     grid_launch_dependents();
     const int c = blockIdx.x * EX_THREADS + threadIdx.x;
     if (16 * c >= pitch_out) return;
@@ -236,6 +245,7 @@ __global__ void __launch_bounds__(EX_THREADS)
 expand_w_bf16_kernel(const uint8_t *__restrict__ W, int N, int K, int pitch_in, int pitch_out, int odd,
                      uint8_t *__restrict__ W16)
 {
+    grid_dependency_wait();
     grid_launch_dependents();
     constexpr uint32_t F = (1u << BITS) - 1u, HALF = 1u << (BITS - 1);
     const int c = blockIdx.x * EX_THREADS + threadIdx.x;
@@ -297,8 +307,8 @@ inline dim3 expand_grid(int64_t chunks, int64_t rows)
 // from `limit` on belong to another tile or lie outside.
 // vec: N is a multiple of 8, so every group of eight columns of a row is a full 32-byte
 // sector, inside or outside the matrix as a whole, and a lane stores its row.  Otherwise the
-// block is turned round in shared memory (`stage`, rows of 33 words: no bank conflicts either
-// way) and a warp stores one row after the other, 128 contiguous bytes at a time.
+// block is turned round in shared memory (`stage`, 128-byte aligned; words XOR-ed with their row:
+// no bank conflicts either way) and a warp stores one row after the other, 128 contiguous bytes at a time.
 // (With two adjacent columns a lane, 4-byte stores for odd N, 2500x1111x1777 3-bit took 22 us,
 // 16 of them in the epilogue; so, and with tiles of 160 columns: 12.5.)
 template <int KIND>
@@ -357,14 +367,14 @@ __device__ __forceinline__ void g8_store_block(const G8Params &p, int m, int n, 
         __syncwarp();
 #pragma unroll
         for (int j = 0; j < 32; ++j)
-            sts_32(stage + 4u * (uint32_t)(lane * 33 + j),
+            sts_32((stage + 132u * (uint32_t)lane) ^ (uint32_t)(4 * j),
                    KIND == G8_BF16 ? r[j] : which ? scaled(r[j], rs) : whole(r[j]));
         __syncwarp();
         if (col < limit) {
             uint32_t *dst = out + (int64_t)m * p.N + col;
 #pragma unroll 8
             for (int i = 0; i < rows; ++i, dst += p.N) {
-                const uint32_t v = lds_32(stage + 4u * (uint32_t)(i * 33 + lane));
+                const uint32_t v = lds_32((stage + 132u * (uint32_t)i) ^ (uint32_t)(4 * lane));
                 *dst = KIND == G8_BF16 ? __float_as_uint(__fmaf_rn(__uint_as_float(v), cs, cb)) : v;
             }
         }
@@ -381,7 +391,7 @@ __device__ __forceinline__ void g8_store_block(const G8Params &p, int m, int n, 
 // which nothing reads any more), adds them to its own in a fixed order and writes
 // those columns.  One tile per cluster.
 template <int KIND, int S>
-__global__ void __launch_bounds__(G8_THREADS, 1)
+__global__ void __maxnreg__(G8_REGS)
 gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
              const __grid_constant__ CUtensorMap tmap_b, const G8Params p)
 {
@@ -394,7 +404,7 @@ gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(tail + 8 * G8_BARS);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tail + 8 * G8_BARS + 8);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t staging = smem_u32(tail + G8_TAIL) + (uint32_t)((warp - G8_WARP_E0) * 32 * 33 * 4);
+    const uint32_t staging = smem_u32(tail + G8_TAIL) + (uint32_t)((warp - G8_WARP_E0) * 32 * 32 * 4);
     const uint32_t crank = cluster_ctarank();
     const uint32_t rank = crank & 1u, split = crank >> 1;       // in the pair; which part of K
     const uint32_t leader = crank & ~1u;
@@ -777,7 +787,7 @@ static int launch_f4(const void *A, const void *B, int64_t M, int64_t N, int64_t
     const size_t kp = round_up((size_t)(K + 1) / 2, 16);
     uint8_t *A4 = (uint8_t *)scratch, *B4 = A4 + round_up((size_t)M * kp, 1024);
     const int st = dsq_launch(expand_rows_f4_kernel<BITS>, expand_grid((int64_t)kp / 16, M + N),
-                              dim3(EX_THREADS), 0, stream, 0, 0, (const uint8_t *)A, (const uint8_t *)B,
+                              dim3(EX_THREADS), 0, stream, dsq_launch_hooks().pdl, 0, (const uint8_t *)A, (const uint8_t *)B,
                               (int)M, (int)N, (int)K, (int)dsq_row_pitch(K, BITS), (int)kp, A4, B4);
     if (st) return st;
     return launch_pass2<G8_F4>(A4, kp, B4, kp, kp, M, N, true, true, p, stream);
@@ -799,7 +809,7 @@ int dsq_gemm8_launch(const void *A_codes, const void *B_codes, int64_t M, int64_
     const int st = dsq_launch(bits == 2   ? expand_rows_kernel<2>
                               : bits == 3 ? expand_rows_kernel<3>
                                           : expand_rows_kernel<4>,
-                              expand_grid((int64_t)kp / 16, M + N), dim3(EX_THREADS), 0, stream, 0, 0,
+                              expand_grid((int64_t)kp / 16, M + N), dim3(EX_THREADS), 0, stream, dsq_launch_hooks().pdl, 0,
                               A, B, (int)M, (int)N, (int)K, pitch_in, (int)kp, A8, B8);
     if (st) return st;
     return launch_pass2<G8_I8>(A8, kp, B8, kp, (size_t)K, M, N, true, false, p, stream);
@@ -837,7 +847,7 @@ int dsq_binary_gemm(const void *A_bits, const void *B_bits, int64_t M, int64_t N
     if (f4_exact(K, 1)) return launch_f4<1>(A_bits, B_bits, M, N, K, p, scratch, (cudaStream_t)stream);
     uint8_t *A8 = scratch, *B8 = scratch + round_up((size_t)M * kp, 1024);
     const int st = dsq_launch(expand_rows_kernel<1>, expand_grid((int64_t)kp / 16, M + N),
-                              dim3(EX_THREADS), 0, (cudaStream_t)stream, 0, 0, (const uint8_t *)A_bits,
+                              dim3(EX_THREADS), 0, (cudaStream_t)stream, dsq_launch_hooks().pdl, 0, (const uint8_t *)A_bits,
                               (const uint8_t *)B_bits, (int)M, (int)N, (int)K,
                               (int)dsq_row_pitch(K, 1), (int)kp, A8, B8);
     if (st) return st;
@@ -882,7 +892,7 @@ int dsq_wgemm_bf16(const void *X_bf16, const void *W_codes, int64_t M, int64_t N
                               : bits == 2 ? expand_w_bf16_kernel<2>
                               : bits == 3 ? expand_w_bf16_kernel<3>
                                           : expand_w_bf16_kernel<4>,
-                              expand_grid(K / 8, N), dim3(EX_THREADS), 0, s, 0, 0, W, (int)N,
+                              expand_grid(K / 8, N), dim3(EX_THREADS), 0, s, dsq_launch_hooks().pdl, 0, W, (int)N,
                               (int)K, pitch_in, (int)wp, odd, W16);
     if (st) return st;
     G8Params p = {};
