@@ -8,7 +8,7 @@
 // Here every row is expanded ONCE:
 //   pass 1  expand_rows_kernel: packed codes -> int8 rows in a scratch area
 //           the caller provides (M*Kp + N*Kp bytes, Kp = K rounded up to 16;
-//           HBM / L2-bound, a few microseconds); codes of 1 and 2 bits -> 4-bit
+//           HBM / L2-bound, a few microseconds); codes of 1 to 3 bits -> 4-bit
 //           floating point (expand_rows_f4_kernel), half of that;
 //   pass 2  gemm8_kernel: a GEMM whose operands go from that scratch straight into
 //           swizzled shared memory by TMA - no thread touches an operand byte.
@@ -67,6 +67,8 @@ struct G8Params {
     int32_t *C_i32;
     const float *row_scale;
     float *D_f32;
+    const int32_t *sums;     // nullable: [parts][M], C = acc + 4 x their sum (expand_rows_f4_kernel<3>)
+    int parts;
     // floating-point problems: Y = fma(acc, col_scale[n], col_bias[n])
     const float *col_scale;
     const float *col_bias;   // nullable
@@ -189,49 +191,91 @@ expand_rows_kernel(const uint8_t *__restrict__ A, const uint8_t *__restrict__ B,
     }
 }
 
-// Integer operands of 1 and 2 bits as 4-bit floating point (E2M1 in steps of 1/2, as
+// Eight 3-bit codes (bits 0 .. 23) -> one in the low three bits of every four; the fourth is
+// anything.
+__device__ __forceinline__ uint32_t spread_nibbles(uint32_t x)
+{
+    const uint32_t y = (x & 0x0000FFFFu) | ((x << 4) & 0xFFFF0000u);
+    const uint32_t z = (y & 0x00FF00FFu) | ((y << 2) & 0xFF00FF00u);
+    return (z & 0x0F0F0F0Fu) | ((z << 1) & 0xF0F0F0F0u);
+}
+// sum of the eight four-bit fields
+__device__ __forceinline__ int sum_nibbles(uint32_t x)
+{
+    return (int)__dp4a((x & 0x0F0F0F0Fu) + ((x >> 4) & 0x0F0F0F0Fu), 0x01010101u, 0u);
+}
+
+// Integer operands of 1 to 3 bits as 4-bit floating point (E2M1 in steps of 1/2, as
 // expand_word_f4; block scales of 2 make the products whole numbers): a chunk of 16 output
 // bytes is 32 values, in the order in which a shift and a mask find them (the same for
 // both operands).  A 2-bit signed code -2 .. 1 is 1010, 1001, 0000, 0001, an unsigned one
 // its own pattern; a bit is 0001 (+1) or 1001 (-1), past K 0.
+// 3 bits: E2M1 has the whole numbers -4 .. 4, so A's codes -4 .. 3 are exact, and B's go less
+// 4: a (q - 4) summed is the result less 4 sum a.  The sums of A's rows are kept for the
+// second pass, one for every 1024 codes (`sums`: [part][M]).
 template <int BITS>
 __global__ void __launch_bounds__(EX_THREADS)
 expand_rows_f4_kernel(const uint8_t *__restrict__ A, const uint8_t *__restrict__ B, int M, int N, int K,
-                      int pitch_in, int pitch_out, uint8_t *__restrict__ A4, uint8_t *__restrict__ B4)
+                      int pitch_in, int pitch_out, uint8_t *__restrict__ A4, uint8_t *__restrict__ B4,
+                      int32_t *__restrict__ sums)
 {
     grid_dependency_wait();
     grid_launch_dependents();
     const int c = blockIdx.x * EX_THREADS + threadIdx.x;
-    if (16 * c >= pitch_out) return;
+    const bool inside = 16 * c < pitch_out;
+    if (BITS == 3 ? 16 * (c & ~31) >= pitch_out : !inside) return;    // (3 bits: warps as a whole)
+    constexpr int WORDS = BITS == 3 ? 3 : BITS == 2 ? 2 : 1;
     for (int r0 = blockIdx.y * EX_ROWS; r0 < M + N; r0 += gridDim.y * EX_ROWS) {
-        uint2 v[EX_ROWS];
+        uint32_t v[EX_ROWS][WORDS];
 #pragma unroll
         for (int i = 0; i < EX_ROWS; ++i) {
             const int r = min(r0 + i, M + N - 1);
             const uint8_t *row = r < M ? A + (int64_t)r * pitch_in : B + (int64_t)(r - M) * pitch_in;
-            if (BITS == 2) v[i] = __ldg(reinterpret_cast<const uint2 *>(row) + c);
-            else v[i].x = __ldg(reinterpret_cast<const uint32_t *>(row) + c);
+            if (BITS == 3) {
+                // (a row may end inside its last chunk)
+#pragma unroll
+                for (int l = 0; l < WORDS; ++l)
+                    v[i][l] = 4 * (3 * c + l) < pitch_in ? __ldg(reinterpret_cast<const uint32_t *>(row) + 3 * c + l)
+                                                         : 0u;
+            } else if (BITS == 2) {
+                const uint2 t = __ldg(reinterpret_cast<const uint2 *>(row) + c);
+                v[i][0] = t.x;
+                v[i][WORDS - 1] = t.y;
+            } else v[i][0] = __ldg(reinterpret_cast<const uint32_t *>(row) + c);
         }
 #pragma unroll
         for (int i = 0; i < EX_ROWS; ++i) {
             const int r = r0 + i;
             if (r >= M + N) break;
-            uint32_t o[4];
+            uint32_t o[4], low = 0u, neg = 0u;
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                if (BITS == 2) {
-                    const uint32_t x = ((j < 2 ? v[i].x : v[i].y) >> (2 * (j & 1))) & 0x33333333u;
+                if (BITS == 3) {
+                    const uint32_t lo = j == 0 ? 0u : v[i][j - 1], hi = j == 3 ? 0u : v[i][j];
+                    const uint32_t f = spread_nibbles(j == 0 ? hi : __funnelshift_r(lo, hi, 32 - 8 * j)) ^
+                                       (r < M ? 0u : 0x44444444u);
+                    // -4 + l is 12 - l
+                    const uint32_t l = f & 0x33333333u, s = f & 0x44444444u;
+                    o[j] = (l ^ ((s >> 2) | (s >> 1))) + ((s >> 2) | (s << 1));
+                    low += l;
+                    neg += s >> 2;
+                } else if (BITS == 2) {
+                    const uint32_t x = ((j < 2 ? v[i][0] : v[i][WORDS - 1]) >> (2 * (j & 1))) & 0x33333333u;
                     const uint32_t hi = x & 0x22222222u, lo = x & 0x11111111u;
                     o[j] = r < M ? (hi << 2) | (hi & ~(lo << 1)) | lo : x;
                 } else {
                     const int left = K - 32 * c;
                     const uint32_t in = left >= 32 ? 0xFFFFFFFFu : (1u << left) - 1u;
                     const uint32_t on = (in >> j) & 0x11111111u;
-                    o[j] = ((on & ~(v[i].x >> j)) << 3) | on;
+                    o[j] = ((on & ~(v[i][0] >> j)) << 3) | on;
                 }
             }
+            if (BITS == 3 && r < M) {
+                const int sum = __reduce_add_sync(0xffffffffu, sum_nibbles(low) - 4 * sum_nibbles(neg));
+                if ((threadIdx.x & 31) == 0) sums[(int64_t)(c >> 5) * M + r] = sum;
+            }
             uint8_t *dst = r < M ? A4 + (int64_t)r * pitch_out : B4 + (int64_t)(r - M) * pitch_out;
-            *reinterpret_cast<uint4 *>(dst + 16 * c) = make_uint4(o[0], o[1], o[2], o[3]);
+            if (BITS != 3 || inside) *reinterpret_cast<uint4 *>(dst + 16 * c) = make_uint4(o[0], o[1], o[2], o[3]);
         }
     }
 }
@@ -313,14 +357,17 @@ inline dim3 expand_grid(int64_t chunks, int64_t rows)
 // 16 of them in the epilogue; so, and with tiles of 160 columns: 12.5.)
 template <int KIND>
 __device__ __forceinline__ void g8_store_block(const G8Params &p, int m, int n, int limit, int lane,
-                                               uint32_t stage, const uint32_t (&r)[32])
+                                               uint32_t stage, const uint32_t (&r)[32], float more)
 {
     constexpr bool FACC = KIND != G8_I8;                  // f32 accumulators
     const int row = m + lane;
     // scaled and, of F4, integer results of an accumulator
-    auto whole = [](uint32_t x) { return FACC ? (uint32_t)__float2int_rn(__uint_as_float(x)) : x; };
-    auto scaled = [](uint32_t x, float rs) {
-        return __float_as_uint(__fmul_rn(FACC ? __uint_as_float(x) : (float)(int)x, rs));
+    // (`more` and the sum are whole numbers below 2^24)
+    auto whole = [more](uint32_t x) {
+        return FACC ? (uint32_t)__float2int_rn(__fadd_rn(__uint_as_float(x), more)) : x;
+    };
+    auto scaled = [more](uint32_t x, float rs) {
+        return __float_as_uint(__fmul_rn(FACC ? __fadd_rn(__uint_as_float(x), more) : (float)(int)x, rs));
     };
     const float rs = KIND != G8_BF16 && p.D_f32 && row < p.M ? __ldg(p.row_scale + row) : 0.0f;
     if (p.vec) {
@@ -379,6 +426,16 @@ __device__ __forceinline__ void g8_store_block(const G8Params &p, int m, int n, 
             }
         }
     }
+}
+
+// what is added to the accumulators of row m: 4-bit operands of 3-bit codes
+template <int KIND>
+__device__ __forceinline__ float g8_row_more(const G8Params &p, int m)
+{
+    int s = 0;
+    if (KIND == G8_F4 && p.sums && m < p.M)
+        for (int i = 0; i < p.parts; ++i) s += __ldg(p.sums + (int64_t)i * p.M + m);
+    return (float)(4 * s);
 }
 
 // KIND: 8-bit integer operands with s32 accumulators (kind::i8), bf16 operands or 4-bit
@@ -556,6 +613,7 @@ gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
             const int b = it & 1;
             const int m = (tile / p.n_tiles) * G8_BM + (int)rank * G8_ROWS + quarter * 32;
             const int n0 = (tile % p.n_tiles) * p.BN, limit = min(p.N, n0 + p.BN);
+            const float more = g8_row_more<KIND>(p, m + lane);
             if (!(ok = wait_bar_warp(bar_acc_full(b), (it >> 1) & 1u, ctl, 24))) break;
             tc_fence_after_sync();
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + b * ACC;
@@ -575,7 +633,7 @@ gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
                 tmem_ld_wait();
                 if (c + 2 >= blocks) release();
                 if (m < p.M && n0 + 32 * c < limit)
-                    g8_store_block<KIND>(p, m, n0 + 32 * c, limit, lane, staging, r);
+                    g8_store_block<KIND>(p, m, n0 + 32 * c, limit, lane, staging, r, more);
             }
         }
     }
@@ -614,6 +672,7 @@ gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
         if (warp >= G8_WARP_E0 && pair < total_tiles) {
             const int m = (pair / p.n_tiles) * G8_BM + (int)rank * G8_ROWS + quarter * 32;
             const int n0 = (pair % p.n_tiles) * p.BN + (int)split * cols, limit = min(p.N, n0 + cols);
+            const float more = g8_row_more<KIND>(p, m + lane);
 #pragma unroll 1
             for (int c0 = 32 * k; c0 < cols; c0 += 64) {
                 uint32_t r[32];
@@ -632,7 +691,7 @@ gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
                                                                            __uint_as_float(w[t]));
                     }
                 if (m < p.M && n0 + c0 < limit)
-                    g8_store_block<KIND>(p, m, n0 + c0, limit, lane, staging, r);
+                    g8_store_block<KIND>(p, m, n0 + c0, limit, lane, staging, r, more);
             }
         }
     }
@@ -760,7 +819,15 @@ inline uint8_t *scratch_of(void *workspace)
 
 }  // namespace
 
-static bool f4_exact(int64_t K, int bits) { return bits < 3 && K * (bits == 2 ? 6 : 1) < (1 << 23); }
+// whether every partial sum of 4-bit operands stays below 2^23 (3 bits: products of -4 .. 4 by
+// -4 .. 3, and the results below 2^24)
+static bool f4_exact(int64_t K, int bits)
+{
+    return bits < 4 && K * (bits == 3 ? 16 : bits == 2 ? 6 : 1) < (1 << 23);
+}
+// bytes of a row, and the parts of a row whose sums are kept
+static size_t f4_pitch(int64_t K) { return round_up((size_t)(K + 1) / 2, 16); }
+static int64_t f4_parts(int64_t K) { return (K + 1023) / 1024; }
 
 // Scratch the two-pass path needs behind the status words (0: the problem is
 // one the fused kernel keeps).
@@ -774,21 +841,30 @@ size_t dsq_gemm8_scratch_bytes(int64_t M, int64_t N, int64_t K, int bits, int fo
         if (!dsq_g8_two_passes(M, N, K, bits, f4, clocks)) return 0;
     }
     const size_t kp = round_up((size_t)K, 16);             // (4-bit operands fill half of it)
-    return round_up((size_t)M * kp, 1024) + round_up((size_t)N * kp, 1024);
+    const size_t need = round_up((size_t)M * kp, 1024) + round_up((size_t)N * kp, 1024);
+    if (bits != 3) return need;
+    const size_t k4 = f4_pitch(K);                         // (more than that only below 128 of K)
+    return std::max(need, round_up((size_t)M * k4, 1024) + round_up((size_t)N * k4, 1024) +
+                              (size_t)(f4_parts(K) * M) * sizeof(int32_t));
 }
 
-// 1- and 2-bit operands as 4-bit floating point where every sum stays below 2^23 (f32
+// 1- to 3-bit operands as 4-bit floating point where every sum stays below 2^23 (f32
 // accumulators then hold it exactly whatever the order of the additions): twice the values
 // per instruction and half of the expanded bytes of int8.
 template <int BITS>
-static int launch_f4(const void *A, const void *B, int64_t M, int64_t N, int64_t K, const G8Params &p,
+static int launch_f4(const void *A, const void *B, int64_t M, int64_t N, int64_t K, G8Params p,
                      void *scratch, cudaStream_t stream)
 {
-    const size_t kp = round_up((size_t)(K + 1) / 2, 16);
+    const size_t kp = f4_pitch(K);
     uint8_t *A4 = (uint8_t *)scratch, *B4 = A4 + round_up((size_t)M * kp, 1024);
+    int32_t *sums = nullptr;
+    if (BITS == 3) {
+        p.sums = sums = (int32_t *)(B4 + round_up((size_t)N * kp, 1024));
+        p.parts = (int)f4_parts(K);
+    }
     const int st = dsq_launch(expand_rows_f4_kernel<BITS>, expand_grid((int64_t)kp / 16, M + N),
                               dim3(EX_THREADS), 0, stream, dsq_launch_hooks().pdl, 0, (const uint8_t *)A, (const uint8_t *)B,
-                              (int)M, (int)N, (int)K, (int)dsq_row_pitch(K, BITS), (int)kp, A4, B4);
+                              (int)M, (int)N, (int)K, (int)dsq_row_pitch(K, BITS), (int)kp, A4, B4, sums);
     if (st) return st;
     return launch_pass2<G8_F4>(A4, kp, B4, kp, kp, M, N, true, true, p, stream);
 }
@@ -800,7 +876,9 @@ int dsq_gemm8_launch(const void *A_codes, const void *B_codes, int64_t M, int64_
     G8Params p = {};
     p.C_i32 = C_i32; p.row_scale = row_scale; p.D_f32 = D_f32;
     p.ws = (int *)workspace;
-    if (f4_exact(K, bits)) return launch_f4<2>(A_codes, B_codes, M, N, K, p, scratch, stream);
+    if (f4_exact(K, bits))
+        return bits == 2 ? launch_f4<2>(A_codes, B_codes, M, N, K, p, scratch, stream)
+                         : launch_f4<3>(A_codes, B_codes, M, N, K, p, scratch, stream);
     const size_t kp = round_up((size_t)K, 16);
     uint8_t *A8 = (uint8_t *)scratch;
     uint8_t *B8 = A8 + round_up((size_t)M * kp, 1024);
