@@ -14,7 +14,7 @@
 //           swizzled shared memory by TMA - no thread touches an operand byte.
 //           CTA pairs on tiles of 256 rows and 64 to 256 columns (tcgen05.mma
 //           cta_group::2, kind::i8 or kind::mxf4, both operands through
-//           shared-memory descriptors), a ring of seven or more stages per CTA,
+//           shared-memory descriptors), a ring of five or more stages per CTA,
 //           and TWO accumulators in tensor memory, so the epilogue of a tile (eight
 //           warps per CTA) overlaps the next tile's instructions.
 // The scratch for 4096^3 is 33.5 MB and stays in the 126 MB L2 between the
@@ -54,6 +54,7 @@ constexpr int G8_BARS = 2 * G8_MAX_STAGES + 4 + 1;
 constexpr int G8_SMEM = 226 * 1024, G8_REGS = 128;
 constexpr int G8_TAIL = 8 * G8_BARS + 24;    // barriers, tensor-memory slot, abort flag
 constexpr int G8_STAGING = G8_E_WARPS * 32 * 32 * 4;     // a 32 x 32 block per epilogue warp
+constexpr int G8_EXCHANGE = 64 * 1024;       // sums of the other pair, at most
 static_assert(G8_TAIL % 128 == 0, "the staging blocks are 128-byte aligned");
 
 struct G8Params {
@@ -347,81 +348,123 @@ inline dim3 expand_grid(int64_t chunks, int64_t rows)
 // ---------------------------------------------------------------------------
 // pass 2: int8 GEMM, CTA pairs
 // ---------------------------------------------------------------------------
+// Integer and scaled outputs of an accumulator (f32 ones of 4-bit operands: `more` and the sum
+// are whole numbers below 2^24).
+template <int KIND>
+__device__ __forceinline__ uint32_t g8_whole(uint32_t x, float more)
+{
+    return KIND == G8_I8 ? x : (uint32_t)__float2int_rn(__fadd_rn(__uint_as_float(x), more));
+}
+template <int KIND>
+__device__ __forceinline__ uint32_t g8_scaled(uint32_t x, float more, float rs)
+{
+    return __float_as_uint(__fmul_rn(KIND == G8_I8 ? (float)(int)x : __fadd_rn(__uint_as_float(x), more), rs));
+}
+
 // Outputs of a 32 x 32 block of accumulators: r[j] is row m + lane, column n + j; columns
 // from `limit` on belong to another tile or lie outside.
-// vec: N is a multiple of 8, so every group of eight columns of a row is a full 32-byte
-// sector, inside or outside the matrix as a whole, and a lane stores its row.  Otherwise the
-// block is turned round in shared memory (`stage`, 128-byte aligned; words XOR-ed with their row:
-// no bank conflicts either way) and a warp stores one row after the other, 128 contiguous bytes at a time.
-// (With two adjacent columns a lane, 4-byte stores for odd N, 2500x1111x1777 3-bit took 22 us,
-// 16 of them in the epilogue; so, and with tiles of 160 columns: 12.5.)
+// Where rows are full 32-byte sectors (p.vec) a lane stores its row from its registers.
+// Elsewhere, and for the last weight-only tile of a CTA (no operands arrive any more), the block
+// is turned round in shared memory (`stage`: rows of 128 bytes, 16-byte units XOR-ed with the
+// row: no bank conflicts either way), and a warp stores whole lines: there a lane's scales and
+// biases are those of eight columns, not of all 32.
+// An SM takes 27 bytes of stores a clock in whole lines, 16 in sectors of 32 lines; beside the
+// next tile's instructions that does not show, and the integer kernels' last tile is no faster
+// turned round (4096^3 4-bit 61.4 us against 60.5).  2500x1111x1777 3-bit with 16-byte
+// stores to shared memory and the next block already on its way 12.7 -> 12.0 us, weight-only
+// 2048x4096x4096 55.5 -> 54.1, 3000x1000x512 11.6 -> 10.6, in a graph.
 template <int KIND>
-__device__ __forceinline__ void g8_store_block(const G8Params &p, int m, int n, int limit, int lane,
-                                               uint32_t stage, const uint32_t (&r)[32], float more)
+__device__ __forceinline__ void g8_store_rows(const G8Params &p, int m, int n, int limit, int lane,
+                                              const uint32_t (&r)[32], float more)
 {
-    constexpr bool FACC = KIND != G8_I8;                  // f32 accumulators
     const int row = m + lane;
-    // scaled and, of F4, integer results of an accumulator
-    // (`more` and the sum are whole numbers below 2^24)
-    auto whole = [more](uint32_t x) {
-        return FACC ? (uint32_t)__float2int_rn(__fadd_rn(__uint_as_float(x), more)) : x;
-    };
-    auto scaled = [more](uint32_t x, float rs) {
-        return __float_as_uint(__fmul_rn(FACC ? __fadd_rn(__uint_as_float(x), more) : (float)(int)x, rs));
-    };
-    const float rs = KIND != G8_BF16 && p.D_f32 && row < p.M ? __ldg(p.row_scale + row) : 0.0f;
-    if (p.vec) {
-        if (row >= p.M) return;
-        const int64_t at = (int64_t)row * p.N + n;
+    if (row >= p.M) return;
+    const float rs = KIND != G8_BF16 && p.D_f32 ? __ldg(p.row_scale + row) : 0.0f;
+    const int64_t at = (int64_t)row * p.N + n;
 #pragma unroll
-        for (int j = 0; j < 32; j += 8) {
-            if (n + j >= limit) break;
-            uint32_t f[8];
-            if (KIND == G8_BF16) {
+    for (int j = 0; j < 32; j += 8) {
+        if (n + j >= limit) break;
+        uint32_t f[8];
+        if (KIND == G8_BF16) {
+#pragma unroll
+            for (int t = 0; t < 8; ++t)
+                f[t] = __float_as_uint(
+                    __fmaf_rn(__uint_as_float(r[j + t]), __ldg(p.col_scale + n + j + t),
+                              p.col_bias ? __ldg(p.col_bias + n + j + t) : 0.0f));
+            stg_256(p.Y_f32 + at + j, f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7]);
+            continue;
+        }
+        if (p.C_i32) {
+#pragma unroll
+            for (int t = 0; t < 8; ++t) f[t] = g8_whole<KIND>(r[j + t], more);
+            stg_256(p.C_i32 + at + j, f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7]);
+        }
+        if (p.D_f32) {
+#pragma unroll
+            for (int t = 0; t < 8; ++t) f[t] = g8_scaled<KIND>(r[j + t], more, rs);
+            stg_256(p.D_f32 + at + j, f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7]);
+        }
+    }
+}
+
+// (`next` is called when r has been read for the last time)
+template <int KIND, class F>
+__device__ __forceinline__ void g8_store_turned(const G8Params &p, int m, int n, int limit, int lane,
+                                                uint32_t stage, const uint32_t (&r)[32], float more, F next)
+{
+    const int rows = min(32, p.M - m);
+    const float rs = KIND != G8_BF16 && p.D_f32 && lane < rows ? __ldg(p.row_scale + m + lane) : 0.0f;
+    const uint32_t mine = stage + 128u * (uint32_t)lane;
+    const int last = KIND != G8_BF16 && p.D_f32 ? 1 : 0;
+#pragma unroll 1
+    for (int which = KIND == G8_BF16 || p.C_i32 ? 0 : 1; which <= last; ++which) {
+        uint32_t *const out = KIND == G8_BF16 ? (uint32_t *)p.Y_f32 : which ? (uint32_t *)p.D_f32 : (uint32_t *)p.C_i32;
+        __syncwarp();                                     // (the block before has been read)
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            uint32_t f[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+                f[t] = KIND == G8_BF16 ? r[4 * u + t] : which ? g8_scaled<KIND>(r[4 * u + t], more, rs) : g8_whole<KIND>(r[4 * u + t], more);
+            sts_128(mine + (uint32_t)((u ^ (lane & 7)) << 4), f[0], f[1], f[2], f[3]);
+        }
+        if (which == last) next();
+        __syncwarp();
+        if (KIND == G8_BF16 && p.vec) {
+            const int u = 2 * (lane & 3), r0 = lane >> 2, col = n + 4 * u;
+            if (col >= limit) continue;
+            float cs[8], cb[8];
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+                cs[t] = __ldg(p.col_scale + col + t);
+                cb[t] = p.col_bias ? __ldg(p.col_bias + col + t) : 0.0f;
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int row = 8 * i + r0;
+                const uint32_t at = stage + 128u * (uint32_t)row;
+                const uint4 x = lds_128(at + (uint32_t)((u ^ (row & 7)) << 4));
+                const uint4 y = lds_128(at + (uint32_t)(((u + 1) ^ (row & 7)) << 4));
+                uint32_t f[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
 #pragma unroll
                 for (int t = 0; t < 8; ++t)
-                    f[t] = __float_as_uint(
-                        __fmaf_rn(__uint_as_float(r[j + t]), __ldg(p.col_scale + n + j + t),
-                                  p.col_bias ? __ldg(p.col_bias + n + j + t) : 0.0f));
-                stg_256(p.Y_f32 + at + j, f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7]);
-                continue;
+                    f[t] = __float_as_uint(__fmaf_rn(__uint_as_float(f[t]), cs[t], cb[t]));
+                if (row < rows)
+                    stg_256(out + (int64_t)(m + row) * p.N + col, f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7]);
             }
-            if (p.C_i32) {
-#pragma unroll
-                for (int t = 0; t < 8; ++t) f[t] = whole(r[j + t]);
-                stg_256(p.C_i32 + at + j, f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7]);
-            }
-            if (p.D_f32) {
-#pragma unroll
-                for (int t = 0; t < 8; ++t) f[t] = scaled(r[j + t], rs);
-                stg_256(p.D_f32 + at + j, f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7]);
-            }
+            continue;
         }
-        return;
-    }
-    const int col = n + lane;
-    const int rows = min(32, p.M - m);
-    float cs = 0.0f, cb = 0.0f;
-    if (KIND == G8_BF16 && col < limit) {
-        cs = __ldg(p.col_scale + col);
-        cb = p.col_bias ? __ldg(p.col_bias + col) : 0.0f;
-    }
-#pragma unroll 1
-    for (int which = 0; which < 2; ++which) {
-        uint32_t *const out = KIND == G8_BF16 ? (uint32_t *)(which ? nullptr : p.Y_f32)
-                                              : which ? (uint32_t *)p.D_f32 : (uint32_t *)p.C_i32;
-        if (!out) continue;
-        __syncwarp();
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-            sts_32((stage + 132u * (uint32_t)lane) ^ (uint32_t)(4 * j),
-                   KIND == G8_BF16 ? r[j] : which ? scaled(r[j], rs) : whole(r[j]));
-        __syncwarp();
+        const int col = n + lane;
         if (col < limit) {
+            float cs = 0.0f, cb = 0.0f;
+            if (KIND == G8_BF16) {
+                cs = __ldg(p.col_scale + col);
+                cb = p.col_bias ? __ldg(p.col_bias + col) : 0.0f;
+            }
             uint32_t *dst = out + (int64_t)m * p.N + col;
 #pragma unroll 8
             for (int i = 0; i < rows; ++i, dst += p.N) {
-                const uint32_t v = lds_32((stage + 132u * (uint32_t)i) ^ (uint32_t)(4 * lane));
+                const uint32_t v = lds_32(stage + (uint32_t)(128 * i + ((lane * 4) ^ ((i & 7) << 4))));
                 *dst = KIND == G8_BF16 ? __float_as_uint(__fmaf_rn(__uint_as_float(v), cs, cb)) : v;
             }
         }
@@ -461,7 +504,10 @@ gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(tail + 8 * G8_BARS);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tail + 8 * G8_BARS + 8);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t staging = smem_u32(tail + G8_TAIL) + (uint32_t)((warp - G8_WARP_E0) * 32 * 32 * 4);
+    // (of the last tile in the ring, which nothing reads any more, behind the exchanged sums; where
+    // every tile needs it, behind the ring)
+    const uint32_t staging = smem_u32(p.vec ? smem + (S > 1 ? G8_EXCHANGE : 0) : tail + G8_TAIL) +
+                             (uint32_t)((warp - G8_WARP_E0) * 32 * 32 * 4);
     const uint32_t crank = cluster_ctarank();
     const uint32_t rank = crank & 1u, split = crank >> 1;       // in the pair; which part of K
     const uint32_t leader = crank & ~1u;
@@ -626,14 +672,31 @@ gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
                     else mbar_arrive(bar_acc_empty(b));
                 }
             };
+            if (p.vec && (KIND != G8_BF16 || tile + npairs < total_tiles)) {
+#pragma unroll 1
+                for (int c = half; c < blocks; c += 2) {
+                    uint32_t r[32];
+                    tmem_ld_32x32(taddr + 32 * c, r);
+                    tmem_ld_wait();
+                    if (c + 2 >= blocks) release();
+                    if (n0 + 32 * c < limit) g8_store_rows<KIND>(p, m, n0 + 32 * c, limit, lane, r, more);
+                }
+                continue;
+            }
+            // (a block is on its way from tensor memory while the one before it is stored)
+            uint32_t r[32];
+            tmem_ld_32x32(taddr + 32 * half, r);
 #pragma unroll 1
             for (int c = half; c < blocks; c += 2) {
-                uint32_t r[32];
-                tmem_ld_32x32(taddr + 32 * c, r);
                 tmem_ld_wait();
                 if (c + 2 >= blocks) release();
+                auto next = [&]() {
+                    if (c + 2 < blocks) tmem_ld_32x32(taddr + 32 * (c + 2), r);
+                };
                 if (m < p.M && n0 + 32 * c < limit)
-                    g8_store_block<KIND>(p, m, n0 + 32 * c, limit, lane, staging, r, more);
+                    g8_store_turned<KIND>(p, m, n0 + 32 * c, limit, lane, staging, r, more, next);
+                else
+                    next();
             }
         }
     }
@@ -690,8 +753,9 @@ gemm8_kernel(const __grid_constant__ CUtensorMap tmap_a,
                                                          : __float_as_uint(__uint_as_float(r[4 * v + t]) +
                                                                            __uint_as_float(w[t]));
                     }
-                if (m < p.M && n0 + c0 < limit)
-                    g8_store_block<KIND>(p, m, n0 + c0, limit, lane, staging, r, more);
+                if (m >= p.M || n0 + c0 >= limit) continue;
+                if (p.vec && KIND != G8_BF16) g8_store_rows<KIND>(p, m, n0 + c0, limit, lane, r, more);
+                else g8_store_turned<KIND>(p, m, n0 + c0, limit, lane, staging, r, more, [] {});
             }
         }
     }
