@@ -58,9 +58,11 @@ inline DsqG8Tile dsq_g8_tile(int64_t M, int64_t N, int64_t kblocks, int widest, 
 // where rows are not whole sectors).  The fused kernel: its rounds of K, the expansion of each row
 // once per tile (3-bit rows one K step a round), the outputs (one word at a time where rows
 // are no multiple of 16 bytes).  The slower path is taken for 32 of them, 0.7 % of time on average
-// (fitted to 292 of them, for 14 of the other 230, 0.7 %).  Fused / two passes, us: 4-bit 1024^3
+// (fitted to 292 of them, for 14 of the other 230, 0.7 %).  The expansion launched
+// dependently costs less than the fits' 6.0 us: with 5.3 (4-bit floating point) and 5.7 the slower
+// path is taken for 29 of 400 other problems, 0.7 % of time on average; with 6.0 for 34, 1.0 %.  Fused / two passes, us: 4-bit 1024^3
 // 6.7 / 8.8, 2048^3 16.0 / 15.6 (either), 3072x3072x1024 20.6 / 18.1, 2500x1111x1777 29 / 12.5; 3-bit
-// 1024^3 10.1 / 8.8, 2048^3 22 / 16; 2-bit 2048^3 16.1 / 13.9.
+// 1024^3 10.1 / 7.8, 2048^3 22 / 14.6; 2-bit 2048^3 16.1 / 13.9.
 inline bool dsq_g8_two_passes(int64_t M, int64_t N, int64_t K, int bits, bool f4, double clocks)
 {
     struct Fused { double fixed, k, nk, out, words, word; };
@@ -71,7 +73,7 @@ inline bool dsq_g8_two_passes(int64_t M, int64_t N, int64_t K, int bits, bool f4
     if ((double)M * (double)N * (double)K >= 1.5e10) return true;
     const double out = (double)M * (double)N * 1e-6, k = (double)K * 1e-3;
     const Fused &f = fused[bits - 2];
-    const double two = 6.0 + clocks / 2310.0 + (N % 8 ? 1.02 : 0.65) * out +
+    const double two = (f4 ? 5.3 : 5.7) + clocks / 2310.0 + (N % 8 ? 1.02 : 0.65) * out +
                        0.157e-6 * (double)(M + N) * (double)K * (bits / 8.0 + (f4 ? 0.5 : 1.0));
     return two < f.fixed + f.k * k + f.nk * out * k + f.out * out + (N % 4 ? f.words + f.word * out : 0.0);
 }
