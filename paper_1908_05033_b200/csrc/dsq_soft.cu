@@ -4,6 +4,10 @@
 // element backward (x and dL/dy in, dL/dx out) plus three scalar reductions.
 #include "dsq_common.cuh"
 #include "dsq_launch.h"
+#include "dsq_ptx.cuh"
+
+using dsq_ptx::grid_dependency_wait;
+using dsq_ptx::grid_launch_dependents;
 
 namespace {
 
@@ -68,6 +72,8 @@ __global__ void __launch_bounds__(256) soft_fwd_kernel(const float *__restrict__
                                                        float *__restrict__ y, int64_t n,
                                                        int64_t head, SoftP p)
 {
+    grid_dependency_wait();
+    grid_launch_dependents();
     const int64_t n8 = (n - head) >> 3;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -131,6 +137,17 @@ __device__ __forceinline__ float soft_bwd_one(float x, float g, const SoftP &p, 
     return x != x ? x : gx;
 }
 
+// Clears the three sums.  The backward kernel, launched dependently behind it, starts when
+// everything ahead of this one has completed and waits for it only before it adds to the sums.
+// With a memset in front, 16384 / 1M / 12.8M elements took 6.2 / 7.7 / 29.2 us in a graph, so 2.7 / 4.5 / 26.7
+// (forward and backward 8.4 / 10.7 / 48.8 -> 4.3 / 7.0 / 44.4).
+__global__ void soft_clear_kernel(double *sums)
+{
+    grid_dependency_wait();
+    grid_launch_dependents();
+    if (threadIdx.x < 3) sums[threadIdx.x] = 0.0;
+}
+
 // 12.8M elements 41.9 -> 28.9 us, 67M 182 -> 126 us (the sums' binary64 additions and the
 // conversions in front of them run beside the loads).
 __global__ void __launch_bounds__(256) soft_bwd_kernel(const float *__restrict__ x,
@@ -182,6 +199,8 @@ __global__ void __launch_bounds__(256) soft_bwd_kernel(const float *__restrict__
     __shared__ double part[3][8];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (lane == 0) { part[0][warp] = aa; part[1][warp] = al; part[2][warp] = au; }
+    grid_dependency_wait();                        // the sums are clear
+    grid_launch_dependents();
     __syncthreads();
     if (threadIdx.x < 3) {
         double s = 0.0;
@@ -250,8 +269,8 @@ extern "C" int dsq_soft_quantize_fwd(const float *x, int64_t n, const dsq_quant_
     if (st) return st;
     if (n <= 0) return DSQ_ERR_SHAPE;
     if (!dsq_aligned16(x) || !dsq_aligned16(y)) return DSQ_ERR_ALIGN;
-    return dsq_launch(soft_fwd_kernel, dim3(soft_grid(n, 16)), dim3(256), 0, (cudaStream_t)stream, 0, 0,
-                      x, y, n, soft_head(x, y, y, n), p);
+    return dsq_launch(soft_fwd_kernel, dim3(soft_grid(n, 16)), dim3(256), 0, (cudaStream_t)stream,
+                      dsq_launch_hooks().pdl, 0, x, y, n, soft_head(x, y, y, n), p);
 }
 
 extern "C" int dsq_soft_quantize_bwd(const float *x, const float *grad_y, int64_t n,
@@ -267,7 +286,9 @@ extern "C" int dsq_soft_quantize_bwd(const float *x, const float *grad_y, int64_
         (reinterpret_cast<uintptr_t>(grad_params) & 7u))
         return DSQ_ERR_ALIGN;
     cudaStream_t s = (cudaStream_t)stream;
-    DSQ_CUDA_TRY(cudaMemsetAsync(grad_params, 0, 3 * sizeof(double), s));
-    return dsq_launch(soft_bwd_kernel, dim3(soft_grid(n, 4)), dim3(256), 0, s, 0, 0, x, grad_y, grad_x,
+    const int pdl = dsq_launch_hooks().pdl;
+    const int st2 = dsq_launch(soft_clear_kernel, dim3(1), dim3(32), 0, s, pdl, 0, grad_params);
+    if (st2) return st2;
+    return dsq_launch(soft_bwd_kernel, dim3(soft_grid(n, 4)), dim3(256), 0, s, pdl, 0, x, grad_y, grad_x,
                       n, soft_head(x, grad_y, grad_x, n), p, grad_params);
 }
