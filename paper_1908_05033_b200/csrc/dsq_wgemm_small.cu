@@ -151,6 +151,21 @@ wgemm_small_kernel(const WsParams p)
             }
     };
     load_w(warp);
+    // A thread's outputs lie in one column.  Its scale and bias come with the first loads where the
+    // loop leaves registers for them (asked for behind the last barrier, in a graph: 48x1000x3000
+    // 3-bit 9.0 us, so 7.9; 8x1024x1024 4-bit 2.3 / 2.1; 17 to 32 rows, blocks of
+    // 32 columns and 16 rows at 3 bits are slower with them: 24x600x5000 2-bit 7.5 / 8.3, 8x1024x1024 3-bit
+    // 2.55 / 2.68).
+    constexpr bool FIRST = MT == 4 || (MT == 1 && NT == 2 && BITS != 3);
+    float cs = 0.f, cb = 0.f;
+    if (FIRST) {
+        static_assert(WARPS * 32 % (8 * NT) == 0, "one column a thread");
+        const int at = n0 + threadIdx.x % (8 * NT);
+        if (at < p.N) {
+            cs = __ldg(p.col_scale + at);
+            if (p.col_bias) cb = __ldg(p.col_bias + at);
+        }
+    }
 #pragma unroll 1
     for (int c = warp; c < chunks; c += WARPS) {
         uint32_t w[NT][BITS];
@@ -224,7 +239,8 @@ wgemm_small_kernel(const WsParams p)
         for (int w = 0; w < 8; ++w) s += part[w][m * NT + t][l][i];
         if (m0 + row < p.M && n0 + col < p.N)
             p.Y[(int64_t)(m0 + row) * p.N + n0 + col] =
-                __fmaf_rn(s, __ldg(p.col_scale + n0 + col), p.col_bias ? __ldg(p.col_bias + n0 + col) : 0.f);
+                FIRST ? __fmaf_rn(s, cs, cb)
+                      : __fmaf_rn(s, __ldg(p.col_scale + n0 + col), p.col_bias ? __ldg(p.col_bias + n0 + col) : 0.f);
     }
 }
 
