@@ -134,8 +134,10 @@ struct DsqSmallTile {
 };
 
 // Fitted to the layers of the ResNet-18- and MobileNetV2-shaped networks at batches of 1, 2 and 4:
-// the longer of a block's chain (0.55 us for every chunk a warp walks) and what the blocks of
-// an SM take together (most of it per warp, whatever it has to do).
+// the longer of a block's chain (0.55 us for every chunk a warp walks, 0.33 where it asks for the next one's
+// activations ahead) and what the blocks of an SM take together (most of it per warp, whatever it
+// has to do).  Of 159 layers of those networks, images of half to 1.2 times their sides, batches of 1 to
+// 12: 1.1 % slower than the fastest of the five forms on average (2.0 % with 0.55 for both).
 inline DsqSmallTile dsq_small_tile(int M, int Ncols, int chunks, int bits, int sms)
 {
     DsqSmallTile best = {0, 0, 0.0};
@@ -146,7 +148,7 @@ inline DsqSmallTile dsq_small_tile(int M, int Ncols, int chunks, int bits, int s
             const double f = bits == 4 ? 1.0 : 2.0;
             const double fixed = mt == 1 ? (warps == 4 ? 0.44 : warps == 8 ? 1.1 : 2.5) : (warps == 4 ? 0.7 : 1.35);
             const double per_block = fixed + f * (mt == 1 ? 0.06 : 0.09) * chunks;
-            const double chain = 1.5 + 0.05 * warps + 0.55 * (bits == 4 ? 1.0 : 1.3) * ((chunks + warps - 1) / warps);
+            const double chain = 1.5 + 0.05 * warps + (mt == 1 ? 0.33 : 0.55) * (bits == 4 ? 1.0 : 1.3) * ((chunks + warps - 1) / warps);
             const double us = std::max(chain, 1.2 + blocks / sms * per_block);
             if (best.mt == 0 || us < best.us) best = DsqSmallTile{mt, warps, us};
         }
@@ -154,7 +156,9 @@ inline DsqSmallTile dsq_small_tile(int M, int Ncols, int chunks, int bits, int s
 }
 
 // And what the other kernel for a layer of M output pixels takes: the window kernel as it says
-// itself; the im2col kernel a floor that grows with K (the few CTAs such a layer has walk it
+// itself; the 1x1 kernel a launch, its outputs and its planes (464 layers of 16 to 1024 outputs, batches
+// of 1 to 16, 6 % off in the mean; more than 3 % slower than the faster kernel 8 of them, 0.3 % on average, where
+// 2.9 + M Cout / 3.7e6 left 73 and 3.0 %); the im2col kernel a floor that grows with K (the few CTAs such a layer has walk it
 // alone) plus its work at full rate, and twice that at 3 bits, where a round is one K step.
 // Measured: 1758 3x3 layers of 64 to 512 channels in and 32 to 1280 out (strides 1 and 2, 2 to
 // 4 bits, both weight grids, batches of 1 to 32): the slower kernel for 23 of them, 0.2 % of time on average;
@@ -162,10 +166,12 @@ inline DsqSmallTile dsq_small_tile(int M, int Ncols, int chunks, int bits, int s
 // 3 to 30 rows: for 32, 1.1 %.  (Without the limit on the outputs, the plain tiles and the factor for
 // 3 bits: 53, 0.6 %; 205, 2.8 %; 72 and 3.4 % without the plain tiles.)
 inline double dsq_small_other(const dsq_nhwc_t *shape, int bits, const dsq_conv_t *conv, int M, int expanded, int lean,
-                              int sms)
+                              int sms, int residual = 0)
 {
     const int ksize = conv->KH;
-    if (ksize == 1 && lean) return 2.9 + (double)M * conv->Cout / 3.7e6;
+    if (ksize == 1 && lean)
+        return 2.9 + 0.9e-6 * (double)M * conv->Cout + 0.41 * conv->Cin / 128.0 + (conv->stride == 2 ? 0.24 : 0.0) +
+               (residual ? 0.73 : 0.0) + (bits == 3 ? 0.72 : 0.0);
     const double window = dsq_conv3_estimate(shape, bits, conv, expanded, sms);
     if (window > 0.0) return window;
     return (bits == 3 ? 2.05 : 1.0) *

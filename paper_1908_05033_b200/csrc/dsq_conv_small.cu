@@ -13,6 +13,13 @@
 //     codes.  tcgen05 would need them in shared or tensor memory first; the fragment
 //     instruction does 1,861 multiply-accumulates a clock and SM (measured), a
 //     quarter of its rate, which is plenty here;
+//   * a warp that walks several chunks asks for the next one's words, activations and
+//     weights, before this one's arithmetic (AHEAD).  At one image the loads and the
+//     arithmetic are 1.3 to 2.6 us of a layer's 3.4 to 4.5, half of it the latency of a chunk's
+//     activations: 14x14 256->256 with residual 4.07 -> 3.21 us, 7x7 512->512 4.47 -> 3.86, two
+//     images 5.60 -> 4.06.  In tiles of two pixel rows the registers for it cost the block
+//     that could sit beside: only where a warp walks four chunks or more (7x7 512->512 at
+//     batch 8 8.84 -> 8.32; 28x28 128->128 at batch 3, two to three chunks, 4.27 -> 4.57);
 //   * the weights of the first chunk, the scales and the biases are fetched before the
 //     wait for the previous kernel, and blocks are small enough to sit beside that
 //     kernel's.
@@ -89,8 +96,8 @@ __device__ __forceinline__ uint32_t byte_word(const uint32_t (&v)[Unit<BITS>::WO
 
 // (NT is 4 wherever it is launched; as a constant of the file the same source compiles to
 // a kernel that is slower for the ResNet-18-shaped network at batch 1, 67.0 -> 69.0 us)
-template <int BITS, int MT, int NT>
-__global__ void __launch_bounds__((MT == 1 ? CS_MAX_WARPS : 8) * 32)
+template <int BITS, int MT, int NT, bool AHEAD>
+__global__ void __launch_bounds__((MT == 1 ? CS_MAX_WARPS : 8) * 32, AHEAD && MT == 1 ? 1 : 0)
 conv_small_kernel(const CsParams p)
 {
     constexpr int WORDS = Unit<BITS>::WORDS, UNIT_BYTES = 4 * WORDS;
@@ -165,10 +172,9 @@ conv_small_kernel(const CsParams p)
                 if (byte0 + b < p.out_pitch) res |= (uint32_t)__ldg(rp + b) << (8 * b);
     }
 
-#pragma unroll 1
-    while (c < p.chunks) {
+    uint32_t an[MT][2][WORDS];
+    auto load_a = [&]() {
         const int kh = p.ksize == 1 ? 0 : (tap * 11) >> 5, kw = tap - kh * p.ksize;
-        uint32_t av[MT][2][WORDS];
 #pragma unroll
         for (int m = 0; m < MT; ++m)
 #pragma unroll
@@ -176,8 +182,20 @@ conv_small_kernel(const CsParams p)
                 const int hi = hb[m][h] + kh, wi = wb[m][h] + kw;
                 const bool in = tap < p.ksize * p.ksize && hi >= 0 && hi < p.H && wi >= 0 && wi < p.W;
                 load_unit<BITS>(p.act + (int64_t)(at0[m][h] + kh * p.W + kw) * p.P + s * UNIT_BYTES, in,
-                                p.P - s * UNIT_BYTES, av[m][h]);
+                                p.P - s * UNIT_BYTES, an[m][h]);
             }
+    };
+    if (AHEAD) load_a();
+#pragma unroll 1
+    while (c < p.chunks) {
+        if (!AHEAD) load_a();
+        uint32_t av[MT][2][WORDS];
+#pragma unroll
+        for (int m = 0; m < MT; ++m)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int i = 0; i < WORDS; ++i) av[m][h][i] = an[m][h][i];
         uint32_t w[NT][WORDS];
 #pragma unroll
         for (int t = 0; t < NT; ++t)
@@ -188,6 +206,7 @@ conv_small_kernel(const CsParams p)
         s += p.d_s;
         if (s >= p.upt) { s -= p.upt; ++tap; }
         load_w();
+        if (AHEAD) load_a();
 #pragma unroll
         for (int q = 0; q < Unit<BITS>::BYTE_WORDS; q += 2) {
             uint32_t a[MT][4];
@@ -290,15 +309,15 @@ conv_small_kernel(const CsParams p)
     }
 }
 
-template <int BITS, int MT, int NT>
+template <int BITS, int MT, int NT, bool AHEAD>
 int launch(const CsParams &p, int warps, cudaStream_t s)
 {
     const size_t smem = (size_t)warps * MT * NT * 32 * 16;
     static std::atomic<unsigned long long> configured{0ull};
-    const int st = dsq_allow_smem((const void *)conv_small_kernel<BITS, MT, NT>, CS_MAX_WARPS * MT * NT * 512,
-                                  &configured);
+    const int st = dsq_allow_smem((const void *)conv_small_kernel<BITS, MT, NT, AHEAD>,
+                                  CS_MAX_WARPS * MT * NT * 512, &configured);
     if (st) return st;
-    return dsq_launch(conv_small_kernel<BITS, MT, NT>,
+    return dsq_launch(conv_small_kernel<BITS, MT, NT, AHEAD>,
                       dim3((p.Ncols + 8 * NT - 1) / (8 * NT), (p.M + 16 * MT - 1) / (16 * MT)),
                       dim3(32 * warps), smem, s, dsq_launch_hooks().pdl, 0, p);
 }
@@ -308,7 +327,8 @@ int pick(CsParams &p, int mt, int warps, cudaStream_t s)
 {
     p.d_tap = 4 * warps / p.upt;
     p.d_s = 4 * warps - p.d_tap * p.upt;
-    return mt == 2 ? launch<BITS, 2, 4>(p, warps, s) : launch<BITS, 1, 4>(p, warps, s);
+    if (mt == 1) return launch<BITS, 1, 4, true>(p, warps, s);
+    return p.chunks > 3 * warps ? launch<BITS, 2, 4, true>(p, warps, s) : launch<BITS, 2, 4, false>(p, warps, s);
 }
 
 }  // namespace
@@ -342,7 +362,8 @@ int dsq_conv_small(const void *act_codes, const dsq_nhwc_t *shape, int bits, con
         return DSQ_ERR_UNSUPPORTED;
     const int sms = dsq_sm_count() > 0 ? dsq_sm_count() : 148;
     const DsqSmallTile best = dsq_small_tile(p.M, p.Ncols, p.chunks, bits, sms);
-    if (best.us > dsq_small_other(shape, bits, conv, p.M, e.half_offset && dsq_launch_hooks().w8, lean, sms))
+    if (best.us > dsq_small_other(shape, bits, conv, p.M, e.half_offset && dsq_launch_hooks().w8, lean, sms,
+                                  e.residual != nullptr))
         return DSQ_ERR_UNSUPPORTED;
     switch (bits) {
     case 2: return pick<2>(p, best.mt, best.warps, stream);
