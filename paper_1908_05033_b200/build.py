@@ -13,9 +13,9 @@ HOST_LIB = os.path.join(HERE, "_dsq_host.so")
 HOST_SOURCE = "dsq_host.cpp"
 OBJ_DIR = os.path.join(HERE, "_build")
 SOURCES = ["dsq_elementwise.cu", "dsq_dwconv.cu", "dsq_tc.cu", "dsq_conv3.cu", "dsq_pw.cu", "dsq_gemm8.cu",
-           "dsq_wgemm_small.cu", "dsq_conv_small.cu",
+           "dsq_wgemm_small.cu", "dsq_gemm_small.cu", "dsq_conv_small.cu",
            "dsq_soft.cu", "dsq_plan.cu", "dsq_workspace.cu"]
-HEADERS = ["dsq_common.cuh", "dsq_conv_rule.h", "dsq_epilogue.cuh", "dsq_gemm8_rule.h", "dsq_ptx.cuh", "dsq_tc_common.cuh",
+HEADERS = ["dsq_common.cuh", "dsq_conv_rule.h", "dsq_epilogue.cuh", "dsq_fragments.cuh", "dsq_gemm8_rule.h", "dsq_ptx.cuh", "dsq_tc_common.cuh",
            "dsq_tc_host.h", "dsq_hooks.h", "dsq_launch.h", "dsq_plan.h",
            os.path.join("..", "..", "include", "dsq.h")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo",

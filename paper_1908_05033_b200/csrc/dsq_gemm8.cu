@@ -912,6 +912,18 @@ size_t dsq_gemm8_scratch_bytes(int64_t M, int64_t N, int64_t K, int bits, int fo
                               (size_t)(f4_parts(K) * M) * sizeof(int32_t));
 }
 
+// What the fused kernel or the two passes, whichever is faster, are expected to take (microseconds).
+double dsq_gemm8_estimate(int64_t M, int64_t N, int64_t K, int bits)
+{
+    const bool f4 = f4_exact(K, bits);
+    const bool two = M >= 128 && N >= 128 && K >= 128;
+    const double clocks = !two ? 0.0
+                          : f4 ? pick_tile<G8_F4>(M, N, (K + 255) / 256).clocks
+                               : pick_tile<G8_I8>(M, N, (K + 127) / 128).clocks;
+    const DsqGemmTimes t = dsq_gemm_times(M, N, K, bits, f4, clocks);
+    return two ? std::min(t.fused, t.two) : t.fused;
+}
+
 // 1- to 3-bit operands as 4-bit floating point where every sum stays below 2^23 (f32
 // accumulators then hold it exactly whatever the order of the additions): twice the values
 // per instruction and half of the expanded bytes of int8.

@@ -63,19 +63,53 @@ inline DsqG8Tile dsq_g8_tile(int64_t M, int64_t N, int64_t kblocks, int widest, 
 // path is taken for 29 of 400 other problems, 0.7 % of time on average; with 6.0 for 34, 1.0 %.  Fused / two passes, us: 4-bit 1024^3
 // 6.7 / 8.8, 2048^3 16.0 / 15.6 (either), 3072x3072x1024 20.6 / 18.1, 2500x1111x1777 29 / 12.5; 3-bit
 // 1024^3 10.1 / 7.8, 2048^3 22 / 14.6; 2-bit 2048^3 16.1 / 13.9.
-inline bool dsq_g8_two_passes(int64_t M, int64_t N, int64_t K, int bits, bool f4, double clocks)
+struct DsqGemmTimes { double fused, two; };
+inline DsqGemmTimes dsq_gemm_times(int64_t M, int64_t N, int64_t K, int bits, bool f4, double clocks)
 {
     struct Fused { double fixed, k, nk, out, words, word; };
     static const Fused fused[3] = {{4.3, 1.76, 0.483, 1.11, 2.5, 4.6},
                                    {4.7, 4.52, 1.015, 0.965, 0.8, 5.5},
                                    {4.3, 1.85, 0.506, 1.21, 0.5, 5.9}};
-    // beyond the range of the fits (4096^3: 75 / 52)
-    if ((double)M * (double)N * (double)K >= 1.5e10) return true;
     const double out = (double)M * (double)N * 1e-6, k = (double)K * 1e-3;
     const Fused &f = fused[bits - 2];
     const double two = (f4 ? 5.3 : 5.7) + clocks / 2310.0 + (N % 8 ? 1.02 : 0.65) * out +
                        0.157e-6 * (double)(M + N) * (double)K * (bits / 8.0 + (f4 ? 0.5 : 1.0));
-    return two < f.fixed + f.k * k + f.nk * out * k + f.out * out + (N % 4 ? f.words + f.word * out : 0.0);
+    return {f.fixed + f.k * k + f.nk * out * k + f.out * out + (N % 4 ? f.words + f.word * out : 0.0), two};
+}
+inline bool dsq_g8_two_passes(int64_t M, int64_t N, int64_t K, int bits, bool f4, double clocks)
+{
+    // beyond the range of the fits (4096^3: 75 / 52)
+    if ((double)M * (double)N * (double)K >= 1.5e10) return true;
+    const DsqGemmTimes t = dsq_gemm_times(M, N, K, bits, f4, clocks);
+    return t.two < t.fused;
+}
+
+// The GEMM with little work (dsq_gemm_small.cu): 16 mt rows x 32 columns a block of `warps` warps, and the
+// microseconds it is expected to take: the longer of a block's chain (its chunks of K a warp)
+// and what the blocks of an SM take together, with the outputs.  units: of a packed row; outs:
+// arrays written.
+// Fitted to 760 problems of 16 to 6144 a side and up to 1.3e9 multiply-accumulates, one or both
+// outputs (11 % off in the mean); of those, with the estimates of the other kernels, 2.0 % slower than the
+// fastest of all on average, 4 more than 3 % slower than the fused kernel or the two passes
+// (without it 1.8 times as long).
+struct DsqGemmSmallTile { int mt, warps; double us; };
+inline DsqGemmSmallTile dsq_gemm_small_tile(int64_t M, int64_t N, int64_t units, int bits, int outs, int sms)
+{
+    const int64_t chunks = (units + 3) / 4;
+    // (instructions a chunk: a 2-bit unit is twice the codes, 3-bit fields take more of them)
+    const double f = bits == 4 ? 1.0 : bits == 3 ? 2.5 : 1.95, chain_f = bits == 4 ? 1.0 : bits == 3 ? 2.0 : 1.67;
+    DsqGemmSmallTile best = {0, 0, 0.0};
+    for (int mt = 1; mt <= 2; ++mt)
+        for (int warps = 4; warps <= 8; warps *= 2) {
+            const double blocks = (double)((M + 16 * mt - 1) / (16 * mt)) * (double)((N + 31) / 32);
+            const double chain = 1.68 + 0.023 * warps + (mt == 1 ? 0.33 : 0.51) * chain_f * (double)((chunks + warps - 1) / warps);
+            const double fixed = mt == 1 ? (warps == 4 ? 0.21 : 0.57) : (warps == 4 ? 0.5 : 1.29);
+            const double all = 1.2 + blocks / sms * (fixed + (mt == 1 ? 0.052 : 0.104) * f * (double)chunks) +
+                               0.82e-6 * (double)M * (double)N * outs;
+            const double us = std::max(chain, all);
+            if (best.mt == 0 || us < best.us) best = DsqGemmSmallTile{mt, warps, us};
+        }
+    return best;
 }
 
 // Whether the weight-only GEMM of few rows does better than two passes of `clocks` in the

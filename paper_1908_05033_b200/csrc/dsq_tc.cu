@@ -1747,10 +1747,18 @@ int dsq_gemm(const void *A_codes, const void *B_codes, int64_t M, int64_t N, int
     if (!dsq_aligned16(workspace)) return DSQ_ERR_ALIGN;
     if (ws_bytes < DSQ_WS_BYTES) return DSQ_ERR_SIZE;
 
+    // little work: a latency-bound kernel of its own (the hooks force the others; up to what its
+    // rule was fitted to)
+    const int two_pass = g_two_pass.load();
+    if (two_pass == 1 && (double)M * (double)N * (double)K < 1e9 && !g_forced_bn.load() && !g_forced_ks.load() &&
+        !g_pair_mode.load() && g_skip_b_round.load() < 0) {
+        st = dsq_gemm_small(A_codes, B_codes, M, N, K, bits, C_i32, row_scale, D_f32,
+                            dsq_gemm8_estimate(M, N, K, bits), (cudaStream_t)stream);
+        if (st != DSQ_ERR_UNSUPPORTED) return st;
+    }
     // large problems, when the caller's workspace has room for the expanded
     // operands (dsq_gemm_workspace_bytes): expand every row once, then an
     // 8-bit GEMM fed by TMA alone
-    const int two_pass = g_two_pass.load();
     const size_t scratch_need = two_pass ? dsq_gemm8_scratch_bytes(M, N, K, bits, two_pass == 2) : 0;
     if (scratch_need) {
         const uintptr_t w0 = reinterpret_cast<uintptr_t>(workspace);
