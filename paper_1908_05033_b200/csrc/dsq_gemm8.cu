@@ -1034,8 +1034,9 @@ int dsq_wgemm_bf16(const void *X_bf16, const void *W_codes, int64_t M, int64_t N
     const size_t wp = round_up((size_t)K, 8) * 2;          // scratch row pitch in bytes
     if (ws_bytes < (size_t)(W16 - (uint8_t *)workspace) + round_up((size_t)N * wp, 1024))
         return DSQ_ERR_SIZE;
-    if (M <= 32 || dsq_wgemm_takes_small(M, N, K, dsq_sm_count() > 0 ? dsq_sm_count() : 148,
-                                         pick_tile<G8_BF16>(M, N, (K + 63) / 64).clocks))
+    const int sms = dsq_sm_count() > 0 ? dsq_sm_count() : 148;
+    const double clocks = M <= 32 ? 0.0 : pick_tile<G8_BF16>(M, N, (K + 63) / 64).clocks;
+    if (M <= 32 || dsq_wgemm_takes_small(M, N, K, sms, clocks) || dsq_wgemm_takes_wide(M, N, K, sms, clocks))
         return dsq_wgemm_small(X_bf16, W_codes, M, N, K, bits, w_offset == 0.5f, col_scale, col_bias,
                                Y_f32, (cudaStream_t)stream);
     const int pitch_in = (int)dsq_row_pitch(K, bits);

@@ -27,6 +27,7 @@
 // 16 x 4096 x 4096, 4-bit: 45.2 us in two passes, 5.9 here.
 #include <cuda_bf16.h>
 
+#include "dsq_gemm8_rule.h"
 #include "dsq_launch.h"
 #include "dsq_tc_host.h"
 
@@ -87,7 +88,8 @@ wgemm_small_kernel(const WsParams p)
     constexpr int D = Fields<BITS>::D, GROUPS = Fields<BITS>::GROUPS, WARPS = Warps<MT>::N;
     constexpr bool ALL = MT <= 2;              // X of a whole chunk in registers
     constexpr int XG = ALL ? GROUPS : 1;
-    __shared__ float part[8][MT * NT][32][4];
+    constexpr int PARTS = MT * NT > 8 ? 4 : 8;
+    __shared__ float part[PARTS][MT * NT][32][4];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n = lane >> 2, j = lane & 3;
     const int n0 = blockIdx.x * 8 * NT, m0 = blockIdx.y * 16 * MT;
@@ -156,7 +158,7 @@ wgemm_small_kernel(const WsParams p)
     // 3-bit 9.0 us, so 7.9; 8x1024x1024 4-bit 2.3 / 2.1; 17 to 32 rows, blocks of
     // 32 columns and 16 rows at 3 bits are slower with them: 24x600x5000 2-bit 7.5 / 8.3, 8x1024x1024 3-bit
     // 2.55 / 2.68).
-    constexpr bool FIRST = MT == 4 || (MT == 1 && NT == 2 && BITS != 3);
+    constexpr bool FIRST = (MT == 4 && NT == 2) || (MT == 1 && NT == 2 && BITS != 3);
     float cs = 0.f, cb = 0.f;
     if (FIRST) {
         static_assert(WARPS * 32 % (8 * NT) == 0, "one column a thread");
@@ -207,7 +209,7 @@ wgemm_small_kernel(const WsParams p)
             }
         }
     }
-    // the warps' sums, added in a fixed order: warps 8 .. 15 into 0 .. 7, those in turn
+    // the warps' sums, added in a fixed order: those from PARTS on into the ones before, those in turn
     auto put = [&](int at) {
 #pragma unroll
         for (int m = 0; m < MT; ++m)
@@ -216,10 +218,11 @@ wgemm_small_kernel(const WsParams p)
                 *reinterpret_cast<float4 *>(part[at][m * NT + t][lane]) =
                     make_float4(acc[m][t][0], acc[m][t][1], acc[m][t][2], acc[m][t][3]);
     };
-    if (WARPS > 8) {
-        if (warp >= 8) put(warp - 8);
+    static_assert(WARPS <= 2 * PARTS, "two rounds of sums");
+    if (WARPS > PARTS) {
+        if (warp >= PARTS) put(warp - PARTS);
         __syncthreads();
-        if (warp < 8)
+        if (warp < PARTS)
 #pragma unroll
             for (int m = 0; m < MT; ++m)
 #pragma unroll
@@ -227,7 +230,7 @@ wgemm_small_kernel(const WsParams p)
 #pragma unroll
                     for (int i = 0; i < 4; ++i) acc[m][t][i] += part[warp][m * NT + t][lane][i];
     }
-    if (warp < 8) put(warp);
+    if (warp < PARTS) put(warp);
     __syncthreads();
     for (int e = threadIdx.x; e < MT * NT * 128; e += WARPS * 32) {
         // element e of the tile in row-major order: row 16 MT, column 8 NT
@@ -236,7 +239,7 @@ wgemm_small_kernel(const WsParams p)
         const int l = (row & 7) * 4 + ((col & 7) >> 1), i = 2 * ((row >> 3) & 1) + (col & 1);
         float s = 0.f;
 #pragma unroll
-        for (int w = 0; w < 8; ++w) s += part[w][m * NT + t][l][i];
+        for (int w = 0; w < PARTS; ++w) s += part[w][m * NT + t][l][i];
         if (m0 + row < p.M && n0 + col < p.N)
             p.Y[(int64_t)(m0 + row) * p.N + n0 + col] =
                 FIRST ? __fmaf_rn(s, cs, cb)
@@ -260,10 +263,11 @@ int pick(const WsParams &p, cudaStream_t s)
     // K = 4096, us with 16 / 32 columns: N = 2048 (128 blocks of 16) 1 row 3.6 / 5.2, 16 rows
     // 4.6 / 5.7, 32 rows 7.2 / 8.3; N = 2400 (150) 5.3 / 5.2, 7.0 / 5.9, 12.7 / 8.5; N = 4096
     // 5.5 / 5.2, 7.2 / 5.9, 13.2 / 8.5.
-    const bool wide = p.N > 16 * (dsq_sm_count() > 0 ? dsq_sm_count() : 148);
+    const int sms = dsq_sm_count() > 0 ? dsq_sm_count() : 148;
+    const bool wide = p.N > 16 * sms;
     if (p.M <= 16) return wide ? launch<BITS, 1, 4>(p, s) : launch<BITS, 1, 2>(p, s);
     if (p.M <= 32) return wide ? launch<BITS, 2, 4>(p, s) : launch<BITS, 2, 2>(p, s);
-    return launch<BITS, 4, 2>(p, s);
+    return dsq_wgemm_small_columns(p.M, p.N, sms) == 32 ? launch<BITS, 4, 4>(p, s) : launch<BITS, 4, 2>(p, s);
 }
 
 }  // namespace
