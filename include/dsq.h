@@ -240,11 +240,11 @@ int dsq_gemm(const void *A_codes, const void *B_codes, int64_t M, int64_t N,
 
 /* Workspace with which dsq_gemm runs this problem fastest.  Any workspace of
  * dsq_workspace_bytes() works (one fused kernel that expands the packed codes
- * tile by tile).  Given this many bytes (the status words, then room for both
+ * tile by tile, or, with little work, one that takes them straight to registers).  Given this many bytes (the status words, then room for both
  * operands as 8-bit rows: about (M + N) * K bytes), problems for which it is
  * the faster way (large ones; smaller ones at 2 and 3 bits, and where N is not
  * a multiple of 4) take two passes instead: every packed row is expanded once,
- * to 8-bit lanes or, at 2 bits, to 4-bit floating point, then a tensor-core
+ * to 8-bit lanes or, at 2 and 3 bits, to 4-bit floating point, then a tensor-core
  * GEMM reads the rows by TMA.  Same results
  * bit for bit.  The area behind the first dsq_workspace_bytes() bytes is
  * scratch: its contents after the call are unspecified, and calls that may

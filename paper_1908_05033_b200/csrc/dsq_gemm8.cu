@@ -14,7 +14,7 @@
 //           swizzled shared memory by TMA - no thread touches an operand byte.
 //           CTA pairs on tiles of 256 rows and 64 to 256 columns (tcgen05.mma
 //           cta_group::2, kind::i8 or kind::mxf4, both operands through
-//           shared-memory descriptors), a ring of five or more stages per CTA,
+//           shared-memory descriptors), a ring of six or more stages per CTA,
 //           and TWO accumulators in tensor memory, so the epilogue of a tile (eight
 //           warps per CTA) overlaps the next tile's instructions.
 // The scratch for 4096^3 is 33.5 MB and stays in the 126 MB L2 between the

@@ -45,8 +45,8 @@ int dsq_set_conv3_window(int mode);
 int dsq_set_conv3_expanded_weights(int on);
 
 /* dsq_gemm with a workspace large enough for the expanded operands: 1 = take
- * the two-pass path where it is the faster one (default: see
- * dsq_gemm_workspace_bytes), 0 = always the fused kernel, 2 = two passes whatever the
+ * the two-pass path where it is the faster one, and the little-work kernel where
+ * that is (default: see dsq_gemm_workspace_bytes), 0 = always the fused kernel, 2 = two passes whatever the
  * size (dsq_gemm_workspace_bytes answers accordingly). */
 int dsq_set_gemm_two_pass(int on);
 
