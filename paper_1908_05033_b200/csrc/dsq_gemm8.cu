@@ -50,8 +50,10 @@ constexpr int G8_E_WARPS = 8;                // per CTA: two per tensor-memory l
 constexpr int G8_THREADS = 32 * (G8_WARP_E0 + G8_E_WARPS);
 constexpr int G8_BARS = 2 * G8_MAX_STAGES + 4 + 1;
 // A block of the next expansion has room beside a CTA: 1 KB of an SM's 228 is the system's for
-// each, and 40 registers for each of 256 threads are left.
+// each, and the registers of both are no more than an SM's (the expansions take 39 at most).
 constexpr int G8_SMEM = 226 * 1024, G8_REGS = 128;
+constexpr int EX_THREADS = 256, EX_BLOCKS = 4, EX_REGS = 65536 / (EX_THREADS * EX_BLOCKS);
+static_assert(G8_THREADS * G8_REGS + EX_THREADS * EX_REGS <= 65536, "a CTA and a block of the next expansion on an SM");
 constexpr int G8_TAIL = 8 * G8_BARS + 24;    // barriers, tensor-memory slot, abort flag
 constexpr int G8_STAGING = G8_E_WARPS * 32 * 32 * 4;     // a 32 x 32 block per epilogue warp
 constexpr int G8_EXCHANGE = 64 * 1024;       // sums of the other pair, at most
@@ -99,7 +101,7 @@ __device__ __forceinline__ uint32_t sign_extend_bytes(uint32_t x)
 // Launched dependently, as every kernel behind another of the library is: the first blocks
 // are on the SMs, beside the kernel ahead, when that ends (2500x1111x1777, 3-bit, among other
 // passes 14.35 -> 13.1 us, 2048x4096x4096 weight-only 69.2 -> 68.5; 4096^3 is bound by power).
-constexpr int EX_ROWS = 4, EX_THREADS = 256;
+constexpr int EX_ROWS = 4;
 
 // `BITS`-bit codes at bit 0 of a word, ascending -> one code per byte, four a word
 template <int BITS>
@@ -151,7 +153,7 @@ __device__ __forceinline__ uint2 load_chunk(const uint8_t *row, int c, int pitch
 // (BITS = 1: both -1 / +1, positions past K 0 so that a row's tail adds nothing;
 // elsewhere the codes past K are spare bits of the packed row: zero).
 template <int BITS>
-__global__ void __launch_bounds__(EX_THREADS)
+__global__ void __launch_bounds__(EX_THREADS, EX_BLOCKS)
 expand_rows_kernel(const uint8_t *__restrict__ A, const uint8_t *__restrict__ B, int M, int N, int K,
                    int pitch_in, int pitch_out, uint8_t *__restrict__ A8, uint8_t *__restrict__ B8)
 {
@@ -215,7 +217,7 @@ __device__ __forceinline__ int sum_nibbles(uint32_t x)
 // 4: a (q - 4) summed is the result less 4 sum a.  The sums of A's rows are kept for the
 // second pass, one for every 1024 codes (`sums`: [part][M]).
 template <int BITS>
-__global__ void __launch_bounds__(EX_THREADS)
+__global__ void __launch_bounds__(EX_THREADS, EX_BLOCKS)
 expand_rows_f4_kernel(const uint8_t *__restrict__ A, const uint8_t *__restrict__ B, int M, int N, int K,
                       int pitch_in, int pitch_out, uint8_t *__restrict__ A4, uint8_t *__restrict__ B4,
                       int32_t *__restrict__ sums)
@@ -286,7 +288,7 @@ expand_rows_f4_kernel(const uint8_t *__restrict__ A, const uint8_t *__restrict__
 // row.  By bit operations: the field (code ^ half) in the low mantissa bits of
 // 128.0 is 128 + field (128 + 2 field + 1), one subtraction leaves the value.
 template <int BITS>
-__global__ void __launch_bounds__(EX_THREADS)
+__global__ void __launch_bounds__(EX_THREADS, EX_BLOCKS)
 expand_w_bf16_kernel(const uint8_t *__restrict__ W, int N, int K, int pitch_in, int pitch_out, int odd,
                      uint8_t *__restrict__ W16)
 {
