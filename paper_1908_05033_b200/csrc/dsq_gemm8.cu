@@ -908,17 +908,20 @@ static bool f4_exact(int64_t K, int bits)
 static size_t f4_pitch(int64_t K) { return round_up((size_t)(K + 1) / 2, 16); }
 static int64_t f4_parts(int64_t K) { return (K + 1023) / 1024; }
 
+// clocks of the second pass
+static double pass2_clocks(int64_t M, int64_t N, int64_t K, int bits)
+{
+    return f4_exact(K, bits) ? pick_tile<G8_F4>(M, N, (K + 255) / 256).clocks
+                             : pick_tile<G8_I8>(M, N, (K + 127) / 128).clocks;
+}
+
 // Scratch the two-pass path needs behind the status words (0: the problem is
 // one the fused kernel keeps).
 size_t dsq_gemm8_scratch_bytes(int64_t M, int64_t N, int64_t K, int bits, int force)
 {
-    if (!force) {
-        if (M < 128 || N < 128 || K < 128) return 0;
-        const bool f4 = f4_exact(K, bits);
-        const double clocks = f4 ? pick_tile<G8_F4>(M, N, (K + 255) / 256).clocks
-                                 : pick_tile<G8_I8>(M, N, (K + 127) / 128).clocks;
-        if (!dsq_g8_two_passes(M, N, K, bits, f4, clocks)) return 0;
-    }
+    if (!force && (!dsq_gemm_may_take_two(M, N, K) ||
+                   !dsq_g8_two_passes(M, N, K, bits, f4_exact(K, bits), pass2_clocks(M, N, K, bits))))
+        return 0;
     const size_t kp = round_up((size_t)K, 16);             // (4-bit operands fill half of it)
     const size_t need = round_up((size_t)M * kp, 1024) + round_up((size_t)N * kp, 1024);
     if (bits != 3) return need;
@@ -927,16 +930,11 @@ size_t dsq_gemm8_scratch_bytes(int64_t M, int64_t N, int64_t K, int bits, int fo
                               (size_t)(f4_parts(K) * M) * sizeof(int32_t));
 }
 
-// What the fused kernel or the two passes, whichever is faster, are expected to take (microseconds).
-double dsq_gemm8_estimate(int64_t M, int64_t N, int64_t K, int bits)
+DsqGemmForm dsq_gemm8_form(int64_t M, int64_t N, int64_t K, int bits, int outs, bool room, bool little)
 {
-    const bool f4 = f4_exact(K, bits);
-    const bool two = M >= 128 && N >= 128 && K >= 128;
-    const double clocks = !two ? 0.0
-                          : f4 ? pick_tile<G8_F4>(M, N, (K + 255) / 256).clocks
-                               : pick_tile<G8_I8>(M, N, (K + 127) / 128).clocks;
-    const DsqGemmTimes t = dsq_gemm_times(M, N, K, bits, f4, clocks);
-    return two ? std::min(t.fused, t.two) : t.fused;
+    return dsq_gemm_form(M, N, K, bits, outs, f4_exact(K, bits),
+                         room && dsq_gemm_may_take_two(M, N, K) ? pass2_clocks(M, N, K, bits) : 0.0, room, little,
+                         dsq_sm_count() > 0 ? dsq_sm_count() : 148);
 }
 
 // 1- to 3-bit operands as 4-bit floating point where every sum stays below 2^23 (f32

@@ -112,6 +112,24 @@ inline DsqGemmSmallTile dsq_gemm_small_tile(int64_t M, int64_t N, int64_t units,
     return best;
 }
 
+// Which kernel dsq_gemm takes.  `room`: the caller's workspace holds the expanded operands; without
+// it the little-work kernel has only the fused one to be faster than (3-bit 439x592x1602: fused 13.4 us,
+// little work 7.9, two passes 8.6).  `little`: that kernel may be taken at all.
+enum DsqGemmForm { DSQ_GEMM_FUSED, DSQ_GEMM_TWO_PASSES, DSQ_GEMM_SMALL };
+inline bool dsq_gemm_may_take_two(int64_t M, int64_t N, int64_t K) { return M >= 128 && N >= 128 && K >= 128; }
+inline DsqGemmForm dsq_gemm_form(int64_t M, int64_t N, int64_t K, int bits, int outs, bool f4, double clocks, bool room,
+                                 bool little, int sms)
+{
+    const bool two = room && dsq_gemm_may_take_two(M, N, K) && dsq_g8_two_passes(M, N, K, bits, f4, clocks);
+    // (up to what its estimate was fitted to, and the rows of a grid)
+    if (little && (double)M * (double)N * (double)K < 1e9 && (M + 15) / 16 <= 65535) {
+        const int64_t units = bits == 2 ? (K + 63) / 64 : (K + 31) / 32;
+        const DsqGemmTimes t = dsq_gemm_times(M, N, K, bits, f4, clocks);
+        if (dsq_gemm_small_tile(M, N, units, bits, outs, sms).us <= (two ? t.two : t.fused)) return DSQ_GEMM_SMALL;
+    }
+    return two ? DSQ_GEMM_TWO_PASSES : DSQ_GEMM_FUSED;
+}
+
 // Columns of a block of the weight-only GEMM of few rows, for more than 32 rows (64 a block): 32
 // take up to 1.5 times as long as 16, which pays where it saves a wave.  16 / 32 columns, us: 64x4096x4096 4-bit
 // 22.8 / 15.4, 150x1500x1000 8.2 / 6.0, 332x659x1136 9.5 / 8.0, 128x1024x1024 (one wave of either) 4.6 / 6.0.

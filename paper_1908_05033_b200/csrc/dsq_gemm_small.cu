@@ -177,7 +177,7 @@ int pick(const GsParams &p, const DsqGemmSmallTile &t, cudaStream_t s)
 }  // namespace
 
 int dsq_gemm_small(const void *A_codes, const void *B_codes, int64_t M, int64_t N, int64_t K, int bits,
-                   int32_t *C_i32, const float *row_scale, float *D_f32, double other_us, cudaStream_t stream)
+                   int32_t *C_i32, const float *row_scale, float *D_f32, cudaStream_t stream)
 {
     GsParams p = {};
     p.A = (const uint8_t *)A_codes;
@@ -188,10 +188,8 @@ int dsq_gemm_small(const void *A_codes, const void *B_codes, int64_t M, int64_t 
     p.shift = 8 - bits;
     p.wide = N % 2 == 0;                               // (outputs are 16-byte aligned)
     p.C_i32 = C_i32; p.row_scale = row_scale; p.D_f32 = D_f32;
-    if ((M + 15) / 16 > 65535) return DSQ_ERR_UNSUPPORTED;
     const DsqGemmSmallTile t = dsq_gemm_small_tile(M, N, p.units, bits, (C_i32 ? 1 : 0) + (D_f32 ? 1 : 0),
                                                    dsq_sm_count() > 0 ? dsq_sm_count() : 148);
-    if (t.us > other_us) return DSQ_ERR_UNSUPPORTED;
     switch (bits) {
     case 2: return pick<2>(p, t, stream);
     case 3: return pick<3>(p, t, stream);

@@ -1747,27 +1747,21 @@ int dsq_gemm(const void *A_codes, const void *B_codes, int64_t M, int64_t N, int
     if (!dsq_aligned16(workspace)) return DSQ_ERR_ALIGN;
     if (ws_bytes < DSQ_WS_BYTES) return DSQ_ERR_SIZE;
 
-    // little work: a latency-bound kernel of its own (the hooks force the others; up to what its
-    // rule was fitted to)
+    // One of three kernels: this one; where the caller's workspace has room for the expanded
+    // operands (dsq_gemm_workspace_bytes) two passes that expand every row once and feed an 8-bit
+    // GEMM by TMA alone; with little work, a latency-bound one (the hooks force the others).
     const int two_pass = g_two_pass.load();
-    if (two_pass == 1 && (double)M * (double)N * (double)K < 1e9 && !g_forced_bn.load() && !g_forced_ks.load() &&
-        !g_pair_mode.load() && g_skip_b_round.load() < 0) {
-        st = dsq_gemm_small(A_codes, B_codes, M, N, K, bits, C_i32, row_scale, D_f32,
-                            dsq_gemm8_estimate(M, N, K, bits), (cudaStream_t)stream);
-        if (st != DSQ_ERR_UNSUPPORTED) return st;
-    }
-    // large problems, when the caller's workspace has room for the expanded
-    // operands (dsq_gemm_workspace_bytes): expand every row once, then an
-    // 8-bit GEMM fed by TMA alone
-    const size_t scratch_need = two_pass ? dsq_gemm8_scratch_bytes(M, N, K, bits, two_pass == 2) : 0;
-    if (scratch_need) {
-        const uintptr_t w0 = reinterpret_cast<uintptr_t>(workspace);
-        const uintptr_t s0 = (w0 + DSQ_WS_BYTES + 1023u) & ~(uintptr_t)1023u;
-        if (ws_bytes >= (s0 - w0) + scratch_need)
-            return dsq_gemm8_launch(A_codes, B_codes, M, N, K, bits, C_i32, row_scale, D_f32,
-                                    workspace, reinterpret_cast<void *>(s0),
-                                    (cudaStream_t)stream);
-    }
+    const uintptr_t w0 = reinterpret_cast<uintptr_t>(workspace);
+    const uintptr_t s0 = (w0 + DSQ_WS_BYTES + 1023u) & ~(uintptr_t)1023u;
+    const bool room = two_pass && ws_bytes >= (s0 - w0) + dsq_gemm8_scratch_bytes(M, N, K, bits, 1);
+    const bool little = !g_forced_bn.load() && !g_forced_ks.load() && !g_pair_mode.load() && g_skip_b_round.load() < 0;
+    const DsqGemmForm form = two_pass != 1 ? (room ? DSQ_GEMM_TWO_PASSES : DSQ_GEMM_FUSED)
+                                           : dsq_gemm8_form(M, N, K, bits, (C_i32 ? 1 : 0) + (D_f32 ? 1 : 0), room, little);
+    if (form == DSQ_GEMM_SMALL)
+        return dsq_gemm_small(A_codes, B_codes, M, N, K, bits, C_i32, row_scale, D_f32, (cudaStream_t)stream);
+    if (form == DSQ_GEMM_TWO_PASSES)
+        return dsq_gemm8_launch(A_codes, B_codes, M, N, K, bits, C_i32, row_scale, D_f32, workspace,
+                                reinterpret_cast<void *>(s0), (cudaStream_t)stream);
 
     const size_t pitch = dsq_row_pitch(K, bits);
     TcParams p = {};

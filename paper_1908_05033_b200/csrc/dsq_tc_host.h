@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include "dsq_epilogue.cuh"
+#include "dsq_gemm8_rule.h"
 #include "dsq_launch.h"
 
 typedef CUresult (*DsqEncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
@@ -67,19 +68,19 @@ static inline int dsq_allow_smem(const void *func, int bytes, std::atomic<unsign
 // force: whatever the size).
 // dsq_gemm8_launch: arguments as dsq_gemm after validation, `scratch`
 // 1024-byte aligned and at least that large.
-// dsq_gemm8_estimate: microseconds of that or the fused kernel, whichever is expected to be faster.
-DSQ_HIDDEN double dsq_gemm8_estimate(int64_t M, int64_t N, int64_t K, int bits);
+// dsq_gemm8_form: the kernel that dsq_gemm takes (dsq_gemm8_rule.h), outs: arrays written.
+DSQ_HIDDEN DsqGemmForm dsq_gemm8_form(int64_t M, int64_t N, int64_t K, int bits, int outs, bool room, bool little);
 DSQ_HIDDEN size_t dsq_gemm8_scratch_bytes(int64_t M, int64_t N, int64_t K, int bits, int force);
 DSQ_HIDDEN int dsq_gemm8_launch(const void *A_codes, const void *B_codes, int64_t M, int64_t N,
                                 int64_t K, int bits, int32_t *C_i32, const float *row_scale,
                                 float *D_f32, void *workspace, void *scratch,
                                 cudaStream_t stream);
 
-// GEMM with little work (dsq_gemm_small.cu): arguments as dsq_gemm after validation; no workspace.
-// DSQ_ERR_UNSUPPORTED where it is expected to take longer than other_us.
+// GEMM with little work (dsq_gemm_small.cu): arguments as dsq_gemm after validation, of problems that
+// dsq_gemm8_form gives it; no workspace.
 DSQ_HIDDEN int dsq_gemm_small(const void *A_codes, const void *B_codes, int64_t M, int64_t N, int64_t K,
                               int bits, int32_t *C_i32, const float *row_scale, float *D_f32,
-                              double other_us, cudaStream_t stream);
+                              cudaStream_t stream);
 
 // Weight-only GEMM for few rows (dsq_wgemm_small.cu): arguments as dsq_wgemm_bf16
 // after validation; no workspace.
