@@ -85,29 +85,41 @@ inline bool dsq_g8_two_passes(int64_t M, int64_t N, int64_t K, int bits, bool f4
 }
 
 // The GEMM with little work (dsq_gemm_small.cu): 16 mt rows x 32 columns a block of `warps` warps, and the
-// microseconds it is expected to take: the longer of a block's chain (its chunks of K a warp)
-// and what the blocks of an SM take together, with the outputs.  units: of a packed row; outs:
-// arrays written.
-// Fitted to 760 problems of 16 to 6144 a side and up to 1.3e9 multiply-accumulates, one or both
-// outputs (11 % off in the mean); of those, with the estimates of the other kernels, 2.0 % slower than the
-// fastest of all on average, 4 more than 3 % slower than the fused kernel or the two passes
-// (without it 1.8 times as long).
+// microseconds it is expected to take.  units: of a packed row; outs: arrays written.
+// An SM holds as many blocks as their registers allow, and each round of them takes a block's chain
+// (its launch, its chunks of K a warp) and what they do beside each other; the outputs come on top.
+// 32 rows a block expand B's rows half as often, at more registers, us with 16 / 32 rows: 3-bit 2177x35x2843
+// 7.4 / 5.3, 4-bit 150x2024x1052 4.9 / 3.9, 4-bit 512^3, one round of either, 2.3 / 2.9.  They count a tenth
+// more than they are expected to take: where it is close, 16 rows are as good or better.
+// Fitted to 1079 problems of 16 to 6144 a side and up to 1.5e9 multiply-accumulates, one or both outputs
+// (8 % off in the mean).  Of 541 others what is taken, among these and the other kernels, is 1.2 %
+// slower than the fastest on average (2.7 % with blocks of 16 rows alone and none above 1e9).
 struct DsqGemmSmallTile { int mt, warps; double us; };
 inline DsqGemmSmallTile dsq_gemm_small_tile(int64_t M, int64_t N, int64_t units, int bits, int outs, int sms)
 {
+    // blocks of four warps that an SM holds; a warp's time for a chunk; an SM's for a block and for a
+    // chunk of one: [mt - 1][bits - 2] and with four and eight warps
+    static const int held[2][3] = {{4, 3, 4}, {3, 2, 3}};
+    static const double walk[2][3] = {{0.103, 0.153, 0.075}, {0.445, 0.338, 0.249}};
+    static const double block[2][3][2] = {{{0.0, 0.128}, {0.023, 0.273}, {0.0, 0.088}},
+                                          {{0.107, 0.129}, {0.347, 0.314}, {0.149, 0.102}}};
+    static const double chunk[2][3][2] = {{{0.066, 0.061}, {0.080, 0.086}, {0.035, 0.035}},
+                                          {{0.076, 0.075}, {0.090, 0.107}, {0.037, 0.040}}};
     const int64_t chunks = (units + 3) / 4;
-    // (instructions a chunk: a 2-bit unit is twice the codes, 3-bit fields take more of them)
-    const double f = bits == 4 ? 1.0 : bits == 3 ? 2.5 : 1.95, chain_f = bits == 4 ? 1.0 : bits == 3 ? 2.0 : 1.67;
     DsqGemmSmallTile best = {0, 0, 0.0};
     for (int mt = 1; mt <= 2; ++mt)
-        for (int warps = 4; warps <= 8; warps *= 2) {
-            const double blocks = (double)((M + 16 * mt - 1) / (16 * mt)) * (double)((N + 31) / 32);
-            const double chain = 1.68 + 0.023 * warps + (mt == 1 ? 0.33 : 0.51) * chain_f * (double)((chunks + warps - 1) / warps);
-            const double fixed = mt == 1 ? (warps == 4 ? 0.21 : 0.57) : (warps == 4 ? 0.5 : 1.29);
-            const double all = 1.2 + blocks / sms * (fixed + (mt == 1 ? 0.052 : 0.104) * f * (double)chunks) +
-                               0.82e-6 * (double)M * (double)N * outs;
-            const double us = std::max(chain, all);
-            if (best.mt == 0 || us < best.us) best = DsqGemmSmallTile{mt, warps, us};
+        for (int eight = 0; eight < 2; ++eight) {
+            const int warps = 4 + 4 * eight, a = mt - 1, b = bits - 2;
+            const int64_t blocks = (M + 16 * mt - 1) / (16 * mt) * ((N + 31) / 32);
+            const int64_t most = held[a][b] / (1 + eight), rounds = blocks / (most * sms);
+            const int64_t rest = (blocks - rounds * most * sms + sms - 1) / sms;
+            const double chain = 0.731 + walk[a][b] * (double)((chunks + warps - 1) / warps);
+            const double beside = block[a][b][eight] + chunk[a][b][eight] * (double)chunks;
+            const double us = 0.867 + (double)rounds * (chain + (double)most * beside) +
+                              (rest ? chain + (double)rest * beside : 0.0) +
+                              (N % 2 ? 1.248e-6 : 1.079e-6) * (double)M * (double)N * outs;
+            const double counted = mt == 2 ? 1.1 * us : us;
+            if (best.mt == 0 || counted < best.us) best = DsqGemmSmallTile{mt, warps, counted};
         }
     return best;
 }
@@ -122,7 +134,7 @@ inline DsqGemmForm dsq_gemm_form(int64_t M, int64_t N, int64_t K, int bits, int 
 {
     const bool two = room && dsq_gemm_may_take_two(M, N, K) && dsq_g8_two_passes(M, N, K, bits, f4, clocks);
     // (up to what its estimate was fitted to, and the rows of a grid)
-    if (little && (double)M * (double)N * (double)K < 1e9 && (M + 15) / 16 <= 65535) {
+    if (little && (double)M * (double)N * (double)K < 1.5e9 && (M + 15) / 16 <= 65535) {
         const int64_t units = bits == 2 ? (K + 63) / 64 : (K + 31) / 32;
         const DsqGemmTimes t = dsq_gemm_times(M, N, K, bits, f4, clocks);
         if (dsq_gemm_small_tile(M, N, units, bits, outs, sms).us <= (two ? t.two : t.fused)) return DSQ_GEMM_SMALL;

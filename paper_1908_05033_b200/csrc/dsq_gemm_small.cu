@@ -9,8 +9,8 @@
 //     their sums in shared memory in a fixed order;
 //   * every lane takes its packed words straight from global memory to the fragments of mma.sync
 //     m16n8k32 (s8 x u8) in registers, the next chunk's before this one's arithmetic.
-// Microseconds in a graph, the faster of the others / this: 4-bit 256^3 3.5 / 1.8, 512^3 4.0 / 2.5,
-// 200x200x4000 10.3 / 3.2; 2-bit 512^3 4.6 / 2.5; 3-bit 5.9 / 4.3, 1024^3 8.7 / 7.8.
+// Microseconds in a graph, the faster of the others / this: 4-bit 256^3 3.3 / 1.6, 512^3 3.9 / 2.3,
+// 200x200x4000 9.6 / 3.1; 2-bit 512^3 4.4 / 2.3; 3-bit 5.7 / 3.4, but 1024^3 7.6 / 15.4.
 // Bound: two to four dependent round trips to memory, and beyond about 0.5 G
 // multiply-accumulates the expansion of both operands once per tile, which is why larger
 // problems go elsewhere (dsq_gemm8_rule.h).

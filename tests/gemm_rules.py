@@ -13,6 +13,7 @@ class Rules:
         lib = self.lib = C.CDLL(so)
         lib.tile.restype = C.c_double
         lib.tile.argtypes = [C.c_int64] * 3 + [C.c_int] + [C.POINTER(C.c_int)] * 2
+        lib.gemm_small.argtypes = [C.c_int64] * 3 + [C.c_int] * 2 + [C.POINTER(C.c_int)] * 2
         lib.gemm_form.argtypes = [C.c_int64] * 3 + [C.c_int] * 2 + [C.c_double, C.c_int]
 
     def tile(self, operands, m, n, k):
@@ -26,6 +27,12 @@ class Rules:
         """Of dsq_gemm with `outs` arrays written: "fused", "two" passes or "small"."""
         _, clocks = self.tile("i8" if bits == 4 else "f4", m, n, k)
         return ("fused", "two", "small")[self.lib.gemm_form(m, n, k, bits, outs, clocks, room)]
+
+    def gemm_small(self, m, n, k, bits, outs):
+        """(rows, warps) of a block of the little-work kernel."""
+        rows, warps = C.c_int(), C.c_int()
+        self.lib.gemm_small(m, n, k, bits, outs, C.byref(rows), C.byref(warps))
+        return rows.value, warps.value
 
 
 @pytest.fixture(scope="session")

@@ -7,4 +7,11 @@ int gemm_form(int64_t M, int64_t N, int64_t K, int bits, int outs, double clocks
 {
     return dsq_gemm_form(M, N, K, bits, outs, bits != 4, clocks, room != 0, true, 148);
 }
+// rows and warps of a block of the little-work kernel
+void gemm_small(int64_t M, int64_t N, int64_t K, int bits, int outs, int *rows, int *warps)
+{
+    const DsqGemmSmallTile t = dsq_gemm_small_tile(M, N, bits == 2 ? (K + 63) / 64 : (K + 31) / 32, bits, outs, 148);
+    *rows = 16 * t.mt;
+    *warps = t.warps;
+}
 }
