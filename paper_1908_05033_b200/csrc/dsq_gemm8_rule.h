@@ -142,9 +142,10 @@ inline DsqGemmForm dsq_gemm_form(int64_t M, int64_t N, int64_t K, int bits, int 
     return two ? DSQ_GEMM_TWO_PASSES : DSQ_GEMM_FUSED;
 }
 
-// Columns of a block of the weight-only GEMM of few rows, for more than 32 rows (64 a block): 32
-// take up to 1.5 times as long as 16, which pays where it saves a wave.  16 / 32 columns, us: 64x4096x4096 4-bit
-// 22.8 / 15.4, 150x1500x1000 8.2 / 6.0, 332x659x1136 9.5 / 8.0, 128x1024x1024 (one wave of either) 4.6 / 6.0.
+// The weight-only GEMM of few rows (dsq_wgemm_small.cu) for more than 32 rows: waves of blocks of 64 rows x 16
+// or 32 columns, 2.6 us for every 1024 of K, three quarters of that at 33 rows; 32 columns take up to 1.5
+// times as long, which pays where it saves a wave.  16 / 32 columns, us, 4-bit: 64x4096x4096
+// 23.1 / 15.9, 150x1500x1000 8.1 / 6.3, 332x659x1136 9.4 / 7.8, 128x1024x1024 (one wave of either) 4.6 / 6.3.
 inline double dsq_wgemm_small_waves(int64_t M, int64_t N, int sms, int columns)
 {
     return std::ceil((double)((N + columns - 1) / columns) * (double)((M + 63) / 64) / sms) * (columns == 32 ? 1.5 : 1.0);
@@ -153,30 +154,29 @@ inline int dsq_wgemm_small_columns(int64_t M, int64_t N, int sms)
 {
     return dsq_wgemm_small_waves(M, N, sms, 32) < dsq_wgemm_small_waves(M, N, sms, 16) ? 32 : 16;
 }
-
-// Whether the weight-only GEMM of few rows does better than two passes of `clocks` in the
-// second, for more than 32 rows (up to those it always does: 4096x4096 4-bit 9.2 us): while its
-// launch - waves of blocks of 64 x 16 outputs, 2.6 us for every 1024 of K, three quarters of that at 33
-// rows - is shorter than the two passes, whose time is fitted to 363 problems of 33 to 700 rows (6 % off in the
-// mean; the rule takes the slower kernel for 17 of them, 0.6 % of time on average).  64
-// rows, this kernel / two passes, us: 4096x4096 23.5 / 20.2, 6144x6144 48.5 / 35.5, 6144x1024 13.0 / 12.6,
-// 1500x2000 7.6 / 13.
-inline bool dsq_wgemm_takes_small(int64_t M, int64_t N, int64_t K, int sms, double clocks)
+inline double dsq_wgemm_small_us(int64_t M, int64_t N, int64_t K, int sms, int columns)
 {
-    const double blocks = (double)((N + 15) / 16) * (double)((M + 63) / 64);
     const double rows = M < 64 ? 0.75 + 0.25 / 31.0 * (double)(M - 33) : 1.0;
-    const double small = 2.2 + std::ceil(blocks / sms) * (double)((K + 1023) / 1024) * 2.6 * rows;
-    return small < 5.5 + 3.2e-7 * (double)N * (double)K + 5.22e-4 * clocks;
+    return 2.2 + dsq_wgemm_small_waves(M, N, sms, columns) * (double)((K + 1023) / 1024) * 2.6 * rows;
+}
+// And two passes, of `clocks` in the second.
+inline double dsq_wgemm_two_us(int64_t N, int64_t K, double clocks)
+{
+    return 5.0 + 3.2e-7 * (double)N * (double)K + 5.22e-4 * clocks;
 }
 
-// The same of its blocks of 32 columns, where they are the better ones: also taken where only they
-// beat the two passes.  Over 300
-// problems of 33 to 1200 rows 0.8 % slower than the fastest of the three on average, 12 more than 5 %
-// (4.1 % with blocks of 16 alone).
+// Whether it does better than two passes, for more than 32 rows (up to those it always does:
+// 4096x4096 4-bit 9.2 us): in blocks of 16 columns, or where those of 32 are the better ones and
+// only they beat the two passes.  Of 360 problems of 33 to 1200 rows, 1 to 4 bits, what is taken is 1.0 % slower
+// than the fastest of the three on average, 22 of them by more than 5 % (1.1 % and 24 with 5.5 us in place of 5.0 for blocks of
+// 16 columns, fitted before the expansion was a dependent launch).  64 rows, 16 columns / 32 / two passes, us, 4-bit:
+// 4096x4096 23.1 / 15.9 / 19.8, 6144x6144 47.8 / 41.8 / 34.8, 6144x1024 12.0 / 11.8 / 11.2, 1500x2000 7.0 / 9.0 / 11.5.
+inline bool dsq_wgemm_takes_small(int64_t M, int64_t N, int64_t K, int sms, double clocks)
+{
+    return dsq_wgemm_small_us(M, N, K, sms, 16) < dsq_wgemm_two_us(N, K, clocks);
+}
 inline bool dsq_wgemm_takes_wide(int64_t M, int64_t N, int64_t K, int sms, double clocks)
 {
-    if (dsq_wgemm_small_columns(M, N, sms) != 32) return false;
-    const double rows = M < 64 ? 0.75 + 0.25 / 31.0 * (double)(M - 33) : 1.0;
-    const double wide = 2.2 + dsq_wgemm_small_waves(M, N, sms, 32) * (double)((K + 1023) / 1024) * 2.6 * rows;
-    return wide < 5.0 + 3.2e-7 * (double)N * (double)K + 5.22e-4 * clocks;
+    return dsq_wgemm_small_columns(M, N, sms) == 32 &&
+           dsq_wgemm_small_us(M, N, K, sms, 32) < dsq_wgemm_two_us(N, K, clocks);
 }

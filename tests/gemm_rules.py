@@ -13,6 +13,7 @@ class Rules:
         lib = self.lib = C.CDLL(so)
         lib.tile.restype = C.c_double
         lib.tile.argtypes = [C.c_int64] * 3 + [C.c_int] + [C.POINTER(C.c_int)] * 2
+        lib.wgemm_form.argtypes = [C.c_int64] * 3 + [C.c_double]
         lib.gemm_small.argtypes = [C.c_int64] * 3 + [C.c_int] * 2 + [C.POINTER(C.c_int)] * 2
         lib.gemm_form.argtypes = [C.c_int64] * 3 + [C.c_int] * 2 + [C.c_double, C.c_int]
 
@@ -33,6 +34,10 @@ class Rules:
         rows, warps = C.c_int(), C.c_int()
         self.lib.gemm_small(m, n, k, bits, outs, C.byref(rows), C.byref(warps))
         return rows.value, warps.value
+
+    def wgemm_form(self, m, n, k):
+        """Of a weight-only GEMM of more than 32 rows: columns of a block of the kernel of few rows, 0: two passes."""
+        return self.lib.wgemm_form(m, n, k, self.tile("bf16", m, n, k)[1])
 
 
 @pytest.fixture(scope="session")

@@ -14,4 +14,10 @@ void gemm_small(int64_t M, int64_t N, int64_t K, int bits, int outs, int *rows, 
     *rows = 16 * t.mt;
     *warps = t.warps;
 }
+// columns of a block of the weight-only kernel of few rows, 0: two passes
+int wgemm_form(int64_t M, int64_t N, int64_t K, double clocks)
+{
+    if (!dsq_wgemm_takes_small(M, N, K, 148, clocks) && !dsq_wgemm_takes_wide(M, N, K, 148, clocks)) return 0;
+    return dsq_wgemm_small_columns(M, N, 148);
+}
 }
