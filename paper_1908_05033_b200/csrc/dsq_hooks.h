@@ -23,10 +23,14 @@ int dsq_set_round_k_steps(int ks);
  * cta_group::2): 0 automatic, 1 never, 2 wherever the shapes allow. */
 int dsq_set_cta_pairs(int mode);
 
-/* Programmatic dependent launch of the tensor-core kernels (default 1): the
- * kernel's set-up may overlap the tail of the previous kernel of the stream;
- * it waits for that kernel (griddepcontrol.wait) before touching global
- * memory.  0 = plain launches. */
+/* Programmatic dependent launch (default 1): a kernel's set-up may overlap the
+ * tail of the previous kernel of the stream; it waits for that kernel
+ * (griddepcontrol.wait) before it touches what that one may read or write, and
+ * lets the next one start only behind that wait.  Ahead of it, layers of a plan
+ * read their constants (dsq_early_constants), and the soft quantiser's backward
+ * kernel its inputs and writes its gradient: what is in front of that one is always
+ * the kernel, or the memset, that clears its sums, and nothing else.  0 = plain
+ * launches. */
 int dsq_set_dependent_launch(int on);
 
 /* Limit of every device-side barrier wait in nanoseconds (default 2 s; 0

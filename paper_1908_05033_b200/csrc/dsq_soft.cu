@@ -137,10 +137,15 @@ __device__ __forceinline__ float soft_bwd_one(float x, float g, const SoftP &p, 
     return x != x ? x : gx;
 }
 
+// Calls of fewer elements have their sums cleared by a memset, outside graphs: the GPU is through
+// with them before the host has enqueued the next, so that the launch that costs the host least is the
+// better one.  Forward and backward one after the other, memset / kernel, us: 21758 elements 10.4 / 11.3,
+// 600000 10.7 / 11.3, 1000000 12.2 / 11.4 (with the hosts of these GPUs; a slower one moves the line up).
 constexpr int64_t SOFT_SMALL = 3 << 18;
 
 // Clears the three sums.  The backward kernel, launched dependently behind it, starts when
-// everything ahead of this one has completed and waits for it only before it adds to the sums.
+// everything ahead of this one has completed (it waits for that before it lets the next one start) and
+// waits for it only before it adds to the sums: until then it reads x and dL/dy and writes dL/dx.
 // With a memset in front, 16384 / 1M / 12.8M elements took 6.2 / 7.7 / 29.2 us in a graph, so 2.7 / 4.5 / 26.7
 // (forward and backward 8.4 / 10.7 / 48.8 -> 4.3 / 7.0 / 44.4).
 __global__ void soft_clear_kernel(double *sums)
@@ -289,10 +294,7 @@ extern "C" int dsq_soft_quantize_bwd(const float *x, const float *grad_y, int64_
         return DSQ_ERR_ALIGN;
     cudaStream_t s = (cudaStream_t)stream;
     const int pdl = dsq_launch_hooks().pdl;
-    // A memset takes 0.7 us less of the host than a launch: it clears the sums of calls that the
-    // GPU is through with before the host has enqueued the next (forward and backward of 21758
-    // elements one after the other 10.4 us with it, 11.3 without; 600000 10.7 / 11.3, 1M 12.2 / 11.4).  In a
-    // graph the host does not matter.
+    // (a memset takes 0.7 us less of the host than a launch; in a graph the host does not matter)
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (n < SOFT_SMALL && !dsq_recording_plan() && cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
         DSQ_CUDA_TRY(cudaMemsetAsync(grad_params, 0, 3 * sizeof(double), s));
