@@ -13,6 +13,7 @@ class Rules:
         lib = self.lib = C.CDLL(so)
         lib.tile.restype = C.c_double
         lib.tile.argtypes = [C.c_int64] * 3 + [C.c_int] + [C.POINTER(C.c_int)] * 2
+        lib.two_passes.argtypes = [C.c_int64] * 3 + [C.c_int] * 2 + [C.c_double]
         lib.wgemm_form.argtypes = [C.c_int64] * 3 + [C.c_double]
         lib.gemm_small.argtypes = [C.c_int64] * 3 + [C.c_int] * 2 + [C.POINTER(C.c_int)] * 2
         lib.gemm_form.argtypes = [C.c_int64] * 3 + [C.c_int] * 2 + [C.c_double, C.c_int]
@@ -28,6 +29,9 @@ class Rules:
         """Of dsq_gemm with `outs` arrays written: "fused", "two" passes or "small"."""
         _, clocks = self.tile("i8" if bits == 4 else "f4", m, n, k)
         return ("fused", "two", "small")[self.lib.gemm_form(m, n, k, bits, outs, clocks, room)]
+
+    def two_passes(self, m, n, k, bits, f4, clocks):
+        return self.lib.two_passes(m, n, k, bits, f4, clocks)
 
     def gemm_small(self, m, n, k, bits, outs):
         """(rows, warps) of a block of the little-work kernel."""

@@ -34,3 +34,16 @@ def test_little_work_blocks(rules, m, n, k, bits, outs, other, a, b, c, d):
     taken = rules.gemm_form(m, n, k, bits, outs, True)
     assert (taken == "small") == (min(times.values()) < other)
     assert times[rules.gemm_small(m, n, k, bits, outs)] <= 1.04 * min(times.values())
+
+
+# M, N, K, the fused kernel's time, two passes' (operands as 4-bit floating point): 3-bit codes
+PASSES = [(2558, 248, 210, 6.3, 6.7), (3015, 1420, 184, 9.7, 11.8), (427, 1516, 265, 6.4, 7.1), (625, 2288, 147, 6.8, 7.7),
+          (4505, 140, 381, 6.0, 7.8), (1039, 848, 322, 6.4, 7.3), (188, 356, 284, 5.4, 7.8), (254, 336, 1271, 10.1, 6.9),
+          (193, 735, 1316, 13.9, 8.7), (145, 1377, 2038, 15.5, 7.8), (473, 273, 505, 7.1, 6.5), (2982, 136, 1471, 11.8, 8.9),
+          (2400, 1114, 2702, 57.7, 17.5), (2286, 428, 3731, 23.9, 12.6), (2497, 1287, 171, 42.7, 15.4)]
+
+
+@pytest.mark.parametrize("m,n,k,fused,two", PASSES)
+def test_three_bits_in_two_passes(rules, m, n, k, fused, two):
+    _, clocks = rules.tile("f4", m, n, k)
+    assert bool(rules.two_passes(m, n, k, 3, True, clocks)) == (two < fused)
