@@ -350,7 +350,7 @@ inline dim3 expand_grid(int64_t chunks, int64_t rows)
 }
 
 // ---------------------------------------------------------------------------
-// pass 2: int8 GEMM, CTA pairs
+// pass 2: GEMM of the expanded rows, CTA pairs
 // ---------------------------------------------------------------------------
 // Integer and scaled outputs of an accumulator (f32 ones of 4-bit operands: `more` and the sum
 // are whole numbers below 2^24).
