@@ -162,14 +162,16 @@ inline double dsq_wgemm_small_us(int64_t M, int64_t N, int64_t K, int sms, int c
 // And two passes, of `clocks` in the second.
 inline double dsq_wgemm_two_us(int64_t N, int64_t K, double clocks)
 {
-    return 5.0 + 3.2e-7 * (double)N * (double)K + 5.22e-4 * clocks;
+    return 5.5 + 3.2e-7 * (double)N * (double)K + 5.22e-4 * clocks;
 }
 
 // Whether it does better than two passes, for more than 32 rows (up to those it always does:
 // 4096x4096 4-bit 9.2 us): in blocks of 16 columns, or where those of 32 are the better ones and
 // only they beat the two passes.  Of 360 problems of 33 to 1200 rows, 1 to 4 bits, what is taken is 1.0 % slower
-// than the fastest of the three on average, 22 of them by more than 5 % (1.1 % and 24 with 5.5 us in place of 5.0 for blocks of
-// 16 columns, fitted before the expansion was a dependent launch).  64 rows, 16 columns / 32 / two passes, us, 4-bit:
+// than the fastest of the three on average, 23 of them by more than 5 %.  (With 5.0 us of launches in
+// place of 5.5 the same, and 22; but where it is close the kernel of few rows is the better one: its sums are closer to
+// those in 64 bits, 5e-8 of the result against 5e-8 to 1e-7 in two passes at K = 2000, 1e-7 / 3e-7 at
+// 5848.)  64 rows, 16 columns / 32 / two passes, us, 4-bit:
 // 4096x4096 23.1 / 15.9 / 19.8, 6144x6144 47.8 / 41.8 / 34.8, 6144x1024 12.0 / 11.8 / 11.2, 1500x2000 7.0 / 9.0 / 11.5.
 inline bool dsq_wgemm_takes_small(int64_t M, int64_t N, int64_t K, int sms, double clocks)
 {

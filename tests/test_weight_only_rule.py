@@ -11,7 +11,7 @@ FORMS = [(208, 2556, 1600, 24.0, 19.8, 12.5), (271, 2718, 3936, 66.6, 42.6, 21.2
          (56, 1287, 1272, 5.6, 7.8, 9.7), (37, 951, 5912, 12.3, 18.8, 18.0), (36, 1956, 656, 3.7, 4.9, 9.2),
          (126, 1613, 1304, 10.0, 8.2, 11.2), (61, 3199, 5848, 29.6, 20.8, 23.8), (41, 4550, 4520, 19.9, 16.1, 26.2),
          (489, 519, 2024, 13.1, 9.6, 10.9), (36, 3017, 2056, 11.2, 8.9, 15.6), (35, 3427, 1120, 8.3, 6.7, 14.3),
-         (162, 903, 1208, 7.8, 7.2, 10.5)]
+         (162, 903, 1208, 7.8, 7.2, 10.5), (148, 1332, 3024, 18.2, 11.9, 13.3)]
 
 
 @pytest.mark.parametrize("m,n,k,narrow,wide,two", FORMS)
