@@ -38,8 +38,8 @@ import dsq_inputs  # noqa: E402
 # DRAM traffic of the tensor-core convolution kernels per launch in this
 # workload, from one ncu capture (profiles/bench_launch_list.txt); valid only
 # for the kernel sources it was taken on (checked by hash)
-TRAFFIC = {"bytes_per_launch": 4973736,
-           "sources_sha256": "08272f632e3587a8d9853bb29bcc5648e04714737da03d20ebfaae7420af527a"}
+TRAFFIC = {"bytes_per_launch": 4973251,
+           "sources_sha256": "a94d6f7e27938f42a1422103c9cbcb9fc4c5459da1c8c7efbda7cc1d6842af45"}
 
 WORKLOAD = "resnet18-shaped stack, 4-bit W/A, batch 64, 56x56x64 stem output, 19 convs"
 METRIC = "4-bit ResNet-18 conv-stack throughput (effective low-bit conv TOPS alongside)"
