@@ -50,12 +50,13 @@ constexpr int G8_E_WARPS = 8;                // per CTA: two per tensor-memory l
 constexpr int G8_THREADS = 32 * (G8_WARP_E0 + G8_E_WARPS);
 constexpr int G8_BARS = 2 * G8_MAX_STAGES + 4 + 1;
 // A block of the next expansion has room beside a CTA: 1 KB of an SM's 228 is the system's for
-// each, and the registers of both are no more than an SM's.  The expansions take 32 a thread, eight
-// blocks an SM (that of 3-bit codes to floating point, which also sums: with 37, six blocks, 2500x1111x1777
-// takes 12.35 us, with 39 12.2, with 48 12.05, so 11.9).
+// each, and the CTA leaves 64 registers a thread for it.  The expansions are bound to 32, eight blocks an
+// SM, which is what they take; the one that also sums rows of 3-bit codes takes 39 and is left unbound: with 32 and with
+// 48 some problems gain 3 to 6 % and others lose 2 to 4 (us with 32 / 39 / 48: 400x2000x4000 13.4 / 12.8 / 12.2,
+// 3394x232x1376 9.0 / 8.9 / 9.2, 1500x1304x1033 9.5 / 9.2 / 9.0, 3001x2001x700 15.0 / 15.5 / 15.5).
 constexpr int G8_SMEM = 226 * 1024, G8_REGS = 128;
-constexpr int EX_THREADS = 256, EX_BLOCKS = 8;
-static_assert(G8_THREADS * G8_REGS + 65536 / EX_BLOCKS <= 65536, "a CTA and a block of the next expansion on an SM");
+constexpr int EX_THREADS = 256, EX_BLOCKS = 8, EX_REGS = 64;
+static_assert(G8_THREADS * G8_REGS + EX_THREADS * EX_REGS <= 65536, "a CTA and a block of the next expansion on an SM");
 constexpr int G8_TAIL = 8 * G8_BARS + 24;    // barriers, tensor-memory slot, abort flag
 constexpr int G8_STAGING = G8_E_WARPS * 32 * 32 * 4;     // a 32 x 32 block per epilogue warp
 constexpr int G8_EXCHANGE = 64 * 1024;       // sums of the other pair, at most
@@ -219,7 +220,7 @@ __device__ __forceinline__ int sum_nibbles(uint32_t x)
 // 4: a (q - 4) summed is the result less 4 sum a.  The sums of A's rows are kept for the
 // second pass, one for every 1024 codes (`sums`: [part][M]).
 template <int BITS>
-__global__ void __launch_bounds__(EX_THREADS, EX_BLOCKS)
+__global__ void __launch_bounds__(EX_THREADS, BITS == 3 ? 0 : EX_BLOCKS)
 expand_rows_f4_kernel(const uint8_t *__restrict__ A, const uint8_t *__restrict__ B, int M, int N, int K,
                       int pitch_in, int pitch_out, uint8_t *__restrict__ A4, uint8_t *__restrict__ B4,
                       int32_t *__restrict__ sums)
